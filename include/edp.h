@@ -29,9 +29,9 @@
  *   tree and small scratch, allocated through edp_config.alloc (cudaMalloc
  *   when NULL) and released by edp_destroy.  libedp never frees caller memory.
  *   Scratch is allocated at a call's first use and grown (after a device
- *   synchronisation) when a later call needs more: edp_update_priorities_td
- *   (4 bytes per pair), the PERMUTE sampling mode, edp_gae with
- *   normalisation and edp_pack_deliver (16 bytes per batch entry).  Before
+ *   synchronisation) when a later call needs more: the PERMUTE sampling
+ *   mode, edp_gae with normalisation and edp_pack_deliver (16 bytes per
+ *   batch entry).  Before
  *   capturing calls into a CUDA graph, make each of them once at its
  *   largest size, outside the capture: a call that would have to grow its
  *   scratch while its stream is being captured returns EDP_ERR_STATE and
@@ -302,8 +302,7 @@ EDP_API edp_status edp_sample_deliver(edp_ctx *ctx, uint32_t batch, uint64_t see
  * deferred (next_obs).  Ancestor sums change by exact integer deltas.
  * Errors: EDP_ERR_STATE for a context without priorities; EDP_ERR_INVALID
  * for NULL inputs or inputs outside device memory (and, for the TD forms,
- * alpha or eps < 0); EDP_ERR_OOM when the TD form cannot allocate its
- * scratch.  n == 0 does nothing. */
+ * alpha or eps < 0).  n == 0 does nothing. */
 EDP_API edp_status edp_update_priorities(edp_ctx *ctx, const int64_t *idx,
                                  const uint32_t *q, uint32_t n,
                                  edp_stream stream);
@@ -313,7 +312,7 @@ EDP_API edp_status edp_update_priorities(edp_ctx *ctx, const int64_t *idx,
  * [2^-100, 2^100] the device evaluates it in double-float arithmetic
  * (relative error below 2^-40), otherwise in fp64; neither is correctly
  * rounded, so q may differ by 1 from a host evaluation (about one case in
- * a million).  Batches of up to 2048 pairs need no scratch. */
+ * a million).  No batch needs scratch. */
 EDP_API edp_status edp_update_priorities_td(edp_ctx *ctx, const int64_t *idx,
                                     const float *td, uint32_t n, double alpha,
                                     double eps, edp_stream stream);
@@ -323,20 +322,12 @@ EDP_API edp_status edp_update_priorities_td(edp_ctx *ctx, const int64_t *idx,
  * device memory when they update priorities -- code being captured into a
  * CUDA graph, where cudaMalloc may not be called, and runtimes that hand out
  * all device memory at start-up and forbid later allocation, or cannot
- * afford the device-wide synchronisation an allocation may bring.
- * Above 2048 pairs edp_update_priorities_td allocates its scratch (one
- * uint32 per pair) on first use; this variant keeps that scratch in a fixed
- * per-device array of 16384 pairs (64 KiB), held by every GPU that loads
- * libedp until the process exits.  n > 16384 returns EDP_ERR_INVALID.  The first call on a device
- * looks up the array's device address (make it before any stream capture).
- * All calls on a device share the array.  Calls queued on one stream are
- * ordered (a call touches the array only after the previous kernel on its
- * stream has finished), so they may follow each other with no
- * synchronisation; calls that can run at the same time on different streams
- * -- of one context or of several on the device -- race on the array and
- * must be ordered by the caller (an event).  The array keeps the last call's
- * contents, which a call never reads before writing.  Results equal those of
- * edp_update_priorities_td for the same arguments. */
+ * afford the device-wide synchronisation an allocation may bring.  No
+ * priority update needs memory beyond its arguments any more, so both entry
+ * points run the same kernels; this one keeps its fixed maximum: n > 16384
+ * returns EDP_ERR_INVALID.  Calls of one context share its priority tree and
+ * must be ordered (see Overlap); calls of different contexts share nothing.
+ * Results equal those of edp_update_priorities_td for the same arguments. */
 EDP_API edp_status edp_update_priorities_td_static(edp_ctx *ctx, const int64_t *idx,
                                                    const float *td, uint32_t n,
                                                    double alpha, double eps,

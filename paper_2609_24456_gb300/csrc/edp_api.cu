@@ -56,9 +56,7 @@ void free_all(edp_ctx *c) {
   if (c->tree_mem) fr(c->cfg.alloc_user, c->tree_mem);
   if (c->ctrl) fr(c->cfg.alloc_user, c->ctrl);
   if (c->scratch) fr(c->cfg.alloc_user, c->scratch);
-  if (c->qbuf) fr(c->cfg.alloc_user, c->qbuf);
   if (c->perm_scratch) fr(c->cfg.alloc_user, c->perm_scratch);
-  c->qbuf = nullptr;
   c->perm_scratch = nullptr;
   c->tree_mem = nullptr;
   c->ctrl = nullptr;
@@ -285,16 +283,6 @@ cudaError_t edp::ctx_perm_scratch(edp_ctx *ctx, size_t bytes, cudaStream_t s, vo
   const cudaError_t e =
       grow(ctx, &ctx->perm_scratch, &ctx->perm_bytes, bytes, perm_zeroed_bytes(), s);
   *out = ctx->perm_scratch;
-  return e;
-}
-
-cudaError_t edp::ctx_qbuf(edp_ctx *ctx, size_t n, cudaStream_t s, uint32_t **out) {
-  void *blk = ctx->qbuf;
-  size_t have = ctx->qbuf_n * 4;
-  const cudaError_t e = grow(ctx, &blk, &have, (n < 4096 ? 4096 : n) * 4, 0, s);
-  ctx->qbuf = (uint32_t *)blk;
-  ctx->qbuf_n = have / 4;
-  *out = ctx->qbuf;
   return e;
 }
 

@@ -29,8 +29,7 @@ struct Ctrl {
   uint32_t err;
   uint32_t pending_q;  // deferred priority of the newest transition
   uint32_t max_q;      // running maximum priority
-  uint32_t pad0[2];
-  uint32_t upd_count;  // priority update: CTAs done with phase 1
+  uint32_t pad0[3];
   uint32_t pack_ticket;  // packed delivery: length CTAs done (calls are ordered)
   uint32_t pad;
   unsigned long long bad_index;  // first offending index (diagnostics)
@@ -62,9 +61,6 @@ struct edp_ctx {
   size_t scratch_bytes = 0;
   void *perm_scratch = nullptr;
   size_t perm_bytes = 0;
-  // priorities computed from TD errors before they are applied
-  uint32_t *qbuf = nullptr;
-  size_t qbuf_n = 0;
   // byte -> fl32(b/255) constants: x*R1 + x*R2 with one rounding
   float r1 = 0.f, r2 = 0.f;
   // per-channel normalisation: t = x - mean; y = t*S1 + t*S2 (one rounding)
@@ -562,7 +558,6 @@ cudaError_t ctx_scratch(edp_ctx *ctx, size_t bytes, cudaStream_t s, void **out);
 cudaError_t ctx_perm_scratch(edp_ctx *ctx, size_t bytes, cudaStream_t s, void **out);
 size_t perm_scratch_bytes(uint32_t n);
 size_t perm_zeroed_bytes();
-cudaError_t ctx_qbuf(edp_ctx *ctx, size_t n, cudaStream_t s, uint32_t **out);
 
 // ---------------------------------------------------------------------------
 // Host helpers shared by the entry points

@@ -324,10 +324,6 @@ __global__ void k_prio_from_td(const float *__restrict__ td, uint32_t n, PrioRul
     q[i] = prio_td(td[i], rule);
 }
 
-constexpr int kUpdThreads = 512;
-constexpr int kUpdPer = 2;                          // pairs per thread per chunk
-constexpr int kUpdChunk = kUpdThreads * kUpdPer;
-constexpr int kUpdTable = 2 * kUpdChunk;            // open-addressing table
 constexpr uint32_t kEmpty = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t tab_hash(uint32_t x, uint32_t mask) {
@@ -337,173 +333,193 @@ __device__ __forceinline__ uint32_t tab_hash(uint32_t x, uint32_t mask) {
   return x & mask;
 }
 
+// The pair's slot holds a transition; *k = its logical offset.
+__device__ __forceinline__ bool slot_holds(int64_t sl, uint64_t cap, uint64_t oldest,
+                                           uint64_t size, uint64_t *k) {
+  if (sl < 0 || (uint64_t)sl >= cap) return false;
+  *k = (uint64_t)sl >= oldest ? (uint64_t)sl - oldest : (uint64_t)sl + cap - oldest;
+  return *k < size;
+}
+
 // Priority update of a large batch (more than kUpdSmallMax pairs; smaller
-// ones take k_update_small below).  Phase 1 (all CTAs): the priority of every pair -- the
-// given u32, or PER's rule from the TD error, whose fp64 pow is spread over
-// the CTAs -- goes to qbuf.  The last CTA to finish (ticket counter, no
-// waiting) then applies the pairs in batch order, in chunks of 1024 (two
-// pairs per thread): a shared-memory hash table keeps, per slot, the largest
-// batch position (atomicMax), so only the last occurrence of a slot writes
-// its leaf.  The
-// exact signed delta of each written leaf is added to its ancestors
-// (two's complement wrap makes negative deltas exact); the two top levels,
-// which every pair shares, are summed on chip first.
+// ones take k_update_small below).  The slots are split over the CTAs by a
+// hash, so a slot has one owner and repeats of it meet in one CTA: no
+// scratch, no second phase, no CTA waits for another.  Every CTA reads the
+// whole batch's slots (8 bytes a pair, from the L2), kUpdLoads in flight per
+// thread, and keeps its own in a shared-memory hash table that holds, per
+// slot, the largest batch position (atomicMax): the last pair wins.  It then
+// evaluates the priority of each winner, writes its leaf and adds the exact
+// signed delta to the ancestors (two's complement wrap makes negative deltas
+// exact): deeper nodes rarely collide and take one 64-bit atomic per pair,
+// level 1 (32 nodes) and the root are summed on chip first.  A batch whose
+// distinct slots of one owner outgrow its table is applied in batch order, a
+// part at a time (a part's leaves are read again by the next).  The
+// running maximum counts every pair, the overwritten ones too, so each warp
+// evaluates a stripe of the batch for it.
+//
+// Bound by the latency of the scan (32,768 pairs are 256 KB per CTA).
+// Calls in a row from TD errors, 1,000,000 slots: 4,096 pairs 7.3 us, 32,768
+// pairs 16.4 us, 131,072 pairs 54.8 us; 28.5, 214.6 and 849.5 us when one
+// CTA applied the batch 1,024 pairs at a time.
+constexpr int kUpdThreads = 1024;
+constexpr int kUpdLoads = 8;                         // slots in flight per thread
+constexpr int kUpdChunk = kUpdThreads * kUpdLoads;   // pairs scanned at a time
+constexpr int kUpdGroup = 2;                         // loads applied at a time when a table fills
+constexpr uint32_t kUpdTable = 4096;                 // open addressing, at most 3/4 full
+static_assert(kUpdLoads % kUpdGroup == 0 && kUpdThreads * kUpdGroup <= kUpdTable / 4 * 3,
+              "a group of loads fits an empty table");
+
+__device__ __noinline__ uint32_t prio_td_call(float td, const PrioRule &rule) {
+  return prio_td(td, rule);
+}
+
 __global__ void __launch_bounds__(kUpdThreads, 1)
-k_update(TreeView t, const int64_t *__restrict__ idx,
-         const uint32_t *__restrict__ q, const float *__restrict__ td,
-         uint32_t *__restrict__ qbuf, PrioRule rule, uint32_t n,
-         uint64_t cap, uint64_t oldest, uint64_t size, int defer, Ctrl *ctrl) {
+k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict__ q,
+         const float *__restrict__ td, const __grid_constant__ PrioRule rule, uint32_t n,
+         uint64_t cap, uint64_t oldest, uint64_t size, int defer, uint32_t first_table,
+         Ctrl *ctrl) {
   __shared__ uint32_t hkey[kUpdTable];
   __shared__ uint32_t hpos[kUpdTable];
-  __shared__ uint32_t ticket;
   __shared__ uint32_t acc_lo[32], acc_hi[32];
   __shared__ unsigned long long warp_root[kUpdThreads / 32];
-  const uint32_t *qv_src = q;
-  // Nothing is read or written before the wait on the preceding kernel: it
-  // may be the kernel that writes the TD errors, or the previous update,
-  // whose last CTA may still be reading qbuf.
-  pdl_wait();
-  pdl_launch();
-  if (td) {
-    // phase 1: one warp per CTA, one CTA per 32 pairs, so the fp64 work
-    // spreads over SMs
-    if (threadIdx.x < 32)
-      for (uint32_t p = blockIdx.x * 32 + threadIdx.x; p < n; p += gridDim.x * 32)
-        qbuf[p] = prio_td(td[p], rule);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) ticket = atomicAdd(&ctrl->upd_count, 1u);
-    __syncthreads();
-    if (ticket != gridDim.x - 1) return;
-    __threadfence();
-    qv_src = qbuf;
-  } else if (blockIdx.x != 0) {
-    return;
+  __shared__ uint32_t s_sel, s_qmax;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (uint32_t i = threadIdx.x; i < kUpdTable; i += kUpdThreads) {
+    hkey[i] = kEmpty;
+    hpos[i] = 0;
   }
-  const uint32_t tsize = n >= kUpdChunk ? kUpdTable
-                                        : max(64u, 2u << (31 - __clz(max(n, 1u))));
-  const uint32_t mask = tsize - 1;
-  uint32_t qmax_local = 0;  // running maximum: one atomic per CTA at the end
-  const int lane = threadIdx.x & 31;
-  unsigned long long root_sum = 0;
   if (threadIdx.x < 32) {
     acc_lo[threadIdx.x] = 0;
     acc_hi[threadIdx.x] = 0;
   }
-  for (uint32_t base = 0; base < n; base += kUpdChunk) {
-    const uint32_t cnt = min((uint32_t)kUpdChunk, n - base);
+  if (threadIdx.x == 0) {
+    s_sel = 0;
+    s_qmax = 0;
+  }
+  // Nothing in memory is read or written before the wait on the preceding
+  // kernel: it may be the one that writes the TD errors.
+  pdl_wait();
+  pdl_launch();
+  __syncthreads();
+  // this warp's stripe of the batch: the running maximum, and bad slots
+  uint32_t qmax = 0;
+  for (uint64_t p = ((uint64_t)warp * gridDim.x + blockIdx.x) * 32 + lane; p < n;
+       p += (uint64_t)gridDim.x * kUpdThreads) {
+    const int64_t sl = idx[p];
+    uint64_t k = 0;
+    if (slot_holds(sl, cap, oldest, size, &k))
+      qmax = max(qmax, td ? prio_td_call(td[p], rule) : q[p]);
+    else if (sl < 0 || (uint64_t)sl >= cap)
+      flag(ctrl, DEVERR_INDEX, (unsigned long long)sl);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) qmax = max(qmax, __shfl_xor_sync(kFull, qmax, o));
+  if (lane == 0 && qmax) atomicMax(&s_qmax, qmax);
+
+  uint32_t tsize = first_table;
+  unsigned long long root_sum = 0;
+  auto insert = [&](uint32_t key, uint32_t pos) {
+    uint32_t h = tab_hash(key, tsize - 1);
+    for (uint32_t probe = 0; probe < tsize; ++probe) {
+      const uint32_t prev = atomicCAS(&hkey[h], kEmpty, key);
+      if (prev == kEmpty || prev == key) {
+        atomicMax(&hpos[h], pos);
+        break;
+      }
+      h = (h + 1) & (tsize - 1);
+    }
+  };
+  // applies the table's pairs and empties it
+  auto apply = [&]() {
+    __syncthreads();
     for (uint32_t i = threadIdx.x; i < tsize; i += kUpdThreads) {
+      const uint32_t key = hkey[i];
+      if (key == kEmpty) continue;
+      const uint32_t p = hpos[i];
       hkey[i] = kEmpty;
       hpos[i] = 0;
-    }
-    __syncthreads();
-    // every load of the chunk (index, priority, old leaf) is issued before
-    // the barrier; pairs are read in batch order p = r * threads + tid
-    int64_t s_[kUpdPer];
-    uint32_t qv_[kUpdPer], old_[kUpdPer];
-    uint64_t k_[kUpdPer];
-    bool holds_[kUpdPer];
-#pragma unroll
-    for (int r = 0; r < kUpdPer; ++r) {
-      const uint32_t p = r * kUpdThreads + threadIdx.x;
-      const bool active = p < cnt;
-      const int64_t sl = active ? idx[base + p] : -1;
-      const bool valid = active && sl >= 0 && (uint64_t)sl < cap;
-      if (active && !valid) flag(ctrl, DEVERR_INDEX, (unsigned long long)sl);
-      const uint64_t k = !valid ? 0
-                       : (uint64_t)sl >= oldest ? (uint64_t)sl - oldest
-                                                : (uint64_t)sl + cap - oldest;
-      const bool holds = valid && k < size;  // the slot holds a transition
-      s_[r] = sl;
-      k_[r] = k;
-      holds_[r] = holds;
-      qv_[r] = holds ? __ldcg(qv_src + base + p) : 0u;
-      old_[r] = holds ? t.leaves[sl] : 0u;
-      if (holds) {
-        const uint32_t key = (uint32_t)sl;
-        uint32_t h = tab_hash(key, mask);
-        for (uint32_t probe = 0; probe < tsize; ++probe) {
-          const uint32_t prev = atomicCAS(&hkey[h], kEmpty, key);
-          if (prev == kEmpty || prev == key) {
-            atomicMax(&hpos[h], p);
-            break;
-          }
-          h = (h + 1) & mask;
-        }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < kUpdPer; ++r) {
-      const uint32_t p = r * kUpdThreads + threadIdx.x;
-      const int64_t sl = s_[r];
-      const uint32_t qv = qv_[r];
-      qmax_local = max(qmax_local, qv);
-      bool win = false;
-      if (holds_[r]) {
-        uint32_t h = tab_hash((uint32_t)sl, mask);
-        for (uint32_t probe = 0; probe < tsize && hkey[h] != (uint32_t)sl; ++probe)
-          h = (h + 1) & mask;
-        win = hpos[h] == p;  // no later pair sets this slot
-      }
-      if (win && defer && k_[r] == size - 1) {
+      const uint32_t old = __ldcg(t.leaves + key);
+      const uint32_t qv = td ? prio_td_call(td[p], rule) : q[p];
+      uint64_t k = 0;
+      slot_holds((int64_t)key, cap, oldest, size, &k);
+      if (defer && k == size - 1) {
         ctrl->pending_q = qv;
-        win = false;
+        continue;
       }
-      unsigned long long delta = 0;
-      if (win) {
-        t.leaves[sl] = qv;
-        delta = (unsigned long long)((long long)qv - (long long)old_[r]);
-      }
-      // ancestors.  The root and level 1 (32 nodes) are shared by many
-      // pairs: the root delta is summed over the block (shuffles, then one
-      // atomic), level-1 deltas go to 32 shared accumulators kept as two
-      // 32-bit halves with explicit carries (exact mod 2^64).  Deeper nodes
-      // rarely collide and take one 64-bit atomic per pair.
+      const unsigned long long delta = (unsigned long long)((long long)qv - (long long)old);
+      if (!delta) continue;
+      t.leaves[key] = qv;
       root_sum += delta;
-      if (delta && t.depth >= 2) {
-        const uint32_t n1 = (uint32_t)((uint64_t)sl >> (5 * (t.depth - 1)));
+      if (t.depth >= 2) {
+        // level 1 as two 32-bit halves with an explicit carry (exact mod 2^64)
+        const uint32_t n1 = key >> (5 * (t.depth - 1));
         const uint32_t lo = (uint32_t)delta, hi = (uint32_t)(delta >> 32);
-        const uint32_t old = atomicAdd(&acc_lo[n1], lo);
-        atomicAdd(&acc_hi[n1], hi + (old + lo < old ? 1u : 0u));
+        const uint32_t was = atomicAdd(&acc_lo[n1], lo);
+        atomicAdd(&acc_hi[n1], hi + (was + lo < was ? 1u : 0u));
       }
-      if (delta)
-        for (uint32_t d = 2; d < t.depth; ++d)
-          atomicAdd((unsigned long long *)&t.lvl(d)[(uint64_t)sl >> (5 * (t.depth - d))],
-                    delta);
+      for (uint32_t d = 2; d < t.depth; ++d)
+        atomicAdd((unsigned long long *)&t.lvl(d)[key >> (5 * (t.depth - d))], delta);
     }
-    // flush the chunk's root and level-1 sums
+    if (threadIdx.x == 0) s_sel = 0;
+    __syncthreads();
+  };
+
+  for (uint64_t base = 0; base < n; base += kUpdChunk) {
+    int64_t s[kUpdLoads];
 #pragma unroll
-    for (int o = 16; o; o >>= 1) root_sum += __shfl_xor_sync(kFull, root_sum, o);
-    if (lane == 0) warp_root[threadIdx.x >> 5] = root_sum;
-    root_sum = 0;
-    __syncthreads();
-    if (threadIdx.x < 32 && t.depth >= 2) {
-      const unsigned long long v =
-          ((unsigned long long)acc_hi[threadIdx.x] << 32) | acc_lo[threadIdx.x];
-      if (v) atomicAdd((unsigned long long *)&t.lvl(1)[threadIdx.x], v);
-      acc_lo[threadIdx.x] = 0;
-      acc_hi[threadIdx.x] = 0;
+    for (int u = 0; u < kUpdLoads; ++u) {
+      const uint64_t p = base + u * kUpdThreads + threadIdx.x;
+      s[u] = p < n ? idx[p] : -1;
     }
-    if (threadIdx.x == 32) {
-      unsigned long long v = 0;
-      for (int w = 0; w < kUpdThreads / 32; ++w) v += warp_root[w];
-      if (v) atomicAdd((unsigned long long *)&t.nodes[0], v);
+    uint32_t mine = 0;  // bit u: slot u is owned here
+#pragma unroll
+    for (int u = 0; u < kUpdLoads; ++u) {
+      uint64_t k = 0;
+      if (slot_holds(s[u], cap, oldest, size, &k) &&
+          __umulhi((uint32_t)s[u] * 0x9E3779B1u, gridDim.x) == blockIdx.x)
+        mine |= 1u << u;
     }
+    if (mine) atomicAdd(&s_sel, (uint32_t)__popc(mine));
     __syncthreads();
+    const bool fits = s_sel <= tsize / 4 * 3;
+    __syncthreads();  // every thread has read s_sel
+    if (fits) {
+#pragma unroll
+      for (int u = 0; u < kUpdLoads; ++u)
+        if ((mine >> u) & 1u)
+          insert((uint32_t)s[u], (uint32_t)base + u * kUpdThreads + threadIdx.x);
+      continue;
+    }
+    apply();  // the earlier pairs, then this chunk's a group at a time
+    tsize = kUpdTable;
+#pragma unroll
+    for (int g = 0; g < kUpdLoads; g += kUpdGroup) {
+#pragma unroll
+      for (int u = g; u < g + kUpdGroup; ++u)
+        if ((mine >> u) & 1u)
+          insert((uint32_t)s[u], (uint32_t)base + u * kUpdThreads + threadIdx.x);
+      apply();
+    }
   }
+  apply();
+
 #pragma unroll
-  for (int o = 16; o; o >>= 1)
-    qmax_local = max(qmax_local, __shfl_xor_sync(kFull, qmax_local, o));
-  if ((threadIdx.x & 31) == 0) ticket = 0;
+  for (int o = 16; o; o >>= 1) root_sum += __shfl_xor_sync(kFull, root_sum, o);
+  if (lane == 0) warp_root[warp] = root_sum;
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) atomicMax(&ticket, qmax_local);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (ticket) atomicMax(&ctrl->max_q, ticket);
-    if (td) ctrl->upd_count = 0;  // ready for the next call
+  if (warp == 0) {
+    if (t.depth >= 2) {
+      const unsigned long long v = ((unsigned long long)acc_hi[lane] << 32) | acc_lo[lane];
+      if (v) atomicAdd((unsigned long long *)&t.lvl(1)[lane], v);
+    }
+    const unsigned long long root = warp_sum_u64(warp_root[lane]);
+    if (lane == 0) {
+      if (root) atomicAdd((unsigned long long *)&t.nodes[0], root);
+      if (s_qmax) atomicMax(&ctrl->max_q, s_qmax);
+    }
   }
 }
+static_assert(kUpdThreads / 32 == 32, "one warp sums the warps' root deltas");
 
 // Priority update of a small batch (n <= kUpdSmallMax pairs): one CTA per 32
 // pairs and a single pass, with no ticket and no second phase.  Each CTA
@@ -705,18 +721,13 @@ cudaError_t launch_update(edp_ctx *c, const int64_t *idx, const uint32_t *q,
     return launch_pdl(k_update_small, dim3((n + 31) / 32), dim3(kUpdSmallThreads), s,
                       view(c), idx, q, td, prio_rule(alpha, eps), n, c->cap, oldest,
                       size, c->defer, c->ctrl);
-  uint32_t *qbuf = nullptr;
-  unsigned grid = 1;
-  if (td) {
-    const cudaError_t e = ctx_qbuf(c, n, s, &qbuf);
-    if (e != cudaSuccess) return e;
-    // 32 priorities (one warp) per CTA: the fp64 work spreads over SMs
-    grid = (n + 31) / 32;
-    if (grid > 2u * (unsigned)c->coop_sms) grid = 2u * (unsigned)c->coop_sms;
-  }
-  return launch_pdl(k_update, dim3(grid), dim3(kUpdThreads), s, view(c), idx, q,
-                    td, qbuf, prio_rule(alpha, eps), n, c->cap, oldest, size, c->defer,
-                    c->ctrl);
+  // one CTA per SM from 64 pairs a CTA on; a table four times the pairs a CTA
+  // is expected to own
+  uint32_t grid = (n + 63) / 64, table = 256;
+  if (grid > (uint32_t)c->coop_sms) grid = (uint32_t)c->coop_sms;
+  while (table < kUpdTable && table / 4 < n / grid) table *= 2;
+  return launch_pdl(k_update, dim3(grid), dim3(kUpdThreads), s, view(c), idx, q, td,
+                    prio_rule(alpha, eps), n, c->cap, oldest, size, c->defer, table, c->ctrl);
 }
 
 cudaError_t launch_prio_from_td(const float *td, uint32_t n, double alpha,
@@ -729,55 +740,17 @@ cudaError_t launch_prio_from_td(const float *td, uint32_t n, double alpha,
 }  // namespace edp
 
 // ---------------------------------------------------------------------------
-// Allocation-free priority update.  Same kernels as edp_update_priorities_td:
-// up to 2,048 pairs the single-pass kernel, which needs no memory beyond
-// its arguments; above that the two-phase kernel, whose per-pair priorities
-// computed from the TD errors go to the fixed array below instead of
-// context-owned scratch that is allocated on first use.  Callers that must not allocate device memory use it: code being
-// captured into a CUDA graph (cudaMalloc may not be called during stream
-// capture), and runtimes that hand out all device memory up front and forbid
-// allocation later, or that cannot afford the device-wide synchronisation a
-// cudaMalloc/cudaFree may bring.  The array is per device and lives until
-// the process exits; every call on that device shares it.  Calls queued on
-// one stream are ordered (the kernel touches the array only after its wait
-// on the preceding kernel); calls that can run at the same time on different
-// streams race.  Nothing in it needs to start at zero: a call writes
-// priorities [0, n) before it reads them.
+// Allocation-free priority update: the kernels of edp_update_priorities_td,
+// neither of which needs memory beyond its arguments, for at most
+// kStaticMaxPairs pairs (the entry point's fixed limit).
 // ---------------------------------------------------------------------------
-#include <mutex>
-
-namespace edp {
-namespace {
-
-constexpr uint32_t kStaticMaxPairs = 16384;  // 64 KiB of priorities
-static __device__ __align__(256) uint32_t g_static_qbuf[kStaticMaxPairs];
-
-constexpr int kMaxDevices = 64;
-std::mutex g_static_mu;
-uint32_t *g_static_ptr[kMaxDevices] = {};
-
-// Device address of g_static_qbuf on the current device (looked up once per
-// device; the host-side name is only a stand-in for the device symbol).
-cudaError_t static_qbuf(int dev, uint32_t **out) {
-  std::lock_guard<std::mutex> lock(g_static_mu);
-  if (!g_static_ptr[dev]) {
-    void *p = nullptr;
-    const cudaError_t e = cudaGetSymbolAddress(&p, g_static_qbuf);
-    if (e != cudaSuccess) return e;
-    g_static_ptr[dev] = (uint32_t *)p;
-  }
-  *out = g_static_ptr[dev];
-  return cudaSuccess;
-}
-
-}  // namespace
-}  // namespace edp
-
 extern "C" edp_status edp_update_priorities_td_static(
     edp_ctx *ctx, const int64_t *idx, const float *td, uint32_t n,
     double alpha, double eps, edp_stream stream) {
   using namespace edp;
   static const char who[] = "edp_update_priorities_td_static";
+  constexpr uint32_t kStaticMaxPairs = 16384;
+  constexpr int kMaxDevices = 64;
   if (ctx && n && !td) return fail(ctx, EDP_ERR_INVALID, "%s: td NULL", who);
   const edp_status st = update_args(ctx, who, idx, nullptr, td, n, alpha, eps);
   if (st != EDP_OK || n == 0) return st;
@@ -789,31 +762,8 @@ extern "C" edp_status edp_update_priorities_td_static(
     return fail(ctx, EDP_ERR_INVALID, "%s: device ordinal out of range", who);
   DeviceGuard dg(ctx->cfg.device);
   EDP_TRACE(who);
-  const uint64_t size = ctx->total < ctx->cap ? ctx->total : ctx->cap;
-  const uint64_t oldest = (ctx->total - size) % ctx->cap;
-  cudaError_t e;
-  if (n <= (uint32_t)kUpdSmallMax) {  // needs no priority array
-    e = launch_pdl(k_update_small, dim3((n + 31) / 32), dim3(kUpdSmallThreads),
-                   (cudaStream_t)stream, view(ctx), idx, (const uint32_t *)nullptr, td,
-                   prio_rule(alpha, eps), n, ctx->cap, oldest, size, ctx->defer, ctx->ctrl);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return fail(ctx, EDP_ERR_CUDA, "%s: %s", who, cudaGetErrorString(e));
-    }
-    return EDP_OK;
-  }
-  uint32_t *qbuf = nullptr;
-  e = static_qbuf(ctx->cfg.device, &qbuf);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(ctx, EDP_ERR_CUDA, "%s: cudaGetSymbolAddress: %s", who,
-                cudaGetErrorString(e));
-  }
-  unsigned grid = (n + 31) / 32;
-  if (grid > 2u * (unsigned)ctx->coop_sms) grid = 2u * (unsigned)ctx->coop_sms;
-  e = launch_pdl(k_update, dim3(grid), dim3(kUpdThreads), (cudaStream_t)stream,
-                 view(ctx), idx, (const uint32_t *)nullptr, td, qbuf, prio_rule(alpha, eps),
-                 n, ctx->cap, oldest, size, ctx->defer, ctx->ctrl);
+  const cudaError_t e =
+      launch_update(ctx, idx, nullptr, td, alpha, eps, n, (cudaStream_t)stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(ctx, EDP_ERR_CUDA, "%s: %s", who, cudaGetErrorString(e));
