@@ -337,7 +337,7 @@ class PerReplay(Workload):
     512, frame stack 4, obs + next_obs fp32, PER alpha 0.6 / beta 0.4 with
     priorities from Exp(1) TD errors; step = sample, deliver, update."""
     name = "per-replay-1M-84x84-B512"
-    kernel = "k_deliver_stack_staged"
+    kernel = "k_deliver_stack"
     dtype = "u8->f32"
     launches_per_round = 3
 

@@ -19,7 +19,7 @@ namespace edp {
 enum : uint32_t {
   DEVERR_INDEX = 1u,    // a slot index outside the sampleable range
   DEVERR_EMPTY = 2u,    // total priority 0 at sampling time
-  DEVERR_TIMEOUT = 4u,  // a bounded device-side wait expired (staged delivery)
+  DEVERR_TIMEOUT = 4u,  // a bounded device-side wait expired (packed delivery)
   DEVERR_TREE = 8u,     // a tree descent found no child holding its target
   DEVERR_OVERFLOW = 16u,  // packed output larger than its buffer (clipped)
 };
@@ -356,11 +356,6 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
 }
 __device__ __forceinline__ void mbar_arrive_tx(unsigned long long *bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-               :: "r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-// Raises the bytes the current phase of `bar` waits for, without arriving.
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, uint32_t bytes) {
-  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;"
                :: "r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ bool mbar_test(unsigned long long *bar, uint32_t parity) {

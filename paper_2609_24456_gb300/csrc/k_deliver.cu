@@ -9,9 +9,7 @@
 // into warp spans whose size is set from the work, not from the grid: a
 // warp runs a few iterations of its unrolled loop per span and the grid
 // holds as many CTAs as that takes (several waves), so the block scheduler
-// balances the tail.  (A large frame-stack batch instead streams its frames
-// through shared memory: k_deliver_stack_staged below.)  A warp walks
-// its span segment by segment (a segment never crosses a frame or image),
+// balances the tail.  A warp walks its span segment by segment (a segment never crosses a frame or image),
 // resolving the sample's slot, episode-boundary mask and source pointer
 // once per segment.  Loads are the payload bytes a lane needs for one
 // 16-byte output store, so every warp-wide store instruction writes 512
@@ -38,8 +36,7 @@ constexpr int kNormUnroll = 6;
 
 // unrolled rows per warp iteration and iterations per warp (chunk span) of
 // each kernel
-constexpr int kStackUnroll = 4;
-constexpr int kStackMinBlocks = 6;  // __launch_bounds__: at most 40 registers
+constexpr int kStackMinBlocks = 5;  // __launch_bounds__: at most 48 registers
 constexpr int kHwcUnroll = 2, kHwcIters = 2;
 constexpr int kNormIters = 2;
 
@@ -134,33 +131,52 @@ __device__ void collate(const Common &c, uint32_t k, bool ok, uint64_t slot,
   }
 }
 
-// The whole batch's collate, importance weights and index reporting by one
-// CTA, for a frame-stack batch small enough to run one chunk per CTA: the
-// streaming CTAs then carry no collate latency (q_min over the batch once, a
-// block reduction, then one sample per thread).
-__device__ void collate_batch(const Common &c) {
+// Minimum of q over the batch (the CTA): every thread gets it.  16-byte loads
+// where q allows them, several in flight.
+__device__ __forceinline__ uint32_t batch_qmin_cta(const Common &c) {
   __shared__ uint32_t s_min[kWarps];
-  const int lane = threadIdx.x & 31;
   uint32_t m = 0xffffffffu;
-  if (c.isw) {
-    for (uint32_t i0 = threadIdx.x; i0 < c.B; i0 += kThreads * 4) {
-      uint32_t v[4];
+  const uint32_t nv = ((uintptr_t)c.q & 15u) == 0 ? c.B / 4 : 0;
+  const uint4 *q4 = reinterpret_cast<const uint4 *>(c.q);
+  for (uint64_t i0 = threadIdx.x; i0 < nv; i0 += kThreads * 4) {
+    uint4 v[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const uint32_t i = i0 + u * kThreads;
-        v[u] = i < c.B ? __ldg(c.q + i) : 0xffffffffu;
-      }
+    for (int u = 0; u < 4; ++u)
+      v[u] = i0 + u * kThreads < nv ? __ldg(q4 + i0 + u * kThreads)
+                                    : make_uint4(~0u, ~0u, ~0u, ~0u);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) m = min(m, v[u]);
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) m = min(m, __shfl_xor_sync(kFull, m, o));
-    if (lane == 0) s_min[threadIdx.x >> 5] = m;
-    __syncthreads();
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) m = min(m, s_min[w]);
+    for (int u = 0; u < 4; ++u) m = min(m, min(min(v[u].x, v[u].y), min(v[u].z, v[u].w)));
   }
-  for (uint32_t k = threadIdx.x; k < c.B; k += kThreads) {
+  for (uint64_t i0 = 4ull * nv + threadIdx.x; i0 < c.B; i0 += kThreads * 4) {
+    uint32_t v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      v[u] = i0 + u * kThreads < c.B ? __ldg(c.q + i0 + u * kThreads) : 0xffffffffu;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) m = min(m, v[u]);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) m = min(m, __shfl_xor_sync(kFull, m, o));
+  if ((threadIdx.x & 31) == 0) s_min[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) m = min(m, s_min[w]);
+  return m;
+}
+
+// Collate, importance weights and index reporting of the batch by CTA `cta`
+// of `ncta`, a sample per thread of its first kCollateThreads (one warp for
+// each fp64 pipe of the SM), so that the streaming CTAs carry no collate
+// latency.  Each CTA takes q_min over the whole batch, so there are at most
+// kCollateCtas.
+constexpr uint32_t kCollateThreads = 128;
+constexpr uint32_t kCollateCtas = 256;
+__device__ void collate_batch(const Common &c, uint32_t cta, uint32_t ncta) {
+  const uint32_t m = c.isw ? batch_qmin_cta(c) : 0xffffffffu;
+  if (threadIdx.x >= kCollateThreads) return;
+  for (uint64_t i = (uint64_t)cta * kCollateThreads + threadIdx.x; i < c.B;
+       i += (uint64_t)ncta * kCollateThreads) {
+    const uint32_t k = (uint32_t)i;
     uint64_t slot = 0, off = 0;
     const bool ok = sample_slot(c, k, &slot, &off, true);
     if (c.act_out) c.act_out[k] = ok ? c.action[slot] : 0;
@@ -200,10 +216,23 @@ __device__ __forceinline__ float byte_f(uint32_t w, int i) {
 // anchor" (zeroes the frame in obs and next_obs) and "at the anchor" (zeroes
 // it in next_obs only).
 //
-// This direct form serves batches too small to fill the GPU with staged
-// pieces (below): one chunk per CTA, no work counter, and one more CTA
-// collates the whole batch (collate_batch) so that no streaming warp waits
-// on it.
+// A warp runs one unrolled iteration: UN loads in flight per lane, a span of
+// 32 UN words, a CTA per kWarps spans, however many waves that makes; the
+// first CTAs collate the batch (collate_batch) so that no streaming warp
+// waits on it.  UN = 8 (256 words) keeps 8 KB of reads in flight per CTA;
+// batches that give an SM less than one CTA at 4 spread over more SMs with 4.
+//
+// Bound by HBM.  Calls in a row, a fresh sample each, in us, and before, when
+// frames were staged through shared memory by bulk copies, 2 CTAs per SM:
+//   84x84, 4 frames + successors   512: 23.0 (23.6)  8,192: 315 (365), 6,799 GB/s
+//   84x84, 1 frame                 8,192: 45.8 (47.6)  32,768: 172 (189)
+//   64x64, 4 + successors          8,192: 184 (198)   128x128 2,048: 184 (196)
+//   48x48, 4 + successors          512: 8.0 (12.0)    8,192: 105 (140)
+//   92x92, 3 frames                512: 11.9 (105: its 529 runs of 16 bytes cut
+//                                  into 23 equal pieces)
+// 4 loads per lane instead of 8 lose up to 20% without successors (half the
+// stores per load); two iterations of 4 are equal at large batches and slower
+// at small ones; a 32x32 frame at 512 6.3 us (10.8).
 // ---------------------------------------------------------------------------
 struct StackArgs {
   const uint8_t *frames;
@@ -211,7 +240,7 @@ struct StackArgs {
   uint32_t W;     // 32-bit words per frame
   uint32_t K;
   uint32_t U;     // frames per sample (K, or K + 1 with next_obs)
-  uint32_t span;  // units per warp per chunk (multiple of 32)
+  uint32_t ncollate;  // CTAs that collate the batch
   float *obs;
   float *next;
 };
@@ -224,7 +253,9 @@ __device__ __forceinline__ void stack_span(const Common &c, const StackArgs &a,
   const uint64_t per = (uint64_t)a.U * a.W;  // units per sample
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
   while (f < end) {
-    const uint32_t k = (uint32_t)(f / per);
+    // 32-bit divisions while they do (a 64-bit one is a long sequence)
+    const uint32_t k = (f | per) <= 0xffffffffu ? (uint32_t)f / (uint32_t)per
+                                                : (uint32_t)(f / per);
     const uint32_t rem = (uint32_t)(f - (uint64_t)k * per);
     const uint32_t m = rem / a.W;
     const uint32_t w_lo = rem - m * a.W;
@@ -301,266 +332,13 @@ k_deliver_stack(Common c, StackArgs a) {
   const uint64_t pol = policy_stream();
   pdl_wait();
   pdl_launch();
-  if (blockIdx.x == 0) {  // CTA 0 collates the batch
-    collate_batch(c);
+  if (blockIdx.x < a.ncollate) {
+    collate_batch(c, blockIdx.x, a.ncollate);
     return;
   }
   const uint64_t total = (uint64_t)c.B * a.U * a.W;
-  const uint64_t f = (uint64_t)(blockIdx.x - 1) * kWarps * a.span + (uint64_t)warp * a.span;
-  if (f < total) stack_span<UN>(c, a, f, min(total, f + a.span), lane, pol);
-}
-
-// ---------------------------------------------------------------------------
-// Frame stack, float32, staged through shared memory (batches that fill the
-// GPU).  A unit is one piece of one frame: piece p of frame m of sample k,
-// where frame m is the one at logical offset off - K + 1 + m (obs slot m for
-// m < K, next_obs slot m - 1 for m >= 1), and the npieces pieces of a frame
-// are equal runs of at most kPiece bytes.  Units are dealt to the CTAs round
-// robin (unit u to CTA u mod grid): equal units, so the split is balanced
-// without a work counter, and no state outlives the launch.  Per CTA:
-//  - warp 0 (producer) resolves 32 of its units at a time, a lane each:
-//    index -> slot and logical offset -> source address, and the done flags
-//    of the frame's window (offsets j .. off).  It issues the bulk copy of
-//    each unit's piece into a free stage as soon as the address is known,
-//    before the flags have arrived (a frame they then zero everywhere is
-//    copied for nothing), and publishes the unit -- which of its output
-//    copies are zero -- with its arrival on the stage once they have;
-//  - warp 1 collates this CTA's samples (k = blockIdx.x mod grid): action,
-//    reward, done, gathered scalars, the importance weight, and the index
-//    when the batch is drawn here;
-//  - warps 2 .. kStageWarps + 1 (consumers) wait for the stage, turn its
-//    bytes into floats and store them to obs and / or next_obs (zeros where
-//    the episode mask says so; each warp-wide store writes 512 contiguous
-//    bytes), then release the stage.
-// A stage's phase completes when the producer has arrived and the copy's
-// bytes have landed.  kStages stages keep several pieces in flight per CTA,
-// so the index -> flags chain is paid once per 32 units, beside the copies.
-// Every wait is bounded (kWaitNs): on expiry the warp records DEVERR_TIMEOUT
-// and stops, the producer after waiting (bounded again) for the copies it
-// has in flight.
-// ---------------------------------------------------------------------------
-constexpr int kStages = 6;
-constexpr uint32_t kPiece = 7168;  // bytes per stage, a multiple of 16
-constexpr int kStageWarps = 7;     // consumer warps
-constexpr int kStagedThreads = 32 * (kStageWarps + 2);
-constexpr int kStagedPerSm = 2;    // CTAs per SM in the grid
-constexpr int kStagedUnroll = 4;
-constexpr uint64_t kWaitNs = 1000000000ull;
-// unit flags (StageSmem::meta)
-constexpr uint32_t kZeroObs = 1u, kZeroNext = 2u, kLoaded = 4u;
-
-struct StageSmem {
-  alignas(128) uint8_t buf[kStages][kPiece];
-  unsigned long long full[kStages];   // producer -> consumers (bytes landed)
-  unsigned long long empty[kStages];  // consumers -> producer (stage free)
-  uint32_t meta[kStages];
-};
-
-// Collate of samples first, first + stride, ... (one warp): q_min over the
-// batch once, then one sample per lane.
-__device__ void collate_strided(const Common &c, uint32_t first, uint32_t stride, int lane) {
-  const uint32_t m = c.isw ? batch_qmin(c, lane) : 0u;
-  for (uint64_t k = first + (uint64_t)lane * stride; k < c.B; k += 32ull * stride) {
-    uint64_t slot = 0, off = 0;
-    const bool ok = sample_slot(c, (uint32_t)k, &slot, &off, true);
-    if (c.act_out) c.act_out[k] = ok ? c.action[slot] : 0;
-    if (c.rew_out) c.rew_out[k] = ok ? c.reward[slot] : 0.f;
-    if (c.done_out) c.done_out[k] = ok ? c.done[slot] : (uint8_t)0;
-    if (c.gdst0) c.gdst0[k] = ok ? c.gsrc0[off] : 0.f;
-    if (c.gdst1) c.gdst1[k] = ok ? c.gsrc1[off] : 0.f;
-    if (c.isw) c.isw[k] = is_weight(m, c.q[k], c.beta);
-  }
-}
-
-// Unit u -> (sample k, frame m, piece p).
-struct Unit {
-  uint32_t k, m, p;
-};
-__device__ __forceinline__ Unit unit_of(uint64_t u, uint32_t U, uint32_t npieces) {
-  const uint32_t per_k = U * npieces;
-  Unit r;
-  r.k = (uint32_t)(u / per_k);
-  const uint32_t rem = (uint32_t)(u - (uint64_t)r.k * per_k);
-  r.m = rem / npieces;
-  r.p = rem - r.m * npieces;
-  return r;
-}
-
-__device__ void stage_producer(const Common &c, const StackArgs &a, StageSmem &sm,
-                               uint32_t npieces, uint32_t piece, uint64_t nmine,
-                               int lane, uint64_t pol) {
-  for (uint64_t i0 = 0; i0 < nmine; i0 += 32) {
-    // lane l resolves unit i0 + l of this CTA: its source now, its episode
-    // flags in flight (used when the unit is published)
-    uint64_t src = 0;
-    bool valid = false, ok = false, has_obs = false, has_next = false;
-    int64_t span = 0;
-    uint32_t bits = 0;
-    if (i0 + lane < nmine) {
-      valid = true;
-      const Unit t = unit_of(blockIdx.x + (i0 + lane) * gridDim.x, a.U, npieces);
-      uint64_t slot = 0, off = 0;
-      ok = sample_slot(c, t.k, &slot, &off, false);
-      const int64_t j = (int64_t)off - (int64_t)(a.K - 1) + (int64_t)t.m;
-      has_obs = t.m < a.K;
-      has_next = a.next && t.m >= 1;
-      if (ok && j >= 0) {
-        uint64_t js = c.oldest + (uint64_t)j;
-        if (js >= c.cap) js -= c.cap;
-        src = (uint64_t)(a.frames + js * a.F + (uint64_t)t.p * piece);
-        span = (int64_t)off - j + 1;  // flags of offsets j .. off (<= K)
-      } else {
-        ok = false;  // zero in every copy
-      }
-      // bit i: done flag of offset j + i
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        if (i < span) {
-          uint64_t ps = c.oldest + (uint64_t)(off - (uint64_t)(span - 1)) + i;
-          if (ps >= c.cap) ps -= c.cap;
-          bits |= (c.done[ps] != 0 ? 1u : 0u) << i;
-        }
-      }
-    }
-    const uint32_t n = (uint32_t)min((uint64_t)32, nmine - i0);
-    uint32_t pub = 0;  // units of the group published so far
-    uint32_t good = 1;
-    // this lane's unit flags: an episode end before the anchor zeroes the
-    // frame in obs and next_obs; one at the anchor zeroes it in next_obs
-    // only (evaluated when the first unit is published: the flag loads are
-    // in flight until then)
-    uint32_t fl = 0;
-    bool fl_ready = false;
-#define EDP_PUBLISH()                                                            \
-    do {                                                                         \
-      if (!fl_ready) {                                                           \
-        const bool end_before = span > 1 && (bits & ((1u << (span - 1)) - 1u)) != 0; \
-        const bool end_at = span > 0 && ((bits >> (span - 1)) & 1u);             \
-        const bool zo = !ok || end_before, zn = zo || end_at;                    \
-        const bool load = (has_obs && !zo) || (has_next && !zn);                 \
-        fl = valid ? (zo ? kZeroObs : 0u) | (zn ? kZeroNext : 0u) | (load ? kLoaded : 0u) \
-                   : 0u;                                                         \
-        fl_ready = true;                                                         \
-      }                                                                          \
-      const uint32_t fl_t = __shfl_sync(kFull, fl, pub);                         \
-      if (lane == 0) {                                                           \
-        const int st_p = (int)((i0 + pub) % kStages);                            \
-        sm.meta[st_p] = fl_t;                                                    \
-        mbar_arrive(&sm.full[st_p]);                                             \
-      }                                                                          \
-      ++pub;                                                                     \
-    } while (0)
-    uint32_t t = 0;
-    for (; t < n; ++t) {
-      const uint64_t i = i0 + t;
-      const int st = (int)(i % kStages);
-      if (i >= kStages) {
-        // the stage's previous occupant (unit i - kStages) must have been
-        // published before the consumers can free the stage
-        while (pub + kStages <= t) EDP_PUBLISH();
-        if (lane == 0)
-          good = mbar_wait(&sm.empty[st], (uint32_t)((i / kStages) - 1) & 1u, kWaitNs);
-        good = __shfl_sync(kFull, good, 0);
-        if (!good) break;
-      }
-      const uint64_t src_t = __shfl_sync(kFull, src, t);
-      if (lane == 0 && src_t) {
-        mbar_expect_tx(&sm.full[st], piece);
-        bulk_load(sm.buf[st], reinterpret_cast<const void *>(src_t), piece, &sm.full[st], pol);
-      }
-    }
-    if (!good) {
-      // units i0 + pub .. i0 + t - 1 are issued but unpublished: publish
-      // them so their phases can complete, then wait (bounded) for the
-      // bytes of the last kStages issued copies, which land in this CTA's
-      // shared memory, before the CTA may exit
-      while (pub < t) EDP_PUBLISH();
-      if (lane == 0) {
-        const uint64_t end = i0 + t;
-        flag(c.ctrl, DEVERR_TIMEOUT, end);
-        for (uint64_t q = end > kStages ? end - kStages : 0; q < end; ++q)
-          mbar_wait(&sm.full[q % kStages], (uint32_t)(q / kStages) & 1u, kWaitNs);
-      }
-      return;
-    }
-    while (pub < n) EDP_PUBLISH();
-#undef EDP_PUBLISH
-  }
-}
-
-__device__ void stage_consumer(const Common &c, const StackArgs &a, StageSmem &sm,
-                               uint32_t npieces, uint32_t piece, uint64_t nmine,
-                               int cw, int lane, uint64_t pol) {
-  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  const uint32_t W = piece / 4;  // words of a piece
-  constexpr uint32_t kRow = 32 * kStageWarps;
-  for (uint64_t i = 0; i < nmine; ++i) {
-    const int st = (int)(i % kStages);
-    if (!mbar_wait(&sm.full[st], (uint32_t)(i / kStages) & 1u, kWaitNs)) {
-      if (lane == 0) flag(c.ctrl, DEVERR_TIMEOUT, i);
-      return;
-    }
-    const uint32_t fl = sm.meta[st];
-    const Unit t = unit_of(blockIdx.x + i * gridDim.x, a.U, npieces);
-    const bool zo = fl & kZeroObs, zn = fl & kZeroNext, loaded = fl & kLoaded;
-    const uint64_t pofs = (uint64_t)t.p * piece;
-    float4 *dobs = t.m < a.K ? reinterpret_cast<float4 *>(
-                                   a.obs + ((uint64_t)t.k * a.K + t.m) * a.F + pofs)
-                             : nullptr;
-    float4 *dnext = (a.next && t.m >= 1)
-                        ? reinterpret_cast<float4 *>(
-                              a.next + ((uint64_t)t.k * a.K + t.m - 1) * a.F + pofs)
-                        : nullptr;
-    const uint32_t *src = reinterpret_cast<const uint32_t *>(sm.buf[st]);
-    for (uint32_t w0 = cw * 32 + lane; w0 < W; w0 += kRow * kStagedUnroll) {
-      uint32_t v[kStagedUnroll];
-#pragma unroll
-      for (int u = 0; u < kStagedUnroll; ++u) {
-        const uint32_t w = w0 + u * kRow;
-        v[u] = (loaded && w < W) ? src[w] : 0u;
-      }
-#pragma unroll
-      for (int u = 0; u < kStagedUnroll; ++u) {
-        const uint32_t w = w0 + u * kRow;
-        if (w >= W) continue;
-        float4 fv;
-        fv.x = unit_f32(byte_f(v[u], 0), c.r1, c.r2);
-        fv.y = unit_f32(byte_f(v[u], 1), c.r1, c.r2);
-        fv.z = unit_f32(byte_f(v[u], 2), c.r1, c.r2);
-        fv.w = unit_f32(byte_f(v[u], 3), c.r1, c.r2);
-        if (dobs) st_stream(dobs + w, zo ? zero4 : fv, pol);
-        if (dnext) st_stream(dnext + w, zn ? zero4 : fv, pol);
-      }
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&sm.empty[st]);
-  }
-}
-
-__global__ void __launch_bounds__(kStagedThreads)
-k_deliver_stack_staged(Common c, StackArgs a, uint32_t npieces, uint32_t piece) {
-  __shared__ StageSmem sm;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < kStages; ++i) {
-      mbar_init(&sm.full[i], 1);
-      mbar_init(&sm.empty[i], kStageWarps);
-    }
-    mbar_init_fence();
-  }
-  __syncthreads();
-  const uint64_t pol = policy_stream();
-  pdl_wait();
-  pdl_launch();
-  const uint64_t units = (uint64_t)c.B * a.U * npieces;
-  const uint64_t nmine =
-      units > blockIdx.x ? (units - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  if (warp == 0)
-    stage_producer(c, a, sm, npieces, piece, nmine, lane, pol);
-  else if (warp == 1)
-    collate_strided(c, blockIdx.x, gridDim.x, lane);
-  else
-    stage_consumer(c, a, sm, npieces, piece, nmine, warp - 2, lane, pol);
+  const uint64_t f = ((uint64_t)(blockIdx.x - a.ncollate) * kWarps + warp) * (32 * UN);
+  if (f < total) stack_span<UN>(c, a, f, min(total, f + 32 * UN), lane, pol);
 }
 
 // ---------------------------------------------------------------------------
@@ -822,25 +600,15 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     a.obs = (float *)out->obs;
     a.next = (float *)out->next_obs;
     a.U = a.K + (a.next ? 1 : 0);
-    // equal pieces: the fewest that divide the frame's 16-byte runs and fit
-    // a stage
-    const uint32_t runs = a.F / 16;
-    uint32_t np = (a.F + kPiece - 1) / kPiece;
-    while (runs % np) ++np;
-    const uint64_t staged_units = (uint64_t)B * a.U * np;
-    const uint64_t staged_grid = (uint64_t)kStagedPerSm * sms;
-    if (staged_units >= 2 * staged_grid) {
-      return launch_pdl(k_deliver_stack_staged, dim3((unsigned)staged_grid),
-                        dim3(kStagedThreads), s, c, a, np, a.F / np);
-    }
-    // a small batch: one span of one unrolled iteration per warp, one chunk
-    // per CTA, and the collate CTA
-    a.span = 32 * kStackUnroll;
-    const uint64_t units = (uint64_t)B * a.U * a.W;
-    const uint64_t chunks = (units + (uint64_t)kWarps * a.span - 1) / ((uint64_t)kWarps * a.span);
-    if (chunks + 1 > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    return launch_pdl(k_deliver_stack<kStackUnroll>, dim3((unsigned)(chunks + 1)),
-                      dim3(kThreads), s, c, a);
+    a.ncollate = (uint32_t)(((uint64_t)B + kCollateThreads - 1) / kCollateThreads);
+    if (a.ncollate > kCollateCtas) a.ncollate = kCollateCtas;
+    const uint64_t per = (uint64_t)a.U * a.W, units = B * per;
+    const bool few = units <= (uint64_t)kWarps * 32 * 4 * sms;
+    const uint64_t each = (uint64_t)kWarps * 32 * (few ? 4 : 8);
+    const uint64_t ctas = (units + each - 1) / each + a.ncollate;
+    if (ctas > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    auto kern = few ? k_deliver_stack<4> : k_deliver_stack<8>;
+    return launch_pdl(kern, dim3((unsigned)ctas), dim3(kThreads), s, c, a);
   } else if (cfg.transform == EDP_XFORM_HWC_CHW_BF16) {
     ChwArgs a{};
     a.obs = ctx->st.obs;
