@@ -37,6 +37,7 @@ constexpr int kNormUnroll = 6;
 // unrolled rows per warp iteration and iterations per warp (chunk span) of
 // each kernel
 constexpr int kStackMinBlocks = 5;  // __launch_bounds__: at most 48 registers
+constexpr int kFlatMinBlocks = 6;   // at most 40
 constexpr int kHwcUnroll = 2, kHwcIters = 2;
 constexpr int kNormIters = 2;
 
@@ -342,6 +343,133 @@ k_deliver_stack(Common c, StackArgs a) {
 }
 
 // ---------------------------------------------------------------------------
+// Frame stack, float32, as one flat range of words: a CTA takes `words`
+// consecutive words of the batch's units (frame m of sample k, as above),
+// whatever frames and samples they belong to, a lane per word and
+// kFlatUnroll loads in flight, so a 128-byte frame fills a warp's access as
+// well as a large one.  The samples it touches are resolved first, a thread
+// each: index -> slot, into shared memory.  Then every thread issues its
+// first loads, and the resolving threads load the K episode flags of their
+// sample beside them and leave the masks of the frames that are zero in obs
+// and in next_obs; a sample's chain is paid once per CTA and not once per
+// frame.  The first `ncollate` CTAs collate the batch.
+//
+// Taken for frames below kFlatFrame bytes, where a span of k_deliver_stack
+// crosses several frames and walks them in turn.  Calls in a row, 32,768
+// samples, in us, here and (k_deliver_stack): 8x16, 1 frame and its
+// successor, 13.5 (120: with 4 loads per lane); 20x20, 4 and their
+// successors, 85 (97.5); 28x28, 4 and their successors, 159 (144).
+// ---------------------------------------------------------------------------
+constexpr uint32_t kFlatFrame = 768;
+constexpr int kFlatUnroll = 4;
+constexpr uint32_t kFlatSamples = kThreads;  // at most touched by a CTA
+struct FlatArgs {
+  uint32_t words;           // per CTA
+  uint32_t per;             // words per sample (U * W)
+  uint32_t div_per, div_w;  // ceil(2^32 / per), ceil(2^32 / W)
+};
+
+__global__ void __launch_bounds__(kThreads, kFlatMinBlocks)
+k_deliver_stack_flat(Common c, StackArgs a, FlatArgs g) {
+  __shared__ uint64_t s_pos[kFlatSamples];    // unwrapped slot of the anchor
+  __shared__ int s_lim[kFlatSamples];         // frames back from the anchor that exist
+  __shared__ uint32_t s_zo[kFlatSamples], s_zn[kFlatSamples];  // bit m: frame m is zero
+  const uint64_t pol = policy_stream();
+  // words [w0, w0 + nw) of the batch; the first is word i_0 of sample k0
+  const uint64_t total = (uint64_t)c.B * g.per;
+  const uint64_t w0 = (uint64_t)(blockIdx.x - a.ncollate) * g.words;
+  const uint64_t k0 = w0 / g.per;
+  const uint32_t i_0 = (uint32_t)(w0 - k0 * g.per);
+  const uint32_t i_1 = i_0 + (uint32_t)min((uint64_t)g.words, total - w0);
+  pdl_wait();
+  pdl_launch();
+  if (blockIdx.x < a.ncollate) {
+    collate_batch(c, blockIdx.x, a.ncollate);
+    return;
+  }
+  const uint32_t ns = (i_1 - 1) / g.per + 1;  // samples touched
+  bool ok = false;
+  uint64_t pos = 0, off = 0;
+  if (threadIdx.x < ns) {
+    uint64_t slot = 0;
+    ok = sample_slot(c, (uint32_t)(k0 + threadIdx.x), &slot, &off, false);
+    pos = c.oldest + off;
+    s_pos[threadIdx.x] = pos;
+    s_lim[threadIdx.x] = ok ? (int)min(off, (uint64_t)a.K) + 1 : -1;
+  }
+  __syncthreads();
+  // word i of sample k0's range: i * per < 2^32, so the rounded-up
+  // reciprocals give the exact quotients
+  uint32_t v[kFlatUnroll];
+  auto load = [&](uint32_t i, bool masked) -> uint32_t {
+    if (i >= i_1) return 0u;
+    const uint32_t s = __umulhi(i, g.div_per), rem = i - s * g.per;
+    const uint32_t m = __umulhi(rem, g.div_w);
+    if ((int)(a.K - 1) - (int)m >= s_lim[s]) return 0u;  // precedes the oldest, or a bad slot
+    if (masked && ((s_zo[s] & s_zn[s]) >> m) & 1u) return 0u;
+    const uint64_t js = s_pos[s] - (a.K - 1) + m;
+    return ld_stream(reinterpret_cast<const uint32_t *>(
+                         a.frames + (js >= c.cap ? js - c.cap : js) * a.F) + (rem - m * a.W),
+                     pol);
+  };
+#pragma unroll
+  for (int u = 0; u < kFlatUnroll; ++u)
+    v[u] = load(i_0 + threadIdx.x + u * kThreads, false);
+  if (threadIdx.x < ns) {
+    uint32_t ends = 0;  // bit i: an episode ends at offset off - K + 1 + i
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const uint32_t back = a.K - 1 - i;
+      if ((uint32_t)i < a.K && ok && off >= back) {
+        const uint64_t ps = pos - back;
+        ends |= (c.done[ps >= c.cap ? ps - c.cap : ps] != 0 ? 1u : 0u) << i;
+      }
+    }
+    // a frame is zero in obs when it precedes the oldest transition or an
+    // episode ends between it and the anchor; in next_obs also when one ends
+    // at the anchor; the anchor's successor (m = K) only with the sample
+    const bool end_at = (ends >> (a.K - 1)) & 1u;
+    uint32_t zo = 0, zn = (ok ? 0u : 1u) << a.K;
+    bool before = false;
+    for (int m = (int)a.K - 1; m >= 0; --m) {
+      if (m < (int)a.K - 1) before |= (ends >> m) & 1u;
+      const bool z = !ok || before || off < a.K - 1 - (uint32_t)m;
+      zo |= (z ? 1u : 0u) << m;
+      zn |= (z || end_at ? 1u : 0u) << m;
+    }
+    s_zo[threadIdx.x] = zo | 1u << a.K;  // the successor is no part of obs,
+    s_zn[threadIdx.x] = a.next ? zn | 1u : ~0u;  // nor the first frame of next_obs
+  }
+  __syncthreads();
+  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (uint32_t i0 = i_0 + threadIdx.x; i0 < i_1; i0 += kThreads * kFlatUnroll) {
+    if (i0 != i_0 + threadIdx.x) {
+#pragma unroll
+      for (int u = 0; u < kFlatUnroll; ++u) v[u] = load(i0 + u * kThreads, true);
+    }
+#pragma unroll
+    for (int u = 0; u < kFlatUnroll; ++u) {
+      const uint32_t i = i0 + u * kThreads;
+      if (i >= i_1) continue;
+      const uint32_t s = __umulhi(i, g.div_per), rem = i - s * g.per;
+      const uint32_t m = __umulhi(rem, g.div_w), w = rem - m * a.W;
+      const uint64_t frame = (k0 + s) * a.K + m;
+      float4 fv;
+      fv.x = unit_f32(byte_f(v[u], 0), c.r1, c.r2);
+      fv.y = unit_f32(byte_f(v[u], 1), c.r1, c.r2);
+      fv.z = unit_f32(byte_f(v[u], 2), c.r1, c.r2);
+      fv.w = unit_f32(byte_f(v[u], 3), c.r1, c.r2);
+      if (m < a.K)
+        st_stream(reinterpret_cast<float4 *>(a.obs) + frame * a.W + w,
+                  (s_zo[s] >> m) & 1u ? zero4 : fv, pol);
+      if (a.next && m >= 1)
+        st_stream(reinterpret_cast<float4 *>(a.next) + (frame - 1) * a.W + w,
+                  (s_zn[s] >> m) & 1u ? zero4 : fv, pol);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // HWC uint8 -> CHW bfloat16 (on-policy mini-batches).  Unit = 8 pixels: a lane
 // converts 8 consecutive pixels: it loads their 8*C interleaved bytes and
 // writes C 16-byte runs, one per channel plane.
@@ -603,6 +731,22 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     a.ncollate = (uint32_t)(((uint64_t)B + kCollateThreads - 1) / kCollateThreads);
     if (a.ncollate > kCollateCtas) a.ncollate = kCollateCtas;
     const uint64_t per = (uint64_t)a.U * a.W, units = B * per;
+    if (a.F < kFlatFrame) {
+      FlatArgs g{};
+      g.per = (uint32_t)per;  // at most 17 frames: words * per < 2^32
+      // 1,024 words (one round of loads), up to 4,096 while every SM keeps
+      // eight CTAs: 8x16, 4 frames and successors, 512 stacks 3.6 / 5.0 / 7.5 us
+      // with 1,024 / 2,048 / 4,096 words, 16x16, 32,768 stacks 64 / 58 / 56 us
+      g.words = 1024;
+      while (g.words < 4096 && units / (2 * g.words) >= 8ull * sms) g.words *= 2;
+      if (g.words > (kFlatSamples - 2) * per)
+        g.words = (uint32_t)((kFlatSamples - 2) * per) & ~31u;
+      g.div_per = (uint32_t)((0x100000000ull + per - 1) / per);
+      g.div_w = (uint32_t)((0x100000000ull + a.W - 1) / a.W);
+      const uint64_t ctas = (units + g.words - 1) / g.words + a.ncollate;
+      if (ctas > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+      return launch_pdl(k_deliver_stack_flat, dim3((unsigned)ctas), dim3(kThreads), s, c, a, g);
+    }
     const bool few = units <= (uint64_t)kWarps * 32 * 4 * sms;
     const uint64_t each = (uint64_t)kWarps * 32 * (few ? 4 : 8);
     const uint64_t ctas = (units + each - 1) / each + a.ncollate;

@@ -2,8 +2,10 @@
 do not divide a warp's span of 128 or 256 words (one 16-byte run more or
 less, primes and squares of primes of runs), with and without successors,
 stacks of 1 to 16, batches on both sides of the kernel's change of span and
-past a multiple of the samples a collating CTA takes; importance weights on
-the prioritized ones."""
+past a multiple of the samples a collating CTA takes; and small frames, which
+take the flat kernel (the smallest, whose CTA touches as many samples as it
+can, and the largest, on either side of its two larger ranges of words);
+importance weights on the prioritized ones."""
 import numpy as np
 import pytest
 import torch
@@ -17,6 +19,9 @@ pytestmark = pytest.mark.gpu
     (4, 1792, 3, True, 129), (4, 1796, 3, True, 400), (92, 92, 3, False, 400),
     (116, 116, 2, True, 60), (16, 1361, 1, False, 97), (16, 64, 4, True, 513),
     (16, 65, 16, True, 70), (32, 32, 1, False, 3000), (4, 260, 5, False, 1),
+    (4, 4, 1, False, 777), (4, 4, 1, True, 20_000), (4, 4, 16, True, 65), (8, 16, 4, True, 5),
+    (4, 36, 3, False, 40_001), (8, 16, 2, True, 50_000), (4, 188, 16, True, 33),
+    (16, 48, 4, True, 1001),
 ])
 def test_frame_sizes(edp_lib, orc, h, w, K, nxt, B):
     edp = edp_lib
