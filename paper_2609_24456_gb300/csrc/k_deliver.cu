@@ -38,7 +38,6 @@ constexpr int kNormUnroll = 6;
 // each kernel
 constexpr int kStackMinBlocks = 5;  // __launch_bounds__: at most 48 registers
 constexpr int kFlatMinBlocks = 6;   // at most 40
-constexpr int kHwcUnroll = 2, kHwcIters = 2;
 constexpr int kNormIters = 2;
 
 struct Common {
@@ -168,10 +167,14 @@ __device__ __forceinline__ uint32_t batch_qmin_cta(const Common &c) {
 // Collate, importance weights and index reporting of the batch by CTA `cta`
 // of `ncta`, a sample per thread of its first kCollateThreads (one warp for
 // each fp64 pipe of the SM), so that the streaming CTAs carry no collate
-// latency.  Each CTA takes q_min over the whole batch, so there are at most
-// kCollateCtas.
+// latency.  With weights each CTA takes q_min over the whole batch, so there
+// are then at most kCollateCtas.
 constexpr uint32_t kCollateThreads = 128;
 constexpr uint32_t kCollateCtas = 256;
+uint32_t collate_ctas(uint32_t B, bool weights) {
+  const uint32_t n = B / kCollateThreads + (B % kCollateThreads != 0);
+  return weights && n > kCollateCtas ? kCollateCtas : n;
+}
 __device__ void collate_batch(const Common &c, uint32_t cta, uint32_t ncta) {
   const uint32_t m = c.isw ? batch_qmin_cta(c) : 0xffffffffu;
   if (threadIdx.x >= kCollateThreads) return;
@@ -472,76 +475,108 @@ k_deliver_stack_flat(Common c, StackArgs a, FlatArgs g) {
 // ---------------------------------------------------------------------------
 // HWC uint8 -> CHW bfloat16 (on-policy mini-batches).  Unit = 8 pixels: a lane
 // converts 8 consecutive pixels: it loads their 8*C interleaved bytes and
-// writes C 16-byte runs, one per channel plane.
+// writes C 16-byte runs, one per channel plane.  A CTA takes `units`
+// consecutive units of the batch, whatever images they belong to: a thread
+// per image it touches resolves the slot into shared memory, then all threads
+// stream the units as one flat range, UN * C loads in flight each, so that
+// images of any size fill a warp.  The first `ncollate` CTAs collate the batch.
+// Bound by HBM; calls in a row, in us, and (before) when a warp walked its
+// span image by image and collated at each: 8x16x1, 65,536 images 5.6 (20.3),
+// 512 images 2.1 (4.9); 16x16x3, 65,536 24.6 (30.1); 64x64x3, 4,096 24.9
+// (25.2), 65,536 352 (353); 84x84x4, 16,384 203 (207).
 // ---------------------------------------------------------------------------
 struct ChwArgs {
   const uint8_t *obs;
   uint32_t HW;   // pixels per image
+  uint32_t units;  // per CTA
+  uint32_t div_g;  // ceil(2^32 / G), G = HW / 8; 0: a CTA spans at most two images
+  uint32_t ncollate;
   __nv_bfloat16 *out;
 };
+constexpr uint32_t kHwcImages = kThreads;  // at most touched by a CTA
 
 template <int C, int UN>
 __global__ void __launch_bounds__(kThreads)
 k_deliver_hwc(Common c, ChwArgs a) {
-  const int lane = threadIdx.x & 31;
+  __shared__ uint64_t s_slot[kHwcImages];  // ~0: a bad index
   const uint64_t pol = policy_stream();
+  const uint32_t G = a.HW / 8;  // 8-pixel groups per image
+  const uint64_t F = (uint64_t)a.HW * C;
+  // units [u0, u0 + n) of the batch; the first is unit i_0 of image k0
+  const uint64_t total = (uint64_t)c.B * G;
+  const uint64_t u0 = (uint64_t)(blockIdx.x - a.ncollate) * a.units;
+  const uint64_t k0 = u0 / G;
+  const uint32_t i_0 = (uint32_t)(u0 - k0 * G);
+  const uint32_t i_1 = i_0 + (uint32_t)min((uint64_t)a.units, total - u0);
   pdl_wait();
   pdl_launch();
-  const uint32_t G = a.HW / 8;  // 8-pixel groups per image
-  const uint64_t total = (uint64_t)c.B * G;
-  const uint64_t F = (uint64_t)a.HW * C;
-  uint64_t f, end;
-  warp_span(total, &f, &end);
-  while (f < end) {
-    const uint32_t k = (uint32_t)(f / G);
-    const uint32_t g_lo = (uint32_t)(f - (uint64_t)k * G);
-    const uint64_t seg_end = min(end, (uint64_t)(k + 1) * G);
-    const uint32_t g_hi = (uint32_t)(seg_end - (uint64_t)k * G);
-    const bool head = g_lo == 0;
+  if (blockIdx.x < a.ncollate) {
+    collate_batch(c, blockIdx.x, a.ncollate);
+    return;
+  }
+  if (threadIdx.x <= (i_1 - 1) / G) {
     uint64_t slot = 0, off = 0;
-    const bool ok = sample_slot(c, k, &slot, &off, head && lane == 0);
-    if (head) collate(c, k, ok, slot, off, lane);
-    const uint2 *src = reinterpret_cast<const uint2 *>(a.obs + slot * F);
-    uint4 *dst = reinterpret_cast<uint4 *>(a.out + (uint64_t)k * F);
-    for (uint32_t g0 = g_lo + lane; g0 < g_hi; g0 += 32 * UN) {
-      uint2 v[UN][C];
+    s_slot[threadIdx.x] =
+        sample_slot(c, (uint32_t)(k0 + threadIdx.x), &slot, &off, false) ? slot : ~0ull;
+  }
+  __syncthreads();
+  for (uint32_t i0 = i_0 + threadIdx.x; i0 < i_1; i0 += kThreads * UN) {
+    uint2 v[UN][C];
 #pragma unroll
-      for (int u = 0; u < UN; ++u) {
-        const uint32_t g = g0 + u * 32;
+    for (int u = 0; u < UN; ++u) {
+      const uint32_t i = i0 + u * kThreads;
+      // i * G < 2^32, so the rounded-up reciprocal gives the exact quotient
+      const uint32_t s = a.div_g ? __umulhi(i, a.div_g) : (i >= G ? 1u : 0u);
+      const uint64_t slot = i < i_1 ? s_slot[s] : ~0ull;
+      const uint2 *src = reinterpret_cast<const uint2 *>(a.obs + slot * F) +
+                         (uint64_t)(i - s * G) * C;
 #pragma unroll
-        for (int q = 0; q < C; ++q)
-          v[u][q] = (ok && g < g_hi) ? ld_stream(src + (uint64_t)g * C + q, pol)
-                                     : make_uint2(0u, 0u);
+      for (int q = 0; q < C; ++q)
+        v[u][q] = slot != ~0ull ? ld_stream(src + q, pol) : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int u = 0; u < UN; ++u) {
+      const uint32_t i = i0 + u * kThreads;
+      if (i >= i_1) continue;
+      const uint32_t s = a.div_g ? __umulhi(i, a.div_g) : (i >= G ? 1u : 0u);
+      uint4 *dst = reinterpret_cast<uint4 *>(a.out + (k0 + s) * F) + (i - s * G);
+      uint32_t wd[2 * C];
+#pragma unroll
+      for (int q = 0; q < C; ++q) {
+        wd[2 * q] = v[u][q].x;
+        wd[2 * q + 1] = v[u][q].y;
       }
 #pragma unroll
-      for (int u = 0; u < UN; ++u) {
-        const uint32_t g = g0 + u * 32;
-        if (g >= g_hi) continue;
-        uint32_t wd[2 * C];
+      for (int ch = 0; ch < C; ++ch) {
+        float fv[8];
 #pragma unroll
-        for (int q = 0; q < C; ++q) {
-          wd[2 * q] = v[u][q].x;
-          wd[2 * q + 1] = v[u][q].y;
+        for (int px = 0; px < 8; ++px) {
+          const int byte = px * C + ch;  // position within the 8*C bytes
+          fv[px] = unit_f32(byte_f(wd[byte >> 2], byte & 3), c.r1, c.r2);
         }
-#pragma unroll
-        for (int ch = 0; ch < C; ++ch) {
-          float fv[8];
-#pragma unroll
-          for (int px = 0; px < 8; ++px) {
-            const int byte = px * C + ch;  // position within the 8*C bytes
-            fv[px] = unit_f32(byte_f(wd[byte >> 2], byte & 3), c.r1, c.r2);
-          }
-          uint4 o;
-          o.x = pack_bf16x2(fv[0], fv[1]);
-          o.y = pack_bf16x2(fv[2], fv[3]);
-          o.z = pack_bf16x2(fv[4], fv[5]);
-          o.w = pack_bf16x2(fv[6], fv[7]);
-          st_stream(dst + (uint64_t)ch * G + g, o, pol);
-        }
+        uint4 o;
+        o.x = pack_bf16x2(fv[0], fv[1]);
+        o.y = pack_bf16x2(fv[2], fv[3]);
+        o.z = pack_bf16x2(fv[4], fv[5]);
+        o.w = pack_bf16x2(fv[6], fv[7]);
+        st_stream(dst + (uint64_t)ch * G, o, pol);
       }
     }
-    f = seg_end;
   }
+}
+
+// One round of UN units per thread: longer ranges (up to 4,096 units while an
+// SM keeps 8 CTAs) were equal on small images and 3-6% slower on large batches.
+template <int C, int UN>
+cudaError_t launch_hwc(const Common &c, ChwArgs a, cudaStream_t s) {
+  const uint64_t G = a.HW / 8, total = c.B * G;
+  uint64_t units = (uint64_t)kThreads * UN;
+  if (units > (kHwcImages - 2) * G) units = ((kHwcImages - 2) * G) & ~31ull;
+  a.units = (uint32_t)units;
+  a.div_g = G < 32768 ? (uint32_t)((0x100000000ull + G - 1) / G) : 0u;
+  const uint64_t ctas = (total + units - 1) / units + a.ncollate;
+  if (ctas > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+  return launch_pdl(k_deliver_hwc<C, UN>, dim3((unsigned)ctas), dim3(kThreads), s, c, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -728,8 +763,7 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     a.obs = (float *)out->obs;
     a.next = (float *)out->next_obs;
     a.U = a.K + (a.next ? 1 : 0);
-    a.ncollate = (uint32_t)(((uint64_t)B + kCollateThreads - 1) / kCollateThreads);
-    if (a.ncollate > kCollateCtas) a.ncollate = kCollateCtas;
+    a.ncollate = collate_ctas(B, out->isw != nullptr);
     const uint64_t per = (uint64_t)a.U * a.W, units = B * per;
     if (a.F < kFlatFrame) {
       FlatArgs g{};
@@ -758,29 +792,12 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     a.obs = ctx->st.obs;
     a.HW = cfg.obs_h * cfg.obs_w;
     a.out = (__nv_bfloat16 *)out->obs;
-    const uint64_t units = (uint64_t)B * (a.HW / 8);
-    constexpr uint64_t it = 32 * kHwcUnroll;
+    a.ncollate = collate_ctas(B, out->isw != nullptr);
     switch (cfg.obs_c) {
-      case 1: {
-        auto kern = k_deliver_hwc<1, kHwcUnroll>;
-        return launch_pdl(kern, dim3(grid_for(kern, units, it, kHwcIters, sms)),
-                          dim3(kThreads), s, c, a);
-      }
-      case 2: {
-        auto kern = k_deliver_hwc<2, kHwcUnroll>;
-        return launch_pdl(kern, dim3(grid_for(kern, units, it, kHwcIters, sms)),
-                          dim3(kThreads), s, c, a);
-      }
-      case 3: {
-        auto kern = k_deliver_hwc<3, kHwcUnroll>;
-        return launch_pdl(kern, dim3(grid_for(kern, units, it, kHwcIters, sms)),
-                          dim3(kThreads), s, c, a);
-      }
-      default: {
-        auto kern = k_deliver_hwc<4, kHwcUnroll>;
-        return launch_pdl(kern, dim3(grid_for(kern, units, it, kHwcIters, sms)),
-                          dim3(kThreads), s, c, a);
-      }
+      case 1: return launch_hwc<1, 4>(c, a, s);
+      case 2: return launch_hwc<2, 2>(c, a, s);
+      case 3: return launch_hwc<3, 2>(c, a, s);
+      default: return launch_hwc<4, 2>(c, a, s);
     }
   } else {
     NormArgs a{};
