@@ -239,6 +239,8 @@ edp_status edp::update_args(edp_ctx *ctx, const char *who, const int64_t *idx,
 
 namespace {
 
+constexpr size_t kLeastScratch = 4096;
+
 // Grow-only block (*blk, *have bytes) to at least `want` bytes; the first
 // `zero_head` bytes of a new block are zeroed.
 cudaError_t grow(edp_ctx *ctx, void **blk, size_t *have, size_t want, size_t zero_head,
@@ -274,6 +276,9 @@ cudaError_t grow(edp_ctx *ctx, void **blk, size_t *have, size_t want, size_t zer
 }  // namespace
 
 cudaError_t edp::ctx_scratch(edp_ctx *ctx, size_t bytes, cudaStream_t s, void **out) {
+  // at least a pair of sums per SM for any GPU this is built for, so that no
+  // call of few environments needs more than another call made room for
+  if (bytes < kLeastScratch) bytes = kLeastScratch;
   const cudaError_t e = grow(ctx, &ctx->scratch, &ctx->scratch_bytes, bytes, 0, s);
   *out = ctx->scratch;
   return e;

@@ -6,11 +6,16 @@
 //   A_t = delta_t + c_t A_{t+1},  c_t = gamma lambda (1 - d_t),  A_T = 0
 //
 // The recurrence is a composition of affine maps x -> b + a x, which is
-// associative, so one warp scans one environment's T steps in parallel:
-// each lane composes the maps of J consecutive steps, a warp-shuffle suffix
-// scan composes lanes (5 levels), and each lane then replays its own steps
-// from the value handed over by its right neighbour.  Chunks of 32*J steps
-// are processed from the end of the rollout backwards, carrying A across.
+// associative, so a CTA scans kE environments' steps in parallel: thread
+// (s, e) composes the maps of kL consecutive steps of environment e (segment
+// s), shuffles compose the segments of a warp, the warps' composites meet in
+// shared memory, and each thread then replays its own steps from the value
+// handed over by the later ones.  Chunks of as many steps as the CTA holds
+// (2,048 / kE at most) are processed from the end of the rollout backwards,
+// carrying A across; the next chunk's inputs are loaded beside a chunk's
+// arithmetic.  With kE = 8 every access of a time-major row moves whole
+// 32-byte sectors; long rollouts of few environments use fewer environments
+// per CTA, so that more SMs and longer chunks share the steps (gae_shape).
 //
 // Arithmetic: GB300's fp64 pipe is narrow (a dependent fp64 FMA costs ~64
 // cycles, fp32 ~4), so the scan -- and each lane's sums of A and A^2 over an
@@ -19,14 +24,24 @@
 // error-free transformations TwoSum (Knuth) and TwoProd via FMA (Dekker),
 // as in the double-double arithmetic of Hida, Li and Bailey -- which keeps
 // ~44 significant bits (relative error ~2^-44 per operation); gamma and
-// gamma*lambda enter as pairs split from fp64.  Only the mean / variance
-// reduction and the normalisation use fp64.  Outputs are rounded to fp32.
+// gamma*lambda enter as pairs split from fp64.  The mean and the variance
+// are formed in fp64 from the CTAs' sums; the normalisation of an element is
+// double-float again (as many bits as its fp32 result can show: its error
+// against 64 bits is the rounding's), fp64 where a value is out of its range.
+// Outputs are rounded to fp32.
+//
+// Bound by latency (a chunk's loads, then its dependent chain) up to ~10^6
+// values, then by HBM.  Calls in a row with all three outputs, in us, and
+// (before) with one warp per environment: 8 x 2,048 steps 13.8 (43.0), 4,096 x
+// 64 14.5 (28.4), 1,024 x 1,024 29.9 (107), 64 x 8,192 44.6 (557), 8 x 128 8.0
+// (9.2).
 //
 // Two kernels chained with programmatic dependent launch: the scan writes A,
-// the returns and per-CTA fp64 sums of A and A^2; the normalisation kernel
+// the returns and per-CTA sums of A and A^2; the normalisation kernel
 // forms mean and the unbiased standard deviation (every CTA reduces the
 // partials in the same fixed order, so all agree bit for bit) and writes
-// the normalised values, one thread per element.  With the environments
+// the normalised values; a rollout that one CTA scans in at most two chunks is
+// normalised by it, without a second kernel.  With the environments
 // sharded over several ranks, the scan's sums are reduced to this rank's
 // (n, sum A, sum A^2) instead (k_gae_stats), the caller sums those over the
 // ranks, and the normalisation reads the totals.
@@ -36,127 +51,189 @@ namespace edp {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kJ = 4;          // steps per lane per chunk
-constexpr int kGaeWarps = 4;   // environments per CTA
-constexpr int kGaeThreads = kGaeWarps * 32;
+constexpr int kL = 4;               // steps per thread and chunk
+constexpr int kGaeThreads = 512;    // at most per CTA
+constexpr int kGaeWarps = kGaeThreads / 32;
 constexpr int kNormThreads = 256;
 
 __device__ __forceinline__ df df_shfl_down(df a, int o) {
   return {__shfl_down_sync(kFull, a.hi, o), __shfl_down_sync(kFull, a.lo, o)};
 }
-// One environment's scan (one warp): writes its advantages and returns and
-// adds this lane's A and A^2 to s1, s2.
-__device__ __forceinline__ void gae_env(const float *__restrict__ r,
-                                        const float *__restrict__ v,
-                                        const uint8_t *__restrict__ d, uint32_t T, uint32_t E,
-                                        uint32_t e, df g, df gl, float *__restrict__ A_out,
-                                        float *__restrict__ ret, double &s1, double &s2) {
-  const int lane = threadIdx.x & 31;
-  const df one = {1.f, 0.f}, zero = {0.f, 0.f};
-  // this lane's A and A^2 summed in double-float (the fp32 pipe), added to
-  // the fp64 accumulators once per environment
-  df a1 = zero, a2 = zero;
-  df carry = zero;  // A at the step after the current chunk
-  for (int64_t te = T; te > 0; te -= 32 * kJ) {
-    const int64_t ts = te - 32 * kJ > 0 ? te - 32 * kJ : 0;
-    df del[kJ], cc[kJ];
-    df a = one, b = zero;  // this lane's steps composed: x -> b + a x
-    // every input of the lane's steps is loaded before any is used, so
-    // the loads share one round trip
-    float rr[kJ], vv[kJ], vn[kJ];
-    bool dd[kJ];
-#pragma unroll
-    for (int i = 0; i < kJ; ++i) {
-      const int64_t t = ts + (int64_t)lane * kJ + i;
-      const uint64_t at = (uint64_t)(t < te ? t : ts) * E + e;
-      rr[i] = r[at];
-      vv[i] = v[at];
-      vn[i] = v[at + E];
-      dd[i] = d[at] != 0;
-    }
-#pragma unroll
-    for (int i = kJ - 1; i >= 0; --i) {
-      const int64_t t = ts + (int64_t)lane * kJ + i;
-      if (t < te) {
-        const bool dn = dd[i];
-        // delta = r + gamma V' (1 - d) - V
-        df x = dn ? df{rr[i], 0.f} : df_add_f(df_mul_f(g, vn[i]), rr[i]);
-        del[i] = df_add_f(x, -vv[i]);
-        cc[i] = dn ? zero : gl;
-        b = df_add(del[i], df_mul(cc[i], b));
-        a = df_mul(cc[i], a);
-      } else {
-        del[i] = zero;
-        cc[i] = one;
-      }
-    }
-    // inclusive suffix scan: lane l gets lanes l..31 composed
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const df a2 = df_shfl_down(a, o);
-      const df b2 = df_shfl_down(b, o);
-      if (lane + o < 32) {
-        b = df_add(b, df_mul(a, b2));
-        a = df_mul(a, a2);
-      }
-    }
-    const df an = df_shfl_down(a, 1);
-    const df bn = df_shfl_down(b, 1);
-    df A = lane < 31 ? df_add(bn, df_mul(an, carry)) : carry;  // A after my steps
-#pragma unroll
-    for (int i = kJ - 1; i >= 0; --i) {
-      const int64_t t = ts + (int64_t)lane * kJ + i;
-      if (t < te) {
-        A = df_add(del[i], df_mul(cc[i], A));
-        const uint64_t at = (uint64_t)t * E + e;
-        if (A_out) A_out[at] = A.hi;
-        if (ret) ret[at] = df_add_f(A, vv[i]).hi;
-        a1 = df_add(a1, A);
-        a2 = df_add(a2, df_mul(A, A));
-      }
-    }
-    const df c0 = df_add(b, df_mul(a, carry));
-    carry = {__shfl_sync(kFull, c0.hi, 0), __shfl_sync(kFull, c0.lo, 0)};
-  }
-  s1 += df_to_d(a1);
-  s2 += df_to_d(a2);
+
+// What the normalisation needs of the whole rollout.
+struct NormStat {
+  double mean, inv;      // inv = 1 / (std + 1e-8); 0 for a single value
+  df neg_mean, inv_df;
+  bool narrow;           // both within double-float's range
+};
+
+// From n values with sums s1 (of A) and s2 (of A^2).
+__device__ __forceinline__ NormStat norm_stat(double nn, double s1, double s2) {
+  NormStat st;
+  st.mean = s1 / nn;
+  double var = nn > 1.0 ? (s2 - s1 * st.mean) / (nn - 1.0) : 0.0;
+  if (var < 0.0) var = 0.0;
+  // a single value equals its mean and normalises to exactly 0; the scale
+  // is 0 so that the fp32 rounding of the stored A (A - mean ~ 2^-24 |A|
+  // here) is not multiplied by 1 / 1e-8
+  st.inv = nn > 1.0 ? 1.0 / (sqrt(var) + 1e-8) : 0.0;
+  st.neg_mean = df_split(-st.mean);
+  st.inv_df = df_split(st.inv);
+  st.narrow = fabs(st.mean) < 1e18 && st.inv > 1e-18 && st.inv < 1e18;
+  return st;
 }
 
+__device__ __forceinline__ float norm_value(float a, const NormStat &st) {
+  if (st.narrow && fabsf(a) < 1e18f) return df_mul(df_add_f(st.neg_mean, a), st.inv_df).hi;
+  return (float)(((double)a - st.mean) * st.inv);
+}
+
+// Inputs of one thread's kL steps t0 .. t0 + kL - 1 of environment e, and the
+// value after each (a step at or past te reads a valid one instead, a value
+// past te the one at te).
+struct GaeIn {
+  float r[kL], v[kL + 1];
+  bool d[kL];
+};
+__device__ __forceinline__ void gae_load(GaeIn &x, const float *__restrict__ r,
+                                         const float *__restrict__ v,
+                                         const uint8_t *__restrict__ d, uint64_t t0, uint64_t te,
+                                         uint32_t E, uint32_t e) {
+#pragma unroll
+  for (int i = 0; i < kL; ++i) {
+    const uint64_t at = min(t0 + i, te - 1) * E + e;
+    x.r[i] = r[at];
+    x.d[i] = d[at] != 0;
+  }
+#pragma unroll
+  for (int i = 0; i <= kL; ++i) x.v[i] = v[min(t0 + i, te) * E + e];
+}
+
+template <int kE>
 __global__ void __launch_bounds__(kGaeThreads)
 k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
            const uint8_t *__restrict__ d, uint32_t T, uint32_t E, double gamma,
-           double lambda, float *__restrict__ A_out, float *__restrict__ ret,
-           double *__restrict__ partial) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  pdl_wait();
+           double lambda, float *A_out, float *__restrict__ ret,
+           double *__restrict__ partial, float *adv_norm) {
+  __shared__ float4 agg[kGaeWarps][kE];  // a warp's composite: a.hi, a.lo, b.hi, b.lo
+  __shared__ float2 s_carry[kE];         // A at the step after the chunk
+  __shared__ float4 s_sum[kGaeWarps];
+  __shared__ NormStat s_stat;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nwarps = blockDim.x >> 5;
+  const uint32_t el = threadIdx.x % kE, seg = threadIdx.x / kE;
+  const uint32_t chunk = blockDim.x / kE * kL;
+  const df one = {1.f, 0.f}, zero = {0.f, 0.f};
   const df g = df_split(gamma);
   const df gl = df_split(gamma * lambda);
-  double s1 = 0.0, s2 = 0.0;
-  for (uint32_t e = blockIdx.x * kGaeWarps + wid; e < E; e += gridDim.x * kGaeWarps)
-    gae_env(r, v, d, T, E, e, g, gl, A_out, ret, s1, s2);
+  pdl_wait();
+  // this thread's A and A^2 summed in double-float (the fp32 pipe)
+  df a1 = zero, a2 = zero;
+  for (uint32_t tile = blockIdx.x; (uint64_t)tile * kE < E; tile += gridDim.x) {
+    const bool real = tile * kE + el < E;
+    const uint32_t e = real ? tile * kE + el : E - 1;
+    if (seg == 0) s_carry[el] = make_float2(0.f, 0.f);  // read after the barrier below
+    GaeIn x;
+    uint32_t te = T, ts = T > chunk ? T - chunk : 0;
+    gae_load(x, r, v, d, (uint64_t)ts + seg * kL, te, E, e);
+    for (;;) {
+      const uint64_t t0 = (uint64_t)ts + seg * kL;
+      const uint32_t te2 = ts, ts2 = ts > chunk ? ts - chunk : 0;
+      GaeIn next;
+      if (te2) gae_load(next, r, v, d, (uint64_t)ts2 + seg * kL, te2, E, e);
+      df del[kL], cc[kL];
+      df a = one, b = zero;  // this thread's steps composed: x -> b + a x
+#pragma unroll
+      for (int i = kL - 1; i >= 0; --i) {
+        if (t0 + i < te) {
+          // delta = r + gamma V' (1 - d) - V
+          const df y = x.d[i] ? df{x.r[i], 0.f} : df_add_f(df_mul_f(g, x.v[i + 1]), x.r[i]);
+          del[i] = df_add_f(y, -x.v[i]);
+          cc[i] = x.d[i] ? zero : gl;
+          b = df_add(del[i], df_mul(cc[i], b));
+          a = df_mul(cc[i], a);
+        } else {
+          del[i] = zero;
+          cc[i] = one;
+        }
+      }
+      // inclusive suffix scan over the warp's segments of each environment
+#pragma unroll
+      for (int o = kE; o < 32; o <<= 1) {
+        const df a2s = df_shfl_down(a, o);
+        const df b2s = df_shfl_down(b, o);
+        if (lane + o < 32) {
+          b = df_add(b, df_mul(a, b2s));
+          a = df_mul(a, a2s);
+        }
+      }
+      if (lane < kE) agg[warp][el] = make_float4(a.hi, a.lo, b.hi, b.lo);
+      __syncthreads();
+      // A at the step after this warp's last one
+      df A = {s_carry[el].x, s_carry[el].y};
+      for (int w = nwarps - 1; w > warp; --w) {
+        const float4 m = agg[w][el];
+        A = df_add(df{m.z, m.w}, df_mul(df{m.x, m.y}, A));
+      }
+      // ... and after this thread's
+      const df an = df_shfl_down(a, kE % 32), bn = df_shfl_down(b, kE % 32);
+      if (lane < 32 - kE) A = df_add(bn, df_mul(an, A));
+#pragma unroll
+      for (int i = kL - 1; i >= 0; --i) {
+        if (t0 + i < te) {
+          A = df_add(del[i], df_mul(cc[i], A));
+          if (real) {
+            const uint64_t at = (t0 + i) * E + e;
+            if (A_out) A_out[at] = A.hi;
+            if (ret) ret[at] = df_add_f(A, x.v[i]).hi;
+            a1 = df_add(a1, A);
+            a2 = df_add(a2, df_mul(A, A));
+          }
+        }
+      }
+      __syncthreads();  // agg and s_carry have been read
+      if (seg == 0) s_carry[el] = make_float2(A.hi, A.lo);
+      if (!te2) break;
+      x = next;
+      te = te2;
+      ts = ts2;
+    }
+  }
   pdl_launch();
-  if (!partial) return;  // no normalisation requested
-  // per-CTA partial sums (fixed order: warps, then lanes by xor tree)
-  __shared__ double ws1[kGaeWarps], ws2[kGaeWarps];
+  if (!partial && !adv_norm) return;  // no normalisation requested
+  // this CTA's sums in a fixed order: a shuffle tree per warp, then over the
+  // warps; fp64 from there on
 #pragma unroll
   for (int o = 16; o; o >>= 1) {
-    s1 += __shfl_xor_sync(kFull, s1, o);
-    s2 += __shfl_xor_sync(kFull, s2, o);
+    a1 = df_add(a1, df_shfl_down(a1, o));
+    a2 = df_add(a2, df_shfl_down(a2, o));
   }
-  if (lane == 0) {
-    ws1[wid] = s1;
-    ws2[wid] = s2;
-  }
+  if (lane == 0) s_sum[warp] = make_float4(a1.hi, a1.lo, a2.hi, a2.lo);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t1 = 0.0, t2 = 0.0;
-    for (int w = 0; w < kGaeWarps; ++w) {
-      t1 += ws1[w];
-      t2 += ws2[w];
+  if (warp == 0) {
+    const float4 m = lane < nwarps ? s_sum[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+    a1 = {m.x, m.y};
+    a2 = {m.z, m.w};
+#pragma unroll
+    for (int o = kGaeWarps / 2; o; o >>= 1) {
+      a1 = df_add(a1, df_shfl_down(a1, o));
+      a2 = df_add(a2, df_shfl_down(a2, o));
     }
-    partial[2 * blockIdx.x] = t1;
-    partial[2 * blockIdx.x + 1] = t2;
+    if (lane == 0) {
+      if (partial) {
+        partial[2 * blockIdx.x] = df_to_d(a1);
+        partial[2 * blockIdx.x + 1] = df_to_d(a2);
+      } else {
+        s_stat = norm_stat((double)((uint64_t)T * E), df_to_d(a1), df_to_d(a2));
+      }
+    }
   }
+  if (partial) return;
+  // one CTA scanned everything: it normalises what it wrote
+  __syncthreads();
+  const NormStat st = s_stat;
+  for (uint64_t i = threadIdx.x; i < (uint64_t)T * E; i += blockDim.x)
+    adv_norm[i] = norm_value(__ldcg(A_out + i), st);
 }
 
 // Sum of the per-CTA partials (sum A, sum A^2) in a fixed order: strided
@@ -199,19 +276,23 @@ k_gae_stats(const double *partial, uint32_t nparts, uint64_t n, double *stats) {
 
 // Normalisation: every CTA reduces the per-CTA partials of the scan in the
 // same fixed order (or reads the statistics (n, sum A, sum A^2) of all ranks
-// when `stats` is given), then one thread per element writes
-// (A - mean) * inv_std.  A is read from A_src (the caller's adv, or adv_norm
-// itself); n is the number of elements here.
+// when `stats` is given), then writes (A - mean) * inv_std, four elements per
+// thread and load where both arrays allow it.  A is read from A_src (the
+// caller's adv, or adv_norm itself); n is the number of elements here.
 __global__ void __launch_bounds__(kNormThreads)
 k_gae_norm(const float *A_src, float *adv_norm, uint64_t n, const double *partial,
            uint32_t nparts, const double *stats) {
   __shared__ double r1[kNormThreads], r2[kNormThreads];
-  __shared__ double stat[2];
+  __shared__ NormStat s_stat;
   pdl_wait();
   pdl_launch();
-  // this thread's first element, loaded beside the partial sums
+  // this thread's first elements, loaded beside the partial sums
+  const bool vec = (((uintptr_t)A_src | (uintptr_t)adv_norm) & 15u) == 0;
+  const uint64_t nv = vec ? n / 4 : 0;
   const uint64_t i0 = blockIdx.x * (uint64_t)kNormThreads + threadIdx.x;
-  const float a0 = i0 < n ? __ldcg(&A_src[i0]) : 0.f;
+  const uint64_t stride = (uint64_t)gridDim.x * kNormThreads;
+  const float4 *src = reinterpret_cast<const float4 *>(A_src);
+  float4 x = i0 < nv ? __ldcg(src + i0) : make_float4(0.f, 0.f, 0.f, 0.f);
   double nn = (double)n, s1, s2;
   if (stats) {
     nn = __ldcg(&stats[0]);
@@ -222,22 +303,58 @@ k_gae_norm(const float *A_src, float *adv_norm, uint64_t n, const double *partia
     s1 = r1[0];
     s2 = r2[0];
   }
-  if (threadIdx.x == 0) {
-    const double mean = s1 / nn;
-    double var = nn > 1.0 ? (s2 - s1 * mean) / (nn - 1.0) : 0.0;
-    if (var < 0.0) var = 0.0;
-    stat[0] = mean;
-    // a single value equals its mean and normalises to exactly 0; the scale
-    // is 0 so that the fp32 rounding of the stored A (A - mean ~ 2^-24 |A|
-    // here) is not multiplied by 1 / 1e-8
-    stat[1] = nn > 1.0 ? 1.0 / (sqrt(var) + 1e-8) : 0.0;
-  }
+  if (threadIdx.x == 0) s_stat = norm_stat(nn, s1, s2);
   __syncthreads();
-  const double mean = stat[0], inv = stat[1];
-  if (i0 < n) adv_norm[i0] = (float)(((double)a0 - mean) * inv);
-  for (uint64_t i = i0 + (uint64_t)gridDim.x * kNormThreads; i < n;
-       i += (uint64_t)gridDim.x * kNormThreads)
-    adv_norm[i] = (float)(((double)__ldcg(&A_src[i]) - mean) * inv);
+  const NormStat st = s_stat;
+  for (uint64_t i = i0; i < nv; i += stride) {
+    if (i != i0) x = __ldcg(src + i);
+    x = make_float4(norm_value(x.x, st), norm_value(x.y, st), norm_value(x.z, st),
+                    norm_value(x.w, st));
+    reinterpret_cast<float4 *>(adv_norm)[i] = x;
+  }
+  for (uint64_t i = 4 * nv + i0; i < n; i += stride)
+    adv_norm[i] = norm_value(__ldcg(&A_src[i]), st);
+}
+
+}  // namespace
+
+namespace {
+
+// Two sums per CTA: a CTA takes eight environments, or fewer while it makes
+// fewer CTAs than SMs, which the least scratch block (ctx_scratch) covers.
+size_t gae_scratch_bytes(uint32_t E) { return ((size_t)E + 3) / 4 * 2 * sizeof(double); }
+
+// Environments per CTA (8, halved while the rollout takes several chunks and
+// half of the SMs would idle), threads per CTA and CTAs of a scan.
+struct GaeShape {
+  uint32_t envs, threads, grid, chunks;
+};
+GaeShape gae_shape(const edp_ctx *c, uint32_t T, uint32_t E) {
+  GaeShape g;
+  g.envs = 8;
+  while (g.envs > 1 && T > kGaeThreads / g.envs * kL &&
+         2 * (((uint64_t)E + g.envs - 1) / g.envs) < (uint64_t)c->coop_sms)
+    g.envs /= 2;
+  const uint64_t want = ((uint64_t)T + kL - 1) / kL * g.envs;
+  g.threads = want < kGaeThreads ? (uint32_t)((want + 31) & ~31ull) : (uint32_t)kGaeThreads;
+  g.grid = (uint32_t)(((uint64_t)E + g.envs - 1) / g.envs);
+  const uint32_t chunk = g.threads / g.envs * kL;
+  g.chunks = T / chunk + (T % chunk != 0);
+  return g;
+}
+
+cudaError_t launch_scan(const GaeShape &g, const float *r, const float *v, const uint8_t *d,
+                        uint32_t T, uint32_t E, double gamma, double lambda, float *A_out,
+                        float *ret, double *partial, float *adv_norm, cudaStream_t s) {
+  auto kern = g.envs == 8 ? k_gae_scan<8> : g.envs == 4 ? k_gae_scan<4>
+            : g.envs == 2 ? k_gae_scan<2> : k_gae_scan<1>;
+  return launch_pdl(kern, dim3(g.grid), dim3(g.threads), s, r, v, d, T, E, gamma, lambda, A_out,
+                    ret, partial, adv_norm);
+}
+
+unsigned norm_grid(const edp_ctx *c, uint64_t n) {
+  const uint64_t most = 4ull * c->coop_sms, want = (n + 4 * kNormThreads - 1) / (4 * kNormThreads);
+  return (unsigned)(want < most ? want : most);
 }
 
 }  // namespace
@@ -246,49 +363,48 @@ cudaError_t launch_gae(edp_ctx *c, const float *r, const float *v,
                        const uint8_t *d, uint32_t T, uint32_t E, double gamma,
                        double lambda, float *adv, float *ret, float *adv_norm,
                        cudaStream_t s) {
-  const uint64_t grid = (E + kGaeWarps - 1) / kGaeWarps;
+  GaeShape g = gae_shape(c, T, E);
   double *partial = nullptr;
   if (adv_norm) {
     void *blk = nullptr;
-    const cudaError_t e = ctx_scratch(c, grid * 2 * sizeof(double), s, &blk);
+    const cudaError_t e = ctx_scratch(c, gae_scratch_bytes(E), s, &blk);
     if (e != cudaSuccess) return e;
     partial = (double *)blk;
   }
-  // A is kept between the kernels in adv, or in adv_norm itself (fp32; the
+  // A is kept for the normalisation in adv, or in adv_norm itself (fp32; the
   // normalisation error this adds is below 2^-24 |A| / std)
   float *A_out = adv ? adv : adv_norm;
-  cudaError_t e = launch_pdl(k_gae_scan, dim3((unsigned)grid), dim3(kGaeThreads), s,
-                             r, v, d, T, E, gamma, lambda, A_out, ret, partial);
+  if (adv_norm && (uint64_t)g.grid * g.chunks <= 2) {
+    g.grid = 1;
+    return launch_scan(g, r, v, d, T, E, gamma, lambda, A_out, ret, nullptr, adv_norm, s);
+  }
+  const cudaError_t e =
+      launch_scan(g, r, v, d, T, E, gamma, lambda, A_out, ret, partial, nullptr, s);
   if (e != cudaSuccess || !adv_norm) return e;
   const uint64_t n = (uint64_t)T * E;
-  uint64_t ng = (n + kNormThreads - 1) / kNormThreads;
-  if (ng > 4ull * c->coop_sms) ng = 4ull * c->coop_sms;
-  return launch_pdl(k_gae_norm, dim3((unsigned)ng), dim3(kNormThreads), s,
-                    (const float *)A_out, adv_norm, n, (const double *)partial,
-                    (uint32_t)grid, (const double *)nullptr);
+  return launch_pdl(k_gae_norm, dim3(norm_grid(c, n)), dim3(kNormThreads), s,
+                    (const float *)A_out, adv_norm, n, (const double *)partial, g.grid,
+                    (const double *)nullptr);
 }
 
 cudaError_t launch_gae_stats(edp_ctx *c, const float *r, const float *v,
                              const uint8_t *d, uint32_t T, uint32_t E, double gamma,
                              double lambda, float *adv, float *ret, double *stats,
                              cudaStream_t s) {
-  const uint64_t grid = (E + kGaeWarps - 1) / kGaeWarps;
+  const GaeShape g = gae_shape(c, T, E);
   void *blk = nullptr;
-  cudaError_t e = ctx_scratch(c, grid * 2 * sizeof(double), s, &blk);
+  cudaError_t e = ctx_scratch(c, gae_scratch_bytes(E), s, &blk);
   if (e != cudaSuccess) return e;
   double *partial = (double *)blk;
-  e = launch_pdl(k_gae_scan, dim3((unsigned)grid), dim3(kGaeThreads), s, r, v, d, T, E,
-                 gamma, lambda, adv, ret, partial);
+  e = launch_scan(g, r, v, d, T, E, gamma, lambda, adv, ret, partial, nullptr, s);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_gae_stats, dim3(1), dim3(kNormThreads), s, (const double *)partial,
-                    (uint32_t)grid, (uint64_t)T * E, stats);
+                    g.grid, (uint64_t)T * E, stats);
 }
 
 cudaError_t launch_gae_normalize(edp_ctx *c, const float *adv, uint64_t n,
                                  const double *stats, float *adv_norm, cudaStream_t s) {
-  uint64_t ng = (n + kNormThreads - 1) / kNormThreads;
-  if (ng > 4ull * c->coop_sms) ng = 4ull * c->coop_sms;
-  return launch_pdl(k_gae_norm, dim3((unsigned)ng), dim3(kNormThreads), s, adv, adv_norm, n,
+  return launch_pdl(k_gae_norm, dim3(norm_grid(c, n)), dim3(kNormThreads), s, adv, adv_norm, n,
                     (const double *)nullptr, 0u, stats);
 }
 

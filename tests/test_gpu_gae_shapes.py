@@ -1,0 +1,61 @@
+"""Advantages against the oracle at the shapes where the scan's split changes:
+one step, one environment, a segment and a chunk more or less, few
+environments over several chunks (fewer environments per CTA), a rollout that
+one CTA normalises, many environments; arrays off 16-byte alignment, and each
+output alone.  The bound is the rounding of the stored fp32 advantages: 4 ulp
+of the value, or of the rollout's largest where it cancels."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import cuda, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+def _shifted(x, k):
+    """x on the device, k elements past an aligned address."""
+    flat = torch.zeros(x.numel() + 8, dtype=x.dtype, device="cuda")
+    out = flat[k:k + x.numel()].view(x.shape)
+    out.copy_(x)
+    return out
+
+
+@pytest.mark.parametrize("T,E", [(1, 1), (1, 9), (3, 8), (4, 1), (5, 16), (128, 8), (256, 8),
+                                 (257, 8), (512, 9), (513, 8), (2048, 1), (2049, 3), (1000, 7),
+                                 (5000, 2), (8192, 64), (64, 1001), (300, 610), (17, 5000)])
+def test_gae_shapes(edp_lib, orc, T, E):
+    edp = edp_lib
+    rng = np.random.default_rng(T * 10007 + E)
+    r = rng.standard_normal((T, E)).astype(np.float32)
+    v = rng.standard_normal((T + 1, E)).astype(np.float32)
+    d = (rng.random((T, E)) < 0.01).astype(np.uint8)
+    ring = edp.Ring(edp.make_config(16, (1, 4, 4), edp.EDP_XFORM_HWC_CHW_BF16), action=False,
+                    reward=False, done=False)
+    A, R = orc.gae(r, v, d, 0.99, 0.95)
+    N, _, _ = orc.normalize(A)
+    want = dict(adv=A, ret=R, adv_norm=N)
+    for k, keep in enumerate([("adv", "ret", "adv_norm"), ("adv_norm",), ("ret", "adv_norm"),
+                              ("ret",), ("adv",)]):
+        out = {n: _shifted(torch.full((T, E), float("nan")), k % 4) for n in keep}
+        edp.edp_gae(ring.ctx, _shifted(cuda(r), k), _shifted(cuda(v), 1), _shifted(cuda(d), 3), T,
+                    E, 0.99, 0.95, **out)
+        edp.edp_sync(ring.ctx)
+        for n in keep:
+            ref = np.asarray(want[n], np.float64).reshape(T, E)
+            bound = 4 * 2.0**-24 * np.maximum(np.abs(ref), np.abs(ref).max())
+            assert (np.abs(to_np(out[n]) - ref) <= bound).all(), (n, keep)
+    stats = torch.zeros(3, dtype=torch.float64, device="cuda")
+    adv = torch.zeros(T, E, device="cuda")
+    edp.edp_gae_stats(ring.ctx, cuda(r), cuda(v), cuda(d), T, E, 0.99, 0.95, adv, stats)
+    edp.edp_gae_normalize(ring.ctx, adv, T * E, stats, adv)
+    edp.edp_sync(ring.ctx)
+    a64 = np.asarray(A, np.float64)
+    s = to_np(stats)
+    assert s[0] == T * E
+    assert abs(s[1] - a64.sum()) <= 1e-11 * np.abs(a64).sum()
+    assert abs(s[2] - (a64**2).sum()) <= 1e-11 * (a64**2).sum()
+    ref = np.asarray(N, np.float64).reshape(T, E)
+    assert (np.abs(to_np(adv) - ref) <= 4 * 2.0**-24 * np.maximum(
+        np.abs(ref), np.abs(ref).max())).all()
+    ring.close()
