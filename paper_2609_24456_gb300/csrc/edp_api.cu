@@ -422,7 +422,10 @@ edp_status edp_create(const edp_config *cfg, const edp_storage *st,
       internal += m;
       m *= kFanout;
     }
-    const size_t bytes = internal * 8 + n * 4;
+    // the root sits 8 bytes below a 256-byte boundary, so that every row of 32
+    // children (256 bytes of sums, 128 of leaves) is whole cache lines
+    const size_t lead = 256 - 8;
+    const size_t bytes = lead + internal * 8 + n * 4;
     c->tree_mem = al(cfg->alloc_user, bytes);
     c->tree_bytes = bytes;
     if (!c->tree_mem) {
@@ -433,11 +436,11 @@ edp_status edp_create(const edp_config *cfg, const edp_storage *st,
     uint64_t off = 0;
     m = 1;
     for (uint32_t d = 0; d < D; ++d) {
-      c->level[d] = (uint64_t *)c->tree_mem + off;
+      c->level[d] = (uint64_t *)((uint8_t *)c->tree_mem + lead) + off;
       off += m;
       m *= kFanout;
     }
-    c->leaves = (uint32_t *)((uint64_t *)c->tree_mem + internal);
+    c->leaves = (uint32_t *)(c->level[0] + internal);
     e = cudaMemset(c->tree_mem, 0, bytes);
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();

@@ -298,18 +298,6 @@ __device__ __forceinline__ uint64_t policy_keep() {
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-__device__ __forceinline__ uint64_t ld_keep(const uint64_t *p, uint64_t pol) {
-  uint64_t v;
-  asm volatile("ld.global.L2::cache_hint.u64 %0, [%1], %2;"
-               : "=l"(v) : "l"(p), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ uint32_t ld_keep(const uint32_t *p, uint64_t pol) {
-  uint32_t v;
-  asm volatile("ld.global.L2::cache_hint.u32 %0, [%1], %2;"
-               : "=r"(v) : "l"(p), "l"(pol));
-  return v;
-}
 __device__ __forceinline__ uint32_t ld_stream(const uint32_t *p, uint64_t pol) {
   uint32_t v;
   asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;"
@@ -407,12 +395,8 @@ __device__ __forceinline__ void flag(Ctrl *c, uint32_t bits,
 // writes are visible, so every such kernel calls it before touching memory
 // the predecessor may write.  pdl_launch() lets the next kernel in the
 // stream start launching.  Both are no-ops for a kernel launched without
-// the attribute.  The samplers, small grids that a one-wave delivery grid
-// follows, call pdl_launch() at their end: triggered at their start, the
-// delivery's CTAs are placed while the sampler's CTAs still hold their SMs,
-// and the block scheduler packs them onto the other SMs up to the occupancy
-// limit (304 CTAs on 88 of the 152 SMs), leaving the rest idle for the
-// whole delivery.
+// the attribute.  Kernels call it right after their wait; the uniform sampler
+// calls it at its end, which makes no difference to the deliveries behind it.
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -34,7 +34,7 @@ __global__ void k_sample_uniform(uint32_t B, uint64_t seed, uint64_t round,
     const uint64_t off = mulhi64(philox_u64(seed, k, round, 0), n_valid);
     idx[k] = (int64_t)((oldest + off) % cap);
   }
-  pdl_launch();  // at the end: see pdl_launch()
+  pdl_launch();
 }
 
 constexpr int kPermThreads = 256;

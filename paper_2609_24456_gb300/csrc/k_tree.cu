@@ -9,10 +9,10 @@
 // (n+1)*32^(D-d)).  Integer sums make every result independent of the order
 // in which threads add, so sums, targets and indices are bit-exact.
 //
-// One warp serves one tree node: a level is one coalesced 256-byte (or
-// 128-byte for leaves) load of the 32 children, a warp-shuffle inclusive
-// prefix sum and a ballot -- D dependent loads per descent instead of the
-// 5*D of a binary tree.
+// A level is one load of a node's 32 children (whole cache lines: 256 bytes of
+// sums, 128 of leaves), a shuffle prefix sum and a ballot -- D dependent loads
+// per descent instead of the 5*D of a binary tree.  A refresh gives a node a
+// warp; a descent gives it eight lanes, four children each.
 #include "edp_internal.cuh"
 
 namespace edp {
@@ -62,135 +62,196 @@ __global__ void k_tree_level(uint64_t *__restrict__ out,
   if (lane == 0) out[node] = v;
 }
 
-// Stratified proportional sampling: one warp per stratum k.  The CTA first
-// copies the top of the tree (levels 1 and 2: 32 + 1024 sums, 8.2 KiB) into
-// shared memory, so a descent of a 1M-leaf tree makes two dependent global
-// loads (level 3, then the leaf row) instead of four.
+// Stratified proportional sampling: eight lanes per stratum k, so a warp
+// descends for four at a time.  The CTA first copies the top of the tree
+// (levels 1 and 2: 32 + 1024 sums, 8.2 KiB) into shared memory, so a descent of
+// a 1M-leaf tree makes two dependent global loads (level 3, then the leaf row)
+// instead of four, and the sampled priority is the child that the last level
+// loaded.  Bound by those round trips (small batches) or by issue (a stratum
+// costs a quarter of what a warp of its own does).  Calls in a row, 1,000,000
+// leaves, in us, and (before) with a warp per stratum: 512 strata 3.1 (3.3),
+// 4,096 3.1 (5.5), 32,768 8.8 (25.4).  The delivery behind it, a grid of many
+// waves, is released at once: a round of 512 stacks of 84x84 frames 31.4 us,
+// 33.8 released at the end.
 constexpr int kSmemLevels = 2;
 constexpr int kSmemNodes = 32 + 1024;
+constexpr int kGroup = 8;                  // lanes per descent
+constexpr int kChildren = kFanout / kGroup;  // of a lane
+constexpr int kSampleThreads = 256;
+constexpr int kSamplePerCta = kSampleThreads / kGroup;
+
+__device__ __forceinline__ ulonglong2 ld_keep2(const uint64_t *p, uint64_t pol) {
+  ulonglong2 v;
+  asm volatile("ld.global.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
+               : "=l"(v.x), "=l"(v.y) : "l"(p), "l"(pol));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_keep4(const uint32_t *p, uint64_t pol) {
+  uint4 v;
+  asm volatile("ld.global.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol));
+  return v;
+}
 
 // Copies levels 1 .. cached of the tree into top (all loads issued before
 // any use); returns the number of cached levels.
 __device__ __forceinline__ uint32_t cache_top(const TreeView &t, uint64_t *top,
                                               uint64_t keep) {
   const uint32_t cached = t.depth - 1 < (uint32_t)kSmemLevels ? t.depth - 1 : kSmemLevels;
-  const uint32_t ncached = cached == 0 ? 0 : (cached == 1 ? 32 : 32 + 1024);
-  uint64_t v5[5];
+  const uint32_t pairs = (cached == 0 ? 0 : (cached == 1 ? 32 : 32 + 1024)) / 2;
+  constexpr int kEach = (kSmemNodes / 2 + kSampleThreads - 1) / kSampleThreads;
+  ulonglong2 v[kEach];
 #pragma unroll
-  for (int u = 0; u < 5; ++u) {
-    const uint32_t i = threadIdx.x + u * 256;
-    v5[u] = i < ncached ? ld_keep(t.nodes + 1 + i, keep) : 0ull;
+  for (int u = 0; u < kEach; ++u) {
+    const uint32_t i = threadIdx.x + u * kSampleThreads;
+    if (i < pairs) v[u] = ld_keep2(t.nodes + 1 + 2 * i, keep);
   }
 #pragma unroll
-  for (int u = 0; u < 5; ++u) {
-    const uint32_t i = threadIdx.x + u * 256;
-    if (i < ncached) top[i] = v5[u];
+  for (int u = 0; u < kEach; ++u) {
+    const uint32_t i = threadIdx.x + u * kSampleThreads;
+    if (i < pairs) reinterpret_cast<ulonglong2 *>(top)[i] = v[u];
   }
   return cached;
 }
 
-// Descent of one target (one warp): the leaf whose prefix range [prefix(i),
-// prefix(i) + q_i) holds `target`, for target < S.  Per level: the 32
-// children, an inclusive warp prefix sum and a ballot.  *ok is cleared if
-// the sums disagree with the children (the leaf then stays in range).
+// Descent of one target by a group of kGroup lanes (all lanes of the warp call
+// it, each group with its own target): the leaf whose prefix range
+// [prefix(i), prefix(i) + q_i) holds `target`, for target < S, and its
+// priority *q.  Per level each lane sums four of the 32 children, a prefix sum
+// over the group places them, and a ballot names the lane that holds the
+// target.  *ok is cleared if the sums disagree with the children (the leaf
+// then stays in range).
 __device__ __forceinline__ uint64_t descend(const TreeView &t, const uint64_t *top,
                                             uint32_t cached, uint64_t target, int lane,
-                                            uint64_t keep, bool *ok) {
+                                            uint64_t keep, bool *ok, uint32_t *q) {
+  const int sub = lane % kGroup, base = lane - sub;
   uint64_t node = 0;
   for (uint32_t d = 1; d <= t.depth; ++d) {
-    const uint64_t c = node * kFanout + lane;
-    uint64_t v;
-    if (d <= cached)
-      v = top[(d == 1 ? 0 : 32) + c];
-    else
-      v = d < t.depth ? ld_keep(t.lvl(d) + c, keep) : (uint64_t)ld_keep(t.leaves + c, keep);
-    uint64_t incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint64_t y = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += y;
+    const uint64_t c = node * kFanout + sub * kChildren;
+    uint64_t v[kChildren];
+    if (d <= cached) {
+      const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(top + (d == 1 ? 0 : 32) + c);
+      const ulonglong2 x = p[0], y = p[1];
+      v[0] = x.x, v[1] = x.y, v[2] = y.x, v[3] = y.y;
+    } else if (d < t.depth) {
+      const ulonglong2 x = ld_keep2(t.lvl(d) + c, keep), y = ld_keep2(t.lvl(d) + c + 2, keep);
+      v[0] = x.x, v[1] = x.y, v[2] = y.x, v[3] = y.y;
+    } else {
+      const uint4 x = ld_keep4(t.leaves + c, keep);
+      v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
     }
-    unsigned m = __ballot_sync(kFull, target < incl);
+    const uint64_t sum = v[0] + v[1] + v[2] + v[3];
+    uint64_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < kGroup; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(kFull, incl, o, kGroup);
+      if (sub >= o) incl += y;
+    }
+    uint32_t m = (__ballot_sync(kFull, target < incl) >> base) & ((1u << kGroup) - 1);
     if (m == 0) {  // sums disagree with children: report, stay in range
       *ok = false;
-      m = 1u << 31;
+      m = 1u << (kGroup - 1);
     }
-    const int f = __ffs(m) - 1;
-    const uint64_t excl = __shfl_sync(kFull, incl - v, f);
+    // in the lane that holds it: the last child that starts at or below the
+    // target (the first one when none does)
+    uint64_t excl = incl - sum, child = v[0];
+    uint32_t f = 0;
+#pragma unroll
+    for (int j = 1; j < kChildren; ++j) {
+      if (target >= excl + child) {
+        excl += child;
+        child = v[j];
+        f = j;
+      }
+    }
+    const int from = base + __ffs(m) - 1;
+    excl = __shfl_sync(kFull, excl, from);
+    f = __shfl_sync(kFull, f, from) + (from - base) * kChildren;
+    if (d == t.depth) *q = (uint32_t)__shfl_sync(kFull, (uint32_t)child, from);
     target = target >= excl ? target - excl : 0;
     node = node * kFanout + f;
   }
   return node;
 }
 
-__global__ void __launch_bounds__(256)
-k_sample_prio(TreeView t, uint32_t B, uint64_t seed, uint64_t round,
+// floor(x / B) with inv = floor((2^64 - 1) / B): the high product is at most
+// two below the quotient.
+__device__ __forceinline__ uint64_t div_by(uint64_t x, uint32_t B, uint64_t inv) {
+  uint64_t q = __umul64hi(x, inv);
+  uint64_t r = x - q * B;
+  if (r >= B) r -= B, ++q;
+  if (r >= B) ++q;
+  return q;
+}
+
+__global__ void __launch_bounds__(kSampleThreads)
+k_sample_prio(TreeView t, uint32_t B, uint64_t inv_b, uint64_t seed, uint64_t round,
               int64_t *__restrict__ idx, uint32_t *__restrict__ qout,
               Ctrl *ctrl) {
-  __shared__ uint64_t top[kSmemNodes];
+  __shared__ __align__(16) uint64_t top[kSmemNodes];
   const int lane = threadIdx.x & 31;
   const uint64_t keep = policy_keep();
+  // Philox and nothing else before the wait
+  uint64_t k = (uint64_t)blockIdx.x * kSamplePerCta + threadIdx.x / kGroup;
+  uint64_t u = philox_u64(seed, (uint32_t)k, round, 1);
   pdl_wait();
+  pdl_launch();
   const uint64_t S = t.nodes[0];  // issued beside the loads of the top levels
   const uint32_t cached = cache_top(t, top, keep);
   __syncthreads();
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < B;
-       k += warps) {
-    if (S == 0) {
-      if (lane == 0) {
-        idx[k] = -1;
-        if (qout) qout[k] = 0;
-        flag(ctrl, DEVERR_EMPTY, k);
-      }
-      continue;
-    }
-    const uint64_t target = stratum_target(S, B, k, seed, round);
+  const uint64_t a = div_by(S, B, inv_b), b = S - a * B;
+  // a warp's groups stay together: the loop ends for all of them at once
+  for (uint64_t k0 = k - lane / kGroup; k0 < B; k0 += (uint64_t)gridDim.x * kSamplePerCta) {
+    const bool mine = k < B;
+    // stratum_target() with the divisions by B as products
+    const uint64_t lo = a * k + div_by(b * k, B, inv_b);
+    const uint64_t hi = a * (k + 1) + div_by(b * (k + 1), B, inv_b);
+    const uint64_t target = lo + mulhi64(u, hi - lo);
     bool ok = true;
-    const uint64_t node = descend(t, top, cached, target, lane, keep, &ok);
-    if (lane == 0) {
-      if (!ok) flag(ctrl, DEVERR_TREE, k);
-      idx[k] = (int64_t)node;
-      if (qout) qout[k] = t.leaves[node];
+    uint32_t q = 0;
+    const uint64_t node = descend(t, top, cached, target, lane, keep, &ok, &q);
+    if (mine && lane % kGroup == 0) {
+      if (S == 0) flag(ctrl, DEVERR_EMPTY, k);
+      else if (!ok) flag(ctrl, DEVERR_TREE, k);
+      idx[k] = S == 0 ? -1 : (int64_t)node;
+      if (qout) qout[k] = S == 0 ? 0 : q;
     }
+    k += (uint64_t)gridDim.x * kSamplePerCta;
+    u = philox_u64(seed, (uint32_t)k, round, 1);
   }
-  pdl_launch();  // at the end: see pdl_launch()
 }
 
 // Descent of given targets (the shard side of a sharded buffer: targets
 // routed here by edp_route_prioritized, each below this tree's total):
-// one warp per target.  A target >= S is reported (DEVERR_INDEX) and
+// eight lanes per target.  A target >= S is reported (DEVERR_INDEX) and
 // gives idx -1, q 0.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSampleThreads)
 k_sample_targets(TreeView t, const uint64_t *__restrict__ targets, uint32_t n,
                  int64_t *__restrict__ idx, uint32_t *__restrict__ qout, Ctrl *ctrl) {
-  __shared__ uint64_t top[kSmemNodes];
+  __shared__ __align__(16) uint64_t top[kSmemNodes];
   const int lane = threadIdx.x & 31;
   const uint64_t keep = policy_keep();
   pdl_wait();
+  pdl_launch();
   const uint64_t S = t.nodes[0];  // issued beside the loads of the top levels
   const uint32_t cached = cache_top(t, top, keep);
   __syncthreads();
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += warps) {
-    const uint64_t target = targets[k];
-    if (target >= S) {
-      if (lane == 0) {
-        idx[k] = -1;
-        if (qout) qout[k] = 0;
-        flag(ctrl, DEVERR_INDEX, target);
-      }
-      continue;
-    }
+  for (uint64_t k0 = (uint64_t)blockIdx.x * kSamplePerCta + threadIdx.x / 32 * (32 / kGroup);
+       k0 < n; k0 += (uint64_t)gridDim.x * kSamplePerCta) {
+    const uint64_t k = k0 + lane / kGroup;
+    const bool mine = k < n;
+    const uint64_t target = mine ? targets[k] : 0;
+    const bool in = target < S;
     bool ok = true;
-    const uint64_t node = descend(t, top, cached, target, lane, keep, &ok);
-    if (lane == 0) {
-      if (!ok) flag(ctrl, DEVERR_TREE, k);
-      idx[k] = (int64_t)node;
-      if (qout) qout[k] = t.leaves[node];
+    uint32_t q = 0;
+    const uint64_t node = descend(t, top, cached, in ? target : 0, lane, keep, &ok, &q);
+    if (mine && lane % kGroup == 0) {
+      if (!in) flag(ctrl, DEVERR_INDEX, target);
+      else if (!ok) flag(ctrl, DEVERR_TREE, k);
+      idx[k] = in ? (int64_t)node : -1;
+      if (qout) qout[k] = in ? q : 0;
     }
   }
-  pdl_launch();  // at the end: see pdl_launch()
 }
 
 // PER priority from a TD error: clamp(rn((|td| + eps)^alpha * 2^20), 1,
@@ -693,23 +754,26 @@ cudaError_t launch_tree_build_all(edp_ctx *c, cudaStream_t s) {
   return launch_tree_refresh(c, 0, c->cap, s);
 }
 
+namespace {
+// A round of descents per CTA, at most eight CTAs per SM.
+dim3 sample_grid(const edp_ctx *c, uint32_t n) {
+  uint64_t blocks = ((uint64_t)n + kSamplePerCta - 1) / kSamplePerCta;
+  if (blocks > 8u * (unsigned)c->coop_sms) blocks = 8u * (unsigned)c->coop_sms;
+  return dim3((unsigned)blocks);
+}
+}  // namespace
+
 cudaError_t launch_sample_targets(edp_ctx *c, const uint64_t *targets, uint32_t n,
                                   int64_t *idx, uint32_t *q, cudaStream_t s) {
-  const unsigned warps_per_block = 8;
-  uint64_t blocks = (n + warps_per_block - 1) / warps_per_block;
-  if (blocks > 8u * (unsigned)c->coop_sms) blocks = 8u * (unsigned)c->coop_sms;
-  return launch_pdl(k_sample_targets, dim3((unsigned)blocks), dim3(warps_per_block * 32),
-                    s, view(c), targets, n, idx, q, c->ctrl);
+  return launch_pdl(k_sample_targets, sample_grid(c, n), dim3(kSampleThreads), s, view(c),
+                    targets, n, idx, q, c->ctrl);
 }
 
 cudaError_t launch_sample_prioritized(edp_ctx *c, uint32_t B, uint64_t seed,
                                       uint64_t round, int64_t *idx, uint32_t *q,
                                       cudaStream_t s) {
-  const unsigned warps_per_block = 8;
-  uint64_t blocks = (B + warps_per_block - 1) / warps_per_block;
-  if (blocks > 8u * (unsigned)c->coop_sms) blocks = 8u * (unsigned)c->coop_sms;
-  return launch_pdl(k_sample_prio, dim3((unsigned)blocks), dim3(warps_per_block * 32),
-                    s, view(c), B, seed, round, idx, q, c->ctrl);
+  return launch_pdl(k_sample_prio, sample_grid(c, B), dim3(kSampleThreads), s, view(c), B,
+                    ~0ull / B, seed, round, idx, q, c->ctrl);
 }
 
 cudaError_t launch_update(edp_ctx *c, const int64_t *idx, const uint32_t *q,
