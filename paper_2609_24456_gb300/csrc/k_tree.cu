@@ -408,8 +408,11 @@ __device__ __forceinline__ bool slot_holds(int64_t sl, uint64_t cap, uint64_t ol
 // scratch, no second phase, no CTA waits for another.  Every CTA reads the
 // whole batch's slots (8 bytes a pair, from the L2), kUpdLoads in flight per
 // thread, and keeps its own in a shared-memory hash table that holds, per
-// slot, the largest batch position (atomicMax): the last pair wins.  It then
-// evaluates the priority of each winner, writes its leaf and adds the exact
+// slot, the largest batch position (atomicMax): the last pair wins.  The owner
+// test comes first, on the slot's low word alone, so that a foreign pair costs
+// a few instructions.  The CTA then evaluates the priority of each winner (a
+// list of the occupied entries keeps the lanes of that evaluation full),
+// writes its leaf and adds the exact
 // signed delta to the ancestors (two's complement wrap makes negative deltas
 // exact): deeper nodes rarely collide and take one 64-bit atomic per pair,
 // level 1 (32 nodes) and the root are summed on chip first.  A batch whose
@@ -418,10 +421,11 @@ __device__ __forceinline__ bool slot_holds(int64_t sl, uint64_t cap, uint64_t ol
 // running maximum counts every pair, the overwritten ones too, so each warp
 // evaluates a stripe of the batch for it.
 //
-// Bound by the latency of the scan (32,768 pairs are 256 KB per CTA).
-// Calls in a row from TD errors, 1,000,000 slots: 4,096 pairs 7.3 us, 32,768
-// pairs 16.4 us, 131,072 pairs 54.8 us; 28.5, 214.6 and 849.5 us when one
-// CTA applied the batch 1,024 pairs at a time.
+// Bound by the scan above ~10,000 pairs (32,768 pairs are 256 KB per CTA, 40
+// MB out of the L2), by latency below.  Calls in a row from TD errors,
+// 1,000,000 slots: 4,096 pairs 7.0 us, 32,768 pairs 13.6 us, 131,072 pairs 40
+// us; 28.5, 214.6 and 849.5 us when one CTA applied the batch 1,024 pairs at a
+// time.
 constexpr int kUpdThreads = 1024;
 constexpr int kUpdLoads = 8;                         // slots in flight per thread
 constexpr int kUpdChunk = kUpdThreads * kUpdLoads;   // pairs scanned at a time
@@ -437,10 +441,11 @@ __device__ __noinline__ uint32_t prio_td_call(float td, const PrioRule &rule) {
 __global__ void __launch_bounds__(kUpdThreads, 1)
 k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict__ q,
          const float *__restrict__ td, const __grid_constant__ PrioRule rule, uint32_t n,
-         uint64_t cap, uint64_t oldest, uint64_t size, int defer, uint32_t first_table,
-         Ctrl *ctrl) {
+         uint64_t cap, uint64_t oldest, uint64_t size, int defer, Ctrl *ctrl) {
   __shared__ uint32_t hkey[kUpdTable];
   __shared__ uint32_t hpos[kUpdTable];
+  __shared__ uint16_t used[kUpdTable / 4 * 3];  // occupied entries, in any order
+  __shared__ uint32_t s_used;
   __shared__ uint32_t acc_lo[32], acc_hi[32];
   __shared__ unsigned long long warp_root[kUpdThreads / 32];
   __shared__ uint32_t s_sel, s_qmax;
@@ -455,6 +460,7 @@ k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict
   }
   if (threadIdx.x == 0) {
     s_sel = 0;
+    s_used = 0;
     s_qmax = 0;
   }
   // Nothing in memory is read or written before the wait on the preceding
@@ -477,28 +483,29 @@ k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict
   for (int o = 16; o; o >>= 1) qmax = max(qmax, __shfl_xor_sync(kFull, qmax, o));
   if (lane == 0 && qmax) atomicMax(&s_qmax, qmax);
 
-  uint32_t tsize = first_table;
   unsigned long long root_sum = 0;
   auto insert = [&](uint32_t key, uint32_t pos) {
-    uint32_t h = tab_hash(key, tsize - 1);
-    for (uint32_t probe = 0; probe < tsize; ++probe) {
+    uint32_t h = tab_hash(key, kUpdTable - 1);
+    for (uint32_t probe = 0; probe < kUpdTable; ++probe) {
       const uint32_t prev = atomicCAS(&hkey[h], kEmpty, key);
+      if (prev == kEmpty) used[atomicAdd(&s_used, 1u)] = (uint16_t)h;
       if (prev == kEmpty || prev == key) {
         atomicMax(&hpos[h], pos);
         break;
       }
-      h = (h + 1) & (tsize - 1);
+      h = (h + 1) & (kUpdTable - 1);
     }
   };
   // applies the table's pairs and empties it
   auto apply = [&]() {
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < tsize; i += kUpdThreads) {
-      const uint32_t key = hkey[i];
-      if (key == kEmpty) continue;
-      const uint32_t p = hpos[i];
-      hkey[i] = kEmpty;
-      hpos[i] = 0;
+    const uint32_t n_used = s_used;
+    for (uint32_t i = threadIdx.x; i < n_used; i += kUpdThreads) {
+      const uint32_t h = used[i];
+      const uint32_t key = hkey[h];
+      const uint32_t p = hpos[h];
+      hkey[h] = kEmpty;
+      hpos[h] = 0;
       const uint32_t old = __ldcg(t.leaves + key);
       const uint32_t qv = td ? prio_td_call(td[p], rule) : q[p];
       uint64_t k = 0;
@@ -521,7 +528,8 @@ k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict
       for (uint32_t d = 2; d < t.depth; ++d)
         atomicAdd((unsigned long long *)&t.lvl(d)[key >> (5 * (t.depth - d))], delta);
     }
-    if (threadIdx.x == 0) s_sel = 0;
+    __syncthreads();  // s_used and the list have been read
+    if (threadIdx.x == 0) s_sel = s_used = 0;
     __syncthreads();
   };
 
@@ -536,13 +544,13 @@ k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict
 #pragma unroll
     for (int u = 0; u < kUpdLoads; ++u) {
       uint64_t k = 0;
-      if (slot_holds(s[u], cap, oldest, size, &k) &&
-          __umulhi((uint32_t)s[u] * 0x9E3779B1u, gridDim.x) == blockIdx.x)
+      if (__umulhi((uint32_t)s[u] * 0x9E3779B1u, gridDim.x) == blockIdx.x &&
+          slot_holds(s[u], cap, oldest, size, &k))
         mine |= 1u << u;
     }
     if (mine) atomicAdd(&s_sel, (uint32_t)__popc(mine));
     __syncthreads();
-    const bool fits = s_sel <= tsize / 4 * 3;
+    const bool fits = s_sel <= kUpdTable / 4 * 3;
     __syncthreads();  // every thread has read s_sel
     if (fits) {
 #pragma unroll
@@ -552,7 +560,6 @@ k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict
       continue;
     }
     apply();  // the earlier pairs, then this chunk's a group at a time
-    tsize = kUpdTable;
 #pragma unroll
     for (int g = 0; g < kUpdLoads; g += kUpdGroup) {
 #pragma unroll
@@ -785,13 +792,12 @@ cudaError_t launch_update(edp_ctx *c, const int64_t *idx, const uint32_t *q,
     return launch_pdl(k_update_small, dim3((n + 31) / 32), dim3(kUpdSmallThreads), s,
                       view(c), idx, q, td, prio_rule(alpha, eps), n, c->cap, oldest,
                       size, c->defer, c->ctrl);
-  // one CTA per SM from 64 pairs a CTA on; a table four times the pairs a CTA
-  // is expected to own
-  uint32_t grid = (n + 63) / 64, table = 256;
+  // one CTA per SM, down to 64 pairs each: fewer CTAs read less but apply more
+  // in turn (8,192 pairs at 64, 128, 256 each: 7.4, 7.8, 8.8 us)
+  uint32_t grid = (n + 63) / 64;
   if (grid > (uint32_t)c->coop_sms) grid = (uint32_t)c->coop_sms;
-  while (table < kUpdTable && table / 4 < n / grid) table *= 2;
   return launch_pdl(k_update, dim3(grid), dim3(kUpdThreads), s, view(c), idx, q, td,
-                    prio_rule(alpha, eps), n, c->cap, oldest, size, c->defer, table, c->ctrl);
+                    prio_rule(alpha, eps), n, c->cap, oldest, size, c->defer, c->ctrl);
 }
 
 cudaError_t launch_prio_from_td(const float *td, uint32_t n, double alpha,
