@@ -11,15 +11,15 @@
 //            count it found is its place in the bucket
 //   scatter  every CTA scans the nb <= 8192 counts in shared memory (the
 //            bucket starts), then puts its (key, j) pairs in their places
-//   rank     a CTA takes whole buckets of about kRankTile pairs, which lie
+//   rank     a CTA takes whole buckets (a few hundred pairs), which lie
 //            side by side, into shared memory: rank_j = bucket start +
 //            #{members < (key_j, j)}; idx[rank_j] = slot of offset j;
 //            re-zero the counters for the next call
 // With nb ~ n/4 buckets (up to 32,768 elements) a bucket holds ~4 keys; above
 // that it holds n / 8192.  The result does not depend on the order of the
-// counting.  Calls in a row: 32,768 elements 13.3 us, 262,144 29.9 us,
-// 1,048,576 134 us; 13.3, 238.5 and 3,366 us when every element read its
-// bucket from the L2.
+// counting.  Calls in a row: 32,768 elements 9.4 us, 262,144 25.3 us,
+// 1,048,576 96 us; 13.3, 238.5 and 3,366 us when every element read its
+// bucket from the L2 and the counts were scanned from 4-byte loads.
 #include "edp_internal.cuh"
 
 namespace edp {
@@ -100,8 +100,24 @@ k_perm_scatter(uint32_t n, int lg, PermScratch sc) {
   const uint32_t nb = 1u << lg;
   pdl_wait();
   pdl_launch();
-  for (uint32_t i = threadIdx.x; i < kMaxBuckets; i += kPermThreads)
-    start[pad32(i)] = i < nb ? __ldcg(&sc.count[i]) : 0u;
+  // 16-byte loads, all in flight before the first is used
+  constexpr int kVecs = kMaxBuckets / 4 / kPermThreads;
+  uint4 c4[kVecs];
+#pragma unroll
+  for (int u = 0; u < kVecs; ++u) {
+    const uint32_t i = 4 * (u * kPermThreads + threadIdx.x);
+    // counts past nb stay zero between calls: whole vectors may be read
+    c4[u] = i < nb ? __ldcg(reinterpret_cast<const uint4 *>(sc.count + i))
+                   : make_uint4(0u, 0u, 0u, 0u);
+  }
+#pragma unroll
+  for (int u = 0; u < kVecs; ++u) {
+    const uint32_t i = pad32(4 * (u * kPermThreads + threadIdx.x));
+    start[i] = c4[u].x;
+    start[i + 1] = c4[u].y;
+    start[i + 2] = c4[u].z;
+    start[i + 3] = c4[u].w;
+  }
   __syncthreads();
   constexpr uint32_t per = kMaxBuckets / kPermThreads;  // 32
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -152,11 +168,15 @@ k_perm_scatter(uint32_t n, int lg, PermScratch sc) {
   }
 }
 
-// Pairs a CTA ranks: buckets_per_cta whole buckets, taken through shared
-// memory kRankTile at a time (one tile unless the buckets are large).
+// The pairs that a CTA ranks are whole buckets, taken through shared memory
+// kRankTile at a time (one tile unless the buckets are large).
 constexpr uint32_t kRankTile = 1024;
-constexpr uint32_t kRankWant = kPermThreads;  // pairs a CTA is given on average
-constexpr uint32_t kRankBuckets = 128;        // at most: a bucket holds over 2 pairs on average
+constexpr uint32_t kRankBuckets = 128;  // at most per CTA: a bucket holds over 2 pairs on average
+// Pairs a CTA is given on average: more, smaller CTAs while the buckets are
+// small (32,768 pairs: 9.4 us per shuffle with 128, 12.5 with 256, 10.0 with
+// 64), a thread each above that (262,144: 25.3 with 256, 27.0 with 128).
+constexpr uint32_t kRankFew = 65536;
+constexpr uint32_t rank_want(uint32_t n) { return n <= kRankFew ? 128 : kPermThreads; }
 
 __global__ void __launch_bounds__(kPermThreads)
 k_perm_rank(uint32_t n, int lg, uint32_t per_cta, PermScratch sc, uint64_t oldest, uint64_t cap,
@@ -210,10 +230,24 @@ k_perm_rank(uint32_t n, int lg, uint32_t per_cta, PermScratch sc, uint64_t oldes
 #pragma unroll
       for (int u = 0; u < kEach; ++u) {
         const uint32_t a = max(blo[u], tlo), z = min(bhi[u], thi);
-        for (uint32_t i = a; i < z; ++i) {
-          const uint64_t k2 = tkey[i - tlo];
-          r[u] += k2 < key[u] || (k2 == key[u] && tj[i - tlo] < j[u]);
+        uint32_t equal = 0;
+        uint32_t i = a;
+        for (; i + 4 <= z; i += 4) {
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
+            const uint64_t k2 = tkey[i + w - tlo];
+            r[u] += k2 < key[u];
+            equal += k2 == key[u];
+          }
         }
+        for (; i < z; ++i) {
+          const uint64_t k2 = tkey[i - tlo];
+          r[u] += k2 < key[u];
+          equal += k2 == key[u];
+        }
+        // equal keys beside the element itself (hardly ever): by offset
+        if (equal > (t0 == e0 ? 1u : 0u))
+          for (i = a; i < z; ++i) r[u] += tkey[i - tlo] == key[u] && tj[i - tlo] < j[u];
       }
     }
 #pragma unroll
@@ -261,7 +295,7 @@ cudaError_t launch_permute(edp_ctx *c, uint32_t n, uint64_t seed,
   const uint64_t oldest = (c->total - size) % c->cap;
   uint64_t grid = (n + (uint64_t)kPermThreads - 1) / kPermThreads;
   if (grid > 4ull * c->coop_sms) grid = 4ull * c->coop_sms;
-  uint32_t per_cta = (uint32_t)((uint64_t)kRankWant * nb / n);  // 2 nb < n + 2: at most 128
+  uint32_t per_cta = (uint32_t)((uint64_t)rank_want(n) * nb / n);
   if (per_cta < 1) per_cta = 1;
   if (per_cta > kRankBuckets) per_cta = kRankBuckets;
   const dim3 g((unsigned)grid), blk(kPermThreads);
