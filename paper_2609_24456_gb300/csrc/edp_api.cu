@@ -166,12 +166,13 @@ edp_status edp::fail(edp_ctx *c, edp_status s, const char *fmt, ...) {
 }
 
 bool edp::device_view(const edp_ctx *c, const void *p, const void **out,
-                      bool allow_host) {
+                      bool allow_host, bool *host) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
+  if (host) *host = a.type == cudaMemoryTypeHost;
   if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) {
     if (a.device != c->cfg.device) return false;
     *out = p;
@@ -184,23 +185,14 @@ bool edp::device_view(const edp_ctx *c, const void *p, const void **out,
   return false;
 }
 
-bool edp::host_memory(const void *p) {
-  if (!p) return false;
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return a.type == cudaMemoryTypeHost;
-}
-
 namespace {
-// Traffic counters: bytes at p (device or page-locked host memory).
-void count_read(edp_ctx *c, const void *p, uint64_t bytes) {
-  if (p && bytes) (host_memory(p) ? c->cnt.link_read : c->cnt.hbm_read) += bytes;
+// Traffic counters: bytes in page-locked host memory (`host`) or in device
+// memory.
+void count_read(edp_ctx *c, bool host, uint64_t bytes) {
+  (host ? c->cnt.link_read : c->cnt.hbm_read) += bytes;
 }
-void count_write(edp_ctx *c, const void *p, uint64_t bytes) {
-  if (p && bytes) (host_memory(p) ? c->cnt.link_write : c->cnt.hbm_write) += bytes;
+void count_write(edp_ctx *c, bool host, uint64_t bytes) {
+  (host ? c->cnt.link_write : c->cnt.hbm_write) += bytes;
 }
 // Device-resident arrays of a call (index, priority and scalar arrays).
 void count_hbm(edp_ctx *c, uint64_t read, uint64_t write) {
@@ -766,20 +758,22 @@ edp_status edp_ingest(edp_ctx *ctx, const edp_fields *src, uint64_t n,
   cudaStream_t s = (cudaStream_t)stream;
   edp_fields f{};
   const void *p;
-  if (!src->obs || !device_view(ctx, src->obs, &p, true) || !aligned16(p))
+  // which sources are page-locked host memory
+  bool h_obs = false, h_tokens = false, h_action = false, h_reward = false, h_done = false;
+  if (!src->obs || !device_view(ctx, src->obs, &p, true, &h_obs) || !aligned16(p))
     return fail(ctx, EDP_ERR_INVALID,
                 "edp_ingest: src.obs must be 16-B aligned device or page-locked memory");
   f.obs = (const uint8_t *)p;
   if ((ctx->tok_bytes > 0) != (src->tokens != nullptr))
     return fail(ctx, EDP_ERR_INVALID, "edp_ingest: src.tokens given iff tokens > 0");
   if (src->tokens) {
-    if (!device_view(ctx, src->tokens, &p, true) || !aligned16(p))
+    if (!device_view(ctx, src->tokens, &p, true, &h_tokens) || !aligned16(p))
       return fail(ctx, EDP_ERR_INVALID, "edp_ingest: bad src.tokens");
     f.tokens = (const int32_t *)p;
   }
 #define EDP_VIEW(field, T)                                                     \
   if (src->field) {                                                            \
-    if (!device_view(ctx, src->field, &p, true))                               \
+    if (!device_view(ctx, src->field, &p, true, &h_##field))                   \
       return fail(ctx, EDP_ERR_INVALID, "edp_ingest: bad src." #field);        \
     f.field = (T)p;                                                            \
   }
@@ -845,12 +839,12 @@ edp_status edp_ingest(edp_ctx *ctx, const edp_fields *src, uint64_t n,
   // and leaves written to HBM
   auto count_ingest = [&]() {
     const uint64_t R = ctx->obs_bytes + ctx->tok_bytes;
-    count_read(ctx, src->obs, n * ctx->obs_bytes);
-    count_read(ctx, src->tokens, n * ctx->tok_bytes);
-    count_read(ctx, src->action, 4 * n);
-    count_read(ctx, src->reward, 4 * n);
-    count_read(ctx, src->done, n);
-    count_read(ctx, q, 4 * n);
+    count_read(ctx, h_obs, n * ctx->obs_bytes);
+    if (src->tokens) count_read(ctx, h_tokens, n * ctx->tok_bytes);
+    if (src->action) count_read(ctx, h_action, 4 * n);
+    if (src->reward) count_read(ctx, h_reward, 4 * n);
+    if (src->done) count_read(ctx, h_done, n);
+    if (q) count_read(ctx, false, 4 * n);
     ctx->cnt.hbm_write += (n - to_host) * R;
     ctx->cnt.link_write += (to_host + demoted) * R;
     ctx->cnt.hbm_read += demoted * R;
@@ -936,9 +930,12 @@ edp_status edp_sample(edp_ctx *ctx, edp_sample_mode mode, uint32_t batch,
 // Argument checks shared by edp_deliver and edp_sample_deliver; *res is
 // the batch with every output resolved to a device-usable address (an
 // output may be page-locked host memory: the kernel then writes it over the
-// host link).
+// host link), and bit i of *host tells that output i is.
+// Outputs in the order of deliver_checks' list.
+enum { OUT_OBS, OUT_NEXT, OUT_ACTION, OUT_REWARD, OUT_DONE, OUT_TOKENS, OUT_ISW, OUT_G0, OUT_G1 };
+
 static edp_status deliver_checks(edp_ctx *ctx, const int64_t *idx, uint32_t batch,
-                                 const edp_batch *out, edp_batch *res) {
+                                 const edp_batch *out, edp_batch *res, uint32_t *host) {
   if (!idx || !out || !out->obs)
     return fail(ctx, EDP_ERR_INVALID, "edp_deliver: idx/out/out->obs is NULL");
   if (batch == 0) return fail(ctx, EDP_ERR_INVALID, "edp_deliver: batch == 0");
@@ -973,12 +970,16 @@ static edp_status deliver_checks(edp_ctx *ctx, const int64_t *idx, uint32_t batc
                    reinterpret_cast<void **>(&res->isw),
                    reinterpret_cast<void **>(&res->gather_dst[0]),
                    reinterpret_cast<void **>(&res->gather_dst[1])};
-  for (void **o : outs) {
+  *host = 0;
+  for (uint32_t i = 0; i < sizeof outs / sizeof *outs; ++i) {
+    void **o = outs[i];
+    bool h = false;
     if (!*o) continue;
-    if (!device_view(ctx, *o, &p, true))
+    if (!device_view(ctx, *o, &p, true, &h))
       return fail(ctx, EDP_ERR_INVALID,
                   "edp_deliver: outputs must be device or page-locked host memory");
     *o = const_cast<void *>(p);
+    *host |= (h ? 1u : 0u) << i;
   }
   if (!aligned16(res->obs) || (res->next_obs && !aligned16(res->next_obs)) ||
       (res->tokens && !aligned16(res->tokens)))
@@ -986,12 +987,12 @@ static edp_status deliver_checks(edp_ctx *ctx, const int64_t *idx, uint32_t batc
   return EDP_OK;
 }
 
-// Traffic of a delivery of B entries into `out` (the caller's pointers):
+// Traffic of a delivery of B entries into `out` (`host` from deliver_checks):
 // per entry the unique source bytes (the K or K + 1 frames of a stack, the
 // image and tokens otherwise) and the scalars read, and every output
 // written to its memory.  A two-tier ring's host rows are counted on the
 // device and moved to link_read by edp_get_counters.
-static void count_deliver(edp_ctx *ctx, uint32_t B, const edp_batch *out) {
+static void count_deliver(edp_ctx *ctx, uint32_t B, const edp_batch *out, uint32_t host) {
   const auto &cfg = ctx->cfg;
   const uint64_t F = ctx->obs_bytes;
   uint64_t per = F, obs_out = 0;
@@ -1006,15 +1007,18 @@ static void count_deliver(edp_ctx *ctx, uint32_t B, const edp_batch *out) {
                            (out->done != nullptr) + 4 * (out->q != nullptr) +
                            4 * (out->gather_src[0] != nullptr) + 4 * (out->gather_src[1] != nullptr);
   ctx->cnt.hbm_read += B * (per + scalars);
-  count_write(ctx, out->obs, B * obs_out);
-  count_write(ctx, out->next_obs, B * obs_out);
-  count_write(ctx, out->tokens, B * ctx->tok_bytes);
-  count_write(ctx, out->action, 4ull * B);
-  count_write(ctx, out->reward, 4ull * B);
-  count_write(ctx, out->done, 1ull * B);
-  count_write(ctx, out->isw, 4ull * B);
-  count_write(ctx, out->gather_dst[0], 4ull * B);
-  count_write(ctx, out->gather_dst[1], 4ull * B);
+  auto wrote = [&](const void *p, int i, uint64_t bytes) {
+    if (p) count_write(ctx, (host >> i) & 1u, bytes);
+  };
+  wrote(out->obs, OUT_OBS, B * obs_out);
+  wrote(out->next_obs, OUT_NEXT, B * obs_out);
+  wrote(out->tokens, OUT_TOKENS, B * ctx->tok_bytes);
+  wrote(out->action, OUT_ACTION, 4ull * B);
+  wrote(out->reward, OUT_REWARD, 4ull * B);
+  wrote(out->done, OUT_DONE, 1ull * B);
+  wrote(out->isw, OUT_ISW, 4ull * B);
+  wrote(out->gather_dst[0], OUT_G0, 4ull * B);
+  wrote(out->gather_dst[1], OUT_G1, 4ull * B);
   ctx->cnt.delivered += B;
   ++ctx->cnt.calls;
 }
@@ -1023,13 +1027,14 @@ edp_status edp_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t batch,
                        const edp_batch *out, edp_stream stream) {
   if (!ctx) return EDP_ERR_INVALID;
   edp_batch res;
-  const edp_status st = deliver_checks(ctx, idx, batch, out, &res);
+  uint32_t host = 0;
+  const edp_status st = deliver_checks(ctx, idx, batch, out, &res, &host);
   if (st != EDP_OK) return st;
   DeviceGuard dg(ctx->cfg.device);
   EDP_TRACE(__func__);
   cudaError_t e = launch_deliver(ctx, idx, batch, &res, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "edp_deliver");
-  count_deliver(ctx, batch, out);
+  count_deliver(ctx, batch, out, host);
   return EDP_OK;
 }
 
@@ -1042,14 +1047,15 @@ edp_status edp_sample_deliver(edp_ctx *ctx, uint32_t batch, uint64_t seed, uint6
     return fail(ctx, EDP_ERR_INVALID,
                 "edp_sample_deliver: uniform draws carry no priorities (q/isw must be NULL)");
   edp_batch res;
-  const edp_status st = deliver_checks(ctx, idx, batch, out, &res);
+  uint32_t host = 0;
+  const edp_status st = deliver_checks(ctx, idx, batch, out, &res, &host);
   if (st != EDP_OK) return st;
   DeviceGuard dg(ctx->cfg.device);
   EDP_TRACE(__func__);
   DrawUniform d{seed, round, idx};
   cudaError_t e = launch_deliver(ctx, idx, batch, &res, (cudaStream_t)stream, &d);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "edp_sample_deliver");
-  count_deliver(ctx, batch, out);  // the drawn indices are written, not read:
+  count_deliver(ctx, batch, out, host);  // the drawn indices are written, not read:
   ctx->cnt.hbm_read -= 8ull * batch;  // the index bytes count once, as a write
   ctx->cnt.hbm_write += 8ull * batch;
   ctx->cnt.sampled += batch;
@@ -1295,9 +1301,11 @@ edp_status edp_pack_deliver(edp_ctx *ctx, const int32_t *tokens, const uint64_t 
     if (o && !device_view(ctx, o, &p, false))
       return fail(ctx, EDP_ERR_INVALID, "edp_pack_deliver: inputs must be device memory");
   void *outs[] = {out_tokens, out_off, out_value};
-  for (void *&o : outs) {
+  bool host[3] = {};
+  for (int i = 0; i < 3; ++i) {
+    void *&o = outs[i];
     if (!o) continue;
-    if (!device_view(ctx, o, &p, true))
+    if (!device_view(ctx, o, &p, true, &host[i]))
       return fail(ctx, EDP_ERR_INVALID,
                   "edp_pack_deliver: outputs must be device or page-locked host memory");
     o = const_cast<void *>(p);
@@ -1309,7 +1317,7 @@ edp_status edp_pack_deliver(edp_ctx *ctx, const int32_t *tokens, const uint64_t 
                               out_cap, (cudaStream_t)stream);
   if (e != cudaSuccess) return launch_fail(ctx, e, "edp_pack_deliver");
   count_hbm(ctx, 24ull * batch, 0);  // indices and sequence offsets; tokens not counted
-  count_write(ctx, out_off, 8ull * (batch + 1));
+  count_write(ctx, host[1], 8ull * (batch + 1));
   ctx->cnt.delivered += batch;
   return EDP_OK;
 }
@@ -1336,9 +1344,11 @@ edp_status edp_grpo_pack_deliver(edp_ctx *ctx, const float *r, const uint64_t *g
     if (o && !device_view(ctx, o, &p, false))
       return fail(ctx, EDP_ERR_INVALID, "edp_grpo_pack_deliver: arrays must be device memory");
   void *outs[] = {out_tokens, out_off, out_value};
-  for (void *&o : outs) {
+  bool host[3] = {};
+  for (int i = 0; i < 3; ++i) {
+    void *&o = outs[i];
     if (!o) continue;
-    if (!device_view(ctx, o, &p, true))
+    if (!device_view(ctx, o, &p, true, &host[i]))
       return fail(ctx, EDP_ERR_INVALID,
                   "edp_grpo_pack_deliver: outputs must be device or page-locked host memory");
     o = const_cast<void *>(p);
@@ -1350,7 +1360,7 @@ edp_status edp_grpo_pack_deliver(edp_ctx *ctx, const float *r, const uint64_t *g
                                    (float *)outs[2], out_cap, (cudaStream_t)stream);
   if (e != cudaSuccess) return launch_fail(ctx, e, "edp_grpo_pack_deliver");
   count_hbm(ctx, 8ull * (n_groups + 1) + 24ull * batch, 0);
-  count_write(ctx, out_off, 8ull * (batch + 1));
+  count_write(ctx, host[1], 8ull * (batch + 1));
   ctx->cnt.delivered += batch;
   return EDP_OK;
 }

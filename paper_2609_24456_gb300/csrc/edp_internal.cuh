@@ -599,11 +599,11 @@ class TraceRange {
 // Resolve a caller pointer to a device-usable address.  Device memory of the
 // context's GPU passes through; page-locked host memory is translated to its
 // mapped device address when allow_host; pageable or foreign memory is
-// rejected (false).
-bool device_view(const edp_ctx *c, const void *p, const void **out, bool allow_host);
-
-// true for page-locked host memory (reached over the host link)
-bool host_memory(const void *p);
+// rejected (false).  *host (where given) tells page-locked host memory from
+// device memory: one query of the pointer serves the check, the translation
+// and the traffic counters.
+bool device_view(const edp_ctx *c, const void *p, const void **out, bool allow_host,
+                 bool *host = nullptr);
 
 // Record a printf-style message as the context's last error; returns s.
 edp_status fail(edp_ctx *c, edp_status s, const char *fmt, ...);

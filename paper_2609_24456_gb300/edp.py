@@ -184,10 +184,27 @@ def ptr(x):
     return x.data_ptr()
 
 
+_current = None
+
+
+def _current_stream():
+    """cudaStream_t of torch's current stream on its current device.  Building
+    torch's Stream object takes longer than a whole call of the library (2.9 us
+    of 8), so the handle is asked for directly where torch has that call."""
+    global _current
+    if _current is None:
+        import torch
+        torch.cuda.current_stream()  # initialises CUDA
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        dev = getattr(torch._C, "_cuda_getDevice", None)
+        _current = ((lambda: raw(dev())) if raw and dev else
+                    (lambda: torch.cuda.current_stream().cuda_stream))
+    return _current()
+
+
 def stream_handle(stream):
     if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
