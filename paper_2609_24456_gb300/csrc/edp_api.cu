@@ -818,7 +818,7 @@ edp_status edp_ingest(edp_ctx *ctx, const edp_fields *src, uint64_t n,
       const uint64_t skip = new_hbm_lo - T;
       e = launch_swap(ctx, lo, f.obs + skip * ctx->obs_bytes,
                       f.tokens ? f.tokens + skip * (ctx->tok_bytes / 4) : nullptr,
-                      hi - lo, s);
+                      hi - lo, &f, n, q, s);
     } else {
       if (hi > lo) e = launch_demote(ctx, lo, hi - lo, s);
       if (e == cudaSuccess && dhi > dlo)
@@ -865,7 +865,7 @@ edp_status edp_ingest(edp_ctx *ctx, const edp_fields *src, uint64_t n,
   // the row copy starts behind the (waiting) metadata and tree kernels and
   // overlaps the last of them, since neither reads the rows
   const bool meta = ctx->st.action || ctx->st.reward || ctx->st.done || ctx->leaves;
-  if (e == cudaSuccess) e = launch_ingest_meta(ctx, &f, n, q, s);
+  if (e == cudaSuccess && !swapped) e = launch_ingest_meta(ctx, &f, n, q, s);
   if (e == cudaSuccess && ctx->depth) e = launch_tree_refresh(ctx, tfirst, tcount, s);
   const uint64_t skip = new_hbm_lo - T, nh = Tn - new_hbm_lo;
   if (e == cudaSuccess && !swapped) {

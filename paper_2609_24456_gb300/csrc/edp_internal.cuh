@@ -437,9 +437,11 @@ cudaError_t launch_demote(edp_ctx *ctx, uint64_t first_id, uint64_t n,
 // Demotion and insertion fused, for the steady state of a full two-tier
 // ring: ids first_id + j leave HBM slot (first_id + j) mod cap_h for host
 // slot (first_id + j) mod cap_c while source rows j of the ingest (obs,
-// tokens) take their HBM slot.
+// tokens) take their HBM slot; and the metadata and leaves of all n_meta
+// transitions of the insertion, as launch_ingest_meta writes them.
 cudaError_t launch_swap(edp_ctx *ctx, uint64_t first_id, const uint8_t *obs,
-                        const int32_t *tokens, uint64_t n, cudaStream_t s);
+                        const int32_t *tokens, uint64_t n, const edp_fields *f, uint64_t n_meta,
+                        const uint32_t *q, cudaStream_t s);
 // payload, metadata and leaves of src ids [L0, L0 + n) into dst's placement
 // as dst ids 0 .. n-1 (dst then has n insertions)
 cudaError_t launch_migrate(const edp_ctx *src, edp_ctx *dst, uint64_t L0, uint64_t n,

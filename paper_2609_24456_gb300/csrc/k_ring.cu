@@ -103,58 +103,6 @@ int sm_count() {
   return sms > 0 ? sms : 1;
 }
 
-// Swap rows through HBM: HBM row (first + j) mod hbm_cap moves to host row
-// (first + j) mod host_cap and source row j takes its place.  One thread
-// handles one 16-byte chunk in all three rows, reading the old HBM value
-// before writing the new one, so no other thread's order matters.  The
-// host-link traffic goes both ways at once (source rows in, demoted rows
-// out), which a demotion followed by a copy would serialise.
-__global__ void __launch_bounds__(kCopyThreads)
-k_swap_rows(uint8_t *__restrict__ hbm, uint64_t hbm_cap, uint8_t *__restrict__ host,
-            uint64_t host_cap, const uint8_t *__restrict__ src, uint64_t first,
-            uint64_t n, uint32_t cpr) {
-  const uint64_t row_bytes = (uint64_t)cpr * 16u;
-  for (uint64_t j = blockIdx.y; j < n; j += gridDim.y) {
-    uint4 *h = reinterpret_cast<uint4 *>(hbm + ((first + j) % hbm_cap) * row_bytes);
-    uint4 *c = reinterpret_cast<uint4 *>(host + ((first + j) % host_cap) * row_bytes);
-    const uint4 *s = reinterpret_cast<const uint4 *>(src + j * row_bytes);
-    const uint32_t step = gridDim.x * kCopyThreads * kCopyUnroll;
-    for (uint32_t w0 = blockIdx.x * kCopyThreads * kCopyUnroll + threadIdx.x;
-         w0 < cpr; w0 += step) {
-      uint4 old_[kCopyUnroll], new_[kCopyUnroll];
-#pragma unroll
-      for (int u = 0; u < kCopyUnroll; ++u) {
-        const uint32_t w = w0 + u * kCopyThreads;
-        if (w < cpr) {
-          old_[u] = h[w];
-          new_[u] = s[w];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kCopyUnroll; ++u) {
-        const uint32_t w = w0 + u * kCopyThreads;
-        if (w < cpr) {
-          c[w] = old_[u];
-          h[w] = new_[u];
-        }
-      }
-    }
-  }
-}
-
-cudaError_t swap_rows(uint8_t *hbm, uint64_t hbm_cap, uint8_t *host, uint64_t host_cap,
-                      const uint8_t *src, uint64_t first, uint64_t n,
-                      uint64_t row_bytes, cudaStream_t s) {
-  if (!n) return cudaSuccess;
-  const uint32_t cpr = (uint32_t)(row_bytes / 16);
-  uint32_t gx = (cpr + kCopyThreads * kCopyUnroll - 1) / (kCopyThreads * kCopyUnroll);
-  if (gx > 64) gx = 64;
-  const uint32_t gy = n < 65535 ? (uint32_t)n : 65535u;
-  k_swap_rows<<<dim3(gx, gy), kCopyThreads, 0, s>>>(hbm, hbm_cap, host, host_cap, src,
-                                                   first, n, cpr);
-  return cudaGetLastError();
-}
-
 // Rows (src_first + j) mod src_cap -> (dst_first + j) mod dst_cap for
 // j < n, as the contiguous runs between the wrap points of either side.
 cudaError_t copy_rows(uint8_t *dst, uint64_t dst_cap, uint64_t dst_first,
@@ -242,6 +190,69 @@ __device__ __forceinline__ void ingest_meta_range(const MetaArgs &a, uint64_t j0
     for (int o = 16; o; o >>= 1)
       qmax_local = max(qmax_local, __shfl_xor_sync(0xffffffffu, qmax_local, o));
     if ((threadIdx.x & 31) == 0 && qmax_local) atomicMax(&a.ctrl->max_q, qmax_local);
+  }
+}
+
+// Swap rows through HBM: HBM row (first + j) mod hbm_cap moves to host row
+// (first + j) mod host_cap and source row j takes its place.  One thread
+// handles one 16-byte chunk in all three rows, reading the old HBM value
+// before writing the new one, so no other thread's order matters.  The
+// host-link traffic goes both ways at once (source rows in, demoted rows
+// out), which a demotion followed by a copy would serialise.  The first obs.gx
+// CTA columns swap the images, the next tok.gx the tokens, and a last one
+// writes the metadata, so that a small insertion is one launch: 64 rows of
+// 27,648 + 512 bytes 9.9 us (12.1 as three kernels without programmatic
+// launch), one row 2.1 us (4.3), 512 rows 75.4 us (77.0; the link's rate out).
+struct SwapRows {
+  uint8_t *hbm;
+  uint8_t *host;
+  const uint8_t *src;
+  uint32_t cpr;  // 16-byte chunks per row
+  uint32_t gx;   // CTA columns
+};
+
+__global__ void __launch_bounds__(kCopyThreads)
+k_swap_rows(SwapRows obs, SwapRows tok, uint64_t hbm_cap, uint64_t host_cap, uint64_t first,
+            uint64_t n, MetaArgs meta) {
+  pdl_wait();
+  pdl_launch();
+  if (blockIdx.x >= obs.gx + tok.gx) {
+    ingest_meta_range(meta, (uint64_t)blockIdx.y * kCopyThreads + threadIdx.x,
+                      (uint64_t)gridDim.y * kCopyThreads);
+    return;
+  }
+  const bool is_tok = blockIdx.x >= obs.gx;
+  uint8_t *const hbm = is_tok ? tok.hbm : obs.hbm;
+  uint8_t *const host = is_tok ? tok.host : obs.host;
+  const uint8_t *const src = is_tok ? tok.src : obs.src;
+  const uint32_t cpr = is_tok ? tok.cpr : obs.cpr;
+  const uint32_t gx = is_tok ? tok.gx : obs.gx;
+  const uint32_t bx = blockIdx.x - (is_tok ? obs.gx : 0u);
+  const uint64_t row_bytes = (uint64_t)cpr * 16u;
+  for (uint64_t j = blockIdx.y; j < n; j += gridDim.y) {
+    uint4 *h = reinterpret_cast<uint4 *>(hbm + ((first + j) % hbm_cap) * row_bytes);
+    uint4 *c = reinterpret_cast<uint4 *>(host + ((first + j) % host_cap) * row_bytes);
+    const uint4 *s = reinterpret_cast<const uint4 *>(src + j * row_bytes);
+    const uint32_t step = gx * kCopyThreads * kCopyUnroll;
+    for (uint32_t w0 = bx * kCopyThreads * kCopyUnroll + threadIdx.x; w0 < cpr; w0 += step) {
+      uint4 old_[kCopyUnroll], new_[kCopyUnroll];
+#pragma unroll
+      for (int u = 0; u < kCopyUnroll; ++u) {
+        const uint32_t w = w0 + u * kCopyThreads;
+        if (w < cpr) {
+          old_[u] = h[w];
+          new_[u] = s[w];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kCopyUnroll; ++u) {
+        const uint32_t w = w0 + u * kCopyThreads;
+        if (w < cpr) {
+          c[w] = old_[u];
+          h[w] = new_[u];
+        }
+      }
+    }
   }
 }
 
@@ -336,6 +347,10 @@ cudaError_t launch_copy_rows(uint8_t *dst, uint64_t dst_cap, uint64_t first,
 }
 
 namespace {
+bool has_meta(const edp_ctx *c) {
+  return c->st.action || c->st.reward || c->st.done || c->leaves;
+}
+
 MetaArgs meta_args(edp_ctx *c, const edp_fields *f, uint64_t n, const uint32_t *q) {
   MetaArgs a{};
   a.action = c->st.action;
@@ -357,8 +372,7 @@ MetaArgs meta_args(edp_ctx *c, const edp_fields *f, uint64_t n, const uint32_t *
 
 cudaError_t launch_ingest_meta(edp_ctx *c, const edp_fields *f, uint64_t n,
                                const uint32_t *q, cudaStream_t s) {
-  if (!c->st.action && !c->st.reward && !c->st.done && !c->leaves)
-    return cudaSuccess;
+  if (!has_meta(c)) return cudaSuccess;
   const int threads = 256;
   uint64_t blocks = (n + threads - 1) / threads;
   if (blocks > 4096) blocks = 4096;
@@ -418,13 +432,21 @@ cudaError_t launch_demote(edp_ctx *c, uint64_t first_id, uint64_t n,
 }
 
 cudaError_t launch_swap(edp_ctx *c, uint64_t first_id, const uint8_t *obs,
-                        const int32_t *tokens, uint64_t n, cudaStream_t s) {
-  cudaError_t e = swap_rows(c->st.obs, c->cap_h, c->st.host_obs, c->cap_c, obs,
-                            first_id, n, c->obs_bytes, s);
-  if (e == cudaSuccess && c->tok_bytes)
-    e = swap_rows((uint8_t *)c->st.tokens, c->cap_h, (uint8_t *)c->st.host_tokens,
-                  c->cap_c, (const uint8_t *)tokens, first_id, n, c->tok_bytes, s);
-  return e;
+                        const int32_t *tokens, uint64_t n, const edp_fields *f, uint64_t n_meta,
+                        const uint32_t *q, cudaStream_t s) {
+  auto rows = [](uint8_t *hbm, uint8_t *host, const uint8_t *src, uint64_t row_bytes) {
+    SwapRows r{hbm, host, src, (uint32_t)(row_bytes / 16), 0};
+    r.gx = (r.cpr + kCopyThreads * kCopyUnroll - 1) / (kCopyThreads * kCopyUnroll);
+    if (r.gx > 64) r.gx = 64;
+    return r;
+  };
+  const SwapRows o = rows(c->st.obs, c->st.host_obs, obs, c->obs_bytes);
+  const SwapRows t = rows((uint8_t *)c->st.tokens, (uint8_t *)c->st.host_tokens,
+                          (const uint8_t *)tokens, c->tok_bytes);
+  const uint32_t gy = n < 65535 ? (uint32_t)n : 65535u;
+  return launch_pdl(k_swap_rows, dim3(o.gx + t.gx + (has_meta(c) ? 1u : 0u), gy),
+                    dim3(kCopyThreads), s, o, t, c->cap_h, c->cap_c, first_id, n,
+                    meta_args(c, f, n_meta, q));
 }
 
 // ---- migration between placements (Sec. 5.3, Alg. 2) ---------------------
