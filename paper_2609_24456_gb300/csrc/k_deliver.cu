@@ -37,7 +37,7 @@ constexpr int kNormUnroll = 6;
 // unrolled rows per warp iteration and iterations per warp (chunk span) of
 // each kernel
 constexpr int kStackMinBlocks = 5;  // __launch_bounds__: at most 48 registers
-constexpr int kFlatMinBlocks = 6;   // at most 40
+constexpr int kFlatMinBlocks = 5;
 constexpr int kNormIters = 2;
 
 struct Common {
@@ -348,8 +348,8 @@ k_deliver_stack(Common c, StackArgs a) {
 // ---------------------------------------------------------------------------
 // Frame stack, float32, as one flat range of words: a CTA takes `words`
 // consecutive words of the batch's units (frame m of sample k, as above),
-// whatever frames and samples they belong to, a lane per word and
-// kFlatUnroll loads in flight, so a 128-byte frame fills a warp's access as
+// whatever frames and samples they belong to, a lane per word and UN loads in
+// flight, so a 128-byte frame fills a warp's access as
 // well as a large one.  The samples it touches are resolved first, a thread
 // each: index -> slot, into shared memory.  Then every thread issues its
 // first loads, and the resolving threads load the K episode flags of their
@@ -360,11 +360,10 @@ k_deliver_stack(Common c, StackArgs a) {
 // Taken for frames below kFlatFrame bytes, where a span of k_deliver_stack
 // crosses several frames and walks them in turn.  Calls in a row, 32,768
 // samples, in us, here and (k_deliver_stack): 8x16, 1 frame and its
-// successor, 13.5 (120: with 4 loads per lane); 20x20, 4 and their
-// successors, 85 (97.5); 28x28, 4 and their successors, 159 (144).
+// successor, 12.5 (120: with 4 loads per lane); 20x20, 4 and their
+// successors, 83 (97.5); 28x28, 4 and their successors, 159 (144).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kFlatFrame = 768;
-constexpr int kFlatUnroll = 4;
 constexpr uint32_t kFlatSamples = kThreads;  // at most touched by a CTA
 struct FlatArgs {
   uint32_t words;           // per CTA
@@ -372,6 +371,7 @@ struct FlatArgs {
   uint32_t div_per, div_w;  // ceil(2^32 / per), ceil(2^32 / W)
 };
 
+template <int UN>
 __global__ void __launch_bounds__(kThreads, kFlatMinBlocks)
 k_deliver_stack_flat(Common c, StackArgs a, FlatArgs g) {
   __shared__ uint64_t s_pos[kFlatSamples];    // unwrapped slot of the anchor
@@ -403,7 +403,7 @@ k_deliver_stack_flat(Common c, StackArgs a, FlatArgs g) {
   __syncthreads();
   // word i of sample k0's range: i * per < 2^32, so the rounded-up
   // reciprocals give the exact quotients
-  uint32_t v[kFlatUnroll];
+  uint32_t v[UN];
   auto load = [&](uint32_t i, bool masked) -> uint32_t {
     if (i >= i_1) return 0u;
     const uint32_t s = __umulhi(i, g.div_per), rem = i - s * g.per;
@@ -416,8 +416,7 @@ k_deliver_stack_flat(Common c, StackArgs a, FlatArgs g) {
                      pol);
   };
 #pragma unroll
-  for (int u = 0; u < kFlatUnroll; ++u)
-    v[u] = load(i_0 + threadIdx.x + u * kThreads, false);
+  for (int u = 0; u < UN; ++u) v[u] = load(i_0 + threadIdx.x + u * kThreads, false);
   if (threadIdx.x < ns) {
     uint32_t ends = 0;  // bit i: an episode ends at offset off - K + 1 + i
 #pragma unroll
@@ -445,13 +444,13 @@ k_deliver_stack_flat(Common c, StackArgs a, FlatArgs g) {
   }
   __syncthreads();
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (uint32_t i0 = i_0 + threadIdx.x; i0 < i_1; i0 += kThreads * kFlatUnroll) {
+  for (uint32_t i0 = i_0 + threadIdx.x; i0 < i_1; i0 += kThreads * UN) {
     if (i0 != i_0 + threadIdx.x) {
 #pragma unroll
-      for (int u = 0; u < kFlatUnroll; ++u) v[u] = load(i0 + u * kThreads, true);
+      for (int u = 0; u < UN; ++u) v[u] = load(i0 + u * kThreads, true);
     }
 #pragma unroll
-    for (int u = 0; u < kFlatUnroll; ++u) {
+    for (int u = 0; u < UN; ++u) {
       const uint32_t i = i0 + u * kThreads;
       if (i >= i_1) continue;
       const uint32_t s = __umulhi(i, g.div_per), rem = i - s * g.per;
@@ -768,10 +767,12 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     if (a.F < kFlatFrame) {
       FlatArgs g{};
       g.per = (uint32_t)per;  // at most 17 frames: words * per < 2^32
-      // 1,024 words (one round of loads), up to 4,096 while every SM keeps
-      // eight CTAs: 8x16, 4 frames and successors, 512 stacks 3.6 / 5.0 / 7.5 us
-      // with 1,024 / 2,048 / 4,096 words, 16x16, 32,768 stacks 64 / 58 / 56 us
-      g.words = 1024;
+      // 1,024 words with 4 loads per lane, one round (8x16, 4 frames and
+      // successors, 512 stacks: 3.6 us, 4.7 with 2,048 words and 8); 2,048 with
+      // 8 from 3.5 CTAs of those per SM on (8,192 stacks: 9.4 us, 10.3), up to
+      // 4,096 while every SM keeps eight CTAs (16x16, 32,768: 55 us, 58)
+      const bool wide = units / 2048 >= 7ull * sms / 2;
+      g.words = wide ? 2048 : 1024;
       while (g.words < 4096 && units / (2 * g.words) >= 8ull * sms) g.words *= 2;
       if (g.words > (kFlatSamples - 2) * per)
         g.words = (uint32_t)((kFlatSamples - 2) * per) & ~31u;
@@ -779,7 +780,8 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
       g.div_w = (uint32_t)((0x100000000ull + a.W - 1) / a.W);
       const uint64_t ctas = (units + g.words - 1) / g.words + a.ncollate;
       if (ctas > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-      return launch_pdl(k_deliver_stack_flat, dim3((unsigned)ctas), dim3(kThreads), s, c, a, g);
+      auto kern = wide ? k_deliver_stack_flat<8> : k_deliver_stack_flat<4>;
+      return launch_pdl(kern, dim3((unsigned)ctas), dim3(kThreads), s, c, a, g);
     }
     const bool few = units <= (uint64_t)kWarps * 32 * 4 * sms;
     const uint64_t each = (uint64_t)kWarps * 32 * (few ? 4 : 8);
