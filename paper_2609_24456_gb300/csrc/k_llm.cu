@@ -266,10 +266,18 @@ __device__ __forceinline__ void pack_copy_cta(PackBuf &sm, uint32_t &uses, const
   const uint32_t ho = min((uint32_t)(((16u - ((uint32_t)(uintptr_t)oc & 15u)) & 15u) >> 2), m);
   const uint32_t q = (m - ho) >> 2;
   if (threadIdx.x < ho) st_stream32(oc + threadIdx.x, sm.tok[threadIdx.x + shift], pol);
+  // the four tokens of a store straddle two 16-byte words of shared memory,
+  // which are read whole (four 4-byte reads would conflict four ways each)
+  const uint32_t off = (ho + shift) & 3u;
+  const uint4 *words = reinterpret_cast<const uint4 *>(sm.tok) + (ho + shift) / 4;
   for (uint32_t i = threadIdx.x; i < q; i += kPackThreads) {
-    const uint32_t t = ho + 4 * i + shift;
-    st_stream(reinterpret_cast<uint4 *>(oc + ho) + i,
-              make_uint4(sm.tok[t], sm.tok[t + 1], sm.tok[t + 2], sm.tok[t + 3]), pol);
+    uint4 x = words[i];
+    if (off) {
+      const uint4 y = words[i + 1];
+      x = off == 1 ? make_uint4(x.y, x.z, x.w, y.x)
+        : off == 2 ? make_uint4(x.z, x.w, y.x, y.y) : make_uint4(x.w, y.x, y.y, y.z);
+    }
+    st_stream(reinterpret_cast<uint4 *>(oc + ho) + i, x, pol);
   }
   const uint32_t to = ho + 4 * q;
   if (threadIdx.x < m - to)
@@ -308,7 +316,7 @@ __device__ __forceinline__ uint64_t pack_offset_cta(const PackEntry *__restrict_
 // entry writes its output offset, that of the last entry out_off[batch] = the
 // total, and flags an overflow.
 // 32 registers, 16.5 KB: 8 CTAs per SM keep more copies in flight than 6 at 38
-// registers (8,192 sequences of 128 to 4,096 tokens 34.7 us, 37.3).
+// registers (8,192 sequences of 128 to 4,096 tokens 34.4 us, 37.3).
 template <bool SPLIT>
 __global__ void __launch_bounds__(kPackThreads, 8)
 k_pack_gather(const int32_t *__restrict__ tokens, const PackEntry *__restrict__ ent,
@@ -443,11 +451,8 @@ cudaError_t launch_grpo(edp_ctx *c, const float *r, const uint64_t *goff, uint32
                         float eps, float *adv, cudaStream_t s) {
   uint64_t blocks = (ng + kGrpoWarps - 1) / kGrpoWarps;
   if (blocks > 16ull * c->coop_sms) blocks = 16ull * c->coop_sms;
-  // A plain launch: behind a large grid (the previous step's gather) an
-  // early-launched k_grpo made the whole step slower (62 vs 46 us for the
-  // 512 x 16 batch); its pdl_wait / pdl_launch are then no-ops.
-  k_grpo<<<dim3((unsigned)blocks), dim3(kGrpoThreads), 0, s>>>(r, goff, ng, eps, adv);
-  return cudaGetLastError();
+  return launch_pdl(k_grpo, dim3((unsigned)blocks), dim3(kGrpoThreads), s, r, goff, ng, eps,
+                    adv);
 }
 
 namespace {
@@ -534,11 +539,9 @@ cudaError_t launch_grpo_pack(edp_ctx *c, const float *r, const uint64_t *goff, u
   if (e != cudaSuccess) return e;
   uint64_t ngc = (ng + kGrpoWarps - 1) / kGrpoWarps;
   if (ngc > 16ull * c->coop_sms) ngc = 16ull * c->coop_sms;
-  // a plain launch, as for k_grpo
-  k_grpo_pack_lengths<<<dim3((unsigned)(ngc + p.G)), dim3(kPackThreads), 0, s>>>(
-      r, goff, ng, eps, adv, (uint32_t)ngc, soff, nseq, idx, B, p.ent, p.part, p.pre, p.work,
-      c->ctrl);
-  e = cudaGetLastError();
+  e = launch_pdl(k_grpo_pack_lengths, dim3((unsigned)(ngc + p.G)), dim3(kPackThreads), s, r,
+                 goff, ng, eps, adv, (uint32_t)ngc, soff, nseq, idx, B, p.ent, p.part, p.pre,
+                 p.work, c->ctrl);
   if (e != cudaSuccess) return e;
   return launch_gather(c, p, tokens, B, adv, otok, ooff, osv, cap, s);
 }
