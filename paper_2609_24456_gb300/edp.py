@@ -413,8 +413,16 @@ class Ring:
     pin_memory for the host tier) and handed to edp_create as raw pointers.
     """
 
+    # rings collected while their thread captured a CUDA graph: destroying a
+    # context synchronises and frees, which would break the capture, so it
+    # waits, with its storage, for the next ring that is made or collected
+    # outside one
+    _waiting = []
+
     def __init__(self, cfg: edp_config, action=True, reward=True, done=True):
         import torch
+        self.ctx = None
+        self._destroy_waiting()
         self.cfg = cfg
         dev = torch.device("cuda", cfg.device)
         ob = cfg.obs_c * cfg.obs_h * cfg.obs_w
@@ -446,9 +454,21 @@ class Ring:
             edp_destroy(self.ctx)
             self.ctx = None
 
+    @classmethod
+    def _destroy_waiting(cls):
+        import torch
+        while cls._waiting and not torch.cuda.is_current_stream_capturing():
+            edp_destroy(cls._waiting.pop()["ctx"])
+
     def __del__(self):
         try:
+            if self.ctx:
+                import torch
+                if torch.cuda.is_current_stream_capturing():
+                    self._waiting.append(dict(self.__dict__))
+                    return
             self.close()
+            self._destroy_waiting()
         except Exception:
             pass
 
