@@ -14,8 +14,8 @@
 // (2,048 / kE at most) are processed from the end of the rollout backwards,
 // carrying A across; the next chunk's inputs are loaded beside a chunk's
 // arithmetic.  With kE = 8 every access of a time-major row moves whole
-// 32-byte sectors; long rollouts of few environments use fewer environments
-// per CTA, so that more SMs and longer chunks share the steps (gae_shape).
+// 32-byte sectors; rollouts of few environments use fewer per CTA, so that more
+// SMs and longer chunks share the steps (gae_shape).
 //
 // Arithmetic: GB300's fp64 pipe is narrow (a dependent fp64 FMA costs ~64
 // cycles, fp32 ~4), so the scan -- and each lane's sums of A and A^2 over an
@@ -32,19 +32,21 @@
 //
 // Bound by latency (a chunk's loads, then its dependent chain) up to ~10^6
 // values, then by HBM.  Calls in a row with all three outputs, in us, and
-// (before) with one warp per environment: 8 x 2,048 steps 13.8 (43.0), 4,096 x
-// 64 14.5 (28.4), 1,024 x 1,024 29.9 (107), 64 x 8,192 44.6 (557), 8 x 128 8.0
-// (9.2).
+// (before) with one warp per environment: 8 x 2,048 steps 12.8 (43.0), 4,096 x
+// 64 13.2 (28.4), 1,024 x 1,024 29.5 (107), 64 x 8,192 41 (557), 8 x 128 7.6
+// (9.2), 8 x 512 8.6.
 //
 // Two kernels chained with programmatic dependent launch: the scan writes A,
 // the returns and per-CTA sums of A and A^2; the normalisation kernel
 // forms mean and the unbiased standard deviation (every CTA reduces the
 // partials in the same fixed order, so all agree bit for bit) and writes
-// the normalised values; a rollout that one CTA scans in at most two chunks is
-// normalised by it, without a second kernel.  With the environments
+// the normalised values; a small rollout is scanned and normalised by one CTA,
+// without a second kernel.  With the environments
 // sharded over several ranks, the scan's sums are reduced to this rank's
 // (n, sum A, sum A^2) instead (k_gae_stats), the caller sums those over the
 // ranks, and the normalisation reads the totals.
+#include <type_traits>
+
 #include "edp_internal.cuh"
 
 namespace edp {
@@ -55,6 +57,7 @@ constexpr int kL = 4;               // steps per thread and chunk
 constexpr int kGaeThreads = 512;    // at most per CTA
 constexpr int kGaeWarps = kGaeThreads / 32;
 constexpr int kNormThreads = 256;
+constexpr int kNormLoads = 8;       // values in flight per thread of a single CTA
 
 __device__ __forceinline__ df df_shfl_down(df a, int o) {
   return {__shfl_down_sync(kFull, a.hi, o), __shfl_down_sync(kFull, a.lo, o)};
@@ -88,25 +91,61 @@ __device__ __forceinline__ float norm_value(float a, const NormStat &st) {
   return (float)(((double)a - st.mean) * st.inv);
 }
 
-// Inputs of one thread's kL steps t0 .. t0 + kL - 1 of environment e, and the
-// value after each (a step at or past te reads a valid one instead, a value
-// past te the one at te).
+// Inputs of one thread's kL steps and the value after each.
 struct GaeIn {
   float r[kL], v[kL + 1];
   bool d[kL];
 };
+// Loads of a chunk [ts, te) by thread (seg, e) of `segs` segments.  With eight
+// environments per CTA a warp's load of one step each touches four rows, whole
+// sectors: the thread loads its own steps ts + seg kL ...  With fewer, adjacent
+// threads load adjacent steps instead (x.r[i] is step ts + i segs + seg), since
+// rows kL apart would take a cache line per lane, and the steps change hands
+// through shared memory (gae_exchange).  A step at or past te reads a valid one
+// instead, a value past te the one at te; x.v[kL] is the value after the
+// thread's last step, or (staged) after the chunk.
+template <bool STAGED>
 __device__ __forceinline__ void gae_load(GaeIn &x, const float *__restrict__ r,
                                          const float *__restrict__ v,
-                                         const uint8_t *__restrict__ d, uint64_t t0, uint64_t te,
-                                         uint32_t E, uint32_t e) {
+                                         const uint8_t *__restrict__ d, uint64_t ts, uint64_t te,
+                                         uint32_t seg, uint32_t segs, uint32_t E, uint32_t e) {
 #pragma unroll
   for (int i = 0; i < kL; ++i) {
-    const uint64_t at = min(t0 + i, te - 1) * E + e;
+    const uint64_t t = STAGED ? ts + (uint64_t)i * segs + seg : ts + (uint64_t)seg * kL + i;
+    const uint64_t at = min(t, te - 1) * E + e;
     x.r[i] = r[at];
     x.d[i] = d[at] != 0;
+    x.v[i] = v[min(t, te) * E + e];
   }
+  x.v[kL] = v[(STAGED ? te : min(ts + (uint64_t)seg * kL + kL, te)) * E + e];
+}
+
+// A chunk's inputs, [step * kE + e], the values one step more.
+struct GaeStage {
+  float r[kGaeThreads * kL];
+  float v[kGaeThreads * kL + 8];
+  bool d[kGaeThreads * kL];
+};
+template <int kE>
+__device__ __forceinline__ void gae_exchange(GaeIn &x, GaeStage &s, uint32_t seg, uint32_t segs,
+                                             uint32_t el) {
 #pragma unroll
-  for (int i = 0; i <= kL; ++i) x.v[i] = v[min(t0 + i, te) * E + e];
+  for (int i = 0; i < kL; ++i) {
+    const uint32_t at = (i * segs + seg) * kE + el;
+    s.r[at] = x.r[i];
+    s.v[at] = x.v[i];
+    s.d[at] = x.d[i];
+  }
+  if (seg == 0) s.v[segs * kL * kE + el] = x.v[kL];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kL; ++i) {
+    const uint32_t at = (seg * kL + i) * kE + el;
+    x.r[i] = s.r[at];
+    x.v[i] = s.v[at];
+    x.d[i] = s.d[at];
+  }
+  x.v[kL] = s.v[(seg * kL + kL) * kE + el];
 }
 
 template <int kE>
@@ -119,10 +158,12 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
   __shared__ float2 s_carry[kE];         // A at the step after the chunk
   __shared__ float4 s_sum[kGaeWarps];
   __shared__ NormStat s_stat;
+  constexpr bool kStaged = kE < 8;
+  __shared__ std::conditional_t<kStaged, GaeStage, char> stage;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
   const uint32_t el = threadIdx.x % kE, seg = threadIdx.x / kE;
-  const uint32_t chunk = blockDim.x / kE * kL;
+  const uint32_t segs = blockDim.x / kE, chunk = segs * kL;
   const df one = {1.f, 0.f}, zero = {0.f, 0.f};
   const df g = df_split(gamma);
   const df gl = df_split(gamma * lambda);
@@ -135,12 +176,13 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
     if (seg == 0) s_carry[el] = make_float2(0.f, 0.f);  // read after the barrier below
     GaeIn x;
     uint32_t te = T, ts = T > chunk ? T - chunk : 0;
-    gae_load(x, r, v, d, (uint64_t)ts + seg * kL, te, E, e);
+    gae_load<kStaged>(x, r, v, d, ts, te, seg, segs, E, e);
     for (;;) {
       const uint64_t t0 = (uint64_t)ts + seg * kL;
       const uint32_t te2 = ts, ts2 = ts > chunk ? ts - chunk : 0;
       GaeIn next;
-      if (te2) gae_load(next, r, v, d, (uint64_t)ts2 + seg * kL, te2, E, e);
+      if (te2) gae_load<kStaged>(next, r, v, d, ts2, te2, seg, segs, E, e);
+      if constexpr (kStaged) gae_exchange<kE>(x, stage, seg, segs, el);
       df del[kL], cc[kL];
       df a = one, b = zero;  // this thread's steps composed: x -> b + a x
 #pragma unroll
@@ -232,8 +274,20 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
   // one CTA scanned everything: it normalises what it wrote
   __syncthreads();
   const NormStat st = s_stat;
-  for (uint64_t i = threadIdx.x; i < (uint64_t)T * E; i += blockDim.x)
-    adv_norm[i] = norm_value(__ldcg(A_out + i), st);
+  const uint64_t n = (uint64_t)T * E;
+  for (uint64_t i0 = threadIdx.x; i0 < n; i0 += kNormLoads * blockDim.x) {
+    float y[kNormLoads];
+#pragma unroll
+    for (int u = 0; u < kNormLoads; ++u) {
+      const uint64_t i = i0 + u * blockDim.x;
+      y[u] = i < n ? __ldcg(A_out + i) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < kNormLoads; ++u) {
+      const uint64_t i = i0 + u * blockDim.x;
+      if (i < n) adv_norm[i] = norm_value(y[u], st);
+    }
+  }
 }
 
 // Sum of the per-CTA partials (sum A, sum A^2) in a fixed order: strided
@@ -324,22 +378,23 @@ namespace {
 // fewer CTAs than SMs, which the least scratch block (ctx_scratch) covers.
 size_t gae_scratch_bytes(uint32_t E) { return ((size_t)E + 3) / 4 * 2 * sizeof(double); }
 
-// Environments per CTA (8, halved while the rollout takes several chunks and
-// half of the SMs would idle), threads per CTA and CTAs of a scan.
+// Environments per CTA, threads per CTA and CTAs of a scan.  A CTA of
+// 512 threads is bound by issue (about 4 us per chunk whatever its shape), so
+// the environments per CTA are halved from 8 while half of the SMs would idle:
+// 8 x 512 steps with 8, 4, 2, 1 environments per CTA 16.2, 17.2, 9.5, 8.6 us
+// per call, 8 x 2,048 36.5, 24.0, 16.0, 12.9, 256 x 128 9.2, 8.8, 9.0, 9.7.
 struct GaeShape {
-  uint32_t envs, threads, grid, chunks;
+  uint32_t envs, threads, grid;
 };
-GaeShape gae_shape(const edp_ctx *c, uint32_t T, uint32_t E) {
+GaeShape gae_shape(const edp_ctx *c, uint32_t T, uint32_t E, bool one_cta) {
   GaeShape g;
   g.envs = 8;
-  while (g.envs > 1 && T > kGaeThreads / g.envs * kL &&
+  while (!one_cta && g.envs > 1 &&
          2 * (((uint64_t)E + g.envs - 1) / g.envs) < (uint64_t)c->coop_sms)
     g.envs /= 2;
   const uint64_t want = ((uint64_t)T + kL - 1) / kL * g.envs;
   g.threads = want < kGaeThreads ? (uint32_t)((want + 31) & ~31ull) : (uint32_t)kGaeThreads;
   g.grid = (uint32_t)(((uint64_t)E + g.envs - 1) / g.envs);
-  const uint32_t chunk = g.threads / g.envs * kL;
-  g.chunks = T / chunk + (T % chunk != 0);
   return g;
 }
 
@@ -352,8 +407,15 @@ cudaError_t launch_scan(const GaeShape &g, const float *r, const float *v, const
                     ret, partial, adv_norm);
 }
 
+// One CTA per SM while that leaves a thread a few elements: each CTA adds the
+// partial sums again and forms the statistics, and several on one SM queue on
+// its fp64 pipe (4,096 x 64: 13.4 us per call, 15.5 with four per SM; 64 x
+// 8,192: 40.0, 44.7); four per SM for the loads of more (1,024 x 1,024: 29.9 us,
+// 33.3 with one).
 unsigned norm_grid(const edp_ctx *c, uint64_t n) {
-  const uint64_t most = 4ull * c->coop_sms, want = (n + 4 * kNormThreads - 1) / (4 * kNormThreads);
+  const uint64_t sms = (uint64_t)c->coop_sms;
+  const uint64_t want = (n + 4 * kNormThreads - 1) / (4 * kNormThreads);
+  const uint64_t most = want <= 4 * sms ? sms : 4 * sms;
   return (unsigned)(want < most ? want : most);
 }
 
@@ -363,7 +425,10 @@ cudaError_t launch_gae(edp_ctx *c, const float *r, const float *v,
                        const uint8_t *d, uint32_t T, uint32_t E, double gamma,
                        double lambda, float *adv, float *ret, float *adv_norm,
                        cudaStream_t s) {
-  GaeShape g = gae_shape(c, T, E);
+  // a rollout of one chunk of eight environments: one CTA scans and normalises
+  // it (8 x 128: 7.6 us per call, 8.4 as two kernels)
+  const bool one_cta = adv_norm && E <= 8 && T <= 128;
+  const GaeShape g = gae_shape(c, T, E, one_cta);
   double *partial = nullptr;
   if (adv_norm) {
     void *blk = nullptr;
@@ -374,10 +439,8 @@ cudaError_t launch_gae(edp_ctx *c, const float *r, const float *v,
   // A is kept for the normalisation in adv, or in adv_norm itself (fp32; the
   // normalisation error this adds is below 2^-24 |A| / std)
   float *A_out = adv ? adv : adv_norm;
-  if (adv_norm && (uint64_t)g.grid * g.chunks <= 2) {
-    g.grid = 1;
+  if (one_cta)
     return launch_scan(g, r, v, d, T, E, gamma, lambda, A_out, ret, nullptr, adv_norm, s);
-  }
   const cudaError_t e =
       launch_scan(g, r, v, d, T, E, gamma, lambda, A_out, ret, partial, nullptr, s);
   if (e != cudaSuccess || !adv_norm) return e;
@@ -391,7 +454,7 @@ cudaError_t launch_gae_stats(edp_ctx *c, const float *r, const float *v,
                              const uint8_t *d, uint32_t T, uint32_t E, double gamma,
                              double lambda, float *adv, float *ret, double *stats,
                              cudaStream_t s) {
-  const GaeShape g = gae_shape(c, T, E);
+  const GaeShape g = gae_shape(c, T, E, false);
   void *blk = nullptr;
   cudaError_t e = ctx_scratch(c, gae_scratch_bytes(E), s, &blk);
   if (e != cudaSuccess) return e;
