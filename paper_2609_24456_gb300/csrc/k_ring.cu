@@ -133,6 +133,8 @@ struct MetaArgs {
   const uint32_t *q;
   Ctrl *ctrl;
   uint64_t cap, total, n;
+  uint64_t head;  // total mod cap: slots come by a subtraction, not by a 64-bit
+                  // remainder (about a hundred instructions) per transition
   int defer;
 };
 
@@ -164,7 +166,8 @@ __device__ __forceinline__ void ingest_meta_range(const MetaArgs &a, uint64_t j0
     for (int b = 0; b < kMetaBatch; ++b) {
       const uint64_t j = jb + b * stride;
       if (j >= a.n) break;
-      const uint64_t m = (a.total + j) % a.cap;
+      const uint64_t s = a.head + j;  // j < n <= cap
+      const uint64_t m = s >= a.cap ? s - a.cap : s;
       if (a.action) a.action[m] = act[b];
       if (a.reward) a.reward[m] = rew[b];
       if (a.done) a.done[m] = dn[b];
@@ -176,7 +179,7 @@ __device__ __forceinline__ void ingest_meta_range(const MetaArgs &a, uint64_t j0
           if (j == 0) {
             // only this thread touches pending_q and the previous newest leaf
             if (a.total >= 1 && a.n < a.cap)
-              a.leaves[(a.total - 1) % a.cap] = a.ctrl->pending_q;
+              a.leaves[(a.head ? a.head : a.cap) - 1] = a.ctrl->pending_q;
             a.ctrl->pending_q = a.q ? a.q[a.n - 1] : qdefault;
           }
         } else {
@@ -193,8 +196,8 @@ __device__ __forceinline__ void ingest_meta_range(const MetaArgs &a, uint64_t j0
   }
 }
 
-// Swap rows through HBM: HBM row (first + j) mod hbm_cap moves to host row
-// (first + j) mod host_cap and source row j takes its place.  One thread
+// Swap rows through HBM: HBM row (hbm_first + j) mod hbm_cap moves to host row
+// (host_first + j) mod host_cap and source row j takes its place.  One thread
 // handles one 16-byte chunk in all three rows, reading the old HBM value
 // before writing the new one, so no other thread's order matters.  The
 // host-link traffic goes both ways at once (source rows in, demoted rows
@@ -212,8 +215,8 @@ struct SwapRows {
 };
 
 __global__ void __launch_bounds__(kCopyThreads)
-k_swap_rows(SwapRows obs, SwapRows tok, uint64_t hbm_cap, uint64_t host_cap, uint64_t first,
-            uint64_t n, MetaArgs meta) {
+k_swap_rows(SwapRows obs, SwapRows tok, uint64_t hbm_cap, uint64_t host_cap,
+            uint64_t hbm_first, uint64_t host_first, uint64_t n, MetaArgs meta) {
   pdl_wait();
   pdl_launch();
   if (blockIdx.x >= obs.gx + tok.gx) {
@@ -230,8 +233,10 @@ k_swap_rows(SwapRows obs, SwapRows tok, uint64_t hbm_cap, uint64_t host_cap, uin
   const uint32_t bx = blockIdx.x - (is_tok ? obs.gx : 0u);
   const uint64_t row_bytes = (uint64_t)cpr * 16u;
   for (uint64_t j = blockIdx.y; j < n; j += gridDim.y) {
-    uint4 *h = reinterpret_cast<uint4 *>(hbm + ((first + j) % hbm_cap) * row_bytes);
-    uint4 *c = reinterpret_cast<uint4 *>(host + ((first + j) % host_cap) * row_bytes);
+    // n is at most either tier's capacity
+    const uint64_t jh = hbm_first + j, jc = host_first + j;
+    uint4 *h = reinterpret_cast<uint4 *>(hbm + (jh >= hbm_cap ? jh - hbm_cap : jh) * row_bytes);
+    uint4 *c = reinterpret_cast<uint4 *>(host + (jc >= host_cap ? jc - host_cap : jc) * row_bytes);
     const uint4 *s = reinterpret_cast<const uint4 *>(src + j * row_bytes);
     const uint32_t step = gx * kCopyThreads * kCopyUnroll;
     for (uint32_t w0 = bx * kCopyThreads * kCopyUnroll + threadIdx.x; w0 < cpr; w0 += step) {
@@ -263,14 +268,12 @@ __global__ void k_ingest_meta(MetaArgs a) {
                     (uint64_t)gridDim.x * blockDim.x);
 }
 
-// One insertion in one launch (replay rings: a single HBM tier, at most
-// kFusedMaxRows rows).  CTA 0 writes the metadata and leaves, then refreshes
+// One insertion in one launch (replay rings: a single HBM tier, a moderate
+// number of rows: ingest_fusable).  CTA 0 writes the metadata and leaves, then refreshes
 // the tree above them level by level (a CTA barrier between levels, so each
 // level reads the sums written below it); the other CTAs copy the payload
 // rows (obs, then tokens).  Nothing of the two parts reads what the other
 // writes, so the metadata chain runs beside the copy.
-constexpr int kFusedThreads = 1024;
-constexpr uint64_t kFusedMaxRows = 16384;
 
 struct TreeRefresh {
   uint64_t *level[kMaxDepth];  // level d: 32^d sums
@@ -280,7 +283,8 @@ struct TreeRefresh {
   uint64_t a0[kMaxDepth], n0[kMaxDepth], a1[kMaxDepth], n1[kMaxDepth];
 };
 
-__global__ void __launch_bounds__(kFusedThreads, 1)
+template <int kFusedThreads>
+__global__ void __launch_bounds__(kFusedThreads, 1024 / kFusedThreads)
 k_ingest_fused(CopyRuns obs, CopyRuns tok, MetaArgs meta, TreeRefresh t) {
   pdl_wait();
   pdl_launch();
@@ -365,6 +369,7 @@ MetaArgs meta_args(edp_ctx *c, const edp_fields *f, uint64_t n, const uint32_t *
   a.cap = c->cap;
   a.total = c->total;
   a.n = n;
+  a.head = c->total % c->cap;
   a.defer = c->defer;
   return a;
 }
@@ -380,8 +385,13 @@ cudaError_t launch_ingest_meta(edp_ctx *c, const edp_fields *f, uint64_t n,
                     meta_args(c, f, n, q));
 }
 
+// While one CTA's metadata hides behind the copy, or costs less than the chain
+// of kernels: rows of 128 bytes with priorities, 4,096 6.0 us (7.5 as a chain),
+// 8,192 9.0 (7.6); of 7,056 bytes, 8,192 20.3 (24.5), 16,384 40.8 (41.5), without
+// priorities 39.4 (35.9).
 bool ingest_fusable(const edp_ctx *c, uint64_t n) {
-  return c->cap_c == 0 && n <= kFusedMaxRows;
+  if (c->cap_c) return false;
+  return n <= 4096 || (c->obs_bytes >= 1024 && n <= (c->depth ? 16384u : 8192u));
 }
 
 cudaError_t launch_ingest_fused(edp_ctx *c, const edp_fields *f, uint64_t n,
@@ -408,12 +418,19 @@ cudaError_t launch_ingest_fused(edp_ctx *c, const edp_fields *f, uint64_t n,
     }
   }
   const uint64_t words = obs.end[2] + tok.end[2];
-  uint64_t blocks = (words + (uint64_t)kFusedThreads * kCopyFlat - 1) /
-                    ((uint64_t)kFusedThreads * kCopyFlat);
-  const uint64_t most = 2ull * sm_count();
+  // CTA 0 is bound by issue: many threads for many transitions.  A few start and
+  // end sooner with less: 4 rows of 7,056 bytes 2.3 us with 256 threads, 2.7
+  // with 512, 3.5 with 1,024; 1,024 rows 3.3, 3.3, 5.1; 4,096 rows with
+  // priorities, of 128 bytes 10.1, 7.2, 6.4, of 7,056 bytes (the copy bounds
+  // them) 12.8, 9.0, 9.9
+  const int threads = n <= 64 ? 256 : n <= 2048 || (n <= 4096 && c->obs_bytes >= 1024) ? 512 : 1024;
+  uint64_t blocks = (words + (uint64_t)threads * kCopyFlat - 1) / ((uint64_t)threads * kCopyFlat);
+  const uint64_t most = 2048ull / threads * sm_count();
   if (blocks > most) blocks = most;
-  return launch_pdl(k_ingest_fused, dim3((unsigned)(blocks + 1)), dim3(kFusedThreads), s, obs,
-                    tok, meta_args(c, f, n, q), t);
+  auto kern = threads == 256 ? k_ingest_fused<256>
+            : threads == 512 ? k_ingest_fused<512> : k_ingest_fused<1024>;
+  return launch_pdl(kern, dim3((unsigned)(blocks + 1)), dim3(threads), s, obs, tok,
+                    meta_args(c, f, n, q), t);
 }
 
 // Two-tier demotion: payload of ids [first_id, first_id+n) moves from HBM
@@ -445,7 +462,8 @@ cudaError_t launch_swap(edp_ctx *c, uint64_t first_id, const uint8_t *obs,
                           (const uint8_t *)tokens, c->tok_bytes);
   const uint32_t gy = n < 65535 ? (uint32_t)n : 65535u;
   return launch_pdl(k_swap_rows, dim3(o.gx + t.gx + (has_meta(c) ? 1u : 0u), gy),
-                    dim3(kCopyThreads), s, o, t, c->cap_h, c->cap_c, first_id, n,
+                    dim3(kCopyThreads), s, o, t, c->cap_h, c->cap_c, first_id % c->cap_h,
+                    first_id % c->cap_c, n,
                     meta_args(c, f, n_meta, q));
 }
 
