@@ -107,17 +107,21 @@ struct GaeIn {
 template <bool STAGED>
 __device__ __forceinline__ void gae_load(GaeIn &x, const float *__restrict__ r,
                                          const float *__restrict__ v,
-                                         const uint8_t *__restrict__ d, uint64_t ts, uint64_t te,
+                                         const uint8_t *__restrict__ d, uint32_t ts, uint32_t te,
                                          uint32_t seg, uint32_t segs, uint32_t E, uint32_t e) {
+  // (T + 1) E < 2^32, and a step past te is less than a chunk past it.  The
+  // eight-environment form keeps 64-bit indices: with fewer registers to hold,
+  // ptxas takes it down to 64 with spills (1,024 x 1,024: 39 us, 29.5)
+  using index = std::conditional_t<STAGED, uint32_t, uint64_t>;
 #pragma unroll
   for (int i = 0; i < kL; ++i) {
-    const uint64_t t = STAGED ? ts + (uint64_t)i * segs + seg : ts + (uint64_t)seg * kL + i;
-    const uint64_t at = min(t, te - 1) * E + e;
+    const index t = STAGED ? (index)ts + i * segs + seg : (index)ts + seg * kL + i;
+    const index at = min(t, (index)(te - 1)) * E + e;
     x.r[i] = r[at];
     x.d[i] = d[at] != 0;
-    x.v[i] = v[min(t, te) * E + e];
+    x.v[i] = v[min(t, (index)te) * E + e];
   }
-  x.v[kL] = v[(STAGED ? te : min(ts + (uint64_t)seg * kL + kL, te)) * E + e];
+  x.v[kL] = v[(STAGED ? (index)te : min((index)ts + seg * kL + kL, (index)te)) * E + e];
 }
 
 // A chunk's inputs, [step * kE + e], the values one step more.
@@ -151,8 +155,8 @@ __device__ __forceinline__ void gae_exchange(GaeIn &x, GaeStage &s, uint32_t seg
 template <int kE>
 __global__ void __launch_bounds__(kGaeThreads)
 k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
-           const uint8_t *__restrict__ d, uint32_t T, uint32_t E, double gamma,
-           double lambda, float *A_out, float *__restrict__ ret,
+           const uint8_t *__restrict__ d, uint32_t T, uint32_t E, float2 g2, float2 gl2,
+           float *A_out, float *__restrict__ ret,
            double *__restrict__ partial, float *adv_norm) {
   __shared__ float4 agg[kGaeWarps][kE];  // a warp's composite: a.hi, a.lo, b.hi, b.lo
   __shared__ float2 s_carry[kE];         // A at the step after the chunk
@@ -165,8 +169,7 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
   const uint32_t el = threadIdx.x % kE, seg = threadIdx.x / kE;
   const uint32_t segs = blockDim.x / kE, chunk = segs * kL;
   const df one = {1.f, 0.f}, zero = {0.f, 0.f};
-  const df g = df_split(gamma);
-  const df gl = df_split(gamma * lambda);
+  const df g = {g2.x, g2.y}, gl = {gl2.x, gl2.y};  // gamma, gamma lambda
   pdl_wait();
   // this thread's A and A^2 summed in double-float (the fp32 pipe)
   df a1 = zero, a2 = zero;
@@ -290,26 +293,58 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
   }
 }
 
-// Sum of the per-CTA partials (sum A, sum A^2) in a fixed order: strided
-// per-thread sums, then a shared-memory tree; the totals end in r1[0],
-// r2[0].  Every CTA that calls it gets the same bits.
+// Sum of the per-CTA partials (sum A, sum A^2) in a fixed order; the totals
+// end in *s1, *s2 of thread 0.  Every CTA that calls it gets the same bits.  Up
+// to kFewParts one warp adds and shuffles them, without a barrier (8 x 2,048:
+// 11.7 us per call, 12.7 with the tree); more take strided per-thread sums and a
+// shared-memory tree, whose levels use fewer and fewer warps of the fp64 pipe
+// (4,096 x 32: 10.3 us, 11.7 with shuffles in every warp).
+constexpr uint32_t kFewParts = 128;
 __device__ __forceinline__ void reduce_partials(const double *partial, uint32_t nparts,
-                                                double *r1, double *r2) {
+                                                double *s1, double *s2) {
+  __shared__ double r1[kNormThreads], r2[kNormThreads];
   double t1 = 0.0, t2 = 0.0;
-  for (unsigned i = threadIdx.x; i < nparts; i += kNormThreads) {
-    t1 += __ldcg(&partial[2 * i]);
-    t2 += __ldcg(&partial[2 * i + 1]);
-  }
-  r1[threadIdx.x] = t1;
-  r2[threadIdx.x] = t2;
-  __syncthreads();
-  for (int w = kNormThreads / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      r1[threadIdx.x] += r1[threadIdx.x + w];
-      r2[threadIdx.x] += r2[threadIdx.x + w];
+  if (nparts <= kFewParts) {
+    if (threadIdx.x < 32) {
+      double p1[kFewParts / 32], p2[kFewParts / 32];
+#pragma unroll
+      for (uint32_t u = 0; u < kFewParts / 32; ++u) {
+        const uint32_t i = threadIdx.x + 32 * u;
+        p1[u] = i < nparts ? __ldcg(&partial[2 * i]) : 0.0;
+        p2[u] = i < nparts ? __ldcg(&partial[2 * i + 1]) : 0.0;
+      }
+#pragma unroll
+      for (uint32_t u = 0; u < kFewParts / 32; ++u) {
+        if (32 * u >= nparts) break;
+        t1 += p1[u];
+        t2 += p2[u];
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        t1 += __shfl_down_sync(kFull, t1, o);
+        t2 += __shfl_down_sync(kFull, t2, o);
+      }
     }
+  } else {
+    for (uint32_t i = threadIdx.x; i < nparts; i += kNormThreads) {
+      t1 += __ldcg(&partial[2 * i]);
+      t2 += __ldcg(&partial[2 * i + 1]);
+    }
+    r1[threadIdx.x] = t1;
+    r2[threadIdx.x] = t2;
     __syncthreads();
+    for (int w = kNormThreads / 2; w > 0; w >>= 1) {
+      if ((int)threadIdx.x < w) {
+        r1[threadIdx.x] += r1[threadIdx.x + w];
+        r2[threadIdx.x] += r2[threadIdx.x + w];
+      }
+      __syncthreads();
+    }
+    t1 = r1[0];
+    t2 = r2[0];
   }
+  *s1 = t1;
+  *s2 = t2;
 }
 
 // This rank's statistics of A for a normalisation over several ranks:
@@ -317,14 +352,14 @@ __device__ __forceinline__ void reduce_partials(const double *partial, uint32_t 
 // order as k_gae_norm reduces them (one CTA).
 __global__ void __launch_bounds__(kNormThreads)
 k_gae_stats(const double *partial, uint32_t nparts, uint64_t n, double *stats) {
-  __shared__ double r1[kNormThreads], r2[kNormThreads];
   pdl_wait();
   pdl_launch();
-  reduce_partials(partial, nparts, r1, r2);
+  double s1, s2;
+  reduce_partials(partial, nparts, &s1, &s2);
   if (threadIdx.x == 0) {
     stats[0] = (double)n;
-    stats[1] = r1[0];
-    stats[2] = r2[0];
+    stats[1] = s1;
+    stats[2] = s2;
   }
 }
 
@@ -336,7 +371,6 @@ k_gae_stats(const double *partial, uint32_t nparts, uint64_t n, double *stats) {
 __global__ void __launch_bounds__(kNormThreads)
 k_gae_norm(const float *A_src, float *adv_norm, uint64_t n, const double *partial,
            uint32_t nparts, const double *stats) {
-  __shared__ double r1[kNormThreads], r2[kNormThreads];
   __shared__ NormStat s_stat;
   pdl_wait();
   pdl_launch();
@@ -353,9 +387,7 @@ k_gae_norm(const float *A_src, float *adv_norm, uint64_t n, const double *partia
     s1 = __ldcg(&stats[1]);
     s2 = __ldcg(&stats[2]);
   } else {
-    reduce_partials(partial, nparts, r1, r2);
-    s1 = r1[0];
-    s2 = r2[0];
+    reduce_partials(partial, nparts, &s1, &s2);  // of thread 0
   }
   if (threadIdx.x == 0) s_stat = norm_stat(nn, s1, s2);
   __syncthreads();
@@ -403,8 +435,12 @@ cudaError_t launch_scan(const GaeShape &g, const float *r, const float *v, const
                         float *ret, double *partial, float *adv_norm, cudaStream_t s) {
   auto kern = g.envs == 8 ? k_gae_scan<8> : g.envs == 4 ? k_gae_scan<4>
             : g.envs == 2 ? k_gae_scan<2> : k_gae_scan<1>;
-  return launch_pdl(kern, dim3(g.grid), dim3(g.threads), s, r, v, d, T, E, gamma, lambda, A_out,
-                    ret, partial, adv_norm);
+  auto split = [](double x) {
+    const float hi = (float)x;
+    return make_float2(hi, (float)(x - (double)hi));
+  };
+  return launch_pdl(kern, dim3(g.grid), dim3(g.threads), s, r, v, d, T, E, split(gamma),
+                    split(gamma * lambda), A_out, ret, partial, adv_norm);
 }
 
 // One CTA per SM while that leaves a thread a few elements: each CTA adds the
