@@ -5,21 +5,21 @@
 // layout and batch shape the learner consumes).
 //
 // Work decomposition: the batch's output is a flat sequence of units (a
-// 32-bit word of a frame, an 8-pixel group, an 8-byte run of a plane), cut
-// into warp spans whose size is set from the work, not from the grid: a
-// warp runs a few iterations of its unrolled loop per span and the grid
-// holds as many CTAs as that takes (several waves), so the block scheduler
-// balances the tail.  A warp walks its span segment by segment (a segment never crosses a frame or image),
-// resolving the sample's slot, episode-boundary mask and source pointer
-// once per segment.  Loads are the payload bytes a lane needs for one
-// 16-byte output store, so every warp-wide store instruction writes 512
-// contiguous bytes.  The byte->float step is x = b (exact),
-// fl32(b/255) = fma(x, r1, x*r2) with one rounding (see unit_f32), then
-// optionally the per-channel normalisation and the round-to-nearest-even
-// bfloat16 conversion.  Where one FMA per byte, bf16(fma(b, A_c, B_c)),
-// gives the same bf16 as that chain for all 256 bytes of every channel
-// (constants searched and checked on the host at creation), the
-// normalising delivery uses it instead of the five-operation chain.
+// 32-bit word of a frame, an 8-pixel group, an 8-byte run of a plane) cut into
+// runs of one or two unrolled rounds, with a CTA per run however many waves
+// that makes, so the block scheduler balances the tail.  The first CTAs collate
+// the batch's scalars.  Frame stacks are cut by warp: a warp resolves slot,
+// episode-boundary mask and source once per frame it meets.  Short frames and
+// all images are cut by CTA: a thread per frame or image the CTA touches
+// resolves it into shared memory, then all threads stream the run.  Loads are
+// the payload bytes a lane needs for one 16-byte output store, so every
+// warp-wide store instruction writes 512 contiguous bytes.  The byte->float
+// step is x = b (exact), fl32(b/255) = fma(x, r1, x*r2) with one rounding (see
+// unit_f32), then optionally the per-channel normalisation and the
+// round-to-nearest-even bfloat16 conversion.  Where one FMA per byte,
+// bf16(fma(b, A_c, B_c)), gives the same bf16 as that chain for all 256 bytes
+// of every channel (constants searched and checked on the host at creation),
+// the normalising delivery uses it instead of the five-operation chain.
 //
 // These kernels are HBM-bound: per sample they read the unique source bytes
 // once and write the (2-8x larger) output once.
@@ -31,14 +31,9 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-// loads in flight per lane (6 x 8 bytes) in the normalising delivery
-constexpr int kNormUnroll = 6;
-
-// unrolled rows per warp iteration and iterations per warp (chunk span) of
-// each kernel
+constexpr int kNormUnroll = 8;  // 8-byte loads in flight per lane in k_deliver_norm
 constexpr int kStackMinBlocks = 5;  // __launch_bounds__: at most 48 registers
 constexpr int kFlatMinBlocks = 5;
-constexpr int kNormIters = 2;
 
 struct Common {
   const int64_t *idx;
@@ -69,7 +64,7 @@ __device__ __forceinline__ bool sample_slot(const Common &c, uint32_t k,
                                             bool report) {
   if (c.draw) {
     // the uniform sampler's draw (Philox stream 0), made where it is used;
-    // the warp that delivers the sample's first unit writes its index
+    // the thread that collates the sample writes its index
     const uint64_t o = mulhi64(philox_u64(c.seed, k, c.round, 0), c.nvalid);
     const uint64_t t = c.oldest + o;
     *slot = t >= c.cap ? t - c.cap : t;
@@ -91,44 +86,6 @@ __device__ __forceinline__ bool sample_slot(const Common &c, uint32_t k,
   *slot = (uint64_t)s;
   *off = o;
   return true;
-}
-
-// Minimum of q over the batch (one warp): loads are issued 8 per lane at a
-// time so a batch of 512 costs two memory round trips, not sixteen.
-__device__ __forceinline__ uint32_t batch_qmin(const Common &c, int lane) {
-  uint32_t m = 0xffffffffu;
-  for (uint32_t i0 = lane; i0 < c.B; i0 += 32 * 8) {
-    uint32_t v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const uint32_t i = i0 + u * 32;
-      v[u] = i < c.B ? __ldg(c.q + i) : 0xffffffffu;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) m = min(m, v[u]);
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) m = min(m, __shfl_xor_sync(kFull, m, o));
-  return m;
-}
-
-// Per-sample collate, importance weight and scalar gathers (one warp).  The
-// head warp of each sample runs this before its payload span, so the fp64
-// chain of the weight overlaps the other warps' streaming.
-__device__ void collate(const Common &c, uint32_t k, bool ok, uint64_t slot,
-                        uint64_t off, int lane) {
-  if (lane == 0) {
-    if (c.act_out) c.act_out[k] = ok ? c.action[slot] : 0;
-    if (c.rew_out) c.rew_out[k] = ok ? c.reward[slot] : 0.f;
-    if (c.done_out) c.done_out[k] = ok ? c.done[slot] : (uint8_t)0;
-    if (c.gdst0) c.gdst0[k] = ok ? c.gsrc0[off] : 0.f;
-    if (c.gdst1) c.gdst1[k] = ok ? c.gsrc1[off] : 0.f;
-  }
-  if (c.isw) {
-    // PER: w = (q_min / q_k)^beta, q_min over the batch; fp64, one rounding
-    const uint32_t m = batch_qmin(c, lane);
-    if (lane == 0) c.isw[k] = is_weight(m, c.q[k], c.beta);
-  }
 }
 
 // Minimum of q over the batch (the CTA): every thread gets it.  16-byte loads
@@ -190,17 +147,6 @@ __device__ void collate_batch(const Common &c, uint32_t cta, uint32_t ncta) {
     if (c.gdst1) c.gdst1[k] = ok ? c.gsrc1[off] : 0.f;
     if (c.isw) c.isw[k] = is_weight(m, c.q[k], c.beta);
   }
-}
-
-// [*f, *end): this warp's contiguous share of `total` units, rounded up to
-// whole 32-unit rows so lanes stay aligned with the rows of the output.
-__device__ __forceinline__ void warp_span(uint64_t total, uint64_t *f,
-                                          uint64_t *end) {
-  const uint64_t nw = (uint64_t)gridDim.x * kWarps;
-  const uint64_t gw = (uint64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
-  const uint64_t span = (((total + nw - 1) / nw) + 31) & ~31ull;
-  *f = gw * span;
-  *end = min(total, *f + span);
 }
 
 // exact integer -> float for a byte: 0x4B0000bb is 2^23 + b
@@ -582,140 +528,165 @@ cudaError_t launch_hwc(const Common &c, ChwArgs a, cudaStream_t s) {
 // CHW uint8 -> per-channel normalised bfloat16 (multimodal payloads), with
 // token collate; optionally two-tier (payload of older transitions in
 // page-locked host memory, read over the host link).  Unit = 8 bytes: a lane
-// converts 8 consecutive bytes of one channel plane to one 16-byte store.
+// converts 8 consecutive bytes of one channel plane to one 16-byte store.  The
+// first `ncollate` CTAs collate the batch, the next `ntok` copy the tokens, and
+// each of the others takes `units` consecutive units of the batch, whatever
+// images they belong to: a thread per image (or token row) it touches resolves
+// the row into shared memory, then all threads stream the units as one flat
+// range, UN loads in flight each.  Bound by HBM for large batches, by the chain
+// of dependent loads for small ones.  Calls in a row, in us, and (before) when a
+// warp walked its span image by image and collated at each image:
+//   images of     64x64x3      96x96x3 + 128   224x224x3 + 512  84x84x1     16x16x1
+//   B = 64        3.1 (3.3)    3.1 (3.6)       5.7 (7.7)        2.8 (4.2)   2.6 (6.2)
+//   B = 256       3.7 (3.6)    5.1 (6.5)       17.9 (17.7)      2.8 (4.4)   2.6 (8.7)
+//   B = 1,024     7.4 (8.9)    13.3 (13.2)     71.3 (71.2)      5.1 (7.8)   2.6 (9.0)
+// 6 units in flight and 4 CTAs per SM, or 8 and 3: 7% slower at 224x224x3, B =
+// 1,024; 4 and 5: 10%.
 // ---------------------------------------------------------------------------
 struct NormArgs {
   const uint8_t *obs_h;   // HBM ring [cap_h][F]
   const uint8_t *obs_c;   // host ring [cap_c][F] (device-mapped) or null
   const int32_t *tok_h;
   const int32_t *tok_c;
-  uint64_t cap_h, cap_c, total, size;
+  uint64_t cap_h, cap_c;
+  // offsets below `cold` (older ones) live in the host tier; physical rows of
+  // the oldest offset there and of offset `cold` in HBM
+  uint64_t cold, first_c, first_h;
   uint32_t F8;    // 8-byte units per image
   uint32_t HW8;   // 8-byte units per channel plane
   uint32_t L16;   // 16-byte units of tokens per transition
+  uint32_t units, tunits;  // image and token units per CTA
+  uint32_t div_f, div_l;  // ceil(2^32 / F8), ceil(2^32 / L16); 0: a CTA spans at most two rows
+  uint32_t ncollate, ntok;
   float mean[4], s1[4], s2[4], sd[4];
   float aa[4], ab[4];  // one-FMA form (AFF): bf16(fma(b, aa, ab))
   int fast;
   __nv_bfloat16 *out;
   int32_t *tok_out;
 };
+constexpr int kNormCtas = 4;               // CTAs per SM
+constexpr uint32_t kNormRows = kThreads;   // at most touched by a CTA
+constexpr uint32_t kTokUnroll = 4;         // 16-byte token loads in flight per lane
+constexpr uint32_t kTokUnits = kThreads * kTokUnroll;
 
-template <int UN, bool AFF>
-__global__ void __launch_bounds__(kThreads)
-k_deliver_norm(Common c, NormArgs a) {
-  const int lane = threadIdx.x & 31;
-  const uint64_t pol = policy_stream();
-  pdl_wait();
-  pdl_launch();
-  const uint64_t total = (uint64_t)c.B * a.F8;
-  uint64_t f, end;
-  warp_span(total, &f, &end);
-  while (f < end) {
-    const uint32_t k = (uint32_t)(f / a.F8);
-    const uint32_t u_lo = (uint32_t)(f - (uint64_t)k * a.F8);
-    const uint64_t seg_end = min(end, (uint64_t)(k + 1) * a.F8);
-    const uint32_t u_hi = (uint32_t)(seg_end - (uint64_t)k * a.F8);
-    const bool head = u_lo == 0;
-    uint64_t slot = 0, off = 0;
-    const bool ok = sample_slot(c, k, &slot, &off, head && lane == 0);
-    if (head) collate(c, k, ok, slot, off, lane);
-    // tier of the logical id L = total - size + off
-    const uint64_t L = a.total - a.size + off;
-    const uint64_t in_hbm = a.total < a.cap_h ? a.total : a.cap_h;
-    const bool hbm = !a.obs_c || L >= a.total - in_hbm;
-    const uint64_t ps = hbm ? L % a.cap_h : L % a.cap_c;
-    const uint8_t *obs = hbm ? a.obs_h : a.obs_c;
-    const uint2 *src = reinterpret_cast<const uint2 *>(obs + ps * a.F8 * 8ull);
-    uint4 *dst = reinterpret_cast<uint4 *>(a.out + (uint64_t)k * a.F8 * 8ull);
-    for (uint32_t u0 = u_lo + lane; u0 < u_hi; u0 += 32 * UN) {
-      uint2 v[UN];
-#pragma unroll
-      for (int u = 0; u < UN; ++u) {
-        const uint32_t w = u0 + u * 32;
-        // HBM tier: streaming non-coherent loads; host tier: plain loads of
-        // the mapped page-locked memory
-        v[u] = (ok && w < u_hi) ? (hbm ? ld_stream(src + w, pol) : src[w])
-                                : make_uint2(0u, 0u);
-      }
-#pragma unroll
-      for (int u = 0; u < UN; ++u) {
-        const uint32_t w = u0 + u * 32;
-        if (w >= u_hi) continue;
-        const uint32_t ch = (w >= a.HW8) + (w >= 2 * a.HW8) + (w >= 3 * a.HW8);
-        float fv[8];
-        if constexpr (AFF) {
-          const float A = a.aa[ch], Bc = a.ab[ch];
-#pragma unroll
-          for (int bb = 0; bb < 8; ++bb)
-            fv[bb] = __fmaf_rn(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), A, Bc);
-        } else {
-          const float mc = a.mean[ch], s1 = a.s1[ch], s2 = a.s2[ch];
-#pragma unroll
-          for (int bb = 0; bb < 8; ++bb) {
-            const float x = unit_f32(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), c.r1, c.r2);
-            const float tt = __fsub_rn(x, mc);
-            fv[bb] = a.fast ? __fmaf_rn(tt, s1, __fmul_rn(tt, s2)) : __fdiv_rn(tt, a.sd[ch]);
-          }
-        }
-        uint4 o;
-        o.x = pack_bf16x2(fv[0], fv[1]);
-        o.y = pack_bf16x2(fv[2], fv[3]);
-        o.z = pack_bf16x2(fv[4], fv[5]);
-        o.w = pack_bf16x2(fv[6], fv[7]);
-        if (!ok) o = make_uint4(0u, 0u, 0u, 0u);
-        st_stream(dst + w, o, pol);
-      }
-    }
-    if (head) {
-      // a two-tier row read over the host link (edp_get_counters)
-      if (lane == 0 && ok && a.obs_c && !hbm)
-        atomicAdd(&c.ctrl->host_bytes,
-                  (unsigned long long)a.F8 * 8ull + (a.tok_out ? a.L16 * 16ull : 0ull));
-      if (a.tok_out) {
-        // the row's tokens, kTokBatch 16-byte loads per lane in flight
-        // before their stores
-        constexpr int kTokBatch = 4;
-        const uint4 *ts = reinterpret_cast<const uint4 *>(
-            (hbm ? a.tok_h : a.tok_c) + ps * a.L16 * 4ull);
-        uint4 *td = reinterpret_cast<uint4 *>(a.tok_out + (uint64_t)k * a.L16 * 4ull);
-        for (uint32_t i0 = lane; i0 < a.L16; i0 += 32 * kTokBatch) {
-          uint4 t4[kTokBatch];
-#pragma unroll
-          for (int u = 0; u < kTokBatch; ++u) {
-            const uint32_t i = i0 + u * 32;
-            t4[u] = (ok && i < a.L16) ? ts[i] : make_uint4(0u, 0u, 0u, 0u);
-          }
-#pragma unroll
-          for (int u = 0; u < kTokBatch; ++u)
-            if (i0 + u * 32 < a.L16) td[i0 + u * 32] = t4[u];
-        }
-      }
-    }
-    f = seg_end;
-  }
+// Physical row of sample k in its tier; false for a bad index.
+__device__ __forceinline__ bool norm_row(const Common &c, const NormArgs &a, uint32_t k,
+                                         uint64_t *row, bool *hbm) {
+  uint64_t slot = 0, off = 0;
+  if (!sample_slot(c, k, &slot, &off, false)) return false;
+  *hbm = off >= a.cold;
+  const uint64_t at = *hbm ? a.first_h + (off - a.cold) : a.first_c + off;
+  const uint64_t cap = *hbm ? a.cap_h : a.cap_c;
+  *row = at >= cap ? at - cap : at;
+  return true;
 }
 
-// Grid size from the work: enough CTAs that each warp runs about `iters`
-// iterations of its unrolled loop (`per_iter` units each), so the block
-// scheduler balances the tail and a CTA that starts late (its SM still busy
-// with another kernel) holds up little work; a small batch is spread over up
-// to one wave (blocks resident per SM x SMs, queried once per kernel) with
-// at least one iteration per warp.
-template <typename Kern>
-unsigned grid_for(Kern kern, uint64_t units, uint64_t per_iter, int iters, int sms) {
-  static int per_sm = 0;  // per template instantiation
-  if (!per_sm) {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0);
-    if (per_sm < 1) per_sm = 1;
+// i / d with inv = ceil(2^32 / d) (i d < 2^32), or for i < 2 d without one.
+__device__ __forceinline__ uint32_t row_of_unit(uint32_t i, uint32_t d, uint32_t inv) {
+  return inv ? __umulhi(i, inv) : (i >= d ? 1u : 0u);
+}
+
+template <int UN, bool AFF, bool TWO>
+__global__ void __launch_bounds__(kThreads, kNormCtas)
+k_deliver_norm(Common c, NormArgs a) {
+  __shared__ uint64_t s_src[kNormRows];  // a row's address (16-byte aligned), its lowest bit
+                                         // set in HBM; 0: a bad index
+  const uint64_t pol = policy_stream();
+  const bool tok = blockIdx.x >= a.ncollate && blockIdx.x < a.ncollate + a.ntok;
+  // units [u0, u0 + n) of the batch's rows of P units; the first is unit i_0 of
+  // row k0
+  const uint32_t P = tok ? a.L16 : a.F8;
+  const uint64_t total = (uint64_t)c.B * P;
+  const uint64_t u0 = tok ? (uint64_t)(blockIdx.x - a.ncollate) * a.tunits
+                          : (uint64_t)(blockIdx.x - a.ncollate - a.ntok) * a.units;
+  const uint64_t k0 = u0 <= 0xffffffffu ? (uint32_t)u0 / P : u0 / P;
+  const uint32_t i_0 = (uint32_t)(u0 - k0 * P);
+  const uint32_t i_1 = i_0 + (uint32_t)min((uint64_t)(tok ? a.tunits : a.units), total - u0);
+  pdl_wait();
+  pdl_launch();
+  if (blockIdx.x < a.ncollate) {
+    collate_batch(c, blockIdx.x, a.ncollate);
+    return;
   }
-  const uint64_t wave = (uint64_t)per_sm * sms;
-  const uint64_t warp_iters = (units + per_iter - 1) / per_iter;
-  uint64_t blocks = (warp_iters + (uint64_t)kWarps * iters - 1) / ((uint64_t)kWarps * iters);
-  if (blocks < wave) {
-    const uint64_t most = (warp_iters + kWarps - 1) / kWarps;
-    blocks = most < wave ? most : wave;
+  if (threadIdx.x <= (i_1 - 1) / P) {
+    uint64_t row = 0, src = 0;
+    bool hbm = true;
+    if (norm_row(c, a, (uint32_t)(k0 + threadIdx.x), &row, &hbm)) {
+      if (tok) {
+        src = (uint64_t)((hbm ? a.tok_h : a.tok_c) + row * a.L16 * 4ull);
+      } else {
+        src = (uint64_t)((hbm ? a.obs_h : a.obs_c) + row * a.F8 * 8ull);
+        // a two-tier row read over the host link (edp_get_counters), counted
+        // where its first unit is read
+        if (!hbm && (threadIdx.x || i_0 == 0))
+          atomicAdd(&c.ctrl->host_bytes,
+                    (unsigned long long)a.F8 * 8ull + (a.tok_out ? a.L16 * 16ull : 0ull));
+      }
+      src |= hbm ? 1u : 0u;
+    }
+    s_src[threadIdx.x] = src;
   }
-  return (unsigned)(blocks ? blocks : 1);
+  __syncthreads();
+  if (tok) {
+    uint4 v[kTokUnroll];
+#pragma unroll
+    for (uint32_t u = 0; u < kTokUnroll; ++u) {
+      const uint32_t i = i_0 + threadIdx.x + u * kThreads;
+      const uint32_t s = P == 1 ? i : row_of_unit(i, P, a.div_l);  // 2^32 / 1 has no 32 bits
+      const uint64_t src = i < i_1 ? s_src[s] & ~1ull : 0;
+      v[u] = src ? reinterpret_cast<const uint4 *>(src)[i - s * P] : make_uint4(0u, 0u, 0u, 0u);
+    }
+    uint4 *dst = reinterpret_cast<uint4 *>(a.tok_out) + k0 * P;
+#pragma unroll
+    for (uint32_t u = 0; u < kTokUnroll; ++u) {
+      const uint32_t i = i_0 + threadIdx.x + u * kThreads;
+      if (i < i_1) dst[i] = v[u];
+    }
+    return;
+  }
+  uint4 *dst = reinterpret_cast<uint4 *>(a.out) + k0 * P;
+  for (uint32_t i0 = i_0 + threadIdx.x; i0 < i_1; i0 += kThreads * UN) {
+    uint2 v[UN];
+#pragma unroll
+    for (int u = 0; u < UN; ++u) {
+      const uint32_t i = i0 + u * kThreads;
+      const uint32_t s = row_of_unit(i, P, a.div_f);
+      const uint64_t src = i < i_1 ? s_src[s] : 0;
+      const uint2 *p = reinterpret_cast<const uint2 *>(src & ~1ull) + (i - s * P);
+      // HBM tier: streaming non-coherent loads; host tier: plain loads of the
+      // mapped page-locked memory
+      v[u] = src ? (!TWO || (src & 1u) ? ld_stream(p, pol) : *p) : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int u = 0; u < UN; ++u) {
+      const uint32_t i = i0 + u * kThreads;
+      if (i >= i_1) continue;
+      const uint32_t s = row_of_unit(i, P, a.div_f), w = i - s * P;
+      const uint32_t ch = (w >= a.HW8) + (w >= 2 * a.HW8) + (w >= 3 * a.HW8);
+      float fv[8];
+      if constexpr (AFF) {
+        const float A = a.aa[ch], Bc = a.ab[ch];
+#pragma unroll
+        for (int bb = 0; bb < 8; ++bb)
+          fv[bb] = __fmaf_rn(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), A, Bc);
+      } else {
+        const float mc = a.mean[ch], s1 = a.s1[ch], s2 = a.s2[ch];
+#pragma unroll
+        for (int bb = 0; bb < 8; ++bb) {
+          const float x = unit_f32(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), c.r1, c.r2);
+          const float tt = __fsub_rn(x, mc);
+          fv[bb] = a.fast ? __fmaf_rn(tt, s1, __fmul_rn(tt, s2)) : __fdiv_rn(tt, a.sd[ch]);
+        }
+      }
+      uint4 o;
+      o.x = pack_bf16x2(fv[0], fv[1]);
+      o.y = pack_bf16x2(fv[2], fv[3]);
+      o.z = pack_bf16x2(fv[4], fv[5]);
+      o.w = pack_bf16x2(fv[6], fv[7]);
+      if (!s_src[s]) o = make_uint4(0u, 0u, 0u, 0u);
+      st_stream(dst + i, o, pol);
+    }
+  }
 }
 
 }  // namespace
@@ -809,8 +780,12 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     a.tok_c = ctx->cap_c ? ctx->st.host_tokens : nullptr;
     a.cap_h = ctx->cap_h;
     a.cap_c = ctx->cap_c ? ctx->cap_c : 1;
-    a.total = ctx->total;
-    a.size = size;
+    // ids total - size + off; the newest min(total, cap_h) of them in HBM at id
+    // mod cap_h, the older ones in the host tier at id mod cap_c
+    const uint64_t in_hbm = ctx->total < ctx->cap_h ? ctx->total : ctx->cap_h;
+    a.cold = size > in_hbm ? size - in_hbm : 0;
+    a.first_h = (ctx->total - size + a.cold) % a.cap_h;
+    a.first_c = (ctx->total - size) % a.cap_c;
     a.F8 = (uint32_t)(ctx->obs_bytes / 8);
     a.HW8 = cfg.obs_h * cfg.obs_w / 8;
     a.L16 = (uint32_t)(ctx->tok_bytes / 16);
@@ -825,13 +800,31 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     a.fast = ctx->norm_fast;
     a.out = (__nv_bfloat16 *)out->obs;
     a.tok_out = out->tokens;
-    const uint64_t units = (uint64_t)B * a.F8;
-    auto kern = ctx->norm_affine ? k_deliver_norm<kNormUnroll, true>
-                                 : k_deliver_norm<kNormUnroll, false>;
-    return launch_pdl(kern, dim3(grid_for(kern, units, 32 * kNormUnroll, kNormIters, sms)),
-                      dim3(kThreads), s, c, a);
+    a.ncollate = collate_ctas(B, out->isw != nullptr);
+    const uint64_t tok_units = a.tok_out ? (uint64_t)B * a.L16 : 0;
+    const uint64_t rows = kNormRows - 2, total = (uint64_t)B * a.F8;
+    a.tunits = rows * a.L16 < kTokUnits ? (uint32_t)(rows * a.L16) : kTokUnits;
+    const uint64_t ntok = tok_units ? (tok_units + a.tunits - 1) / a.tunits : 0;
+    a.ntok = (uint32_t)ntok;
+    // One round per CTA up to two waves of CTAs, two rounds above (us, one
+    // round against two, B images of 64x64x3: 1,024 7.4, 8.7; 4,096 24.4, 24.4;
+    // of 96x96x3: 256 5.1, 5.9; 1,024 13.9, 13.3; of 224x224x3: 64 5.7, 6.4;
+    // 256 18.9, 17.9; 1,024 71.7, 71.3); three and more lose 1-5%.
+    uint64_t units = (uint64_t)kThreads * kNormUnroll;
+    if (total > 2 * (uint64_t)kNormCtas * sms * units) units *= 2;
+    if (units > rows * a.F8) units = (rows * a.F8) & ~31ull;
+    a.units = (uint32_t)units;
+    a.div_f = a.F8 < 32768 ? (uint32_t)((0x100000000ull + a.F8 - 1) / a.F8) : 0u;
+    a.div_l = a.L16 && a.L16 < 32768 ? (uint32_t)((0x100000000ull + a.L16 - 1) / a.L16) : 0u;
+    const uint64_t ctas = (total + units - 1) / units + a.ncollate + a.ntok;
+    if (ctas > 0x7FFFFFFFull || ntok > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    auto kern = ctx->norm_affine
+                    ? (a.obs_c ? k_deliver_norm<kNormUnroll, true, true>
+                               : k_deliver_norm<kNormUnroll, true, false>)
+                    : (a.obs_c ? k_deliver_norm<kNormUnroll, false, true>
+                               : k_deliver_norm<kNormUnroll, false, false>);
+    return launch_pdl(kern, dim3((unsigned)ctas), dim3(kThreads), s, c, a);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace edp
