@@ -406,33 +406,39 @@ __device__ __forceinline__ bool slot_holds(int64_t sl, uint64_t cap, uint64_t ol
 // ones take k_update_small below).  The slots are split over the CTAs by a
 // hash, so a slot has one owner and repeats of it meet in one CTA: no
 // scratch, no second phase, no CTA waits for another.  Every CTA reads the
-// whole batch's slots (8 bytes a pair, from the L2), kUpdLoads in flight per
-// thread, and keeps its own in a shared-memory hash table that holds, per
-// slot, the largest batch position (atomicMax): the last pair wins.  The owner
-// test comes first, on the slot's low word alone, so that a foreign pair costs
-// a few instructions.  The CTA then evaluates the priority of each winner (a
-// list of the occupied entries keeps the lanes of that evaluation full),
-// writes its leaf and adds the exact
-// signed delta to the ancestors (two's complement wrap makes negative deltas
-// exact): deeper nodes rarely collide and take one 64-bit atomic per pair,
-// level 1 (32 nodes) and the root are summed on chip first.  A batch whose
-// distinct slots of one owner outgrow its table is applied in batch order, a
-// part at a time (a part's leaves are read again by the next).  The
-// running maximum counts every pair, the overwritten ones too, so each warp
-// evaluates a stripe of the batch for it.
+// low words of the whole batch's slots (out of the L2), kUpdLow in flight per
+// thread, and lists the positions of its own.  The owner test is a product on
+// the low word, so that a foreign pair costs a few instructions; all else is
+// done for the listed pairs, whose lanes are full.  They enter a shared-memory
+// hash table that holds, per slot, the largest batch position (atomicMax): the
+// last pair wins.  The CTA then evaluates the priority of each winner (a list
+// of the occupied entries), writes its leaf and adds the exact signed delta to
+// the ancestors (two's complement wrap makes negative deltas exact): deeper
+// nodes rarely collide and take one 64-bit atomic per pair, level 1 (32 nodes)
+// and the root are summed on chip first.  A batch of more pairs per CTA than
+// half of the list, or with more pairs of one owner than the list holds, is
+// entered in batch order, a part at a time where its distinct slots outgrow the
+// table (a part's leaves are read again by the next).  The running maximum
+// counts every pair, the overwritten ones too, so each warp evaluates a stripe
+// of the batch for it.
 //
-// Bound by the scan above ~10,000 pairs (32,768 pairs are 256 KB per CTA, 40
-// MB out of the L2), by latency below.  Calls in a row from TD errors,
-// 1,000,000 slots: 4,096 pairs 7.0 us, 32,768 pairs 13.6 us, 131,072 pairs 40
-// us; 28.5, 214.6 and 849.5 us when one CTA applied the batch 1,024 pairs at a
-// time.
+// Bound by latency up to ~10,000 pairs, by the scan above.  Calls in a row from
+// TD errors, 1,000,000 slots, and (one CTA that applied the batch 1,024 pairs at
+// a time): 4,096 pairs 6.4 us (28.5), 32,768 pairs 9.0 (214.6), 131,072 pairs
+// 19.5 (849.5).  With every pair tested in full and entered where it was found,
+// at one pair in 32 lanes: 7.0, 13.6 and 40; halves of the scan by pairs of CTAs
+// that enter each other's tables over the cluster: no gain over that.
 constexpr int kUpdThreads = 1024;
 constexpr int kUpdLoads = 8;                         // slots in flight per thread
 constexpr int kUpdChunk = kUpdThreads * kUpdLoads;   // pairs scanned at a time
 constexpr int kUpdGroup = 2;                         // loads applied at a time when a table fills
 constexpr uint32_t kUpdTable = 4096;                 // open addressing, at most 3/4 full
-static_assert(kUpdLoads % kUpdGroup == 0 && kUpdThreads * kUpdGroup <= kUpdTable / 4 * 3,
+constexpr uint32_t kUpdMost = kUpdTable / 4 * 3;
+constexpr int kUpdLow = 8;                          // low words in flight per thread
+constexpr uint32_t kUpdList = 2048;                  // pairs of an owner listed by the scan
+static_assert(kUpdLoads % kUpdGroup == 0 && kUpdThreads * kUpdGroup <= kUpdMost,
               "a group of loads fits an empty table");
+static_assert(kUpdList <= kUpdMost, "the listed pairs fit an empty table");
 
 __device__ __noinline__ uint32_t prio_td_call(float td, const PrioRule &rule) {
   return prio_td(td, rule);
@@ -444,8 +450,9 @@ k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict
          uint64_t cap, uint64_t oldest, uint64_t size, int defer, Ctrl *ctrl) {
   __shared__ uint32_t hkey[kUpdTable];
   __shared__ uint32_t hpos[kUpdTable];
-  __shared__ uint16_t used[kUpdTable / 4 * 3];  // occupied entries, in any order
-  __shared__ uint32_t s_used;
+  __shared__ uint16_t used[kUpdMost];  // occupied entries, in any order
+  __shared__ uint32_t list[kUpdList];   // batch positions
+  __shared__ uint32_t s_used, s_listed;
   __shared__ uint32_t acc_lo[32], acc_hi[32];
   __shared__ unsigned long long warp_root[kUpdThreads / 32];
   __shared__ uint32_t s_sel, s_qmax;
@@ -461,6 +468,7 @@ k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict
   if (threadIdx.x == 0) {
     s_sel = 0;
     s_used = 0;
+    s_listed = 0;
     s_qmax = 0;
   }
   // Nothing in memory is read or written before the wait on the preceding
@@ -533,40 +541,84 @@ k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict
     __syncthreads();
   };
 
-  for (uint64_t base = 0; base < n; base += kUpdChunk) {
-    int64_t s[kUpdLoads];
+  auto owned = [&](uint32_t low) {
+    return __umulhi(low * 0x9E3779B1u, gridDim.x) == blockIdx.x;
+  };
+  // The scan lists the positions of the pairs owned here; no warp waits for
+  // another until the batch has been read.
+  const bool scan = n <= gridDim.x * (kUpdList / 2);
+  if (scan) {
+    const uint2 *slots = reinterpret_cast<const uint2 *>(idx);
+    for (uint32_t base = 0; base < n; base += kUpdThreads * kUpdLow) {
+      uint32_t low[kUpdLow], mine = 0;
+      if (base + kUpdThreads * kUpdLow <= n) {
 #pragma unroll
-    for (int u = 0; u < kUpdLoads; ++u) {
-      const uint64_t p = base + u * kUpdThreads + threadIdx.x;
-      s[u] = p < n ? idx[p] : -1;
-    }
-    uint32_t mine = 0;  // bit u: slot u is owned here
+        for (int u = 0; u < kUpdLow; ++u)
+          low[u] = __ldg(&slots[base + u * kUpdThreads + threadIdx.x].x);
 #pragma unroll
-    for (int u = 0; u < kUpdLoads; ++u) {
-      uint64_t k = 0;
-      if (__umulhi((uint32_t)s[u] * 0x9E3779B1u, gridDim.x) == blockIdx.x &&
-          slot_holds(s[u], cap, oldest, size, &k))
-        mine |= 1u << u;
+        for (int u = 0; u < kUpdLow; ++u) mine |= owned(low[u]) ? 1u << u : 0u;
+      } else {
+#pragma unroll
+        for (int u = 0; u < kUpdLow; ++u) {
+          const uint32_t p = base + u * kUpdThreads + threadIdx.x;
+          low[u] = p < n ? __ldg(&slots[p].x) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < kUpdLow; ++u)
+          mine |= owned(low[u]) && base + u * kUpdThreads + threadIdx.x < n ? 1u << u : 0u;
+      }
+      if (!mine) continue;
+      uint32_t at = atomicAdd(&s_listed, (uint32_t)__popc(mine));
+      do {
+        if (at < kUpdList) list[at] = base + (__ffs(mine) - 1) * kUpdThreads + threadIdx.x;
+        ++at;
+        mine &= mine - 1;
+      } while (mine);
     }
-    if (mine) atomicAdd(&s_sel, (uint32_t)__popc(mine));
     __syncthreads();
-    const bool fits = s_sel <= kUpdTable / 4 * 3;
-    __syncthreads();  // every thread has read s_sel
-    if (fits) {
-#pragma unroll
-      for (int u = 0; u < kUpdLoads; ++u)
-        if ((mine >> u) & 1u)
-          insert((uint32_t)s[u], (uint32_t)base + u * kUpdThreads + threadIdx.x);
-      continue;
+  }
+  if (scan && s_listed <= kUpdList) {
+    for (uint32_t i = threadIdx.x; i < s_listed; i += kUpdThreads) {
+      const int64_t sl = idx[list[i]];
+      uint64_t k = 0;
+      if (slot_holds(sl, cap, oldest, size, &k)) insert((uint32_t)sl, list[i]);
     }
-    apply();  // the earlier pairs, then this chunk's a group at a time
+  } else {
+    // A batch beyond the list, or most of it on few owners: in order, as many
+    // pairs at a time as the table holds.
+    for (uint64_t base = 0; base < n; base += kUpdChunk) {
+      int64_t s[kUpdLoads];
 #pragma unroll
-    for (int g = 0; g < kUpdLoads; g += kUpdGroup) {
+      for (int u = 0; u < kUpdLoads; ++u) {
+        const uint64_t p = base + u * kUpdThreads + threadIdx.x;
+        s[u] = p < n ? idx[p] : -1;
+      }
+      uint32_t mine = 0;  // bit u: slot u is owned here
 #pragma unroll
-      for (int u = g; u < g + kUpdGroup; ++u)
-        if ((mine >> u) & 1u)
-          insert((uint32_t)s[u], (uint32_t)base + u * kUpdThreads + threadIdx.x);
-      apply();
+      for (int u = 0; u < kUpdLoads; ++u) {
+        uint64_t k = 0;
+        if (owned((uint32_t)s[u]) && slot_holds(s[u], cap, oldest, size, &k)) mine |= 1u << u;
+      }
+      if (mine) atomicAdd(&s_sel, (uint32_t)__popc(mine));
+      __syncthreads();
+      const bool fits = s_sel <= kUpdMost;
+      __syncthreads();  // every thread has read s_sel
+      if (fits) {
+#pragma unroll
+        for (int u = 0; u < kUpdLoads; ++u)
+          if ((mine >> u) & 1u)
+            insert((uint32_t)s[u], (uint32_t)base + u * kUpdThreads + threadIdx.x);
+        continue;
+      }
+      apply();  // the earlier pairs, then this chunk's a group at a time
+#pragma unroll
+      for (int g = 0; g < kUpdLoads; g += kUpdGroup) {
+#pragma unroll
+        for (int u = g; u < g + kUpdGroup; ++u)
+          if ((mine >> u) & 1u)
+            insert((uint32_t)s[u], (uint32_t)base + u * kUpdThreads + threadIdx.x);
+        apply();
+      }
     }
   }
   apply();

@@ -56,3 +56,17 @@ def test_large_update(edp_lib, orc, big, n, slots):
     edp.edp_sync(m.ring.ctx)
     orc.update_leaves(m.st, m.total, idx, qu)
     check_tree(orc, m.ring, m.st)
+
+
+@pytest.mark.parametrize("slots", ["spread", "few"])
+def test_beyond_the_list(edp_lib, orc, big, slots):
+    """More pairs per CTA than the scan lists: entered in batch order."""
+    edp, m = edp_lib, big
+    n = 1024 * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    rng = np.random.default_rng(5)
+    idx = rng.choice(CAP if slots == "spread" else 40, size=n).astype(np.int64)
+    qu = rng.integers(0, 1 << 32, size=n, dtype=np.uint64).astype(np.uint32)
+    edp.edp_update_priorities(m.ring.ctx, cuda(idx), cuda(qu), n)
+    edp.edp_sync(m.ring.ctx)
+    orc.update_leaves(m.st, m.total, idx, qu)
+    check_tree(orc, m.ring, m.st)
