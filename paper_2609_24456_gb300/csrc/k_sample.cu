@@ -17,9 +17,11 @@
 //            re-zero the counters for the next call
 // With nb ~ n/4 buckets (up to 32,768 elements) a bucket holds ~4 keys; above
 // that it holds n / 8192.  The result does not depend on the order of the
-// counting.  Calls in a row: 32,768 elements 9.4 us, 262,144 25.3 us,
-// 1,048,576 96 us; 13.3, 238.5 and 3,366 us when every element read its
-// bucket from the L2 and the counts were scanned from 4-byte loads.
+// counting.  Bound by the latency of the three kernels' chains up to ~100,000
+// elements, by the counting atomics and the 16-byte scattered writes above.
+// Calls in a row: 32,768 elements 7.8 us, 262,144 20.1 us, 1,048,576 78.6 us;
+// 13.3, 238.5 and 3,366 us when every element read its bucket from the L2 and
+// the counts were scanned from 4-byte loads.
 #include "edp_internal.cuh"
 
 namespace edp {
@@ -89,62 +91,58 @@ k_perm_keys(uint32_t n, uint64_t seed, uint64_t round, int lg, PermScratch sc) {
   }
 }
 
-// Exclusive scan of the nb bucket counts into smem start[] (padded layout:
-// each thread scans 32 consecutive entries without bank conflicts).
-__device__ __forceinline__ uint32_t pad32(uint32_t i) { return i + i / 32; }
-
 __global__ void __launch_bounds__(kPermThreads)
 k_perm_scatter(uint32_t n, int lg, PermScratch sc) {
-  __shared__ uint32_t start[kMaxBuckets + kMaxBuckets / 32];
+  // Exclusive scan of the bucket counts: a warp takes 1,024 consecutive ones as
+  // rows of 16-byte vectors, all in flight before the first is used, and scans
+  // the vectors' sums by shuffles (48 a lane; 96 loads and stores of shared
+  // memory when each thread scanned 32 counts there).
+  __shared__ __align__(16) uint32_t start[kMaxBuckets];
   __shared__ uint32_t warp_tot[kPermThreads / 32];
   const uint32_t nb = 1u << lg;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int kVecs = kMaxBuckets / 4 / kPermThreads;
+  const uint32_t v0 = wid * 32 * kVecs + lane;
   pdl_wait();
   pdl_launch();
-  // 16-byte loads, all in flight before the first is used
-  constexpr int kVecs = kMaxBuckets / 4 / kPermThreads;
   uint4 c4[kVecs];
 #pragma unroll
   for (int u = 0; u < kVecs; ++u) {
-    const uint32_t i = 4 * (u * kPermThreads + threadIdx.x);
+    const uint32_t i = 4 * (v0 + u * 32);
     // counts past nb stay zero between calls: whole vectors may be read
     c4[u] = i < nb ? __ldcg(reinterpret_cast<const uint4 *>(sc.count + i))
                    : make_uint4(0u, 0u, 0u, 0u);
   }
+  uint32_t before[kVecs], run = 0;
 #pragma unroll
   for (int u = 0; u < kVecs; ++u) {
-    const uint32_t i = pad32(4 * (u * kPermThreads + threadIdx.x));
-    start[i] = c4[u].x;
-    start[i + 1] = c4[u].y;
-    start[i + 2] = c4[u].z;
-    start[i + 3] = c4[u].w;
+    const uint32_t sum = c4[u].x + c4[u].y + c4[u].z + c4[u].w;
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    before[u] = run + incl - sum;
+    run += __shfl_sync(0xffffffffu, incl, 31);
   }
+  if (lane == 0) warp_tot[wid] = run;
   __syncthreads();
-  constexpr uint32_t per = kMaxBuckets / kPermThreads;  // 32
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint32_t b0 = threadIdx.x * per;
-  uint32_t run = 0;
+  uint32_t acc = 0;
 #pragma unroll
-  for (uint32_t i = 0; i < per; ++i) run += start[pad32(b0 + i)];
-  uint32_t incl = run;
+  for (int w = 0; w < kPermThreads / 32; ++w) acc += w < wid ? warp_tot[w] : 0u;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) warp_tot[wid] = incl;
-  __syncthreads();
-  uint32_t acc = incl - run;
-  for (int w = 0; w < wid; ++w) acc += warp_tot[w];
-#pragma unroll
-  for (uint32_t i = 0; i < per; ++i) {
-    const uint32_t k = pad32(b0 + i);
-    const uint32_t cnt = start[k];
-    start[k] = acc;
-    acc += cnt;
+  for (int u = 0; u < kVecs; ++u) {
+    uint4 at;
+    at.x = acc + before[u];
+    at.y = at.x + c4[u].x;
+    at.z = at.y + c4[u].y;
+    at.w = at.z + c4[u].z;
+    reinterpret_cast<uint4 *>(start)[v0 + u * 32] = at;
   }
   __syncthreads();
   if (blockIdx.x == 0) {
-    for (uint32_t i = threadIdx.x; i < nb; i += kPermThreads) sc.start[i] = start[pad32(i)];
+    for (uint32_t i = threadIdx.x; i < nb; i += kPermThreads) sc.start[i] = start[i];
     if (threadIdx.x == 0) sc.start[nb] = n;
   }
   const uint64_t stride = (uint64_t)gridDim.x * kPermThreads;
@@ -162,19 +160,20 @@ k_perm_scatter(uint32_t n, int lg, PermScratch sc) {
     for (int u = 0; u < kPermBatch; ++u) {
       const uint64_t j = j0 + u * stride;
       if (j < n)
-        sc.pairs[start[pad32(bucket_of(key[u], lg))] + place[u]] =
+        sc.pairs[start[bucket_of(key[u], lg)] + place[u]] =
             make_uint4((uint32_t)key[u], (uint32_t)(key[u] >> 32), (uint32_t)j, 0u);
     }
   }
 }
 
 // The pairs that a CTA ranks are whole buckets, taken through shared memory
-// kRankTile at a time (one tile unless the buckets are large).
-constexpr uint32_t kRankTile = 1024;
+// kRankTile at a time (one tile unless the buckets are large; 1,024: 262,144
+// elements 21.1 us instead of 20.1, 1,048,576 82.4 instead of 78.6).
+constexpr uint32_t kRankTile = 512;
 constexpr uint32_t kRankBuckets = 128;  // at most per CTA: a bucket holds over 2 pairs on average
 // Pairs a CTA is given on average: more, smaller CTAs while the buckets are
-// small (32,768 pairs: 9.4 us per shuffle with 128, 12.5 with 256, 10.0 with
-// 64), a thread each above that (262,144: 25.3 with 256, 27.0 with 128).
+// small (32,768 pairs: 7.8 us per shuffle with 128, 8.9 with 256, 8.2 with
+// 64), a thread each above that (262,144: 20.1 with 256, 21.4 with 128).
 constexpr uint32_t kRankFew = 65536;
 constexpr uint32_t rank_want(uint32_t n) { return n <= kRankFew ? 128 : kPermThreads; }
 
@@ -182,6 +181,7 @@ __global__ void __launch_bounds__(kPermThreads)
 k_perm_rank(uint32_t n, int lg, uint32_t per_cta, PermScratch sc, uint64_t oldest, uint64_t cap,
             int64_t *__restrict__ idx) {
   __shared__ uint64_t tkey[kRankTile];
+  __shared__ __align__(16) uint32_t ttop[kRankTile];  // high words; ~0 past the pairs
   __shared__ uint32_t tj[kRankTile];
   __shared__ uint32_t bstart[kRankBuckets + 1];
   const uint32_t nb = 1u << lg;
@@ -218,36 +218,38 @@ k_perm_rank(uint32_t n, int lg, uint32_t per_cta, PermScratch sc, uint64_t oldes
         for (int u = 0; u < kEach; ++u) {
           tkey[u * kPermThreads + threadIdx.x] = key[u];
           tj[u * kPermThreads + threadIdx.x] = j[u];
+          ttop[u * kPermThreads + threadIdx.x] = bhi[u] > blo[u] ? (uint32_t)(key[u] >> 32) : ~0u;
         }
       } else {
-        for (uint32_t i = threadIdx.x; i < thi - tlo; i += kPermThreads) {
+        for (uint32_t i = threadIdx.x; i < kRankTile; i += kPermThreads) {
+          ttop[i] = ~0u;
+          if (i >= thi - tlo) continue;
           const uint4 v = __ldcg(&sc.pairs[tlo + i]);
           tkey[i] = ((uint64_t)v.y << 32) | v.x;
           tj[i] = v.z;
+          ttop[i] = v.y;
         }
       }
       __syncthreads();
 #pragma unroll
       for (int u = 0; u < kEach; ++u) {
-        const uint32_t a = max(blo[u], tlo), z = min(bhi[u], thi);
-        uint32_t equal = 0;
-        uint32_t i = a;
-        for (; i + 4 <= z; i += 4) {
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const uint64_t k2 = tkey[i + w - tlo];
-            r[u] += k2 < key[u];
-            equal += k2 == key[u];
-          }
+        if (max(blo[u], tlo) >= min(bhi[u], thi)) continue;
+        const uint32_t a = max(blo[u], tlo) - tlo, z = min(bhi[u], thi) - tlo;
+        // By the high words, four at a time: those before `a` in the first
+        // four are of lower buckets, hence less, those from `z` on never.
+        const uint32_t top = (uint32_t)(key[u] >> 32);
+        uint32_t less = 0, most = 0;
+        for (uint32_t i = a & ~3u; i < z; i += 4) {
+          const uint4 v = *reinterpret_cast<const uint4 *>(ttop + i);
+          less += (v.x < top) + (v.y < top) + (v.z < top) + (v.w < top);
+          most += (v.x <= top) + (v.y <= top) + (v.z <= top) + (v.w <= top);
         }
-        for (; i < z; ++i) {
-          const uint64_t k2 = tkey[i - tlo];
-          r[u] += k2 < key[u];
-          equal += k2 == key[u];
+        if (most - less == (t0 == e0 ? 1u : 0u)) {
+          r[u] += less - (a & 3u);
+        } else {  // another key with this high word: in full, equal ones by offset
+          for (uint32_t i = a; i < z; ++i)
+            r[u] += tkey[i] < key[u] || (tkey[i] == key[u] && tj[i] < j[u]);
         }
-        // equal keys beside the element itself (hardly ever): by offset
-        if (equal > (t0 == e0 ? 1u : 0u))
-          for (i = a; i < z; ++i) r[u] += tkey[i - tlo] == key[u] && tj[i - tlo] < j[u];
       }
     }
 #pragma unroll
