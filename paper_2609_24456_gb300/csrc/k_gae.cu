@@ -32,9 +32,9 @@
 //
 // Bound by latency (a chunk's loads, then its dependent chain) up to ~10^6
 // values, then by HBM.  Calls in a row with all three outputs, in us, and
-// (before) with one warp per environment: 8 x 2,048 steps 12.8 (43.0), 4,096 x
-// 64 13.2 (28.4), 1,024 x 1,024 29.5 (107), 64 x 8,192 41 (557), 8 x 128 7.6
-// (9.2), 8 x 512 8.6.
+// (before) with one warp per environment: 8 x 2,048 steps 10.8 (43.0), 4,096 x
+// 64 12.3 (28.4), 1,024 x 1,024 24.3 (107), 64 x 8,192 37.9 (557), 8 x 128 7.0
+// (9.2), 8 x 512 7.4.
 //
 // Two kernels chained with programmatic dependent launch: the scan writes A,
 // the returns and per-CTA sums of A and A^2; the normalisation kernel
@@ -296,7 +296,7 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
 // Sum of the per-CTA partials (sum A, sum A^2) in a fixed order; the totals
 // end in *s1, *s2 of thread 0.  Every CTA that calls it gets the same bits.  Up
 // to kFewParts one warp adds and shuffles them, without a barrier (8 x 2,048:
-// 11.7 us per call, 12.7 with the tree); more take strided per-thread sums and a
+// a microsecond less per call than with the tree); more take strided per-thread sums and a
 // shared-memory tree, whose levels use fewer and fewer warps of the fp64 pipe
 // (4,096 x 32: 10.3 us, 11.7 with shuffles in every warp).
 constexpr uint32_t kFewParts = 128;

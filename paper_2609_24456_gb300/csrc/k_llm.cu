@@ -451,8 +451,11 @@ cudaError_t launch_grpo(edp_ctx *c, const float *r, const uint64_t *goff, uint32
                         float eps, float *adv, cudaStream_t s) {
   uint64_t blocks = (ng + kGrpoWarps - 1) / kGrpoWarps;
   if (blocks > 16ull * c->coop_sms) blocks = 16ull * c->coop_sms;
-  return launch_pdl(k_grpo, dim3((unsigned)blocks), dim3(kGrpoThreads), s, r, goff, ng, eps,
-                    adv);
+  // Launched plainly (its pdl_wait / pdl_launch are then no-ops): released early
+  // behind a gather of thousands of CTAs, advantages then delivery take 48.1 us
+  // for 512 x 16 responses instead of 38.0.
+  k_grpo<<<dim3((unsigned)blocks), dim3(kGrpoThreads), 0, s>>>(r, goff, ng, eps, adv);
+  return cudaGetLastError();
 }
 
 namespace {
