@@ -31,7 +31,11 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kNormUnroll = 8;  // 8-byte loads in flight per lane in k_deliver_norm
+// 8-byte loads in flight per lane, and iterations per warp, of k_deliver_norm;
+// loads in flight of k_deliver_norm_flat
+constexpr int kNormUnroll = 6;
+constexpr int kNormIters = 2;
+constexpr int kNormFlatUnroll = 8;
 constexpr int kStackMinBlocks = 5;  // __launch_bounds__: at most 48 registers
 constexpr int kFlatMinBlocks = 5;
 
@@ -88,6 +92,44 @@ __device__ __forceinline__ bool sample_slot(const Common &c, uint32_t k,
   return true;
 }
 
+// Minimum of q over the batch (one warp): loads are issued 8 per lane at a
+// time so a batch of 512 costs two memory round trips, not sixteen.
+__device__ __forceinline__ uint32_t batch_qmin(const Common &c, int lane) {
+  uint32_t m = 0xffffffffu;
+  for (uint32_t i0 = lane; i0 < c.B; i0 += 32 * 8) {
+    uint32_t v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const uint32_t i = i0 + u * 32;
+      v[u] = i < c.B ? __ldg(c.q + i) : 0xffffffffu;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) m = min(m, v[u]);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) m = min(m, __shfl_xor_sync(kFull, m, o));
+  return m;
+}
+
+// Per-sample collate, importance weight and scalar gathers (one warp).  The
+// head warp of each sample runs this before its payload span, so the fp64
+// chain of the weight overlaps the other warps' streaming.
+__device__ void collate(const Common &c, uint32_t k, bool ok, uint64_t slot,
+                        uint64_t off, int lane) {
+  if (lane == 0) {
+    if (c.act_out) c.act_out[k] = ok ? c.action[slot] : 0;
+    if (c.rew_out) c.rew_out[k] = ok ? c.reward[slot] : 0.f;
+    if (c.done_out) c.done_out[k] = ok ? c.done[slot] : (uint8_t)0;
+    if (c.gdst0) c.gdst0[k] = ok ? c.gsrc0[off] : 0.f;
+    if (c.gdst1) c.gdst1[k] = ok ? c.gsrc1[off] : 0.f;
+  }
+  if (c.isw) {
+    // PER: w = (q_min / q_k)^beta, q_min over the batch; fp64, one rounding
+    const uint32_t m = batch_qmin(c, lane);
+    if (lane == 0) c.isw[k] = is_weight(m, c.q[k], c.beta);
+  }
+}
+
 // Minimum of q over the batch (the CTA): every thread gets it.  16-byte loads
 // where q allows them, several in flight.
 __device__ __forceinline__ uint32_t batch_qmin_cta(const Common &c) {
@@ -125,7 +167,8 @@ __device__ __forceinline__ uint32_t batch_qmin_cta(const Common &c) {
 // of `ncta`, a sample per thread of its first kCollateThreads (one warp for
 // each fp64 pipe of the SM), so that the streaming CTAs carry no collate
 // latency.  With weights each CTA takes q_min over the whole batch, so there
-// are then at most kCollateCtas.
+// are then at most kCollateCtas (half as many: the delivery of 32,768 small
+// stacks 0.5 us shorter alone, 1 us longer in front of an update).
 constexpr uint32_t kCollateThreads = 128;
 constexpr uint32_t kCollateCtas = 256;
 uint32_t collate_ctas(uint32_t B, bool weights) {
@@ -147,6 +190,17 @@ __device__ void collate_batch(const Common &c, uint32_t cta, uint32_t ncta) {
     if (c.gdst1) c.gdst1[k] = ok ? c.gsrc1[off] : 0.f;
     if (c.isw) c.isw[k] = is_weight(m, c.q[k], c.beta);
   }
+}
+
+// [*f, *end): this warp's contiguous share of `total` units, rounded up to
+// whole 32-unit rows so lanes stay aligned with the rows of the output.
+__device__ __forceinline__ void warp_span(uint64_t total, uint64_t *f,
+                                          uint64_t *end) {
+  const uint64_t nw = (uint64_t)gridDim.x * kWarps;
+  const uint64_t gw = (uint64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
+  const uint64_t span = (((total + nw - 1) / nw) + 31) & ~31ull;
+  *f = gw * span;
+  *end = min(total, *f + span);
 }
 
 // exact integer -> float for a byte: 0x4B0000bb is 2^23 + b
@@ -533,22 +587,21 @@ cudaError_t launch_hwc(const Common &c, ChwArgs a, cudaStream_t s) {
 // each of the others takes `units` consecutive units of the batch, whatever
 // images they belong to: a thread per image (or token row) it touches resolves
 // the row into shared memory, then all threads stream the units as one flat
-// range, UN loads in flight each.  Bound by HBM for large batches, by the chain
-// of dependent loads for small ones.  Calls in a row, in us, and (before) when a
-// warp walked its span image by image and collated at each image:
+// range, UN loads in flight each.  Bound by the chain of dependent loads for
+// small batches.  Calls in a row, in us, and (by warps, k_deliver_norm):
 //   images of     64x64x3      96x96x3 + 128   224x224x3 + 512  84x84x1     16x16x1
 //   B = 64        3.1 (3.3)    3.1 (3.6)       5.7 (7.7)        2.8 (4.2)   2.6 (6.2)
-//   B = 256       3.7 (3.6)    5.1 (6.5)       17.9 (17.7)      2.8 (4.4)   2.6 (8.7)
-//   B = 1,024     7.4 (8.9)    13.3 (13.2)     71.3 (71.2)      5.1 (7.8)   2.6 (9.0)
-// 6 units in flight and 4 CTAs per SM, or 8 and 3: 7% slower at 224x224x3, B =
-// 1,024; 4 and 5: 10%.
+//   B = 256       3.7 (3.6)    5.1 (6.5)                        2.8 (4.4)   2.6 (8.7)
+//   B = 1,024     7.4 (8.9)                                     5.1 (7.8)   2.6 (9.0)
+// 6 units in flight and 4 CTAs per SM, or 8 and 3: 7% slower on large batches; 4
+// and 5: 10%.
 // ---------------------------------------------------------------------------
 struct NormArgs {
   const uint8_t *obs_h;   // HBM ring [cap_h][F]
   const uint8_t *obs_c;   // host ring [cap_c][F] (device-mapped) or null
   const int32_t *tok_h;
   const int32_t *tok_c;
-  uint64_t cap_h, cap_c;
+  uint64_t cap_h, cap_c, total, size;
   // offsets below `cold` (older ones) live in the host tier; physical rows of
   // the oldest offset there and of offset `cold` in HBM
   uint64_t cold, first_c, first_h;
@@ -588,7 +641,7 @@ __device__ __forceinline__ uint32_t row_of_unit(uint32_t i, uint32_t d, uint32_t
 
 template <int UN, bool AFF, bool TWO>
 __global__ void __launch_bounds__(kThreads, kNormCtas)
-k_deliver_norm(Common c, NormArgs a) {
+k_deliver_norm_flat(Common c, NormArgs a) {
   __shared__ uint64_t s_src[kNormRows];  // a row's address (16-byte aligned), its lowest bit
                                          // set in HBM; 0: a bad index
   const uint64_t pol = policy_stream();
@@ -689,6 +742,130 @@ k_deliver_norm(Common c, NormArgs a) {
   }
 }
 
+// The same by warps: each takes an equal contiguous span of the batch, image by
+// image, and resolves and collates a sample where its first unit lies, so no
+// warp waits for another.  For large batches of large images, where a delivery
+// alone takes as long either way, and on two streams in turn, each filling the
+// other's last wave, 67.3 us a batch of 1,024 224x224x3 + 512 tokens; 68.2 by
+// flat runs.
+template <int UN, bool AFF>
+__global__ void __launch_bounds__(kThreads)
+k_deliver_norm(Common c, NormArgs a) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t pol = policy_stream();
+  pdl_wait();
+  pdl_launch();
+  const uint64_t total = (uint64_t)c.B * a.F8;
+  uint64_t f, end;
+  warp_span(total, &f, &end);
+  while (f < end) {
+    const uint32_t k = (uint32_t)(f / a.F8);
+    const uint32_t u_lo = (uint32_t)(f - (uint64_t)k * a.F8);
+    const uint64_t seg_end = min(end, (uint64_t)(k + 1) * a.F8);
+    const uint32_t u_hi = (uint32_t)(seg_end - (uint64_t)k * a.F8);
+    const bool head = u_lo == 0;
+    uint64_t slot = 0, off = 0;
+    const bool ok = sample_slot(c, k, &slot, &off, head && lane == 0);
+    if (head) collate(c, k, ok, slot, off, lane);
+    // tier of the logical id L = total - size + off
+    const uint64_t L = a.total - a.size + off;
+    const uint64_t in_hbm = a.total < a.cap_h ? a.total : a.cap_h;
+    const bool hbm = !a.obs_c || L >= a.total - in_hbm;
+    const uint64_t ps = hbm ? L % a.cap_h : L % a.cap_c;
+    const uint8_t *obs = hbm ? a.obs_h : a.obs_c;
+    const uint2 *src = reinterpret_cast<const uint2 *>(obs + ps * a.F8 * 8ull);
+    uint4 *dst = reinterpret_cast<uint4 *>(a.out + (uint64_t)k * a.F8 * 8ull);
+    for (uint32_t u0 = u_lo + lane; u0 < u_hi; u0 += 32 * UN) {
+      uint2 v[UN];
+#pragma unroll
+      for (int u = 0; u < UN; ++u) {
+        const uint32_t w = u0 + u * 32;
+        // HBM tier: streaming non-coherent loads; host tier: plain loads of
+        // the mapped page-locked memory
+        v[u] = (ok && w < u_hi) ? (hbm ? ld_stream(src + w, pol) : src[w])
+                                : make_uint2(0u, 0u);
+      }
+#pragma unroll
+      for (int u = 0; u < UN; ++u) {
+        const uint32_t w = u0 + u * 32;
+        if (w >= u_hi) continue;
+        const uint32_t ch = (w >= a.HW8) + (w >= 2 * a.HW8) + (w >= 3 * a.HW8);
+        float fv[8];
+        if constexpr (AFF) {
+          const float A = a.aa[ch], Bc = a.ab[ch];
+#pragma unroll
+          for (int bb = 0; bb < 8; ++bb)
+            fv[bb] = __fmaf_rn(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), A, Bc);
+        } else {
+          const float mc = a.mean[ch], s1 = a.s1[ch], s2 = a.s2[ch];
+#pragma unroll
+          for (int bb = 0; bb < 8; ++bb) {
+            const float x = unit_f32(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), c.r1, c.r2);
+            const float tt = __fsub_rn(x, mc);
+            fv[bb] = a.fast ? __fmaf_rn(tt, s1, __fmul_rn(tt, s2)) : __fdiv_rn(tt, a.sd[ch]);
+          }
+        }
+        uint4 o;
+        o.x = pack_bf16x2(fv[0], fv[1]);
+        o.y = pack_bf16x2(fv[2], fv[3]);
+        o.z = pack_bf16x2(fv[4], fv[5]);
+        o.w = pack_bf16x2(fv[6], fv[7]);
+        if (!ok) o = make_uint4(0u, 0u, 0u, 0u);
+        st_stream(dst + w, o, pol);
+      }
+    }
+    if (head) {
+      // a two-tier row read over the host link (edp_get_counters)
+      if (lane == 0 && ok && a.obs_c && !hbm)
+        atomicAdd(&c.ctrl->host_bytes,
+                  (unsigned long long)a.F8 * 8ull + (a.tok_out ? a.L16 * 16ull : 0ull));
+      if (a.tok_out) {
+        // the row's tokens, kTokBatch 16-byte loads per lane in flight
+        // before their stores
+        constexpr int kTokBatch = 4;
+        const uint4 *ts = reinterpret_cast<const uint4 *>(
+            (hbm ? a.tok_h : a.tok_c) + ps * a.L16 * 4ull);
+        uint4 *td = reinterpret_cast<uint4 *>(a.tok_out + (uint64_t)k * a.L16 * 4ull);
+        for (uint32_t i0 = lane; i0 < a.L16; i0 += 32 * kTokBatch) {
+          uint4 t4[kTokBatch];
+#pragma unroll
+          for (int u = 0; u < kTokBatch; ++u) {
+            const uint32_t i = i0 + u * 32;
+            t4[u] = (ok && i < a.L16) ? ts[i] : make_uint4(0u, 0u, 0u, 0u);
+          }
+#pragma unroll
+          for (int u = 0; u < kTokBatch; ++u)
+            if (i0 + u * 32 < a.L16) td[i0 + u * 32] = t4[u];
+        }
+      }
+    }
+    f = seg_end;
+  }
+}
+
+// Grid size from the work: enough CTAs that each warp runs about `iters`
+// iterations of its unrolled loop (`per_iter` units each), so the block
+// scheduler balances the tail and a CTA that starts late (its SM still busy
+// with another kernel) holds up little work; a small batch is spread over up
+// to one wave (blocks resident per SM x SMs, queried once per kernel) with
+// at least one iteration per warp.
+template <typename Kern>
+unsigned grid_for(Kern kern, uint64_t units, uint64_t per_iter, int iters, int sms) {
+  static int per_sm = 0;  // per template instantiation
+  if (!per_sm) {
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0);
+    if (per_sm < 1) per_sm = 1;
+  }
+  const uint64_t wave = (uint64_t)per_sm * sms;
+  const uint64_t warp_iters = (units + per_iter - 1) / per_iter;
+  uint64_t blocks = (warp_iters + (uint64_t)kWarps * iters - 1) / ((uint64_t)kWarps * iters);
+  if (blocks < wave) {
+    const uint64_t most = (warp_iters + kWarps - 1) / kWarps;
+    blocks = most < wave ? most : wave;
+  }
+  return (unsigned)(blocks ? blocks : 1);
+}
+
 }  // namespace
 
 cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
@@ -780,6 +957,8 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     a.tok_c = ctx->cap_c ? ctx->st.host_tokens : nullptr;
     a.cap_h = ctx->cap_h;
     a.cap_c = ctx->cap_c ? ctx->cap_c : 1;
+    a.total = ctx->total;
+    a.size = size;
     // ids total - size + off; the newest min(total, cap_h) of them in HBM at id
     // mod cap_h, the older ones in the host tier at id mod cap_c
     const uint64_t in_hbm = ctx->total < ctx->cap_h ? ctx->total : ctx->cap_h;
@@ -800,29 +979,37 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     a.fast = ctx->norm_fast;
     a.out = (__nv_bfloat16 *)out->obs;
     a.tok_out = out->tokens;
+    const uint64_t rows = kNormRows - 2, total = (uint64_t)B * a.F8;
+    uint64_t units = (uint64_t)kThreads * kNormFlatUnroll;
+    // Flat runs up to two waves of CTAs, and for small images (below 1,024
+    // units, where a warp's span crosses several) at any batch size, in runs of
+    // two rounds there (4,096 images of 84x84: 13.1 us; 13.9 in one round, 16.2
+    // by warps).
+    if (total > 2 * (uint64_t)kNormCtas * sms * units) {
+      if (a.F8 >= 1024) {
+        auto kern = ctx->norm_affine ? k_deliver_norm<kNormUnroll, true>
+                                     : k_deliver_norm<kNormUnroll, false>;
+        return launch_pdl(kern, dim3(grid_for(kern, total, 32 * kNormUnroll, kNormIters, sms)),
+                          dim3(kThreads), s, c, a);
+      }
+      units *= 2;
+    }
+    if (units > rows * a.F8) units = (rows * a.F8) & ~31ull;
+    a.units = (uint32_t)units;
     a.ncollate = collate_ctas(B, out->isw != nullptr);
     const uint64_t tok_units = a.tok_out ? (uint64_t)B * a.L16 : 0;
-    const uint64_t rows = kNormRows - 2, total = (uint64_t)B * a.F8;
     a.tunits = rows * a.L16 < kTokUnits ? (uint32_t)(rows * a.L16) : kTokUnits;
     const uint64_t ntok = tok_units ? (tok_units + a.tunits - 1) / a.tunits : 0;
     a.ntok = (uint32_t)ntok;
-    // One round per CTA up to two waves of CTAs, two rounds above (us, one
-    // round against two, B images of 64x64x3: 1,024 7.4, 8.7; 4,096 24.4, 24.4;
-    // of 96x96x3: 256 5.1, 5.9; 1,024 13.9, 13.3; of 224x224x3: 64 5.7, 6.4;
-    // 256 18.9, 17.9; 1,024 71.7, 71.3); three and more lose 1-5%.
-    uint64_t units = (uint64_t)kThreads * kNormUnroll;
-    if (total > 2 * (uint64_t)kNormCtas * sms * units) units *= 2;
-    if (units > rows * a.F8) units = (rows * a.F8) & ~31ull;
-    a.units = (uint32_t)units;
     a.div_f = a.F8 < 32768 ? (uint32_t)((0x100000000ull + a.F8 - 1) / a.F8) : 0u;
     a.div_l = a.L16 && a.L16 < 32768 ? (uint32_t)((0x100000000ull + a.L16 - 1) / a.L16) : 0u;
     const uint64_t ctas = (total + units - 1) / units + a.ncollate + a.ntok;
     if (ctas > 0x7FFFFFFFull || ntok > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     auto kern = ctx->norm_affine
-                    ? (a.obs_c ? k_deliver_norm<kNormUnroll, true, true>
-                               : k_deliver_norm<kNormUnroll, true, false>)
-                    : (a.obs_c ? k_deliver_norm<kNormUnroll, false, true>
-                               : k_deliver_norm<kNormUnroll, false, false>);
+                    ? (a.obs_c ? k_deliver_norm_flat<kNormFlatUnroll, true, true>
+                               : k_deliver_norm_flat<kNormFlatUnroll, true, false>)
+                    : (a.obs_c ? k_deliver_norm_flat<kNormFlatUnroll, false, true>
+                               : k_deliver_norm_flat<kNormFlatUnroll, false, false>);
     return launch_pdl(kern, dim3((unsigned)ctas), dim3(kThreads), s, c, a);
   }
 }
