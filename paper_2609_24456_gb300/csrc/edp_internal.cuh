@@ -396,7 +396,8 @@ __device__ __forceinline__ void flag(Ctrl *c, uint32_t bits,
 // the predecessor may write.  pdl_launch() lets the next kernel in the
 // stream start launching.  Both are no-ops for a kernel launched without
 // the attribute.  Kernels call it right after their wait; the uniform sampler
-// calls it at its end, which makes no difference to the deliveries behind it.
+// calls it at its end, which makes no difference to the deliveries behind it,
+// and the frame-stack delivery leaves it out (k_deliver_stack says why).
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -405,12 +406,12 @@ __device__ __forceinline__ void pdl_launch() {
 }
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block,
-                       cudaStream_t s, Args... args) {
+cudaError_t launch_pdl_smem(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                            cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -418,6 +419,11 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block,
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block,
+                       cudaStream_t s, Args... args) {
+  return launch_pdl_smem(kern, grid, block, 0, s, args...);
 }
 
 // ---------------------------------------------------------------------------

@@ -38,6 +38,7 @@ constexpr int kNormIters = 2;
 constexpr int kNormFlatUnroll = 8;
 constexpr int kStackMinBlocks = 5;  // __launch_bounds__: at most 48 registers
 constexpr int kFlatMinBlocks = 5;
+constexpr size_t kFourPerSm = 47000;  // shared memory of which an SM holds four
 
 struct Common {
   const int64_t *idx;
@@ -228,7 +229,7 @@ __device__ __forceinline__ float byte_f(uint32_t w, int i) {
 //
 // Bound by HBM.  Calls in a row, a fresh sample each, in us, and before, when
 // frames were staged through shared memory by bulk copies, 2 CTAs per SM:
-//   84x84, 4 frames + successors   512: 23.0 (23.6)  8,192: 315 (365), 6,799 GB/s
+//   84x84, 4 frames + successors   512: 22.7 (23.6)  8,192: 314 (365), 6,820 GB/s
 //   84x84, 1 frame                 8,192: 45.8 (47.6)  32,768: 172 (189)
 //   64x64, 4 + successors          8,192: 184 (198)   128x128 2,048: 184 (196)
 //   48x48, 4 + successors          512: 8.0 (12.0)    8,192: 105 (140)
@@ -334,8 +335,9 @@ __global__ void __launch_bounds__(kThreads, kStackMinBlocks)
 k_deliver_stack(Common c, StackArgs a) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint64_t pol = policy_stream();
+  // No early release: the next kernel's CTAs, waiting on this one in the last
+  // waves' places, made a round of sampling, delivery and update 30.2 us; 29.7.
   pdl_wait();
-  pdl_launch();
   if (blockIdx.x < a.ncollate) {
     collate_batch(c, blockIdx.x, a.ncollate);
     return;
@@ -936,7 +938,15 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     const uint64_t ctas = (units + each - 1) / each + a.ncollate;
     if (ctas > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     auto kern = few ? k_deliver_stack<4> : k_deliver_stack<8>;
-    return launch_pdl(kern, dim3((unsigned)ctas), dim3(kThreads), s, c, a);
+    // With successors and more than two and a half waves, four CTAs per SM
+    // instead of five, held there by shared memory that they don't use: as fast
+    // alone (84x84, 4 frames, 512: 22.7 us, 22.9), and the small kernels of other
+    // streams find room among its waves (sampling and update beside it: a round
+    // 22.6 us, 24.4).  Without successors four are 12% slower (8,192: 195 us,
+    // 171), between one wave and two up to 15%.
+    const bool four = a.next && 2 * ctas >= 5ull * kStackMinBlocks * sms;
+    return launch_pdl_smem(kern, dim3((unsigned)ctas), dim3(kThreads), four ? kFourPerSm : 0, s,
+                           c, a);
   } else if (cfg.transform == EDP_XFORM_HWC_CHW_BF16) {
     ChwArgs a{};
     a.obs = ctx->st.obs;
