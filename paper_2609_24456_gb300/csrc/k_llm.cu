@@ -316,7 +316,10 @@ __device__ __forceinline__ uint64_t pack_offset_cta(const PackEntry *__restrict_
 // entry writes its output offset, that of the last entry out_off[batch] = the
 // total, and flags an overflow.
 // 32 registers, 16.5 KB: 8 CTAs per SM keep more copies in flight than 6 at 38
-// registers (8,192 sequences of 128 to 4,096 tokens 34.4 us, 37.3).
+// registers (8,192 sequences of 128 to 4,096 tokens 34.4 us, 37.3).  Neither
+// this kernel nor k_pack_gather_short releases the next one early: its CTAs, which
+// can only wait, took places from the last waves (that call 33.6 us, with its
+// lengths and advantages 37.3, 39.3 before; 65,536 short sequences 28.0, 28.9).
 template <bool SPLIT>
 __global__ void __launch_bounds__(kPackThreads, 8)
 k_pack_gather(const int32_t *__restrict__ tokens, const PackEntry *__restrict__ ent,
@@ -330,7 +333,6 @@ k_pack_gather(const int32_t *__restrict__ tokens, const PackEntry *__restrict__ 
   uint32_t uses = 0;
   const uint64_t pol = policy_stream();
   pdl_wait();
-  pdl_launch();
   const uint32_t k = blockIdx.x;
   const uint64_t first = SPLIT ? (uint64_t)blockIdx.y * chunk : 0;
   if (SPLIT && blockIdx.y && ent[k].len <= first) return;  // no chunk is left
@@ -383,7 +385,6 @@ k_pack_gather_short(const int32_t *__restrict__ tokens, const PackEntry *__restr
   const uint32_t warp = threadIdx.x >> 5;
   const uint64_t pol = policy_stream();
   pdl_wait();
-  pdl_launch();
   const uint32_t each = kPackWarps * per_warp;  // 8, 16 or 32: divides the 256-entry chunk
   const uint32_t k0 = blockIdx.x * each;
   const uint32_t ne = min(each, B - k0);
