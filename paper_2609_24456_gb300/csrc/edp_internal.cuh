@@ -397,7 +397,8 @@ __device__ __forceinline__ void flag(Ctrl *c, uint32_t bits,
 // stream start launching.  Both are no-ops for a kernel launched without
 // the attribute.  Kernels call it right after their wait; the uniform sampler
 // calls it at its end, which makes no difference to the deliveries behind it,
-// and the frame-stack delivery and the packed gathers leave it out (they say why).
+// and the frame-stack delivery, the packed gathers and the row copy leave it out
+// (they say why).
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -65,10 +65,12 @@ __device__ __forceinline__ void copy_tiles(const CopyRuns &r, uint64_t cta, uint
   }
 }
 
+// No early release of the next kernel, whose CTAs would wait in the last tiles'
+// places: a rollout of 32,768 64x64x3 images, then GAE, shuffle and delivery,
+// 330.9 us instead of 332.8; alone it makes no difference.
 __global__ void __launch_bounds__(kCopyThreads)
 k_copy_flat(CopyRuns r, int wait_first) {
   if (wait_first) pdl_wait();
-  pdl_launch();
   copy_tiles<kCopyThreads>(r, blockIdx.x, gridDim.x);
   if (!wait_first) pdl_wait();
 }
