@@ -458,7 +458,15 @@ class Ring:
     def _destroy_waiting(cls):
         import torch
         while cls._waiting and not torch.cuda.is_current_stream_capturing():
-            edp_destroy(cls._waiting.pop()["ctx"])
+            try:
+                state = cls._waiting.pop()
+            except IndexError:  # another thread took the last one
+                return
+            # the status is not this caller's: an error of the device shows in
+            # the next call on it.  `state` holds the storage until the context
+            # is gone.
+            lib().edp_destroy(state["ctx"])
+            del state
 
     def __del__(self):
         try:

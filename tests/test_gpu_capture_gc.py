@@ -16,8 +16,10 @@ def test_ring_collected_during_capture(edp_lib):
     def make():
         return edp.Ring(edp.make_config(16, (1, 4, 4), edp.EDP_XFORM_HWC_CHW_BF16))
 
+    gc.collect()  # rings of earlier tests are not collected in the capture
     lost = make()
     lost.itself = lost  # only the cyclic collector can find it
+    ctx = lost.ctx
     x = torch.zeros(8, device="cuda")
     torch.cuda.synchronize()
     g = torch.cuda.CUDAGraph()
@@ -29,7 +31,7 @@ def test_ring_collected_during_capture(edp_lib):
             gc.collect()
     finally:
         gc.enable()
-    assert len(edp.Ring._waiting) == 1
+    assert [w["ctx"] for w in edp.Ring._waiting] == [ctx]
     g.replay()
     torch.cuda.synchronize()
     assert (x == 1).all()
