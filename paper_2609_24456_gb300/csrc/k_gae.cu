@@ -18,13 +18,16 @@
 // SMs and longer chunks share the steps (gae_shape).
 //
 // Arithmetic: GB300's fp64 pipe is narrow (a dependent fp64 FMA costs ~64
-// cycles, fp32 ~4), so the scan -- and each lane's sums of A and A^2 over an
-// environment -- run in double-float arithmetic -- a value
+// cycles, fp32 ~4), so the scan -- and a thread's sums of A and A^2 over its
+// steps of a chunk -- run in double-float arithmetic -- a value
 // is an unevaluated pair hi + lo of fp32 numbers, combined with the
 // error-free transformations TwoSum (Knuth) and TwoProd via FMA (Dekker),
 // as in the double-double arithmetic of Hida, Li and Bailey -- which keeps
 // ~44 significant bits (relative error ~2^-44 per operation); gamma and
-// gamma*lambda enter as pairs split from fp64.  The mean and the variance
+// gamma*lambda enter as pairs split from fp64.  The sums over chunks, threads
+// and warps carry three words and round once per CTA, to fp64 (in double-float
+// the variance lost up to a digit against fp64: 24 rollouts of 2,048 steps,
+// mean 1e5 deviations, 1.3e-5 off; 3.9e-6 so).  The mean and the variance
 // are formed in fp64 from the CTAs' sums; the normalisation of an element is
 // double-float again (as many bits as its fp32 result can show: its error
 // against 64 bits is the rounding's), fp64 where a value is out of its range.
@@ -56,11 +59,42 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kL = 4;               // steps per thread and chunk
 constexpr int kGaeThreads = 512;    // at most per CTA
 constexpr int kGaeWarps = kGaeThreads / 32;
+static_assert(kGaeWarps <= 16, "half a warp adds the warps' sums");
 constexpr int kNormThreads = 256;
 constexpr int kNormLoads = 8;       // values in flight per thread of a single CTA
 
 __device__ __forceinline__ df df_shfl_down(df a, int o) {
   return {__shfl_down_sync(kFull, a.hi, o), __shfl_down_sync(kFull, a.lo, o)};
+}
+
+// A sum of three fp32 numbers, for the sums over a CTA's threads, which were
+// fp64: each addition keeps about 70 significant bits (the errors of two_sum are
+// carried in full, only the third words' sum rounds), so the total rounds
+// once, to fp64.  fp64 itself would take 16 instructions a warp of the narrow
+// pipe, about 64 cycles each.  (A and A^2 share a tree, half a warp each, so this
+// takes no longer than two trees in double-float: 8 x 2,048 10.7 us both, 1 x
+// 262,144 83.2 then, 60.7 now, 1,024 x 1,024 24.2 and 24.8.)
+struct tf {
+  float a, b, c;
+};
+__device__ __forceinline__ tf tf_add(tf x, tf y) {
+  const df s = two_sum(x.a, y.a), t = two_sum(x.b, y.b);
+  const df m = two_sum(s.lo, t.hi);
+  const float c = __fadd_rn(__fadd_rn(x.c, y.c), __fadd_rn(t.lo, m.lo));
+  const df p = two_sum(s.hi, m.hi);
+  const df q = two_sum(p.lo, c);
+  return {p.hi, q.hi, q.lo};
+}
+__device__ __forceinline__ tf tf_shfl_down16(tf x, int o) {  // within half a warp
+  return {__shfl_down_sync(kFull, x.a, o, 16), __shfl_down_sync(kFull, x.b, o, 16),
+          __shfl_down_sync(kFull, x.c, o, 16)};
+}
+__device__ __forceinline__ tf tf_shfl_xor16(tf x) {
+  return {__shfl_xor_sync(kFull, x.a, 16), __shfl_xor_sync(kFull, x.b, 16),
+          __shfl_xor_sync(kFull, x.c, 16)};
+}
+__device__ __forceinline__ double tf_to_d(tf x) {
+  return (double)x.a + ((double)x.b + (double)x.c);
 }
 
 // What the normalisation needs of the whole rollout.
@@ -160,7 +194,7 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
            double *__restrict__ partial, float *adv_norm) {
   __shared__ float4 agg[kGaeWarps][kE];  // a warp's composite: a.hi, a.lo, b.hi, b.lo
   __shared__ float2 s_carry[kE];         // A at the step after the chunk
-  __shared__ float4 s_sum[kGaeWarps];
+  __shared__ tf s_sum[2][kGaeWarps];  // of A, of A^2
   __shared__ NormStat s_stat;
   constexpr bool kStaged = kE < 8;
   __shared__ std::conditional_t<kStaged, GaeStage, char> stage;
@@ -171,8 +205,10 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
   const df one = {1.f, 0.f}, zero = {0.f, 0.f};
   const df g = {g2.x, g2.y}, gl = {gl2.x, gl2.y};  // gamma, gamma lambda
   pdl_wait();
-  // this thread's A and A^2 summed in double-float (the fp32 pipe)
+  // this thread's A and A^2: a chunk's in double-float (the fp32 pipe), the
+  // chunks' in three words
   df a1 = zero, a2 = zero;
+  tf t1 = {0.f, 0.f, 0.f}, t2 = t1;
   for (uint32_t tile = blockIdx.x; (uint64_t)tile * kE < E; tile += gridDim.x) {
     const bool real = tile * kE + el < E;
     const uint32_t e = real ? tile * kE + el : E - 1;
@@ -239,6 +275,9 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
       __syncthreads();  // agg and s_carry have been read
       if (seg == 0) s_carry[el] = make_float2(A.hi, A.lo);
       if (!te2) break;
+      t1 = tf_add(t1, tf{a1.hi, a1.lo, 0.f});
+      t2 = tf_add(t2, tf{a2.hi, a2.lo, 0.f});
+      a1 = a2 = zero;
       x = next;
       te = te2;
       ts = ts2;
@@ -247,30 +286,29 @@ k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
   pdl_launch();
   if (!partial && !adv_norm) return;  // no normalisation requested
   // this CTA's sums in a fixed order: a shuffle tree per warp, then over the
-  // warps; fp64 from there on
+  // warps, the lower half of a warp for A and the upper for A^2
+  t1 = tf_add(t1, tf{a1.hi, a1.lo, 0.f});
+  t2 = tf_add(t2, tf{a2.hi, a2.lo, 0.f});
+  const int half = lane >> 4, hl = lane & 15;
+  tf t = tf_add(half ? t2 : t1, tf_shfl_xor16(half ? t1 : t2));
 #pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    a1 = df_add(a1, df_shfl_down(a1, o));
-    a2 = df_add(a2, df_shfl_down(a2, o));
+  for (int o = 8; o; o >>= 1) t = tf_add(t, tf_shfl_down16(t, o));
+  if (nwarps > 1) {
+    if (hl == 0) s_sum[half][warp] = t;
+    __syncthreads();
   }
-  if (lane == 0) s_sum[warp] = make_float4(a1.hi, a1.lo, a2.hi, a2.lo);
-  __syncthreads();
   if (warp == 0) {
-    const float4 m = lane < nwarps ? s_sum[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
-    a1 = {m.x, m.y};
-    a2 = {m.z, m.w};
+    if (nwarps > 1) {
+      t = hl < nwarps ? s_sum[half][hl] : tf{0.f, 0.f, 0.f};
 #pragma unroll
-    for (int o = kGaeWarps / 2; o; o >>= 1) {
-      a1 = df_add(a1, df_shfl_down(a1, o));
-      a2 = df_add(a2, df_shfl_down(a2, o));
+      for (int o = kGaeWarps / 2; o; o >>= 1)
+        if (o < nwarps) t = tf_add(t, tf_shfl_down16(t, o));
     }
-    if (lane == 0) {
-      if (partial) {
-        partial[2 * blockIdx.x] = df_to_d(a1);
-        partial[2 * blockIdx.x + 1] = df_to_d(a2);
-      } else {
-        s_stat = norm_stat((double)((uint64_t)T * E), df_to_d(a1), df_to_d(a2));
-      }
+    const double sum = tf_to_d(t), other = __shfl_xor_sync(kFull, sum, 16);
+    if (partial) {
+      if (hl == 0) partial[2 * blockIdx.x + half] = sum;
+    } else if (lane == 0) {
+      s_stat = norm_stat((double)((uint64_t)T * E), sum, other);
     }
   }
   if (partial) return;

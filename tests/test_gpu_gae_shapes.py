@@ -4,6 +4,8 @@ environments over several chunks (fewer environments per CTA), a rollout that
 one CTA normalises, many environments; arrays off 16-byte alignment, and each
 output alone.  The bound is the rounding of the stored fp32 advantages: 4 ulp
 of the value, or of the rollout's largest where it cancels."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -58,4 +60,36 @@ def test_gae_shapes(edp_lib, orc, T, E):
     ref = np.asarray(N, np.float64).reshape(T, E)
     assert (np.abs(to_np(adv) - ref) <= 4 * 2.0**-24 * np.maximum(
         np.abs(ref), np.abs(ref).max())).all()
+    ring.close()
+
+
+@pytest.mark.parametrize("T,E", [(2048, 1), (128, 8), (2048, 8), (8192, 2), (128, 256)])
+@pytest.mark.parametrize("mean", [0.0, 10.0, 1e3, 1e5])
+def test_sums_keep_64_bits(edp_lib, T, E, mean):
+    """Sums of A and A^2 of advantages whose mean is up to 1e5 of their
+    deviations (the variance is a difference of the two): every step ends an
+    episode and V = 0, so A = r.  The bound on the root mean square over 24
+    rollouts is 2^-51, four roundings to fp64 (a thread's few double-float
+    additions average out: 3.7e-16 at most); reductions of a CTA in double-float
+    gave 5e-16 to 2e-15 in the first four shapes."""
+    edp = edp_lib
+    ring = edp.Ring(edp.make_config(16, (1, 4, 4), edp.EDP_XFORM_HWC_CHW_BF16), action=False,
+                    reward=False, done=False)
+    v = torch.zeros(T + 1, E, device="cuda")
+    d = torch.ones(T, E, dtype=torch.uint8, device="cuda")
+    adv = torch.zeros(T, E, device="cuda")
+    stats = torch.zeros(3, dtype=torch.float64, device="cuda")
+    off = []
+    for seed in range(24):
+        rng = np.random.default_rng(seed * 1000 + T + E)
+        r = (mean + rng.standard_normal((T, E))).astype(np.float32)
+        edp.edp_gae_stats(ring.ctx, cuda(r), v, d, T, E, 0.99, 0.95, adv, stats)
+        edp.edp_sync(ring.ctx)
+        n, s1, s2 = to_np(stats)
+        assert n == T * E and np.array_equal(to_np(adv), r)
+        x = r.astype(np.float64).ravel()
+        want = math.fsum(x * x)  # the squares of fp32 values are exact in fp64
+        off.append((s2 - want) / want)
+        assert abs(s1 - math.fsum(x)) <= 2.0**-51 * math.fsum(np.abs(x))
+    assert math.sqrt(np.mean(np.square(off))) <= 2.0**-51
     ring.close()
