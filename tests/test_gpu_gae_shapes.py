@@ -5,6 +5,7 @@ one CTA normalises, many environments; arrays off 16-byte alignment, and each
 output alone.  The bound is the rounding of the stored fp32 advantages: 4 ulp
 of the value, or of the rollout's largest where it cancels."""
 import math
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -92,4 +93,42 @@ def test_sums_keep_64_bits(edp_lib, T, E, mean):
         off.append((s2 - want) / want)
         assert abs(s1 - math.fsum(x)) <= 2.0**-51 * math.fsum(np.abs(x))
     assert math.sqrt(np.mean(np.square(off))) <= 2.0**-51
+    ring.close()
+
+
+@pytest.mark.parametrize("mean,std", [(1000.37, 1.0), (-731.0123456789, 0.9), (3e-4, 1.7),
+                                      (0.0, 2.5), (-5e12, 7e9), (2e-19, 1e-18), (1.25, 0.0)])
+def test_normalised_values_round_once(edp_lib, mean, std):
+    """(A - mean) / (std + 1e-8) for values next to the mean, where the
+    difference cancels, and for ordinary, large and infinite ones: within 0.51 ulp
+    of the exact product of fp64's mean and scale (half an ulp is the result's
+    own rounding; fp64 arithmetic gives 0.56 at a mean of 1e3 deviations, a mean
+    held in two fp32 words 2).  The scale is formed from s2 - s1 mean, contracted
+    or not: the two differ by 2^-53 s2, below 1e-9 of the variance for a mean of
+    up to 1e3 deviations and nothing at all at 1.25 (exact products)."""
+    edp = edp_lib
+    ring = edp.Ring(edp.make_config(16, (1, 4, 4), edp.EDP_XFORM_HWC_CHW_BF16), action=False,
+                    reward=False, done=False)
+    nn = 4096.0
+    s1 = nn * mean
+    m = s1 / nn
+    s2 = s1 * m + (nn - 1.0) * std * std
+    inv = 1.0 / (math.sqrt(max((s2 - s1 * m) / (nn - 1.0), 0.0)) + 1e-8)
+    near = np.float32(m) + np.spacing(np.float32(m)) * np.arange(-300, 301, dtype=np.float32)
+    rng = np.random.default_rng(1)
+    x = np.concatenate([near, (m + (std + 1e-8) * rng.standard_normal(400)), [0.0, 1e30, -2e19]])
+    a = np.concatenate([x.astype(np.float32), np.array([np.inf, -np.inf, np.nan], np.float32)])
+    stats = torch.tensor([nn, s1, s2], dtype=torch.float64, device="cuda")
+    out = torch.zeros(len(a), device="cuda")
+    edp.edp_gae_normalize(ring.ctx, cuda(a), len(a), stats, out)
+    edp.edp_sync(ring.ctx)
+    y = to_np(out)
+    assert y[-3] == np.inf and y[-2] == -np.inf and np.isnan(y[-1])
+    for got, v in zip(y[:-3], a[:-3]):
+        want = (Fraction(float(v)) - Fraction(m)) * Fraction(inv)
+        if abs(want) > 3e38:
+            assert np.isinf(got) and (got > 0) == (want > 0)
+            continue
+        ulp = Fraction(float(np.spacing(np.float32(abs(float(want))))))
+        assert abs(Fraction(float(got)) - want) <= Fraction(51, 100) * ulp, (v, got)
     ring.close()
