@@ -393,7 +393,10 @@ __device__ __forceinline__ void flag(Ctrl *c, uint32_t bits,
 // launch_pdl may be scheduled while its predecessor in the stream is still
 // running; pdl_wait() blocks until the predecessor has completed and its
 // writes are visible, so every such kernel calls it before touching memory
-// the predecessor may write.  pdl_launch() lets the next kernel in the
+// the predecessor may write.  No pointer parameter of such a kernel is
+// __restrict__: for the compiler, nothing but the kernel itself then touches what
+// it points to, the wait's memory clobber does not bind its loads, and they may
+// be moved above the wait.  pdl_launch() lets the next kernel in the
 // stream start launching.  Both are no-ops for a kernel launched without
 // the attribute.  Kernels call it right after their wait; the uniform sampler
 // calls it at its end, which makes no difference to the deliveries behind it,

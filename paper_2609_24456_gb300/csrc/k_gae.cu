@@ -170,9 +170,8 @@ struct GaeIn {
 // instead, a value past te the one at te; x.v[kL] is the value after the
 // thread's last step, or (staged) after the chunk.
 template <bool STAGED>
-__device__ __forceinline__ void gae_load(GaeIn &x, const float *__restrict__ r,
-                                         const float *__restrict__ v,
-                                         const uint8_t *__restrict__ d, uint32_t ts, uint32_t te,
+__device__ __forceinline__ void gae_load(GaeIn &x, const float *r, const float *v,
+                                         const uint8_t *d, uint32_t ts, uint32_t te,
                                          uint32_t seg, uint32_t segs, uint32_t E, uint32_t e) {
   // (T + 1) E < 2^32, and a step past te is less than a chunk past it.  The
   // eight-environment form keeps 64-bit indices: with fewer registers to hold,
@@ -219,10 +218,8 @@ __device__ __forceinline__ void gae_exchange(GaeIn &x, GaeStage &s, uint32_t seg
 
 template <int kE>
 __global__ void __launch_bounds__(kGaeThreads)
-k_gae_scan(const float *__restrict__ r, const float *__restrict__ v,
-           const uint8_t *__restrict__ d, uint32_t T, uint32_t E, float2 g2, float2 gl2,
-           float *A_out, float *__restrict__ ret,
-           double *__restrict__ partial, float *adv_norm) {
+k_gae_scan(const float *r, const float *v, const uint8_t *d, uint32_t T, uint32_t E, float2 g2,
+           float2 gl2, float *A_out, float *ret, double *partial, float *adv_norm) {
   __shared__ float4 agg[kGaeWarps][kE];  // a warp's composite: a.hi, a.lo, b.hi, b.lo
   __shared__ float2 s_carry[kE];         // A at the step after the chunk
   __shared__ tf s_sum[2][kGaeWarps];  // of A, of A^2

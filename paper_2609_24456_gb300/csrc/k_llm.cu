@@ -36,10 +36,9 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // Groups g = first, first + stride, ... of one warp.
-__device__ __forceinline__ void grpo_groups(const float *__restrict__ r,
-                                            const uint64_t *__restrict__ goff, uint32_t ng,
-                                            float eps, float *__restrict__ adv,
-                                            uint64_t first, uint64_t stride) {
+__device__ __forceinline__ void grpo_groups(const float *r, const uint64_t *goff, uint32_t ng,
+                                            float eps, float *adv, uint64_t first,
+                                            uint64_t stride) {
   const int lane = threadIdx.x & 31;
   for (uint64_t g = first; g < ng; g += stride) {
     const uint64_t lo = goff[g], hi = goff[g + 1];
@@ -62,8 +61,7 @@ __device__ __forceinline__ void grpo_groups(const float *__restrict__ r,
 }
 
 __global__ void __launch_bounds__(kGrpoThreads)
-k_grpo(const float *__restrict__ r, const uint64_t *__restrict__ goff, uint32_t ng,
-       float eps, float *__restrict__ adv) {
+k_grpo(const float *r, const uint64_t *goff, uint32_t ng, float eps, float *adv) {
   pdl_wait();
   pdl_launch();
   grpo_groups(r, goff, ng, eps, adv, (uint64_t)blockIdx.x * kGrpoWarps + (threadIdx.x >> 5),
@@ -100,12 +98,9 @@ __device__ __forceinline__ uint64_t block_sum(uint64_t v, uint64_t *red) {
 // and resets the ticket.
 // Chunk `cta` of `ncta` (the CTA's role; the fused GRPO kernel runs it
 // beside the advantages).
-__device__ __forceinline__ void pack_lengths_cta(const uint64_t *__restrict__ soff,
-                                                 uint64_t nseq,
-                                                 const int64_t *__restrict__ idx, uint32_t B,
-                                                 PackEntry *__restrict__ ent,
-                                                 uint64_t *__restrict__ part,
-                                                 uint64_t *__restrict__ pre, uint32_t *work,
+__device__ __forceinline__ void pack_lengths_cta(const uint64_t *soff, uint64_t nseq,
+                                                 const int64_t *idx, uint32_t B, PackEntry *ent,
+                                                 uint64_t *part, uint64_t *pre, uint32_t *work,
                                                  Ctrl *ctrl, uint32_t cta, uint32_t ncta) {
   __shared__ uint64_t red[kPackThreads / 32];
   __shared__ uint32_t ticket;
@@ -165,10 +160,8 @@ __device__ __forceinline__ void pack_lengths_cta(const uint64_t *__restrict__ so
 }
 
 __global__ void __launch_bounds__(kPackThreads)
-k_pack_lengths(const uint64_t *__restrict__ soff, uint64_t nseq,
-               const int64_t *__restrict__ idx, uint32_t B, PackEntry *__restrict__ ent,
-               uint64_t *__restrict__ part, uint64_t *__restrict__ pre, uint32_t *work,
-               Ctrl *ctrl) {
+k_pack_lengths(const uint64_t *soff, uint64_t nseq, const int64_t *idx, uint32_t B, PackEntry *ent,
+               uint64_t *part, uint64_t *pre, uint32_t *work, Ctrl *ctrl) {
   pdl_wait();
   pdl_launch();
   pack_lengths_cta(soff, nseq, idx, B, ent, part, pre, work, ctrl, blockIdx.x, gridDim.x);
@@ -178,11 +171,9 @@ k_pack_lengths(const uint64_t *__restrict__ soff, uint64_t nseq,
 // (two warps each, so the groups spread over the SMs), the others the
 // batch's length pass, which needs no advantage (the gather reads them).
 __global__ void __launch_bounds__(kPackThreads)
-k_grpo_pack_lengths(const float *__restrict__ r, const uint64_t *__restrict__ goff,
-                    uint32_t ng, float eps, float *__restrict__ adv, uint32_t ngc,
-                    const uint64_t *__restrict__ soff, uint64_t nseq,
-                    const int64_t *__restrict__ idx, uint32_t B, PackEntry *__restrict__ ent,
-                    uint64_t *__restrict__ part, uint64_t *__restrict__ pre, uint32_t *work,
+k_grpo_pack_lengths(const float *r, const uint64_t *goff, uint32_t ng, float eps, float *adv,
+                    uint32_t ngc, const uint64_t *soff, uint64_t nseq, const int64_t *idx,
+                    uint32_t B, PackEntry *ent, uint64_t *part, uint64_t *pre, uint32_t *work,
                     Ctrl *ctrl) {
   pdl_wait();
   pdl_launch();
@@ -296,9 +287,8 @@ __device__ __forceinline__ void pack_buf_init(PackBuf &sm) {
 // Output offset of batch entry k (the CTA): the prefix of its 256-entry chunk
 // (from `pre`, or the chunk sums before it) plus the lengths before it in the
 // chunk, in one round trip and a block sum.
-__device__ __forceinline__ uint64_t pack_offset_cta(const PackEntry *__restrict__ ent,
-                                                    const uint64_t *__restrict__ part,
-                                                    const uint64_t *__restrict__ pre, uint32_t k,
+__device__ __forceinline__ uint64_t pack_offset_cta(const PackEntry *ent, const uint64_t *part,
+                                                    const uint64_t *pre, uint32_t k,
                                                     uint64_t *red) {
   const uint32_t c = k / kPackThreads;
   const uint32_t j = c * kPackThreads + threadIdx.x;
@@ -322,11 +312,9 @@ __device__ __forceinline__ uint64_t pack_offset_cta(const PackEntry *__restrict_
 // lengths and advantages 37.3, 39.3 before; 65,536 short sequences 28.0, 28.9).
 template <bool SPLIT>
 __global__ void __launch_bounds__(kPackThreads, 8)
-k_pack_gather(const int32_t *__restrict__ tokens, const PackEntry *__restrict__ ent,
-              const uint64_t *__restrict__ part, const uint64_t *__restrict__ pre, uint32_t B,
-              const float *__restrict__ sv, int32_t *__restrict__ otok,
-              uint64_t *__restrict__ ooff, float *__restrict__ osv, uint64_t cap,
-              uint32_t chunk, Ctrl *ctrl) {
+k_pack_gather(const int32_t *tokens, const PackEntry *ent, const uint64_t *part,
+              const uint64_t *pre, uint32_t B, const float *sv, int32_t *otok, uint64_t *ooff,
+              float *osv, uint64_t cap, uint32_t chunk, Ctrl *ctrl) {
   __shared__ uint64_t red[kPackThreads / 32];
   __shared__ PackBuf sm;
   pack_buf_init(sm);
@@ -370,11 +358,9 @@ constexpr uint32_t kPackWarps = kPackThreads / 32;
 constexpr uint32_t kShortEntries = 32;  // per CTA at most: the lanes of a warp
 
 __global__ void __launch_bounds__(kPackThreads, 6)
-k_pack_gather_short(const int32_t *__restrict__ tokens, const PackEntry *__restrict__ ent,
-                    const uint64_t *__restrict__ part, const uint64_t *__restrict__ pre,
-                    uint32_t B, const float *__restrict__ sv, int32_t *__restrict__ otok,
-                    uint64_t *__restrict__ ooff, float *__restrict__ osv, uint64_t cap,
-                    uint32_t per_warp, Ctrl *ctrl) {
+k_pack_gather_short(const int32_t *tokens, const PackEntry *ent, const uint64_t *part,
+                    const uint64_t *pre, uint32_t B, const float *sv, int32_t *otok,
+                    uint64_t *ooff, float *osv, uint64_t cap, uint32_t per_warp, Ctrl *ctrl) {
   __shared__ uint64_t red[kPackThreads / 32];
   __shared__ PackBuf sm;
   __shared__ uint32_t s_long;  // bit i: entry k0 + i is left to the CTA

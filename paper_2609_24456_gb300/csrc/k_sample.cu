@@ -27,9 +27,8 @@
 namespace edp {
 namespace {
 
-__global__ void k_sample_uniform(uint32_t B, uint64_t seed, uint64_t round,
-                                 uint64_t n_valid, uint64_t oldest,
-                                 uint64_t cap, int64_t *__restrict__ idx) {
+__global__ void k_sample_uniform(uint32_t B, uint64_t seed, uint64_t round, uint64_t n_valid,
+                                 uint64_t oldest, uint64_t cap, int64_t *idx) {
   pdl_wait();
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < B;
        k += gridDim.x * blockDim.x) {
@@ -179,7 +178,7 @@ constexpr uint32_t rank_want(uint32_t n) { return n <= kRankFew ? 128 : kPermThr
 
 __global__ void __launch_bounds__(kPermThreads)
 k_perm_rank(uint32_t n, int lg, uint32_t per_cta, PermScratch sc, uint64_t oldest, uint64_t cap,
-            int64_t *__restrict__ idx) {
+            int64_t *idx) {
   __shared__ uint64_t tkey[kRankTile];
   __shared__ __align__(16) uint32_t ttop[kRankTile];  // high words; ~0 past the pairs
   __shared__ uint32_t tj[kRankTile];

@@ -29,7 +29,7 @@ namespace {
 constexpr uint32_t kMaxShards = 1024;
 constexpr int kRouteThreads = 256;
 
-__global__ void k_tree_total(const uint64_t *__restrict__ root, uint64_t *__restrict__ out) {
+__global__ void k_tree_total(const uint64_t *root, uint64_t *out) {
   pdl_wait();
   pdl_launch();
   if (threadIdx.x == 0) *out = *root;
@@ -39,9 +39,9 @@ __global__ void k_tree_total(const uint64_t *__restrict__ root, uint64_t *__rest
 // targets in stratum order and per-shard counts.  One CTA (a round routes a
 // few hundred strata; the work is a Philox draw and a binary search each).
 __global__ void __launch_bounds__(kRouteThreads)
-k_route_prio(const uint64_t *__restrict__ totals, uint32_t G, uint32_t B, uint32_t k0,
-             uint32_t n, uint64_t seed, uint64_t round, uint64_t *__restrict__ local_t,
-             int64_t *__restrict__ counts, Ctrl *ctrl) {
+k_route_prio(const uint64_t *totals, uint32_t G, uint32_t B, uint32_t k0,
+             uint32_t n, uint64_t seed, uint64_t round, uint64_t *local_t, int64_t *counts,
+             Ctrl *ctrl) {
   __shared__ uint64_t prefix[kMaxShards + 1];
   __shared__ uint32_t cnt[kMaxShards];
   __shared__ int bad;
@@ -88,7 +88,7 @@ k_route_prio(const uint64_t *__restrict__ totals, uint32_t G, uint32_t B, uint32
 // Minimum of q[0..n) as int64 (2^32 - 1 for n == 0, the neutral element of
 // the minimum over ranks).  One CTA.
 __global__ void __launch_bounds__(256)
-k_batch_qmin(const uint32_t *__restrict__ q, uint32_t n, int64_t *__restrict__ out) {
+k_batch_qmin(const uint32_t *q, uint32_t n, int64_t *out) {
   __shared__ uint32_t wmin[8];
   pdl_wait();
   pdl_launch();
@@ -106,9 +106,8 @@ k_batch_qmin(const uint32_t *__restrict__ q, uint32_t n, int64_t *__restrict__ o
 
 // w[k] = (q_min / q[k])^beta, fp64, one rounding to fp32 -- the delivery's
 // importance weight with q_min given (the global batch minimum).
-__global__ void k_is_weights(const uint32_t *__restrict__ q, uint32_t n,
-                             const int64_t *__restrict__ qmin, double beta,
-                             float *__restrict__ w) {
+__global__ void k_is_weights(const uint32_t *q, uint32_t n, const int64_t *qmin, double beta,
+                             float *w) {
   pdl_wait();
   pdl_launch();
   const uint32_t m = (uint32_t)*qmin;

@@ -46,10 +46,8 @@ __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
 }
 
 // Recompute nodes [a0, a0+n0) and [a1, a1+n1) of level d from level d+1.
-__global__ void k_tree_level(uint64_t *__restrict__ out,
-                             const uint64_t *__restrict__ child64,
-                             const uint32_t *__restrict__ child32, uint64_t a0,
-                             uint64_t n0, uint64_t a1, uint64_t n1) {
+__global__ void k_tree_level(uint64_t *out, const uint64_t *child64, const uint32_t *child32,
+                             uint64_t a0, uint64_t n0, uint64_t a1, uint64_t n1) {
   pdl_wait();
   pdl_launch();
   const uint64_t w = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
@@ -186,8 +184,7 @@ __device__ __forceinline__ uint64_t div_by(uint64_t x, uint32_t B, uint64_t inv)
 
 __global__ void __launch_bounds__(kSampleThreads)
 k_sample_prio(TreeView t, uint32_t B, uint64_t inv_b, uint64_t seed, uint64_t round,
-              int64_t *__restrict__ idx, uint32_t *__restrict__ qout,
-              Ctrl *ctrl) {
+              int64_t *idx, uint32_t *qout, Ctrl *ctrl) {
   __shared__ __align__(16) uint64_t top[kSmemNodes];
   const int lane = threadIdx.x & 31;
   const uint64_t keep = policy_keep();
@@ -226,8 +223,8 @@ k_sample_prio(TreeView t, uint32_t B, uint64_t inv_b, uint64_t seed, uint64_t ro
 // eight lanes per target.  A target >= S is reported (DEVERR_INDEX) and
 // gives idx -1, q 0.
 __global__ void __launch_bounds__(kSampleThreads)
-k_sample_targets(TreeView t, const uint64_t *__restrict__ targets, uint32_t n,
-                 int64_t *__restrict__ idx, uint32_t *__restrict__ qout, Ctrl *ctrl) {
+k_sample_targets(TreeView t, const uint64_t *targets, uint32_t n, int64_t *idx, uint32_t *qout,
+                 Ctrl *ctrl) {
   __shared__ __align__(16) uint64_t top[kSmemNodes];
   const int lane = threadIdx.x & 31;
   const uint64_t keep = policy_keep();
@@ -445,8 +442,8 @@ __device__ __noinline__ uint32_t prio_td_call(float td, const PrioRule &rule) {
 }
 
 __global__ void __launch_bounds__(kUpdThreads, 1)
-k_update(TreeView t, const int64_t *__restrict__ idx, const uint32_t *__restrict__ q,
-         const float *__restrict__ td, const __grid_constant__ PrioRule rule, uint32_t n,
+k_update(TreeView t, const int64_t *idx, const uint32_t *q, const float *td,
+         const __grid_constant__ PrioRule rule, uint32_t n,
          uint64_t cap, uint64_t oldest, uint64_t size, int defer, Ctrl *ctrl) {
   __shared__ uint32_t hkey[kUpdTable];
   __shared__ uint32_t hpos[kUpdTable];
@@ -658,8 +655,7 @@ constexpr int kUpdScan = kUpdSmallThreads - 32;                        // scanni
 constexpr int kUpdScanPer = (kUpdSmallMax + kUpdScan - 1) / kUpdScan;  // slots each loads
 
 __global__ void __launch_bounds__(kUpdSmallThreads)
-k_update_small(TreeView t, const int64_t *__restrict__ idx,
-               const uint32_t *__restrict__ q, const float *__restrict__ td,
+k_update_small(TreeView t, const int64_t *idx, const uint32_t *q, const float *td,
                PrioRule rule, uint32_t n, uint64_t cap, uint64_t oldest,
                uint64_t size, int defer, Ctrl *ctrl) {
   __shared__ uint32_t bkey[kUpdSmallMax];  // slot of each pair, kEmpty if it sets none
