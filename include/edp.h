@@ -30,7 +30,7 @@
  *   when NULL) and released by edp_destroy.  libedp never frees caller memory.
  *   Scratch is allocated at a call's first use and grown (after a device
  *   synchronisation) when a later call needs more: the PERMUTE sampling
- *   mode, edp_gae with normalisation and edp_pack_deliver (16 bytes per
+ *   mode, edp_gae with normalisation and edp_pack_deliver (20 bytes per
  *   batch entry).  Before
  *   capturing calls into a CUDA graph, make each of them once at its
  *   largest size, outside the capture: a call that would have to grow its

@@ -29,9 +29,10 @@ struct Ctrl {
   uint32_t err;
   uint32_t pending_q;  // deferred priority of the newest transition
   uint32_t max_q;      // running maximum priority
-  uint32_t pad0[3];
-  uint32_t pack_ticket;  // packed delivery: length CTAs done (calls are ordered)
-  uint32_t pad;
+  // packed delivery (calls are ordered), each 0 between calls: length CTAs done,
+  // long sequences listed, gather CTAs done with the list
+  uint32_t pack_ticket, pack_long, pack_left;
+  uint32_t pad[2];
   unsigned long long bad_index;  // first offending index (diagnostics)
   unsigned long long host_bytes;  // two-tier deliveries: bytes read from the host tier
 };

@@ -12,10 +12,10 @@
 // chunk sums before its chunk plus the lengths before it in the chunk -- and
 // moves its tokens (neither the source nor the destination offset is aligned
 // to more than a token), writing the value beside each token: a CTA per
-// sequence, several CTAs per long sequence, or a warp per short one
-// (launch_gather).  Up to kDirectChunks chunks the copying CTAs add the
-// chunk sums themselves; beyond that the last lengths CTA turns them into
-// prefixes once.  The copy is HBM-bound.
+// sequence, several CTAs per long sequence, or a warp per short one, the long
+// ones among them by CTAs from a list (launch_gather).  Up to kDirectChunks
+// chunks the copying CTAs add the chunk sums themselves; beyond that the last
+// lengths CTA turns them into prefixes once.  The copy is HBM-bound.
 #include "edp_internal.cuh"
 
 namespace edp {
@@ -78,6 +78,31 @@ struct PackEntry {
 };
 constexpr uint32_t kNoSeq = 0xffffffffu;
 
+// What k_pack_gather_short does with the long entries (above kShortTokens) of a
+// CTA's `each` neighbouring ones: the first of them, up to `keep` tokens together,
+// the CTA copies itself, the others the lengths kernel lists (in any order) for
+// whichever CTA takes them.  entry null: no list is wanted.
+constexpr uint32_t kShortTokens = 1024;
+struct LongList {
+  uint32_t *entry;  // [B]
+  uint32_t each;    // 8, 16 or 32: lanes of a warp, and divides the 256-entry chunk
+  uint32_t keep;    // 0: CTAs apart from the others take the list
+};
+enum class Copy { kWarp, kCta, kList };
+// Lane i of a group of `each` lanes: how its entry of `len` tokens is copied.
+__device__ __forceinline__ Copy copy_of(uint32_t len, const LongList &l) {
+  const bool is_long = len > kShortTokens;
+  if (!__any_sync(kFull, is_long)) return Copy::kWarp;
+  const uint32_t g = threadIdx.x & (l.each - 1);
+  uint64_t sum = is_long ? len : 0u;
+#pragma unroll
+  for (uint32_t o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(kFull, sum, o);
+    if (g >= o) sum += y;
+  }
+  return !is_long ? Copy::kWarp : sum <= l.keep ? Copy::kCta : Copy::kList;
+}
+
 __device__ __forceinline__ uint64_t block_sum(uint64_t v, uint64_t *red) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
@@ -100,7 +125,7 @@ __device__ __forceinline__ uint64_t block_sum(uint64_t v, uint64_t *red) {
 // beside the advantages).
 __device__ __forceinline__ void pack_lengths_cta(const uint64_t *soff, uint64_t nseq,
                                                  const int64_t *idx, uint32_t B, PackEntry *ent,
-                                                 uint64_t *part, uint64_t *pre, uint32_t *work,
+                                                 uint64_t *part, uint64_t *pre, LongList longs,
                                                  Ctrl *ctrl, uint32_t cta, uint32_t ncta) {
   __shared__ uint64_t red[kPackThreads / 32];
   __shared__ uint32_t ticket;
@@ -120,6 +145,16 @@ __device__ __forceinline__ void pack_lengths_cta(const uint64_t *soff, uint64_t 
     }
     ent[k] = PackEntry{a, seq, (uint32_t)len};
   }
+  if (longs.entry) {  // one atomic per warp that has any
+    const int lane = threadIdx.x & 31;
+    const bool listed = copy_of((uint32_t)len, longs) == Copy::kList;  // the length as stored
+    const unsigned m = __ballot_sync(kFull, listed);
+    if (m) {
+      uint32_t at = lane == 0 ? atomicAdd(&ctrl->pack_long, (uint32_t)__popc(m)) : 0u;
+      at = __shfl_sync(kFull, at, 0) + __popc(m & ((1u << lane) - 1u));
+      if (listed && at < B) longs.entry[at] = (uint32_t)k;
+    }
+  }
   const uint64_t sum = block_sum(len, red);
   if (!pre) {
     if (threadIdx.x == 0) part[cta] = sum;
@@ -128,7 +163,7 @@ __device__ __forceinline__ void pack_lengths_cta(const uint64_t *soff, uint64_t 
   if (threadIdx.x == 0) {
     part[cta] = sum;
     __threadfence();
-    ticket = atomicAdd(&work[0], 1u);
+    ticket = atomicAdd(&ctrl->pack_ticket, 1u);
   }
   __syncthreads();
   if (ticket != ncta - 1) return;
@@ -156,15 +191,15 @@ __device__ __forceinline__ void pack_lengths_cta(const uint64_t *soff, uint64_t 
     for (int w = 0; w < kPackThreads / 32; ++w) tile += red[w];
     carry += tile;
   }
-  if (threadIdx.x == 0) work[0] = 0u;  // every CTA has taken its ticket
+  if (threadIdx.x == 0) ctrl->pack_ticket = 0u;  // every CTA has taken its ticket
 }
 
 __global__ void __launch_bounds__(kPackThreads)
 k_pack_lengths(const uint64_t *soff, uint64_t nseq, const int64_t *idx, uint32_t B, PackEntry *ent,
-               uint64_t *part, uint64_t *pre, uint32_t *work, Ctrl *ctrl) {
+               uint64_t *part, uint64_t *pre, LongList longs, Ctrl *ctrl) {
   pdl_wait();
   pdl_launch();
-  pack_lengths_cta(soff, nseq, idx, B, ent, part, pre, work, ctrl, blockIdx.x, gridDim.x);
+  pack_lengths_cta(soff, nseq, idx, B, ent, part, pre, longs, ctrl, blockIdx.x, gridDim.x);
 }
 
 // The GRPO step's first kernel: CTAs [0, ngc) compute the group advantages
@@ -173,7 +208,7 @@ k_pack_lengths(const uint64_t *soff, uint64_t nseq, const int64_t *idx, uint32_t
 __global__ void __launch_bounds__(kPackThreads)
 k_grpo_pack_lengths(const float *r, const uint64_t *goff, uint32_t ng, float eps, float *adv,
                     uint32_t ngc, const uint64_t *soff, uint64_t nseq, const int64_t *idx,
-                    uint32_t B, PackEntry *ent, uint64_t *part, uint64_t *pre, uint32_t *work,
+                    uint32_t B, PackEntry *ent, uint64_t *part, uint64_t *pre, LongList longs,
                     Ctrl *ctrl) {
   pdl_wait();
   pdl_launch();
@@ -184,7 +219,7 @@ k_grpo_pack_lengths(const float *r, const uint64_t *goff, uint32_t ng, float eps
                   (uint64_t)ngc * kGrpoWarps);
     return;
   }
-  pack_lengths_cta(soff, nseq, idx, B, ent, part, pre, work, ctrl, blockIdx.x - ngc,
+  pack_lengths_cta(soff, nseq, idx, B, ent, part, pre, longs, ctrl, blockIdx.x - ngc,
                    gridDim.x - ngc);
 }
 
@@ -343,92 +378,125 @@ k_pack_gather(const int32_t *tokens, const PackEntry *ent, const uint64_t *part,
                   ctrl);
 }
 
-// Short sequences, many of them: a CTA takes kWarps * per_warp neighbouring
-// entries, resolves the output offset of the first as above and those of the
-// others from their lengths, and each warp copies its entries by 4-byte loads
-// and stores, kShortUnroll in flight per lane.  An entry above kShortTokens
-// is left to the whole CTA afterwards.  Bound by the chain of a CTA (entries,
-// offset, tokens) that few waves hide.  Calls in a row, lengths U[8, 256]:
-// 65,536 sequences 23.2 us (171 with a CTA each: two block barriers, a bulk
-// copy and an mbarrier for 132 tokens), 4,096 4.8 us (13.4); U[64, 1,024],
-// 8,192 12.2 us (26.2).
-constexpr uint32_t kShortTokens = 1024;
+// Short sequences, many of them: a CTA takes 8, 16 or 32 neighbouring entries,
+// resolves the output offset of the first as above and those of the others from
+// their lengths, and each warp copies its entries by 4-byte loads and stores,
+// kShortUnroll in flight per lane.  A long entry (above kShortTokens) is copied by
+// a whole CTA as in k_pack_gather: by its own one while that has little of such
+// work (LongList::keep), else by the one that its place in the lengths kernel's
+// list names, so that long sequences run side by side however they lie in the
+// batch; batches of less than a wave of CTAs get kServersPerSm CTAs per SM for the
+// list alone.  Bound by the chain of a CTA (entries, offset, tokens) that few
+// waves hide.  Calls in a row, in us, here, (with the long ones left to the CTA of
+// their neighbours) and [a CTA each, k_pack_gather]:
+//   lengths U[8, 256]        65,536: 22.9 (22.5) [171]     4,096: 5.0 (4.8) [13.4]
+//   U[64, 1,024]              8,192: 12.0 (11.7) [25.8]
+//   2% of 16,000, first, 64   1,024: 7.2 (26.7) [7.2]     65,536: 50 (430) [192]
+//   10% of 8,000 at random    1,024: 5.9 (10.0) [8.7]      8,192: 14.1 (19.2) [30.0]
+//   50% of 1,500 at random    8,192: 16.7 (15.6) [25.7]   65,536: 133 (116) [191]
+// kKeepTokens 12,288 or 4,096: 5% slower on one of the last three or another.
 constexpr int kShortUnroll = 8;
 constexpr uint32_t kPackWarps = kPackThreads / 32;
 constexpr uint32_t kShortEntries = 32;  // per CTA at most: the lanes of a warp
+constexpr uint32_t kServersPerSm = 4;
+constexpr uint32_t kKeepTokens = 6144;
 
 __global__ void __launch_bounds__(kPackThreads, 6)
 k_pack_gather_short(const int32_t *tokens, const PackEntry *ent, const uint64_t *part,
                     const uint64_t *pre, uint32_t B, const float *sv, int32_t *otok,
-                    uint64_t *ooff, float *osv, uint64_t cap, uint32_t per_warp, Ctrl *ctrl) {
+                    uint64_t *ooff, float *osv, uint64_t cap, uint32_t server0,
+                    LongList longs, Ctrl *ctrl) {
   __shared__ uint64_t red[kPackThreads / 32];
   __shared__ PackBuf sm;
-  __shared__ uint32_t s_long;  // bit i: entry k0 + i is left to the CTA
-  if (threadIdx.x == 0) s_long = 0;
+  __shared__ uint32_t s_listed;
   pack_buf_init(sm);
   uint32_t uses = 0;
   const int lane = threadIdx.x & 31;
   const uint32_t warp = threadIdx.x >> 5;
   const uint64_t pol = policy_stream();
   pdl_wait();
-  const uint32_t each = kPackWarps * per_warp;  // 8, 16 or 32: divides the 256-entry chunk
-  const uint32_t k0 = blockIdx.x * each;
-  const uint32_t ne = min(each, B - k0);
+  const uint32_t each = longs.each, per_warp = each / kPackWarps;
+  const uint64_t first = (uint64_t)blockIdx.x * each;
+  const uint32_t k0 = (uint32_t)min(first, (uint64_t)B);
+  const uint32_t ne = min(each, B - k0);  // 0: a CTA for the list alone
+  const uint32_t server = blockIdx.x - server0, nserver = gridDim.x - server0;
+  const uint32_t next = !ne && server < B ? longs.entry[server] : 0u;  // beside the length
+  if (threadIdx.x == 0) s_listed = min(__ldcg(&ctrl->pack_long), B);
+  if (!ne) __syncthreads();  // else one follows
   // lane i of every warp: entry k0 + i, and its value
   PackEntry mine{0, kNoSeq, 0};
   if ((uint32_t)lane < ne) mine = ent[k0 + lane];
   float value = 0.f;
   if (osv && mine.seq != kNoSeq) value = __ldcg(&sv[mine.seq]);
-  uint64_t dst = mine.len;  // inclusive, then exclusive prefix
+  if (ne) {
+    uint64_t dst = mine.len;  // inclusive, then exclusive prefix
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint64_t y = __shfl_up_sync(kFull, dst, o);
-    if (lane >= o) dst += y;
-  }
-  dst += pack_offset_cta(ent, part, pre, k0, red) - mine.len;
-  if (warp == 0 && (uint32_t)lane < ne) {
-    ooff[k0 + lane] = dst;
-    if (mine.len > kShortTokens) atomicOr(&s_long, 1u << lane);
-    if (k0 + lane == B - 1) {
-      ooff[B] = dst + mine.len;
-      if (dst + mine.len > cap)
-        flag(ctrl, DEVERR_OVERFLOW, (unsigned long long)(dst + mine.len));
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(kFull, dst, o);
+      if (lane >= o) dst += y;
+    }
+    dst += pack_offset_cta(ent, part, pre, k0, red) - mine.len;
+    if (warp == 0 && (uint32_t)lane < ne) {
+      ooff[k0 + lane] = dst;
+      if (k0 + lane == B - 1) {
+        ooff[B] = dst + mine.len;
+        if (dst + mine.len > cap)
+          flag(ctrl, DEVERR_OVERFLOW, (unsigned long long)(dst + mine.len));
+      }
+    }
+    for (uint32_t i = warp * per_warp; i < min(ne, (warp + 1) * per_warp); ++i) {
+      const uint32_t len = __shfl_sync(kFull, mine.len, i);
+      const uint64_t d = __shfl_sync(kFull, dst, i);
+      const uint64_t src = __shfl_sync(kFull, mine.src, i);
+      const uint32_t vbits = __float_as_uint(__shfl_sync(kFull, value, i));
+      if (len > kShortTokens || d >= cap) continue;
+      const uint32_t n = (uint32_t)min((uint64_t)len, cap - d);
+      const int32_t *sc = tokens + src;
+      for (uint32_t t0 = lane; t0 < n; t0 += 32 * kShortUnroll) {
+        int32_t v[kShortUnroll];
+#pragma unroll
+        for (int u = 0; u < kShortUnroll; ++u)
+          if (t0 + u * 32 < n) v[u] = __ldg(sc + t0 + u * 32);
+#pragma unroll
+        for (int u = 0; u < kShortUnroll; ++u)
+          if (t0 + u * 32 < n) {
+            st_stream32(otok + d + t0 + u * 32, (uint32_t)v[u], pol);
+            if (osv) st_stream32(osv + d + t0 + u * 32, vbits, pol);
+          }
+      }
+    }
+    const Copy how = copy_of(mine.len, longs);
+    for (uint32_t left = __ballot_sync(kFull, how == Copy::kCta); left; left &= left - 1) {
+      const int i = __ffs(left) - 1;  // the same in every warp
+      const uint32_t len = __shfl_sync(kFull, mine.len, i);
+      const uint64_t d = __shfl_sync(kFull, dst, i);
+      const uint64_t src = __shfl_sync(kFull, mine.src, i);
+      const float val = __shfl_sync(kFull, value, i);
+      if (d >= cap) continue;
+      const uint64_t n = min((uint64_t)len, cap - d);
+      for (uint64_t c0 = 0; c0 < n; c0 += kPackChunk)
+        pack_copy_cta(sm, uses, tokens + src, otok + d, osv ? osv + d : nullptr,
+                      __float_as_uint(val), c0, (uint32_t)min((uint64_t)kPackChunk, n - c0), k0 + i,
+                      pol, ctrl);
     }
   }
-  for (uint32_t i = warp * per_warp; i < min(ne, (warp + 1) * per_warp); ++i) {
-    const uint32_t len = __shfl_sync(kFull, mine.len, i);
-    const uint64_t d = __shfl_sync(kFull, dst, i);
-    const uint64_t src = __shfl_sync(kFull, mine.src, i);
-    const uint32_t vbits = __float_as_uint(__shfl_sync(kFull, value, i));
-    if (len > kShortTokens || d >= cap) continue;
-    const uint32_t n = (uint32_t)min((uint64_t)len, cap - d);
-    const int32_t *sc = tokens + src;
-    for (uint32_t t0 = lane; t0 < n; t0 += 32 * kShortUnroll) {
-      int32_t v[kShortUnroll];
-#pragma unroll
-      for (int u = 0; u < kShortUnroll; ++u)
-        if (t0 + u * 32 < n) v[u] = __ldg(sc + t0 + u * 32);
-#pragma unroll
-      for (int u = 0; u < kShortUnroll; ++u)
-        if (t0 + u * 32 < n) {
-          st_stream32(otok + d + t0 + u * 32, (uint32_t)v[u], pol);
-          if (osv) st_stream32(osv + d + t0 + u * 32, vbits, pol);
-        }
+  if (blockIdx.x >= server0) {
+    const uint32_t listed = s_listed;  // thread 0's, so that all of the CTA go by one value
+    for (uint32_t i = server; i < listed; i += nserver) {
+      const uint32_t k = !ne && i == server ? next : longs.entry[i];
+      const PackEntry e = ent[k];
+      const uint64_t d = pack_offset_cta(ent, part, pre, k, red);
+      if (d >= cap) continue;
+      const float val = osv && e.seq != kNoSeq ? __ldcg(&sv[e.seq]) : 0.f;
+      const uint64_t n = min((uint64_t)e.len, cap - d);
+      for (uint64_t c0 = 0; c0 < n; c0 += kPackChunk)
+        pack_copy_cta(sm, uses, tokens + e.src, otok + d, osv ? osv + d : nullptr,
+                      __float_as_uint(val), c0, (uint32_t)min((uint64_t)kPackChunk, n - c0), k,
+                      pol, ctrl);
     }
-  }
-  __syncthreads();
-  for (uint32_t left = s_long; left; left &= left - 1) {
-    const int i = __ffs(left) - 1;
-    const uint32_t len = __shfl_sync(kFull, mine.len, i);
-    const uint64_t d = __shfl_sync(kFull, dst, i);
-    const uint64_t src = __shfl_sync(kFull, mine.src, i);
-    const float val = __shfl_sync(kFull, value, i);
-    if (d >= cap) continue;
-    const uint64_t n = min((uint64_t)len, cap - d);
-    for (uint64_t c0 = 0; c0 < n; c0 += kPackChunk)
-      pack_copy_cta(sm, uses, tokens + src, otok + d, osv ? osv + d : nullptr,
-                    __float_as_uint(val), c0, (uint32_t)min((uint64_t)kPackChunk, n - c0), k0 + i,
-                    pol, ctrl);
+    // the last CTA that is done with the list clears it for the next call
+    if (listed && threadIdx.x == 0 && atomicInc(&ctrl->pack_left, nserver - 1) == nserver - 1)
+      ctrl->pack_long = 0;
   }
 }
 
@@ -447,34 +515,43 @@ cudaError_t launch_grpo(edp_ctx *c, const float *r, const uint64_t *goff, uint32
 
 namespace {
 
+// A wave of gather CTAs.
+uint64_t pack_wave(const edp_ctx *c) { return 6ull * (uint64_t)c->coop_sms; }
+
 struct PackPlan {
   PackEntry *ent;
   uint64_t *part, *pre;
-  uint32_t *work;
+  LongList longs;  // entry null: k_pack_gather
   uint32_t G;
 };
 
-cudaError_t pack_plan(edp_ctx *c, uint32_t B, cudaStream_t s, PackPlan *p) {
+cudaError_t pack_plan(edp_ctx *c, uint32_t B, uint64_t cap, cudaStream_t s, PackPlan *p) {
   p->G = (B + kPackThreads - 1) / kPackThreads;
   const size_t ent_bytes = ((size_t)B * sizeof(PackEntry) + 255) & ~(size_t)255;
   void *blk = nullptr;
-  const cudaError_t e =
-      ctx_scratch(c, ent_bytes + 2 * (size_t)p->G * sizeof(uint64_t), s, &blk);
+  const cudaError_t e = ctx_scratch(
+      c, ent_bytes + 2 * (size_t)p->G * sizeof(uint64_t) + (size_t)B * sizeof(uint32_t), s, &blk);
   if (e != cudaSuccess) return e;
   uint8_t *scr = (uint8_t *)blk;
   p->ent = (PackEntry *)scr;
   p->part = (uint64_t *)(scr + ent_bytes);
   p->pre = p->G > kDirectChunks ? p->part + p->G : nullptr;
-  // packed deliveries share the scratch above, so they are ordered, and one
-  // ticket serves them all
-  p->work = &c->ctrl->pack_ticket;
+  p->longs = LongList{};
+  const uint64_t wave = pack_wave(c);
+  if (B > wave && cap / B <= kShortTokens) {  // k_pack_gather_short (launch_gather)
+    p->longs.entry = (uint32_t *)(p->part + 2 * (size_t)p->G);
+    uint32_t &each = p->longs.each = kShortEntries;
+    while (each > kPackWarps && B < 2 * wave * each) each /= 2;
+    p->longs.keep = (B + each - 1) / each < wave ? 0 : kKeepTokens;
+  }
   return cudaSuccess;
 }
 
 // How the batch is copied follows from its size and from the room the caller
 // gave it, which bounds the mean length (the lengths are on the device):
 //  - more sequences than about a wave of CTAs, at most kShortTokens of room
-//    each on average: k_pack_gather_short;
+//    each on average: k_pack_gather_short (1,024 sequences U[1, 256] 3.9 us, 4.9
+//    with a CTA each; exponential lengths of mean 512 5.7, 5.4);
 //  - otherwise a CTA per sequence, and where that leaves the chip idle and
 //    the room allows long sequences, several CTAs per sequence on chunks of
 //    1,024 tokens or more (64 sequences U[2,048, 32,768]: 5.9 us, 12.3 with
@@ -482,15 +559,16 @@ cudaError_t pack_plan(edp_ctx *c, uint32_t B, cudaStream_t s, PackPlan *p) {
 cudaError_t launch_gather(edp_ctx *c, const PackPlan &p, const int32_t *tokens, uint32_t B,
                           const float *sv, int32_t *otok, uint64_t *ooff, float *osv,
                           uint64_t cap, cudaStream_t s) {
-  const uint64_t wave = 6ull * (uint64_t)c->coop_sms;
+  const uint64_t wave = pack_wave(c);
   const uint64_t room = cap / B;
-  if (B > wave && room <= kShortTokens) {
-    uint32_t per_warp = kShortEntries / kPackWarps;
-    while (per_warp > 1 && B < 2 * wave * kPackWarps * per_warp) per_warp /= 2;
-    const uint32_t each = kPackWarps * per_warp;
-    return launch_pdl(k_pack_gather_short, dim3((B + each - 1) / each), dim3(kPackThreads), s,
-                      tokens, (const PackEntry *)p.ent, (const uint64_t *)p.part,
-                      (const uint64_t *)p.pre, B, sv, otok, ooff, osv, cap, per_warp, c->ctrl);
+  if (p.longs.entry) {
+    const uint32_t ctas = (B + p.longs.each - 1) / p.longs.each;
+    const bool apart = !p.longs.keep;
+    return launch_pdl(k_pack_gather_short,
+                      dim3(apart ? ctas + kServersPerSm * (unsigned)c->coop_sms : ctas),
+                      dim3(kPackThreads), s, tokens, (const PackEntry *)p.ent,
+                      (const uint64_t *)p.part, (const uint64_t *)p.pre, B, sv, otok, ooff, osv,
+                      cap, apart ? ctas : 0u, p.longs, c->ctrl);
   }
   uint32_t chunk = kPackChunk;
   while (chunk > 1024 && (uint64_t)B * ((room + chunk - 1) / chunk) < wave) chunk /= 2;
@@ -511,10 +589,10 @@ cudaError_t launch_pack(edp_ctx *c, const int32_t *tokens, const uint64_t *soff,
                         int32_t *otok, uint64_t *ooff, float *osv, uint64_t cap,
                         cudaStream_t s) {
   PackPlan p;
-  cudaError_t e = pack_plan(c, B, s, &p);
+  cudaError_t e = pack_plan(c, B, cap, s, &p);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(k_pack_lengths, dim3(p.G), dim3(kPackThreads), s, soff, nseq,
-                             idx, B, p.ent, p.part, p.pre, p.work, c->ctrl);
+  e = launch_pdl(k_pack_lengths, dim3(p.G), dim3(kPackThreads), s, soff, nseq, idx, B,
+                 p.ent, p.part, p.pre, p.longs, c->ctrl);
   if (e != cudaSuccess) return e;
   return launch_gather(c, p, tokens, B, sv, otok, ooff, osv, cap, s);
 }
@@ -525,13 +603,13 @@ cudaError_t launch_grpo_pack(edp_ctx *c, const float *r, const uint64_t *goff, u
                              uint32_t B, int32_t *otok, uint64_t *ooff, float *osv,
                              uint64_t cap, cudaStream_t s) {
   PackPlan p;
-  cudaError_t e = pack_plan(c, B, s, &p);
+  cudaError_t e = pack_plan(c, B, cap, s, &p);
   if (e != cudaSuccess) return e;
   uint64_t ngc = (ng + kGrpoWarps - 1) / kGrpoWarps;
   if (ngc > 16ull * c->coop_sms) ngc = 16ull * c->coop_sms;
   e = launch_pdl(k_grpo_pack_lengths, dim3((unsigned)(ngc + p.G)), dim3(kPackThreads), s, r,
                  goff, ng, eps, adv, (uint32_t)ngc, soff, nseq, idx, B, p.ent, p.part, p.pre,
-                 p.work, c->ctrl);
+                 p.longs, c->ctrl);
   if (e != cudaSuccess) return e;
   return launch_gather(c, p, tokens, B, adv, otok, ooff, osv, cap, s);
 }
