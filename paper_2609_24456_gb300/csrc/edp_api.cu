@@ -1314,7 +1314,7 @@ edp_status edp_pack_deliver(edp_ctx *ctx, const int32_t *tokens, const uint64_t 
   EDP_TRACE(__func__);
   cudaError_t e = launch_pack(ctx, tokens, seq_off, n_seq, idx, batch, seq_value,
                               (int32_t *)outs[0], (uint64_t *)outs[1], (float *)outs[2],
-                              out_cap, (cudaStream_t)stream);
+                              out_cap, host[0] || host[2], (cudaStream_t)stream);
   if (e != cudaSuccess) return launch_fail(ctx, e, "edp_pack_deliver");
   count_hbm(ctx, 24ull * batch, 0);  // indices and sequence offsets; tokens not counted
   count_write(ctx, host[1], 8ull * (batch + 1));
@@ -1357,7 +1357,8 @@ edp_status edp_grpo_pack_deliver(edp_ctx *ctx, const float *r, const uint64_t *g
   EDP_TRACE(__func__);
   cudaError_t e = launch_grpo_pack(ctx, r, group_off, n_groups, eps, adv, tokens, seq_off,
                                    n_seq, idx, batch, (int32_t *)outs[0], (uint64_t *)outs[1],
-                                   (float *)outs[2], out_cap, (cudaStream_t)stream);
+                                   (float *)outs[2], out_cap, host[0] || host[2],
+                                   (cudaStream_t)stream);
   if (e != cudaSuccess) return launch_fail(ctx, e, "edp_grpo_pack_deliver");
   count_hbm(ctx, 8ull * (n_groups + 1) + 24ull * batch, 0);
   count_write(ctx, host[1], 8ull * (batch + 1));

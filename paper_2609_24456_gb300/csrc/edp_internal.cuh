@@ -472,18 +472,19 @@ struct DrawUniform {
 cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
                            const edp_batch *out, cudaStream_t s,
                            const DrawUniform *draw = nullptr);
-// LLM post-training: group-relative advantages and packed delivery
+// LLM post-training: group-relative advantages and packed delivery (host_out: tokens
+// or values go to page-locked host memory)
 cudaError_t launch_grpo(edp_ctx *ctx, const float *r, const uint64_t *goff, uint32_t ng,
                         float eps, float *adv, cudaStream_t s);
 cudaError_t launch_pack(edp_ctx *ctx, const int32_t *tokens, const uint64_t *soff,
                         uint64_t nseq, const int64_t *idx, uint32_t B, const float *sv,
-                        int32_t *otok, uint64_t *ooff, float *osv, uint64_t cap,
+                        int32_t *otok, uint64_t *ooff, float *osv, uint64_t cap, bool host_out,
                         cudaStream_t s);
 cudaError_t launch_grpo_pack(edp_ctx *ctx, const float *r, const uint64_t *goff, uint32_t ng,
                              float eps, float *adv, const int32_t *tokens,
                              const uint64_t *soff, uint64_t nseq, const int64_t *idx,
                              uint32_t B, int32_t *otok, uint64_t *ooff, float *osv,
-                             uint64_t cap, cudaStream_t s);
+                             uint64_t cap, bool host_out, cudaStream_t s);
 cudaError_t launch_tree_refresh(edp_ctx *ctx, uint64_t first_leaf,
                                 uint64_t count, cudaStream_t s);
 // Nodes of each level d that cover leaves [first, first + count) (mod the

@@ -525,7 +525,8 @@ struct PackPlan {
   uint32_t G;
 };
 
-cudaError_t pack_plan(edp_ctx *c, uint32_t B, uint64_t cap, cudaStream_t s, PackPlan *p) {
+cudaError_t pack_plan(edp_ctx *c, uint32_t B, uint64_t cap, bool host_out, cudaStream_t s,
+                      PackPlan *p) {
   p->G = (B + kPackThreads - 1) / kPackThreads;
   const size_t ent_bytes = ((size_t)B * sizeof(PackEntry) + 255) & ~(size_t)255;
   void *blk = nullptr;
@@ -538,7 +539,7 @@ cudaError_t pack_plan(edp_ctx *c, uint32_t B, uint64_t cap, cudaStream_t s, Pack
   p->pre = p->G > kDirectChunks ? p->part + p->G : nullptr;
   p->longs = LongList{};
   const uint64_t wave = pack_wave(c);
-  if (B > wave && cap / B <= kShortTokens) {  // k_pack_gather_short (launch_gather)
+  if (B > wave && cap / B <= kShortTokens && !host_out) {  // k_pack_gather_short (launch_gather)
     p->longs.entry = (uint32_t *)(p->part + 2 * (size_t)p->G);
     uint32_t &each = p->longs.each = kShortEntries;
     while (each > kPackWarps && B < 2 * wave * each) each /= 2;
@@ -551,7 +552,10 @@ cudaError_t pack_plan(edp_ctx *c, uint32_t B, uint64_t cap, cudaStream_t s, Pack
 // gave it, which bounds the mean length (the lengths are on the device):
 //  - more sequences than about a wave of CTAs, at most kShortTokens of room
 //    each on average: k_pack_gather_short (1,024 sequences U[1, 256] 3.9 us, 4.9
-//    with a CTA each; exponential lengths of mean 512 5.7, 5.4);
+//    with a CTA each; exponential lengths of mean 512 5.7, 5.4).  Not into
+//    page-locked host memory, where its 4-byte stores of any alignment make more
+//    and smaller writes on the link: 4,096 sequences U[64, 1,024] 154 us, 111 with a
+//    CTA each, 16,384 U[8, 256] 153, 126;
 //  - otherwise a CTA per sequence, and where that leaves the chip idle and
 //    the room allows long sequences, several CTAs per sequence on chunks of
 //    1,024 tokens or more (64 sequences U[2,048, 32,768]: 5.9 us, 12.3 with
@@ -586,10 +590,10 @@ cudaError_t launch_gather(edp_ctx *c, const PackPlan &p, const int32_t *tokens, 
 
 cudaError_t launch_pack(edp_ctx *c, const int32_t *tokens, const uint64_t *soff,
                         uint64_t nseq, const int64_t *idx, uint32_t B, const float *sv,
-                        int32_t *otok, uint64_t *ooff, float *osv, uint64_t cap,
+                        int32_t *otok, uint64_t *ooff, float *osv, uint64_t cap, bool host_out,
                         cudaStream_t s) {
   PackPlan p;
-  cudaError_t e = pack_plan(c, B, cap, s, &p);
+  cudaError_t e = pack_plan(c, B, cap, host_out, s, &p);
   if (e != cudaSuccess) return e;
   e = launch_pdl(k_pack_lengths, dim3(p.G), dim3(kPackThreads), s, soff, nseq, idx, B,
                  p.ent, p.part, p.pre, p.longs, c->ctrl);
@@ -601,9 +605,9 @@ cudaError_t launch_grpo_pack(edp_ctx *c, const float *r, const uint64_t *goff, u
                              float eps, float *adv, const int32_t *tokens,
                              const uint64_t *soff, uint64_t nseq, const int64_t *idx,
                              uint32_t B, int32_t *otok, uint64_t *ooff, float *osv,
-                             uint64_t cap, cudaStream_t s) {
+                             uint64_t cap, bool host_out, cudaStream_t s) {
   PackPlan p;
-  cudaError_t e = pack_plan(c, B, cap, s, &p);
+  cudaError_t e = pack_plan(c, B, cap, host_out, s, &p);
   if (e != cudaSuccess) return e;
   uint64_t ngc = (ng + kGrpoWarps - 1) / kGrpoWarps;
   if (ngc > 16ull * c->coop_sms) ngc = 16ull * c->coop_sms;

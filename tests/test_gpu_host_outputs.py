@@ -2,8 +2,8 @@
 batch over the host link): bit-identical to the same deliveries into device
 memory, for the three transforms -- frame stacks with collate and
 importance weights, HWC -> CHW bf16 with gathered advantages and returns,
-normalised bf16 with tokens from a two-tier ring -- and pageable host
-outputs rejected."""
+normalised bf16 with tokens from a two-tier ring -- and for packed
+sequences, many short ones among them; pageable host outputs rejected."""
 import numpy as np
 import pytest
 import torch
@@ -30,7 +30,7 @@ def test_frame_stack_per_into_host(edp_lib, orc):
     m = MirroredDqn(1200, prioritized=True)
     for sl in (slice(0, 700), slice(700, 1500)):  # wraps the ring
         m.ingest(orc, frames[sl], action[sl], reward[sl], done[sl], q=q[sl])
-    for B in (32, 700):  # one chunk per CTA, and the staged path
+    for B in (32, 700):  # a few CTAs, and more than a wave
         idx = torch.empty(B, dtype=torch.int64, device="cuda")
         qs = torch.empty(B, dtype=torch.int32, device="cuda")
         edp.edp_sample(m.ring.ctx, edp.EDP_SAMPLE_PRIORITIZED, B, 5, B, idx, qs)
@@ -87,3 +87,34 @@ def test_two_tier_norm_into_host(edp_lib, orc):
         edp.edp_deliver(ring.ctx, idx, B, edp.make_batch(torch.empty((B, C, H, W),
                                                                      dtype=torch.bfloat16)))
     assert e.value.status == edp.EDP_ERR_INVALID
+
+
+@pytest.mark.parametrize("B,lmax", [(1500, 90), (9000, 40), (100, 3000)])
+@pytest.mark.parametrize("pin", [(True, True), (True, False), (False, True), (True, None)])
+def test_packed_into_host(edp_lib, B, lmax, pin):
+    """Tokens and values each into either memory, or no values."""
+    edp = edp_lib
+    rng = np.random.default_rng(B)
+    lens = rng.integers(0, lmax + 1, size=B)
+    lens[B // 2] = 2500
+    off = np.zeros(B + 1, np.uint64)
+    np.cumsum(lens, out=off[1:])
+    total = int(off[-1])
+    tok, idx = rng.integers(0, 1 << 30, size=total, dtype=np.int32), rng.permutation(B)
+    t = [cuda(x) for x in (tok, off, idx.astype(np.int64),
+                           rng.standard_normal(B).astype(np.float32))]
+    ring = edp.Ring(edp.make_config(16, (1, 4, 4), edp.EDP_XFORM_HWC_CHW_BF16), action=False,
+                    reward=False, done=False)
+    dev = [torch.full((total,), -3, dtype=torch.int32, device="cuda"),
+           torch.full((total,), -3.0, device="cuda"),
+           torch.zeros(B + 1, dtype=torch.int64, device="cuda")]
+    host = [_pinned_like(x) if p else torch.empty_like(x) for x, p in zip(dev, (*pin, pin[0]))]
+    for o in (dev, host):
+        edp.edp_pack_deliver(ring.ctx, t[0], t[1], B, t[2], B, o[0], o[2], total,
+                             seq_value=t[3] if pin[1] is not None else None,
+                             out_value=o[1] if pin[1] is not None else None)
+    edp.edp_sync(ring.ctx)
+    if pin[1] is None:
+        dev, host = [dev[0], dev[2]], [host[0], host[2]]
+    _same(dev, host)
+    ring.close()
