@@ -71,6 +71,10 @@ struct edp_ctx {
   float naff_a[4] = {}, naff_b[4] = {};
   int norm_affine = 0;
   int coop_sms = 0;
+  // stream of the last sampling or priority update (a handle that is compared,
+  // never used): a delivery on another one runs beside such kernels
+  cudaStream_t sampler_stream = nullptr;
+  bool sampler_known = false;
   edp_counters cnt{};  // host-side traffic counters (edp_get_counters)
   uint64_t host_bytes_base = 0;  // the device's host-tier byte count at the last reset
   std::string err;
@@ -555,6 +559,12 @@ size_t perm_zeroed_bytes();
 // ---------------------------------------------------------------------------
 // Host helpers shared by the entry points
 // ---------------------------------------------------------------------------
+
+// Notes the stream of a sampling or a priority update.
+inline void samples_on(edp_ctx *c, cudaStream_t s) {
+  c->sampler_stream = s;
+  c->sampler_known = true;
+}
 
 // Makes `dev` the calling thread's current device for the guard's lifetime
 // and gives the thread its previous current device back afterwards, so an

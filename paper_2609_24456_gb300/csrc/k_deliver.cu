@@ -221,11 +221,12 @@ __device__ __forceinline__ float byte_f(uint32_t w, int i) {
 // anchor" (zeroes the frame in obs and next_obs) and "at the anchor" (zeroes
 // it in next_obs only).
 //
-// A warp runs one unrolled iteration: UN loads in flight per lane, a span of
-// 32 UN words, a CTA per kWarps spans, however many waves that makes; the
-// first CTAs collate the batch (collate_batch) so that no streaming warp
-// waits on it.  UN = 8 (256 words) keeps 8 KB of reads in flight per CTA;
-// batches that give an SM less than one CTA at 4 spread over more SMs with 4.
+// A warp runs one unrolled iteration (or two, launch_deliver): UN loads in
+// flight per lane, a span of 32 UN words or twice that, a CTA per kWarps spans,
+// however many waves that makes; the first CTAs collate the batch
+// (collate_batch) so that no streaming warp waits on it.  UN = 8 (256 words) keeps
+// 8 KB of reads in flight per CTA; batches that give an SM less than one CTA at 4
+// spread over more SMs with 4.
 //
 // Bound by HBM.  Calls in a row, a fresh sample each, in us, and before, when
 // frames were staged through shared memory by bulk copies, 2 CTAs per SM:
@@ -246,6 +247,7 @@ struct StackArgs {
   uint32_t K;
   uint32_t U;     // frames per sample (K, or K + 1 with next_obs)
   uint32_t ncollate;  // CTAs that collate the batch
+  uint32_t span;      // words per warp, a multiple of 32 UN
   float *obs;
   float *next;
 };
@@ -343,8 +345,8 @@ k_deliver_stack(Common c, StackArgs a) {
     return;
   }
   const uint64_t total = (uint64_t)c.B * a.U * a.W;
-  const uint64_t f = ((uint64_t)(blockIdx.x - a.ncollate) * kWarps + warp) * (32 * UN);
-  if (f < total) stack_span<UN>(c, a, f, min(total, f + 32 * UN), lane, pol);
+  const uint64_t f = ((uint64_t)(blockIdx.x - a.ncollate) * kWarps + warp) * a.span;
+  if (f < total) stack_span<UN>(c, a, f, min(total, f + a.span), lane, pol);
 }
 
 // ---------------------------------------------------------------------------
@@ -934,17 +936,28 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
       return launch_pdl(kern, dim3((unsigned)ctas), dim3(kThreads), s, c, a, g);
     }
     const bool few = units <= (uint64_t)kWarps * 32 * 4 * sms;
-    const uint64_t each = (uint64_t)kWarps * 32 * (few ? 4 : 8);
-    const uint64_t ctas = (units + each - 1) / each + a.ncollate;
-    if (ctas > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    auto kern = few ? k_deliver_stack<4> : k_deliver_stack<8>;
+    a.span = 32 * (few ? 4 : 8);
+    uint64_t ctas = (units + (uint64_t)kWarps * a.span - 1) / ((uint64_t)kWarps * a.span);
     // With successors and more than two and a half waves, four CTAs per SM
     // instead of five, held there by shared memory that they don't use: as fast
     // alone (84x84, 4 frames, 512: 22.7 us, 22.9), and the small kernels of other
     // streams find room among its waves (sampling and update beside it: a round
     // 22.6 us, 24.4).  Without successors four are 12% slower (8,192: 195 us,
     // 171), between one wave and two up to 15%.
-    const bool four = a.next && 2 * ctas >= 5ull * kStackMinBlocks * sms;
+    const bool four = a.next && 2 * (ctas + a.ncollate) >= 5ull * kStackMinBlocks * sms;
+    // On another stream than the context's sampling and updates, two iterations
+    // per warp up to 16 waves: in half the waves those kernels, on which the next
+    // delivery waits, get through sooner.  That round 21.6 us instead of 22.6 for
+    // 512 stacks, 43.3 instead of 43.9 for 1,024, 83.8 instead of 84.4 for 2,048
+    // (8,192: 327.5, 326.6).  On their stream it is slower, the last wave being
+    // longer: 30.5 instead of 29.7, the delivery alone 23.7 instead of 22.8.
+    if (four && ctas <= 64ull * sms && ctx->sampler_known && s != ctx->sampler_stream) {
+      a.span *= 2;
+      ctas = (ctas + 1) / 2;
+    }
+    ctas += a.ncollate;
+    if (ctas > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    auto kern = few ? k_deliver_stack<4> : k_deliver_stack<8>;
     return launch_pdl_smem(kern, dim3((unsigned)ctas), dim3(kThreads), four ? kFourPerSm : 0, s,
                            c, a);
   } else if (cfg.transform == EDP_XFORM_HWC_CHW_BF16) {

@@ -267,6 +267,7 @@ k_perm_rank(uint32_t n, int lg, uint32_t per_cta, PermScratch sc, uint64_t oldes
 
 cudaError_t launch_sample_uniform(edp_ctx *c, uint32_t B, uint64_t seed,
                                   uint64_t round, int64_t *idx, cudaStream_t s) {
+  samples_on(c, s);
   const uint64_t size = c->total < c->cap ? c->total : c->cap;
   const uint64_t oldest = (c->total - size) % c->cap;
   const uint64_t nv = size - c->defer;

@@ -820,6 +820,7 @@ dim3 sample_grid(const edp_ctx *c, uint32_t n) {
 
 cudaError_t launch_sample_targets(edp_ctx *c, const uint64_t *targets, uint32_t n,
                                   int64_t *idx, uint32_t *q, cudaStream_t s) {
+  samples_on(c, s);
   return launch_pdl(k_sample_targets, sample_grid(c, n), dim3(kSampleThreads), s, view(c),
                     targets, n, idx, q, c->ctrl);
 }
@@ -827,6 +828,7 @@ cudaError_t launch_sample_targets(edp_ctx *c, const uint64_t *targets, uint32_t 
 cudaError_t launch_sample_prioritized(edp_ctx *c, uint32_t B, uint64_t seed,
                                       uint64_t round, int64_t *idx, uint32_t *q,
                                       cudaStream_t s) {
+  samples_on(c, s);
   return launch_pdl(k_sample_prio, sample_grid(c, B), dim3(kSampleThreads), s, view(c), B,
                     ~0ull / B, seed, round, idx, q, c->ctrl);
 }
@@ -834,6 +836,7 @@ cudaError_t launch_sample_prioritized(edp_ctx *c, uint32_t B, uint64_t seed,
 cudaError_t launch_update(edp_ctx *c, const int64_t *idx, const uint32_t *q,
                           const float *td, double alpha, double eps, uint32_t n,
                           cudaStream_t s) {
+  samples_on(c, s);
   const uint64_t size = c->total < c->cap ? c->total : c->cap;
   const uint64_t oldest = (c->total - size) % c->cap;
   if (n <= (uint32_t)kUpdSmallMax)

@@ -68,3 +68,34 @@ def test_frame_sizes(edp_lib, orc, h, w, K, nxt, B):
         ulp = to_np(isw).view(np.int32) - orc.is_weights(u32(qs), 0.5).view(np.int32)
         assert np.abs(ulp).max() <= 1
     ring.close()
+
+
+@pytest.mark.parametrize("h,w,K,B", [(84, 84, 4, 512), (4, 1796, 3, 700), (64, 64, 2, 1501),
+                                     (4, 4228, 1, 601), (84, 84, 4, 2300)])
+def test_beside_the_sampler(edp_lib, h, w, K, B):
+    """A delivery on another stream than the sampling may give its warps twice the
+    span (up to 16 waves): the same bits as on the sampler's stream, with a bad
+    slot and importance weights."""
+    edp = edp_lib
+    F, cap = h * w, 300
+    frames, action, reward, done = fx.dqn_transitions(h + w, cap + 37, F, done_p=0.05)
+    ring = edp.Ring(edp.make_config(cap, (1, h, w), edp.EDP_XFORM_STACK_F32, frame_stack=K,
+                                    next_obs=True, prioritized=True))
+    for lo, hi in [(0, cap), (cap, cap + 37)]:
+        edp.edp_ingest(ring.ctx, cuda(frames[lo:hi]), hi - lo, action=cuda(action[lo:hi]),
+                       reward=cuda(reward[lo:hi]), done=cuda(done[lo:hi]))
+    idx = torch.zeros(B, dtype=torch.int64, device="cuda")
+    q = torch.zeros(B, dtype=torch.int32, device="cuda")
+    edp.edp_sample(ring.ctx, edp.EDP_SAMPLE_PRIORITIZED, B, 5, 0, idx, q)
+    idx[B // 2] = cap + 1
+    outs = []
+    for stream in (torch.cuda.current_stream(), torch.cuda.Stream()):
+        out = list(dqn_outputs(B, K, F)) + [torch.full((B,), -1.0, device="cuda")]
+        torch.cuda.synchronize()
+        edp.edp_deliver(ring.ctx, idx, B, edp.make_batch(*out[:5], q=q, isw=out[5], beta=0.5),
+                        stream=stream)
+        assert edp.edp_sync_status(ring.ctx, stream)[0] == edp.EDP_ERR_INVALID
+        outs.append([bits(t) for t in out])
+    for x, y in zip(*outs):
+        assert np.array_equal(x, y)
+    ring.close()
