@@ -225,8 +225,7 @@ __device__ __forceinline__ float byte_f(uint32_t w, int i) {
 // flight per lane, a span of 32 UN words or twice that, a CTA per kWarps spans,
 // however many waves that makes; the first CTAs collate the batch
 // (collate_batch) so that no streaming warp waits on it.  UN = 8 (256 words) keeps
-// 8 KB of reads in flight per CTA; batches that give an SM less than one CTA at 4
-// spread over more SMs with 4.
+// 8 KB of reads in flight per CTA; small batches spread over more SMs with 4.
 //
 // Bound by HBM.  Calls in a row, a fresh sample each, in us, and before, when
 // frames were staged through shared memory by bulk copies, 2 CTAs per SM:
@@ -935,7 +934,10 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
       auto kern = wide ? k_deliver_stack_flat<8> : k_deliver_stack_flat<4>;
       return launch_pdl(kern, dim3((unsigned)ctas), dim3(kThreads), s, c, a, g);
     }
-    const bool few = units <= (uint64_t)kWarps * 32 * 4 * sms;
+    // 4 loads per lane up to three such CTAs per SM (84x84, 4 frames and
+    // successors, 48: 4.1 us, 4.6 with 8; 64: 4.7, 4.6; 128x128, 16: 3.6, 4.1; one
+    // frame, 192: 3.6, 3.8)
+    const bool few = units <= 3ull * kWarps * 32 * 4 * sms;
     a.span = 32 * (few ? 4 : 8);
     uint64_t ctas = (units + (uint64_t)kWarps * a.span - 1) / ((uint64_t)kWarps * a.span);
     // With successors and more than two and a half waves, four CTAs per SM
