@@ -231,13 +231,15 @@ k_sample_targets(TreeView t, const uint64_t *targets, uint32_t n, int64_t *idx, 
   pdl_wait();
   pdl_launch();
   const uint64_t S = t.nodes[0];  // issued beside the loads of the top levels
+  const uint64_t first =
+      (uint64_t)blockIdx.x * kSamplePerCta + threadIdx.x / 32 * (32 / kGroup);
+  uint64_t target = first + lane / kGroup < n ? targets[first + lane / kGroup] : 0;  // likewise
   const uint32_t cached = cache_top(t, top, keep);
   __syncthreads();
-  for (uint64_t k0 = (uint64_t)blockIdx.x * kSamplePerCta + threadIdx.x / 32 * (32 / kGroup);
-       k0 < n; k0 += (uint64_t)gridDim.x * kSamplePerCta) {
+  for (uint64_t k0 = first; k0 < n; k0 += (uint64_t)gridDim.x * kSamplePerCta) {
     const uint64_t k = k0 + lane / kGroup;
     const bool mine = k < n;
-    const uint64_t target = mine ? targets[k] : 0;
+    if (k0 != first) target = mine ? targets[k] : 0;
     const bool in = target < S;
     bool ok = true;
     uint32_t q = 0;
