@@ -850,15 +850,15 @@ k_deliver_norm(Common c, NormArgs a) {
 // iterations of its unrolled loop (`per_iter` units each), so the block
 // scheduler balances the tail and a CTA that starts late (its SM still busy
 // with another kernel) holds up little work; a small batch is spread over up
-// to one wave (blocks resident per SM x SMs, queried once per kernel) with
-// at least one iteration per warp.
-template <typename Kern>
-unsigned grid_for(Kern kern, uint64_t units, uint64_t per_iter, int iters, int sms) {
-  static int per_sm = 0;  // per template instantiation
-  if (!per_sm) {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0);
-    if (per_sm < 1) per_sm = 1;
-  }
+// to one wave (blocks resident per SM x SMs, queried once for each kernel: the
+// library runs on one kind of GPU) with at least one iteration per warp.
+template <auto kern>
+unsigned grid_for(uint64_t units, uint64_t per_iter, int iters, int sms) {
+  static const int per_sm = [] {
+    int n = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kThreads, 0);
+    return n < 1 ? 1 : n;
+  }();
   const uint64_t wave = (uint64_t)per_sm * sms;
   const uint64_t warp_iters = (units + per_iter - 1) / per_iter;
   uint64_t blocks = (warp_iters + (uint64_t)kWarps * iters - 1) / ((uint64_t)kWarps * iters);
@@ -1012,10 +1012,12 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     // by warps).
     if (total > 2 * (uint64_t)kNormCtas * sms * units) {
       if (a.F8 >= 1024) {
-        auto kern = ctx->norm_affine ? k_deliver_norm<kNormUnroll, true>
-                                     : k_deliver_norm<kNormUnroll, false>;
-        return launch_pdl(kern, dim3(grid_for(kern, total, 32 * kNormUnroll, kNormIters, sms)),
-                          dim3(kThreads), s, c, a);
+        constexpr auto one_fma = k_deliver_norm<kNormUnroll, true>;
+        constexpr auto chain = k_deliver_norm<kNormUnroll, false>;
+        const unsigned grid =
+            ctx->norm_affine ? grid_for<one_fma>(total, 32 * kNormUnroll, kNormIters, sms)
+                             : grid_for<chain>(total, 32 * kNormUnroll, kNormIters, sms);
+        return launch_pdl(ctx->norm_affine ? one_fma : chain, dim3(grid), dim3(kThreads), s, c, a);
       }
       units *= 2;
     }
