@@ -416,8 +416,8 @@ __device__ __forceinline__ bool slot_holds(int64_t sl, uint64_t cap, uint64_t ol
 // nodes rarely collide and take one 64-bit atomic per pair, level 1 (32 nodes)
 // and the root are summed on chip first.  A batch of more pairs per CTA than
 // half of the list, or with more pairs of one owner than the list holds, is
-// entered in batch order, a part at a time where its distinct slots outgrow the
-// table (a part's leaves are read again by the next).  The running maximum
+// entered in batch order, a part at a time where its pairs outgrow the table (a
+// part's leaves are read again by the next).  The running maximum
 // counts every pair, the overwritten ones too, so each warp evaluates a stripe
 // of the batch for it.
 //
@@ -873,7 +873,6 @@ extern "C" edp_status edp_update_priorities_td_static(
   using namespace edp;
   static const char who[] = "edp_update_priorities_td_static";
   constexpr uint32_t kStaticMaxPairs = 16384;
-  constexpr int kMaxDevices = 64;
   if (ctx && n && !td) return fail(ctx, EDP_ERR_INVALID, "%s: td NULL", who);
   const edp_status st = update_args(ctx, who, idx, nullptr, td, n, alpha, eps);
   if (st != EDP_OK || n == 0) return st;
@@ -881,8 +880,6 @@ extern "C" edp_status edp_update_priorities_td_static(
     return fail(ctx, EDP_ERR_INVALID,
                 "%s: n exceeds the fixed maximum of 16384 pairs (use "
                 "edp_update_priorities_td)", who);
-  if (ctx->cfg.device < 0 || ctx->cfg.device >= kMaxDevices)
-    return fail(ctx, EDP_ERR_INVALID, "%s: device ordinal out of range", who);
   DeviceGuard dg(ctx->cfg.device);
   EDP_TRACE(who);
   const cudaError_t e =

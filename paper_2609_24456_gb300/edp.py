@@ -279,8 +279,8 @@ def edp_update_priorities_td(ctx, idx, td, n, alpha, eps, stream=None):
 
 
 def edp_update_priorities_td_static(ctx, idx, td, n, alpha, eps, stream=None):
-    """Allocation-free edp_update_priorities_td (fixed per-device scratch of
-    16384 pairs; see include/edp.h)."""
+    """edp_update_priorities_td for callers that cannot allocate (neither entry
+    point does), at most 16384 pairs; see include/edp.h."""
     return _check(ctx, lib().edp_update_priorities_td_static(
         ctx, ptr(idx), ptr(td), n, alpha, eps, stream_handle(stream)),
         "edp_update_priorities_td_static")

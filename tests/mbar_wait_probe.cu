@@ -1,5 +1,5 @@
-// Test probe (not part of libedp): the bounded mbarrier wait that the staged
-// frame-stack delivery uses, run on its own.  One thread initialises an
+// Test probe (not part of libedp): the bounded mbarrier wait that the packed
+// delivery's bulk copies use, run on its own.  One thread initialises an
 // mbarrier expecting one arrival and waits for phase 0 with a time limit:
 // first with nothing arriving (the wait must give up after about the limit
 // and report false), then after its own arrival (true at once).  Times are
@@ -17,7 +17,8 @@ __global__ void k_mbar_wait_probe(uint64_t limit_ns, unsigned long long *out) {
   const uint64_t t0 = edp::global_ns();
   const bool got = edp::mbar_wait(&bar, 0, limit_ns);  // nothing arrives
   const uint64_t t1 = edp::global_ns();
-  edp::mbar_arrive(&bar);                              // completes phase 0
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];"  // completes phase 0
+               :: "r"(edp::smem_addr(&bar)) : "memory");
   const bool got2 = edp::mbar_wait(&bar, 0, limit_ns);
   const uint64_t t2 = edp::global_ns();
   out[0] = got;

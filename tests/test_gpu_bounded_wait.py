@@ -1,10 +1,10 @@
-"""The bounded mbarrier wait of the staged frame-stack delivery expires
+"""The bounded mbarrier wait of the packed delivery's bulk copies expires
 instead of hanging.  The probe (tests/mbar_wait_probe.cu, built by the
 package's build step) runs libedp's wait helper on an mbarrier that nothing
 arrives on: the wait must return false after about its limit (here 2 ms),
 with the GPU context still usable; after the thread's own arrival the same
-wait returns true at once.  The delivery kernel uses the same helper (with a
-1 s limit) and reports an expiry as DEVERR_TIMEOUT."""
+wait returns true at once.  The packed gathers use the same helper (with a 1 s
+limit) and report an expiry as DEVERR_TIMEOUT."""
 import ctypes as C
 
 import pytest
