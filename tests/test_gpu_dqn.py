@@ -110,10 +110,10 @@ def test_dqn_host_pinned_ingest_source(edp_lib, orc):
 
 
 @pytest.mark.parametrize("fw", [112, 560])
-def test_staged_stack_multi_piece_frames_and_bad_indices(edp_lib, orc, fw):
-    """Frames larger than one shared-memory stage (84 x 112 = 9,408 B in two
-    pieces, 84 x 560 = 47,040 B in seven) through the staged delivery (a
-    batch of 300 stacks fills the GPU), with episode ends and a wrapped ring;
+def test_large_frames_and_bad_indices(edp_lib, orc, fw):
+    """Frames that take many warps' spans each (84 x 112 = 9,408 B in ten of
+    1,024 B, 84 x 560 = 47,040 B in 46), in a batch of 300 stacks that fills the
+    GPU, with episode ends and a wrapped ring;
     slots outside the sampleable range (-1, capacity, the newest slot, whose
     successor does not exist) give zero rows and a device flag, and every
     other row equals the oracle's."""

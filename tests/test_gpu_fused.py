@@ -1,8 +1,8 @@
 """The fused uniform sample -> deliver call (edp_sample_deliver) through the
 C ABI: the same indices as edp_sample(UNIFORM) with the same seed and round
 (and as the oracle's sampler), and outputs bit-identical to edp_deliver of
-those indices, for the three transforms -- frame stacks (one chunk per CTA
-and the staged path), HWC -> CHW bf16, and normalised bf16 over a
+those indices, for the three transforms -- frame stacks (a few CTAs and
+many waves), HWC -> CHW bf16, and normalised bf16 over a
 two-tier ring; plus its argument errors."""
 import numpy as np
 import pytest

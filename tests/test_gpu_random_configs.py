@@ -1,9 +1,10 @@
 """Randomised configurations against the oracle, to reach the corners of
 the launch logic the fixed-size tests do not: frame stacks of K = 1..16 with
-and without next_obs, frame sizes of one and several shared-memory pieces,
+and without next_obs, frame sizes on both sides of the flat kernel's limit,
 dense and sparse episode ends, rings filled in random chunk sizes past a wrap
-(insertions take the one-launch path up to 16,384 rows, the kernel chain
-above), batches on both sides of the staged delivery's threshold; and
+(insertions take the one-launch path up to 4,096 rows, or 16,384 of large
+rows, the kernel chain above), batches on both sides of the delivery's change of
+span; and
 normalised deliveries of 1 to 4 channels, with and without tokens, on one
 and two tiers.  Every output bit-exact against the oracle."""
 import numpy as np

@@ -1,8 +1,8 @@
 """Randomised prioritized-replay rounds against the oracle: rings of 40 to
 40,000 slots filled past a wrap in random chunks with random priorities
 (some zero, some at the running maximum), frame stacks of 1 to 8 with and
-without next_obs, batches of 1 to 2,000 on both sides of the staged
-delivery's threshold; per round the indices, priorities and whole batch
+without next_obs, batches of 1 to 2,000 on both sides of the
+delivery's change of span; per round the indices, priorities and whole batch
 bit-exact, IS weights within 1 ulp, then a priority update (u32 or from TD
 errors, with repeats, the deferred newest transition and slots that hold
 nothing) after which every node of the tree is compared."""

@@ -1,13 +1,12 @@
-"""The staged path of the frame-stack delivery, under concurrency.
+"""Frame-stack deliveries that fill the GPU, under concurrency.
 
-A batch that fills the GPU (here 1,024 stacks, 5,120 frame pieces) is
-delivered by the staged kernel: pieces are dealt to the CTAs round robin,
-so a launch shares no state with any other and leaves none behind.  Here it
-is delivered many times: from two streams at once, 40 times in a row inside
-a CUDA graph, and 40 deliveries that may all run at once -- released
-together on eight streams, eagerly and from a graph replayed twice.  Every
-delivery must equal the first bit for bit, and the first must equal the
-oracle on a strided sample of rows.
+A batch of 1,024 stacks of four 84x84 frames and their successors is 4,410
+CTAs, each of which writes its own words of the batch: a launch shares no state
+with any other and leaves none behind.  Here it is delivered many times: from
+two streams at once, 40 times in a row inside a CUDA graph, and 40 deliveries
+that may all run at once -- released together on eight streams, eagerly and
+from a graph replayed twice.  Every delivery must equal the first bit for bit,
+and the first must equal the oracle on a strided sample of rows.
 """
 import numpy as np
 import pytest
@@ -20,7 +19,7 @@ pytestmark = pytest.mark.gpu
 B, CAP, N_INGEST = 1024, 3000, 2900
 
 
-def test_concurrent_and_repeated_staged_deliveries(edp_lib, orc):
+def test_concurrent_and_repeated_deliveries(edp_lib, orc):
     edp = edp_lib
     frames, action, reward, done = fx.dqn_transitions(40, N_INGEST, done_p=0.05)
     m = MirroredDqn(CAP)
@@ -74,8 +73,8 @@ def test_concurrent_and_repeated_staged_deliveries(edp_lib, orc):
 @pytest.mark.parametrize("B", [37, 1024])
 def test_outputs_16_byte_aligned_only(edp_lib, orc, B):
     """Outputs 16 bytes past a 32-byte boundary (the alignment the ABI
-    requires, and no more) give the same batches as aligned ones, on the
-    one-chunk-per-CTA and the staged paths."""
+    requires, and no more) give the same batches as aligned ones, in small and
+    in large grids."""
     edp = edp_lib
     frames, action, reward, done = fx.dqn_transitions(42, N_INGEST, done_p=0.05)
     m = MirroredDqn(CAP)

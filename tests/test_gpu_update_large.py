@@ -1,8 +1,8 @@
 """Priority updates above the single-pass kernel's 2,048 pairs: at the edges
 of the scan's chunk of 8,192 pairs, with every pair on one slot, with few
-slots, and with more distinct slots of one owner CTA than its table holds
-(they are then applied in parts).  Every node of the tree against the
-oracle, bit for bit."""
+slots, with every pair of one owner CTA (more than its list and table hold: they
+are then applied in parts), and with more distinct slots of one owner than its
+table.  Every node of the tree against the oracle, bit for bit."""
 import numpy as np
 import pytest
 import torch
@@ -26,10 +26,10 @@ def big(edp_lib, orc):
     m.ring.close()
 
 
-def _one_owner(n):
+def _one_owner(n, cap=CAP):
     """Slots that one CTA of an n-pair update owns (the kernel's split)."""
     grid = min((n + 63) // 64, torch.cuda.get_device_properties(0).multi_processor_count)
-    s = np.arange(CAP, dtype=np.uint64)
+    s = np.arange(cap, dtype=np.uint64)
     owner = (((s * np.uint64(0x9E3779B1)) & np.uint64(0xFFFFFFFF)) * np.uint64(grid)) >> np.uint64(32)
     return np.flatnonzero(owner == 1)
 
@@ -70,3 +70,24 @@ def test_beyond_the_list(edp_lib, orc, big, slots):
     edp.edp_sync(m.ring.ctx)
     orc.update_leaves(m.st, m.total, idx, qu)
     check_tree(orc, m.ring, m.st)
+
+
+@pytest.mark.parametrize("n", [8192, 30_011])
+def test_more_slots_of_one_owner_than_its_table(edp_lib, orc, n):
+    edp, cap, fill = edp_lib, 600_000, 600_500
+    rng = np.random.default_rng(n)
+    m = MirroredDqn(cap, F=84 * 4, prioritized=True)
+    q = rng.integers(1, 1 << 24, size=fill).astype(np.uint32)
+    for lo, hi in [(0, cap), (cap, fill)]:
+        k = hi - lo
+        m.ingest(orc, np.zeros((k, 84 * 4), np.uint8), np.zeros(k, np.int32),
+                 np.zeros(k, np.float32), np.zeros(k, np.uint8), q=q[lo:hi])
+    idx = rng.choice(_one_owner(n, cap), size=n).astype(np.int64)
+    assert len(np.unique(idx)) > 3072  # the table takes no more
+    idx[5] = (m.total - 1) % cap
+    qu = rng.integers(0, 1 << 32, size=n, dtype=np.uint64).astype(np.uint32)
+    edp.edp_update_priorities(m.ring.ctx, cuda(idx), cuda(qu), n)
+    edp.edp_sync(m.ring.ctx)
+    orc.update_leaves(m.st, m.total, idx, qu)
+    check_tree(orc, m.ring, m.st)
+    m.ring.close()

@@ -2,15 +2,14 @@
 
 edp_update_priorities_td_static serves callers that cannot allocate device
 memory while they update priorities (for instance while a CUDA graph is being
-captured, or under a runtime that hands out all device memory at start-up):
-it keeps its per-pair scratch in a fixed per-device array instead of
-allocating it.  Its results must equal those of the allocating
-edp_update_priorities_td on the same arguments -- here compared on the whole
-priority tree (leaves, every internal sum, the deferred and the running
-maximum priority), bit for bit, after two calls in a row, and after two
-calls queued back to back on one stream; and against the oracle.  This
-file is collected last so that a failure here leaves every other test
-already run.
+captured, or under a runtime that hands out all device memory at start-up).
+Neither it nor edp_update_priorities_td allocates; it keeps a maximum size.
+Its results are compared with the oracle's and with those of
+edp_update_priorities_td on the same arguments, on the whole priority tree
+(leaves, every internal sum, the deferred and the running maximum priority),
+bit for bit, after two calls in a row, and after two calls queued back to back
+on one stream.  This file is collected last so that a failure here leaves
+every other test already run.
 """
 import numpy as np
 import pytest
@@ -34,12 +33,20 @@ def _twin_rings(orc, cap, n):
     return rings
 
 
-def test_static_update_matches_allocating_update(edp_lib, orc):
+def _device_rule(edp, ring, d_td, n):
+    """The priorities that the device's rule gives for these TD errors."""
+    qd = torch.zeros(n, dtype=torch.int32, device="cuda")
+    edp.edp_priorities_from_td(ring.ctx, d_td, n, ALPHA, EPS, qd)
+    edp.edp_sync(ring.ctx)
+    return qd.cpu().numpy().view(np.uint32)
+
+
+def test_static_update_matches_the_oracle_and_the_other(edp_lib, orc):
     edp = edp_lib
     cap, n_ingest = 3000, 2500
     a, b = _twin_rings(orc, cap, n_ingest)
     rng = np.random.default_rng(22)
-    for call in range(2):  # two calls in a row share the fixed array
+    for call in range(2):
         n = 700 + 300 * call
         idx = rng.integers(0, n_ingest, size=n).astype(np.int64)
         idx[::5] = idx[1]  # duplicates: the last pair wins
@@ -59,6 +66,8 @@ def test_static_update_matches_allocating_update(edp_lib, orc):
         assert (pa, ma) == (pb, mb)
         # and the update did happen: the leaves of the updated slots moved
         assert not np.array_equal(la[:cap], b.st.leaves)
+        orc.update_leaves(b.st, b.total, idx, _device_rule(edp, b.ring, d_td, n))
+        check_tree(orc, b.ring, b.st)
     # then a pair of calls queued back to back on one stream, with nothing
     # between them: stream order alone keeps them apart
     pairs = []
@@ -66,11 +75,11 @@ def test_static_update_matches_allocating_update(edp_lib, orc):
         n = 4000
         idx = rng.integers(0, n_ingest, size=n).astype(np.int64)
         idx[: n // 2] = rng.integers(0, 300, size=n // 2)  # slots both calls hit
-        pairs.append((cuda(idx), cuda(fx.td_errors(200 + call, n)), n))
+        pairs.append((cuda(idx), cuda(fx.td_errors(200 + call, n)), n, idx))
     torch.cuda.synchronize()
-    for d_idx, d_td, n in pairs:
+    for d_idx, d_td, n, _ in pairs:
         edp.edp_update_priorities_td(a.ring.ctx, d_idx, d_td, n, ALPHA, EPS)
-    for d_idx, d_td, n in pairs:
+    for d_idx, d_td, n, _ in pairs:
         edp.edp_update_priorities_td_static(b.ring.ctx, d_idx, d_td, n, ALPHA, EPS)
     edp.edp_sync(a.ring.ctx)
     edp.edp_sync(b.ring.ctx)
@@ -80,6 +89,9 @@ def test_static_update_matches_allocating_update(edp_lib, orc):
     for d, (x, y) in enumerate(zip(lva, lvb)):
         assert np.array_equal(x, y), d
     assert (pa, ma) == (pb, mb)
+    for _, d_td, n, idx in pairs:
+        orc.update_leaves(b.st, b.total, idx, _device_rule(edp, b.ring, d_td, n))
+    check_tree(orc, b.ring, b.st)
 
 
 def test_static_updates_back_to_back_match_oracle(edp_lib, orc):
