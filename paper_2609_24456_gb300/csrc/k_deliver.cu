@@ -362,9 +362,12 @@ k_deliver_stack(Common c, StackArgs a) {
 //
 // Taken for frames below kFlatFrame bytes, where a span of k_deliver_stack
 // crosses several frames and walks them in turn.  Calls in a row, 32,768
-// samples, in us, here and (k_deliver_stack): 8x16, 1 frame and its
-// successor, 12.5 (120: with 4 loads per lane); 20x20, 4 and their
-// successors, 83 (97.5); 28x28, 4 and their successors, 159 (144).
+// samples, in us, here and (k_deliver_stack): 8x16, 1 frame and its successor,
+// 12.5 (120: with 4 loads per lane); 4 frames and their successors of 320 bytes
+// 67 (89), 448 91 (108), 512 102 (94: its frames end where spans do), 704 139
+// (148), 768 150 (140), 784 154 (162), 1,024 198 (185).  8,192: 320 bytes 21.3
+// (24.4), 704 39.2 (40.3), 784 42.4 (43.9).  Up to 2,048 samples the two cross
+// at 320 to 384 bytes: 320 8.2 (8.1), 448 9.8 (9.3), 704 13.4 (12.2).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kFlatFrame = 768;
 constexpr uint32_t kFlatSamples = kThreads;  // at most touched by a CTA

@@ -35,9 +35,9 @@
 //
 // Bound by latency (a chunk's loads, then its dependent chain) up to ~10^6
 // values, then by HBM.  Calls in a row with all three outputs, in us, and
-// (before) with one warp per environment: 8 x 2,048 steps 10.8 (43.0), 4,096 x
-// 64 12.3 (28.4), 1,024 x 1,024 24.3 (107), 64 x 8,192 37.9 (557), 8 x 128 7.0
-// (9.2), 8 x 512 7.4.
+// (before) with one warp per environment: 8 x 2,048 steps 10.3 (43.0), 4,096 x
+// 64 12.3 (28.4), 1,024 x 1,024 24.8 (107), 64 x 8,192 37.9 (557), 8 x 128 6.8
+// (9.2), 8 x 512 7.0 (16.0).
 //
 // Two kernels chained with programmatic dependent launch: the scan writes A,
 // the returns and per-CTA sums of A and A^2; the normalisation kernel
@@ -361,10 +361,10 @@ k_gae_scan(const float *r, const float *v, const uint8_t *d, uint32_t T, uint32_
 
 // Sum of the per-CTA partials (sum A, sum A^2) in a fixed order; the totals
 // end in *s1, *s2 of thread 0.  Every CTA that calls it gets the same bits.  Up
-// to kFewParts one warp adds and shuffles them, without a barrier (8 x 2,048:
-// 10.9 us per call, 11.9 with the tree); more take strided per-thread sums and a
-// shared-memory tree, whose levels use fewer and fewer warps of the fp64 pipe
-// (4,096 x 32: 10.3 us, 11.7 with shuffles in every warp).
+// to kFewParts one warp adds and shuffles them, without a barrier (a call of 8 x
+// 2,048 takes 1.0 us longer with the tree); more take strided per-thread sums and
+// a shared-memory tree, whose levels use fewer and fewer warps of the fp64 pipe
+// (4,096 x 32: 1.4 us longer with shuffles in every warp).
 constexpr uint32_t kFewParts = 128;
 __device__ __forceinline__ void reduce_partials(const double *partial, uint32_t nparts,
                                                 double *s1, double *s2) {
@@ -479,8 +479,8 @@ size_t gae_scratch_bytes(uint32_t E) { return ((size_t)E + 3) / 4 * 2 * sizeof(d
 // Environments per CTA, threads per CTA and CTAs of a scan.  A CTA of
 // 512 threads is bound by issue (about 4 us per chunk whatever its shape), so
 // the environments per CTA are halved from 8 while half of the SMs would idle:
-// 8 x 512 steps with 8, 4, 2, 1 environments per CTA 12.9, 9.4, 7.8, 7.4 us
-// per call, 8 x 2,048 35.1, 21.0, 13.9, 10.9, 256 x 128 7.8, 7.6, 8.0, 9.6.
+// 8 x 512 steps with 8, 4, 2, 1 environments per CTA 12.7, 9.4, 7.8, 7.2 us
+// per call, 8 x 2,048 35.9, 21.5, 13.8, 10.3, 256 x 128 7.6, 7.4, 7.6, 9.1.
 struct GaeShape {
   uint32_t envs, threads, grid;
 };
@@ -511,8 +511,8 @@ cudaError_t launch_scan(const GaeShape &g, const float *r, const float *v, const
 
 // One CTA per SM while that leaves a thread a few elements: each CTA adds the
 // partial sums again and forms the statistics, and several on one SM queue on
-// its fp64 pipe (4,096 x 64: 12.3 us per call, 13.0 with four per SM); four per
-// SM for the loads of more (1,024 x 1,024: 24.3 us, 27.9 with one).
+// its fp64 pipe (4,096 x 64: 12.7 us per call, 13.2 with four per SM); four per
+// SM for the loads of more (1,024 x 1,024: 25.3 us, 29.6 with one).
 unsigned norm_grid(const edp_ctx *c, uint64_t n) {
   const uint64_t sms = (uint64_t)c->coop_sms;
   const uint64_t want = (n + 4 * kNormThreads - 1) / (4 * kNormThreads);
@@ -527,7 +527,7 @@ cudaError_t launch_gae(edp_ctx *c, const float *r, const float *v,
                        double lambda, float *adv, float *ret, float *adv_norm,
                        cudaStream_t s) {
   // a rollout of one chunk of eight environments: one CTA scans and normalises
-  // it (8 x 128: 7.2 us either way from a graph; one launch instead of two)
+  // it (8 x 128: 6.8 us; equal either way from a graph, one launch instead of two)
   const bool one_cta = adv_norm && E <= 8 && T <= 128;
   const GaeShape g = gae_shape(c, T, E, one_cta);
   double *partial = nullptr;

@@ -388,9 +388,12 @@ cudaError_t launch_ingest_meta(edp_ctx *c, const edp_fields *f, uint64_t n,
 }
 
 // While one CTA's metadata hides behind the copy, or costs less than the chain
-// of kernels: rows of 128 bytes with priorities, 4,096 6.0 us (7.5 as a chain),
-// 8,192 9.0 (7.6); of 7,056 bytes, 8,192 20.3 (24.5), 16,384 40.8 (41.5), without
-// priorities 39.4 (35.9).
+// of kernels.  With priorities, as one launch and (as a chain), us: rows of 128 or
+// 512 bytes, 4,096 6.0 (7.2), 5,120 7.5 (7.4), 8,192 9.0 (7.6); of 1,024 bytes, 8,192
+// 9.2 (8.8), 6,144 8.0 (8.2); of 2,304, 12,288 13.0 (13.6), 16,384 17.1 (16.6); of
+// 7,056, 8,192 20.6 (24.8), 16,384 41.0 (41.4).  Without priorities the chain is two
+// kernels and ahead from 2,048 rows of up to 1,024 bytes on (4,096 of 128: 5.1,
+// 2.9); of 7,056 bytes 4,096 8.6 (8.7), 8,192 20.6 (19.5), 16,384 40.1 (35.9).
 bool ingest_fusable(const edp_ctx *c, uint64_t n) {
   if (c->cap_c) return false;
   return n <= 4096 || (c->obs_bytes >= 1024 && n <= (c->depth ? 16384u : 8192u));

@@ -1,7 +1,7 @@
 """Randomised configurations against the oracle, to reach the corners of
 the launch logic the fixed-size tests do not: frame stacks of K = 1..16 with
-and without next_obs, frame sizes on both sides of the flat kernel's limit,
-dense and sparse episode ends, rings filled in random chunk sizes past a wrap
+and without next_obs, frames of 1,680 to 9,408 bytes (no whole number of warps'
+spans), dense and sparse episode ends, rings filled in random chunk sizes past a wrap
 (insertions take the one-launch path up to 4,096 rows, or 16,384 of large
 rows, the kernel chain above), batches on both sides of the delivery's change of
 span; and
