@@ -645,6 +645,34 @@ __device__ __forceinline__ uint32_t row_of_unit(uint32_t i, uint32_t d, uint32_t
   return inv ? __umulhi(i, inv) : (i >= d ? 1u : 0u);
 }
 
+// The eight bytes of unit w of an image, normalised.
+template <bool AFF>
+__device__ __forceinline__ uint4 norm_unit(const Common &c, const NormArgs &a, uint2 v,
+                                           uint32_t w) {
+  const uint32_t ch = (w >= a.HW8) + (w >= 2 * a.HW8) + (w >= 3 * a.HW8);
+  float fv[8];
+  if constexpr (AFF) {
+    const float A = a.aa[ch], Bc = a.ab[ch];
+#pragma unroll
+    for (int bb = 0; bb < 8; ++bb)
+      fv[bb] = __fmaf_rn(byte_f(bb < 4 ? v.x : v.y, bb & 3), A, Bc);
+  } else {
+    const float mc = a.mean[ch], s1 = a.s1[ch], s2 = a.s2[ch];
+#pragma unroll
+    for (int bb = 0; bb < 8; ++bb) {
+      const float x = unit_f32(byte_f(bb < 4 ? v.x : v.y, bb & 3), c.r1, c.r2);
+      const float tt = __fsub_rn(x, mc);
+      fv[bb] = a.fast ? __fmaf_rn(tt, s1, __fmul_rn(tt, s2)) : __fdiv_rn(tt, a.sd[ch]);
+    }
+  }
+  uint4 o;
+  o.x = pack_bf16x2(fv[0], fv[1]);
+  o.y = pack_bf16x2(fv[2], fv[3]);
+  o.z = pack_bf16x2(fv[4], fv[5]);
+  o.w = pack_bf16x2(fv[6], fv[7]);
+  return o;
+}
+
 template <int UN, bool AFF, bool TWO>
 __global__ void __launch_bounds__(kThreads, kNormCtas)
 k_deliver_norm_flat(Common c, NormArgs a) {
@@ -721,27 +749,7 @@ k_deliver_norm_flat(Common c, NormArgs a) {
       const uint32_t i = i0 + u * kThreads;
       if (i >= i_1) continue;
       const uint32_t s = row_of_unit(i, P, a.div_f), w = i - s * P;
-      const uint32_t ch = (w >= a.HW8) + (w >= 2 * a.HW8) + (w >= 3 * a.HW8);
-      float fv[8];
-      if constexpr (AFF) {
-        const float A = a.aa[ch], Bc = a.ab[ch];
-#pragma unroll
-        for (int bb = 0; bb < 8; ++bb)
-          fv[bb] = __fmaf_rn(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), A, Bc);
-      } else {
-        const float mc = a.mean[ch], s1 = a.s1[ch], s2 = a.s2[ch];
-#pragma unroll
-        for (int bb = 0; bb < 8; ++bb) {
-          const float x = unit_f32(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), c.r1, c.r2);
-          const float tt = __fsub_rn(x, mc);
-          fv[bb] = a.fast ? __fmaf_rn(tt, s1, __fmul_rn(tt, s2)) : __fdiv_rn(tt, a.sd[ch]);
-        }
-      }
-      uint4 o;
-      o.x = pack_bf16x2(fv[0], fv[1]);
-      o.y = pack_bf16x2(fv[2], fv[3]);
-      o.z = pack_bf16x2(fv[4], fv[5]);
-      o.w = pack_bf16x2(fv[6], fv[7]);
+      uint4 o = norm_unit<AFF>(c, a, v[u], w);
       if (!s_src[s]) o = make_uint4(0u, 0u, 0u, 0u);
       st_stream(dst + i, o, pol);
     }
@@ -795,27 +803,7 @@ k_deliver_norm(Common c, NormArgs a) {
       for (int u = 0; u < UN; ++u) {
         const uint32_t w = u0 + u * 32;
         if (w >= u_hi) continue;
-        const uint32_t ch = (w >= a.HW8) + (w >= 2 * a.HW8) + (w >= 3 * a.HW8);
-        float fv[8];
-        if constexpr (AFF) {
-          const float A = a.aa[ch], Bc = a.ab[ch];
-#pragma unroll
-          for (int bb = 0; bb < 8; ++bb)
-            fv[bb] = __fmaf_rn(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), A, Bc);
-        } else {
-          const float mc = a.mean[ch], s1 = a.s1[ch], s2 = a.s2[ch];
-#pragma unroll
-          for (int bb = 0; bb < 8; ++bb) {
-            const float x = unit_f32(byte_f(bb < 4 ? v[u].x : v[u].y, bb & 3), c.r1, c.r2);
-            const float tt = __fsub_rn(x, mc);
-            fv[bb] = a.fast ? __fmaf_rn(tt, s1, __fmul_rn(tt, s2)) : __fdiv_rn(tt, a.sd[ch]);
-          }
-        }
-        uint4 o;
-        o.x = pack_bf16x2(fv[0], fv[1]);
-        o.y = pack_bf16x2(fv[2], fv[3]);
-        o.z = pack_bf16x2(fv[4], fv[5]);
-        o.w = pack_bf16x2(fv[6], fv[7]);
+        uint4 o = norm_unit<AFF>(c, a, v[u], w);
         if (!ok) o = make_uint4(0u, 0u, 0u, 0u);
         st_stream(dst + w, o, pol);
       }
