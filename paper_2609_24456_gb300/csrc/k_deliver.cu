@@ -931,13 +931,15 @@ cudaError_t launch_deliver(edp_ctx *ctx, const int64_t *idx, uint32_t B,
     const bool few = units <= 3ull * kWarps * 32 * 4 * sms;
     a.span = 32 * (few ? 4 : 8);
     uint64_t ctas = (units + (uint64_t)kWarps * a.span - 1) / ((uint64_t)kWarps * a.span);
-    // With successors and more than two and a half waves, four CTAs per SM
-    // instead of five, held there by shared memory that they don't use: as fast
-    // alone (84x84, 4 frames, 512: 22.7 us, 22.9), and the small kernels of other
-    // streams find room among its waves (sampling and update beside it: a round
-    // 22.6 us, 24.4).  Without successors four are 12% slower (8,192: 195 us,
-    // 171), between one wave and two up to 15%.
-    const bool four = a.next && 2 * (ctas + a.ncollate) >= 5ull * kStackMinBlocks * sms;
+    // Stacks of three frames or more with successors, from 2.8 waves on: four CTAs
+    // per SM instead of five, held there by shared memory that they don't use: as
+    // fast alone (84x84, 4 frames, 512: 22.7 us, 22.9; 3 frames, 2.7 waves: 19.1, 18.7),
+    // and the small kernels of other streams find room among its waves (sampling
+    // and update beside it: a round 22.6 us, 24.4).  Fewer stores per load need the
+    // fifth: 84x84, 1 frame and successor, 4,096: 51.8 us, 45.7; 2 frames, 768: 18.6,
+    // 16.6; without successors 8,192: 195, 171.
+    const bool four =
+        a.next && a.K >= 3 && 5 * (ctas + a.ncollate) >= 14ull * kStackMinBlocks * sms;
     // On another stream than the context's sampling and updates, two iterations
     // per warp up to 16 waves: in half the waves those kernels, on which the next
     // delivery waits, get through sooner.  That round 21.6 us instead of 22.6 for
