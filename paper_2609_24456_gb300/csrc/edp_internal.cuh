@@ -274,9 +274,6 @@ __device__ __forceinline__ df df_split(double x) {
   const float hi = (float)x;
   return {hi, (float)(x - (double)hi)};
 }
-__device__ __forceinline__ double df_to_d(df a) {
-  return (double)a.hi + (double)a.lo;
-}
 
 // Importance weight (q_min / q_k)^beta in fp64, one rounding to fp32 (PER:
 // (N P(i))^-beta over its batch maximum, in which N and the total cancel).

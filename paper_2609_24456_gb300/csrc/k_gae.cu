@@ -18,25 +18,23 @@
 // SMs and longer chunks share the steps (gae_shape).
 //
 // Arithmetic: GB300's fp64 pipe is narrow (a dependent fp64 FMA costs ~64
-// cycles, fp32 ~4), so the scan -- and a thread's sums of A and A^2 over its
-// steps of a chunk -- run in double-float arithmetic -- a value
+// cycles, fp32 ~4), so the scan runs in double-float arithmetic -- a value
 // is an unevaluated pair hi + lo of fp32 numbers, combined with the
 // error-free transformations TwoSum (Knuth) and TwoProd via FMA (Dekker),
 // as in the double-double arithmetic of Hida, Li and Bailey -- which keeps
 // ~44 significant bits (relative error ~2^-44 per operation); gamma and
-// gamma*lambda enter as pairs split from fp64.  The sums over chunks, threads
-// and warps carry three words and round once per CTA, to fp64 (in double-float
-// the variance lost up to a digit against fp64: 24 rollouts of 2,048 steps,
-// mean 1e5 deviations, 1.3e-5 off; 3.9e-6 so).  The mean and the variance
-// are formed in fp64 from the CTAs' sums; the normalisation of an element takes
-// the mean in three fp32 words and the scale in two (norm_value), fp64 where a
-// value is out of their range.
+// gamma*lambda enter as pairs split from fp64.  The sums of A and A^2 carry three
+// words and round once per CTA, to fp64 (in double-float the variance lost up to
+// a digit against fp64: 24 rollouts of 2,048 steps, mean 1e5 deviations, 1.3e-5
+// off, 7.8e-7 so).  The mean and the variance are formed in fp64 from the CTAs'
+// sums; the normalisation of an element takes the mean in three fp32 words and
+// the scale in two (norm_value), fp64 where a value is out of their range.
 // Outputs are rounded to fp32.
 //
 // Bound by latency (a chunk's loads, then its dependent chain) up to ~10^6
 // values, then by HBM.  Calls in a row with all three outputs, in us, and
 // (before) with one warp per environment: 8 x 2,048 steps 10.3 (43.0), 4,096 x
-// 64 12.3 (28.4), 1,024 x 1,024 24.8 (107), 64 x 8,192 37.9 (557), 8 x 128 6.8
+// 64 12.3 (28.4), 1,024 x 1,024 24.6 (107), 64 x 8,192 37.9 (557), 8 x 128 6.8
 // (9.2), 8 x 512 7.0 (16.0).
 //
 // Two kernels chained with programmatic dependent launch: the scan writes A,
@@ -67,23 +65,34 @@ __device__ __forceinline__ df df_shfl_down(df a, int o) {
   return {__shfl_down_sync(kFull, a.hi, o), __shfl_down_sync(kFull, a.lo, o)};
 }
 
-// A sum of three fp32 numbers, for the sums over a CTA's threads, which were
-// fp64: each addition keeps about 70 significant bits (the errors of two_sum are
-// carried in full, only the third words' sum rounds), so the total rounds
-// once, to fp64.  fp64 itself would take 16 instructions a warp of the narrow
-// pipe, about 64 cycles each.  (A and A^2 share a tree, half a warp each, so this
-// takes no longer than two trees in double-float: 8 x 2,048 10.7 us both, 1 x
-// 262,144 83.2 then, 60.7 now, 1,024 x 1,024 24.2 and 24.8.)
+// A sum of three fp32 numbers, for the sums over a CTA's values: each addition
+// keeps about 70 significant bits (the errors of two_sum are carried in full, only
+// the third words' sum rounds), so the total rounds once, to fp64.  fp64 itself
+// would take 16 instructions a warp of the narrow pipe, about 64 cycles each.  In
+// us, environments x steps, and with sums and trees in double-float: 262,144 x 1
+// 60.4 (83.3: A and A^2 share a tree, half a warp each), 8 x 2,048 10.3 (10.7),
+// 1,024 x 1,024 24.6 (24.3); long rollouts in many CTAs pay for the third word,
+// most at 977 x 2,048 41.9 (40.9).
 struct tf {
   float a, b, c;
 };
+__device__ __forceinline__ tf tf_norm(tf x) {
+  const df p = two_sum(x.a, x.b);
+  const df q = two_sum(p.lo, x.c);
+  return {p.hi, q.hi, q.lo};
+}
 __device__ __forceinline__ tf tf_add(tf x, tf y) {
   const df s = two_sum(x.a, y.a), t = two_sum(x.b, y.b);
   const df m = two_sum(s.lo, t.hi);
-  const float c = __fadd_rn(__fadd_rn(x.c, y.c), __fadd_rn(t.lo, m.lo));
-  const df p = two_sum(s.hi, m.hi);
-  const df q = two_sum(p.lo, c);
-  return {p.hi, q.hi, q.lo};
+  return tf_norm({s.hi, m.hi, __fadd_rn(__fadd_rn(x.c, y.c), __fadd_rn(t.lo, m.lo))});
+}
+// x + y for a running sum, in the operations of a double-float addition: the
+// words overlap by the logarithm of the number of values, which tf_norm takes up
+// before it counts.
+__device__ __forceinline__ tf tf_acc(tf x, df y) {
+  const df s = two_sum(x.a, y.hi), t = two_sum(x.b, y.lo);
+  const df m = two_sum(s.lo, t.hi);
+  return {s.hi, m.hi, __fadd_rn(x.c, __fadd_rn(t.lo, m.lo))};
 }
 __device__ __forceinline__ tf tf_shfl_down16(tf x, int o) {  // within half a warp
   return {__shfl_down_sync(kFull, x.a, o, 16), __shfl_down_sync(kFull, x.b, o, 16),
@@ -233,10 +242,7 @@ k_gae_scan(const float *r, const float *v, const uint8_t *d, uint32_t T, uint32_
   const df one = {1.f, 0.f}, zero = {0.f, 0.f};
   const df g = {g2.x, g2.y}, gl = {gl2.x, gl2.y};  // gamma, gamma lambda
   pdl_wait();
-  // this thread's A and A^2: a chunk's in double-float (the fp32 pipe), the
-  // chunks' in three words
-  df a1 = zero, a2 = zero;
-  tf t1 = {0.f, 0.f, 0.f}, t2 = t1;
+  tf t1 = {0.f, 0.f, 0.f}, t2 = t1;  // this thread's sums of A and A^2
   for (uint32_t tile = blockIdx.x; (uint64_t)tile * kE < E; tile += gridDim.x) {
     const bool real = tile * kE + el < E;
     const uint32_t e = real ? tile * kE + el : E - 1;
@@ -249,6 +255,8 @@ k_gae_scan(const float *r, const float *v, const uint8_t *d, uint32_t T, uint32_
       const uint32_t te2 = ts, ts2 = ts > chunk ? ts - chunk : 0;
       GaeIn next;
       if (te2) gae_load<kStaged>(next, r, v, d, ts2, te2, seg, segs, E, e);
+      t1 = tf_norm(t1);  // while the loads are under way
+      t2 = tf_norm(t2);
       if constexpr (kStaged) gae_exchange<kE>(x, stage, seg, segs, el);
       df del[kL], cc[kL];
       df a = one, b = zero;  // this thread's steps composed: x -> b + a x
@@ -295,17 +303,15 @@ k_gae_scan(const float *r, const float *v, const uint8_t *d, uint32_t T, uint32_
             const uint64_t at = (t0 + i) * E + e;
             if (A_out) A_out[at] = A.hi;
             if (ret) ret[at] = df_add_f(A, x.v[i]).hi;
-            a1 = df_add(a1, A);
-            a2 = df_add(a2, df_mul(A, A));
+            t1 = tf_acc(t1, A);
+            const float sq = __fmul_rn(A.hi, A.hi);
+            t2 = tf_acc(t2, df{sq, __fmaf_rn(2.f * A.hi, A.lo, __fmaf_rn(A.hi, A.hi, -sq))});
           }
         }
       }
       __syncthreads();  // agg and s_carry have been read
       if (seg == 0) s_carry[el] = make_float2(A.hi, A.lo);
       if (!te2) break;
-      t1 = tf_add(t1, tf{a1.hi, a1.lo, 0.f});
-      t2 = tf_add(t2, tf{a2.hi, a2.lo, 0.f});
-      a1 = a2 = zero;
       x = next;
       te = te2;
       ts = ts2;
@@ -315,8 +321,6 @@ k_gae_scan(const float *r, const float *v, const uint8_t *d, uint32_t T, uint32_
   if (!partial && !adv_norm) return;  // no normalisation requested
   // this CTA's sums in a fixed order: a shuffle tree per warp, then over the
   // warps, the lower half of a warp for A and the upper for A^2
-  t1 = tf_add(t1, tf{a1.hi, a1.lo, 0.f});
-  t2 = tf_add(t2, tf{a2.hi, a2.lo, 0.f});
   const int half = lane >> 4, hl = lane & 15;
   tf t = tf_add(half ? t2 : t1, tf_shfl_xor16(half ? t1 : t2));
 #pragma unroll
