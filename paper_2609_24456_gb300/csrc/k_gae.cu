@@ -34,7 +34,7 @@
 // Bound by latency (a chunk's loads, then its dependent chain) up to ~10^6
 // values, then by HBM.  Calls in a row with all three outputs, in us, and
 // (before) with one warp per environment: 8 x 2,048 steps 10.3 (43.0), 4,096 x
-// 64 12.3 (28.4), 1,024 x 1,024 24.6 (107), 64 x 8,192 37.9 (557), 8 x 128 6.8
+// 64 11.9 (28.4), 1,024 x 1,024 24.6 (107), 64 x 8,192 36.9 (557), 8 x 128 6.8
 // (9.2), 8 x 512 7.0 (16.0).
 //
 // Two kernels chained with programmatic dependent launch: the scan writes A,
@@ -72,7 +72,7 @@ __device__ __forceinline__ df df_shfl_down(df a, int o) {
 // us, environments x steps, and with sums and trees in double-float: 262,144 x 1
 // 60.4 (83.3: A and A^2 share a tree, half a warp each), 8 x 2,048 10.3 (10.7),
 // 1,024 x 1,024 24.6 (24.3); long rollouts in many CTAs pay for the third word,
-// most at 977 x 2,048 41.9 (40.9).
+// most at 977 x 2,048 41.7 (40.9).
 struct tf {
   float a, b, c;
 };
@@ -255,8 +255,6 @@ k_gae_scan(const float *r, const float *v, const uint8_t *d, uint32_t T, uint32_
       const uint32_t te2 = ts, ts2 = ts > chunk ? ts - chunk : 0;
       GaeIn next;
       if (te2) gae_load<kStaged>(next, r, v, d, ts2, te2, seg, segs, E, e);
-      t1 = tf_norm(t1);  // while the loads are under way
-      t2 = tf_norm(t2);
       if constexpr (kStaged) gae_exchange<kE>(x, stage, seg, segs, el);
       df del[kL], cc[kL];
       df a = one, b = zero;  // this thread's steps composed: x -> b + a x
@@ -312,6 +310,11 @@ k_gae_scan(const float *r, const float *v, const uint8_t *d, uint32_t T, uint32_
       __syncthreads();  // agg and s_carry have been read
       if (seg == 0) s_carry[el] = make_float2(A.hi, A.lo);
       if (!te2) break;
+      // kL values since the last; ahead of the exchange above instead, under the
+      // loads, it delayed a rollout of one chunk: an iteration of 256 x 128 with its
+      // delivery 190.4 us, 188.7 so
+      t1 = tf_norm(t1);
+      t2 = tf_norm(t2);
       x = next;
       te = te2;
       ts = ts2;
